@@ -38,7 +38,8 @@ DAMPING = 0.85
 WL = synth.PAGERANK_RMAT22
 PROFILE = os.path.join(REPO, "profiles", "superstep_pagerank_rmat22.txt")
 PROFILE_CC = os.path.join(REPO, "profiles", "superstep_cc_er24_8parts.txt")
-KERNEL_SRC = os.path.join(REPO, "paper_2203_13005_gb300", "csrc", "sell.cu")
+KERNEL_SRC = os.path.join(REPO, "paper_2203_13005_gb300", "csrc", "sweep.cu")     # one partition
+KERNEL_SRC_CC = os.path.join(REPO, "paper_2203_13005_gb300", "csrc", "sell.cu")   # several
 
 
 def algorithmic_bytes(n_vertices: int, n_edges: int) -> int:
@@ -63,7 +64,7 @@ def measured_peaks() -> dict:
     return {"hbm_gbs": 6800.0, "source": "fallback"}
 
 
-def profiled_traffic(profile=None):
+def profiled_traffic(profile=None, kernel_src=None):
     """Per-launch DRAM bytes from a committed ncu summary (the PageRank one by
     default), if it was taken on the current kernel source (its sha256 is
     recorded there); else None."""
@@ -75,7 +76,7 @@ def profiled_traffic(profile=None):
         if ":" in ln and not ln.startswith("#"):
             k, v = ln.split(":", 1)
             kv[k.strip()] = v.strip()
-    sha = hashlib.sha256(open(KERNEL_SRC, "rb").read()).hexdigest()
+    sha = hashlib.sha256(open(kernel_src or KERNEL_SRC, "rb").read()).hexdigest()
     if kv.get("kernel_source_sha256") != sha or "dram_bytes_per_launch" not in kv:
         return None
     return float(kv["dram_bytes_per_launch"])
@@ -370,10 +371,8 @@ def run_sssp(args):
         "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": "u32", "data": "synthetic",
         "config": {"workload": wl.name, "vertices": n, "edges": m, "source": 0, "supersteps": steps,
-                   "step": ("one gxp_run to convergence: " + (
-                       f"{st['persistent_launches']} persistent cooperative launch(es), grid barrier between "
-                       "supersteps" if st["persistent_launches"] else
-                       "a CUDA graph whose WHILE node repeats superstep + control")),
+                   "step": (f"one gxp_run to convergence: {st['persistent_launches']} persistent cooperative "
+                            "launch(es), grid barrier between supersteps"),
                    "value": "supersteps x edges / run time (the Jacobi sweeps the run stands for)",
                    "l2": (f"{bytes_sweep / 1e6:.0f} MB working set: "
                           + ("L2-resident" if bytes_sweep < 129e6 else "larger than L2")),
@@ -384,13 +383,13 @@ def run_sssp(args):
                    "graph500_gteps": m / (ms * 1e-3) / 1e9},
         "roofline": {"bound": "hbm", "achieved": bytes_sweep / (k_us * 1e-6) / 1e9, "peak": peaks["hbm_gbs"],
                      "unit": "GB/s", "frac": bytes_sweep / (k_us * 1e-6) / 1e9 / peaks["hbm_gbs"], "traffic": None,
-                     "peak_source": peaks["source"], "kernel": "k_sell<SSSP>", "avg_launch_us": k_us,
+                     "peak_source": peaks["source"], "kernel": "k_sweep<SSSP>", "avg_launch_us": k_us,
                      "algorithmic_bytes_per_launch": bytes_sweep},
         "e2e": {"value": steps * m / e2e_s / 1e9, "unit": "GTEPS", "h2d_bytes_per_step": 8 * (n + 1) + 8 * m,
                 "d2h_bytes_per_step": 4 * n, "ms_per_step": e2e_s * 1e3},
         # per run: initial values, identity slot and frontier seed, then the
-        # persistent loop's launches or the graph's superstep + control kernels
-        "gpu_launches": reps * (3 + (st["persistent_launches"] or 2 * steps)),
+        # persistent kernel's launches
+        "gpu_launches": reps * (3 + st["persistent_launches"]),
         "clocks": clk.summary(),
     }
     line.update(cpu)
@@ -534,7 +533,7 @@ def run_cc(args):
         "superstep_with_sync_us": [round(x * 1e3, 1) for x in s_ms],
         "roofline": {"bound": "hbm", "achieved": bytes_sweep / (k_us * 1e-6) / 1e9, "peak": peaks["hbm_gbs"],
                      "unit": "GB/s", "frac": bytes_sweep / (k_us * 1e-6) / 1e9 / peaks["hbm_gbs"],
-                     "traffic": profiled_traffic(PROFILE_CC) if args.cc_scale == 24 else None,
+                     "traffic": profiled_traffic(PROFILE_CC, KERNEL_SRC_CC) if args.cc_scale == 24 else None,
                      "peak_source": peaks["source"], "kernel": "k_sell<CC>",
                      "avg_launch_us": k_us, "algorithmic_bytes_per_launch": bytes_sweep,
                      "launches_averaged": f"the {n_sweep} pull supersteps (every edge read) "
@@ -1057,7 +1056,7 @@ def main():
                          "frac": achieved / peaks["hbm_gbs"], "traffic": traffic,
                          "peak_source": peaks["source"], "algorithmic_bytes_per_launch": bytes_launch,
                          "frac_with_old_rank_read": bytes_launch_old_rank / avg_kernel_s / 1e9 / peaks["hbm_gbs"],
-                         "kernel": "k_sell<PR>", "avg_launch_us": avg_kernel_s * 1e6},
+                         "kernel": "k_sweep<PR>", "avg_launch_us": avg_kernel_s * 1e6},
             "e2e": {"value": ITERS * m / e2e_s / 1e9, "unit": "GTEPS",
                     "h2d_bytes_per_step": 8 * (n + 1) + 4 * m, "d2h_bytes_per_step": 4 * n,
                     "ms_per_step": e2e_s * 1e3},

@@ -71,9 +71,12 @@ typedef enum gxp_status {
  *               statistics finds its delivery mark missing: GXP_E_LOST, and
  *               the context is poisoned.
  *  - TIMEOUT:   every bounded device-side wait gives up at once (it then
- *               waits for its own copies in flight): GXP_E_TIMEOUT. Only the
- *               kernel of gxp_superstep_min_noalloc waits on the device, and
- *               it reads the GXP_FAULT variable ("timeout") on every call. */
+ *               waits for its own copies in flight): GXP_E_TIMEOUT. Waits
+ *               on the device: the grid barriers of the persistent kernels
+ *               (gxp_run of SSSP, CC and PageRank on one partition, resident
+ *               gxp_sssp_batch) and the bulk copies of
+ *               gxp_superstep_min_noalloc, which reads the GXP_FAULT
+ *               variable ("timeout") on every call. */
 typedef enum gxp_fault {
     GXP_FAULT_NONE = 0,
     GXP_FAULT_ALLOC = 1,
@@ -207,8 +210,8 @@ typedef struct gxp_stats {
     double   last_kernel_ms;        /* device time of the last superstep's compute kernel alone
                                        (MSGGen + MSGMerge + MSGApply, without its sync); gxp_run's
                                        device-driven loop: the average superstep */
-    uint64_t persistent_launches;   /* gxp_run launches of the persistent superstep loop since
-                                       gxp_begin (small single-partition SSSP / CC graphs: one
+    uint64_t persistent_launches;   /* gxp_run launches of the persistent superstep kernel since
+                                       gxp_begin (single-partition SSSP, CC and PageRank: one
                                        cooperative kernel runs up to 32 supersteps) */
     uint64_t reserved[2];
 } gxp_stats;
@@ -323,11 +326,12 @@ GXP_API gxp_status gxp_cache_get(gxp_ctx* ctx, uint32_t part, uint32_t* ids, uin
  * vertex (SSSP, CC, LP) or max_steps of them (always max_steps for
  * PageRank; LP need not settle: the paper caps it at 15). Starts with
  * gxp_begin(algo, source, damping). *steps_done (nullable) counts supersteps
- * run, including the final one that changed nothing. SSSP and CC on one
- * partition run the loop on the device (a CUDA graph whose conditional
- * node repeats superstep + stop test, up to 32 supersteps per launch, one
- * host synchronization per launch); the others enqueue supersteps in
- * chunks and read their changed counts once per chunk. */
+ * run, including the final one that changed nothing. SSSP, CC and PageRank on
+ * one partition run the loop on the device (a persistent cooperative kernel,
+ * up to 32 supersteps and one host synchronization per launch; with a
+ * timeout_ns below the default a launch per superstep, which waits for
+ * nothing); the others enqueue supersteps in chunks and read their changed
+ * counts once per chunk. */
 GXP_API gxp_status gxp_run(gxp_ctx* ctx, gxp_algo algo, uint32_t source, float damping,
                            uint32_t max_steps, uint32_t* steps_done);
 

@@ -24,6 +24,7 @@ void cuda_check(cudaError_t e, const char* what) {
 
 namespace {
 
+constexpr uint64_t kDefaultTimeoutNs = 2000000000ull;
 constexpr uint32_t kDefaultTile = 2048;   // edges per hub part; rows above tile/2 in-edges are hubs
 
 inline size_t pad4(size_t n) { return ((n + 3) & ~size_t(3)) + 4; }
@@ -48,7 +49,7 @@ Engine::Engine(int device, const gxp_config* cfg) : device_(device) {
     auto_tiles_ = cfg_.tile_items == 0 && cfg_.hub_items == 0;
     if (cfg_.tile_items == 0) cfg_.tile_items = kDefaultTile;
     if (cfg_.hub_items == 0) cfg_.hub_items = cfg_.tile_items / 2;
-    if (cfg_.timeout_ns == 0) cfg_.timeout_ns = 2000000000ull;
+    if (cfg_.timeout_ns == 0) cfg_.timeout_ns = kDefaultTimeoutNs;
     if (cfg_.max_slots == 0) cfg_.max_slots = 64;
     if (cfg_.pipeline_depth == 0) cfg_.pipeline_depth = 3;
     if (cfg_.push_div == 0) cfg_.push_div = 8;
@@ -60,6 +61,9 @@ Engine::Engine(int device, const gxp_config* cfg) : device_(device) {
     cuda_check(cudaGetDeviceCount(&n_dev), "cudaGetDeviceCount");
     if (device < 0 || device >= n_dev) fail(GXP_E_INVAL, "no such CUDA device");
     cuda_check(cudaSetDevice(device), "cudaSetDevice");
+    int sms = 0;
+    cuda_check(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device), "multiprocessors");
+    sms_ = (uint32_t)sms;
     cuda_check(cudaStreamCreateWithFlags(&own_stream_, cudaStreamNonBlocking), "cudaStreamCreate");
     stream_ = own_stream_;
     cudaMemPoolProps props{};
@@ -82,8 +86,7 @@ Engine::~Engine() {
     if (ev_a_) cudaEventDestroy(ev_a_);
     if (ev_b_) cudaEventDestroy(ev_b_);
     if (ev_k_) cudaEventDestroy(ev_k_);
-    if (h_ctl_) cudaFreeHost(h_ctl_);
-    if (h_ring_) cudaFreeHost(h_ring_);
+    if (h_run_) cudaFreeHost(h_run_);
     if (stream_) cudaStreamSynchronize(stream_);   // the frees above
     if (pool_) cudaMemPoolDestroy(pool_);
     if (own_stream_) cudaStreamDestroy(own_stream_);
@@ -135,12 +138,8 @@ void* Engine::dalloc(size_t bytes) {
 void Engine::free_graph_device() {
     if (stream_) cudaStreamSynchronize(stream_);
     free_batch();   // graphs and pinned buffers that refer to the device buffers below
-    for (auto& g : run_graph_) {
-        if (g) cudaGraphExecDestroy(g);
-        g = nullptr;
-    }
-    d_ctl_ = nullptr;
     d_bar_ = nullptr;
+    bar_passed_ = 0;
     h_old2new_.clear();
     lp_ = LpLists{};
     lru_ = Lru{};
@@ -152,8 +151,9 @@ void Engine::free_graph_device() {
     d_parts_ = nullptr;
     d_slices_ = nullptr;
     d_hubs_ = nullptr;
-    n_slices_ = n_hubs_ = n_zero_slices_ = 0;
-    d_hub_val_ = d_hub_arrive_ = nullptr;
+    n_slices_ = n_hubs_ = 0;
+    d_hub_val_ = nullptr;
+    d_hub_arrive_ = nullptr;
     d_outdeg_ = nullptr;
     d_own_[0] = d_own_[1] = nullptr;
     d_rank_[0] = d_rank_[1] = nullptr;
@@ -173,6 +173,7 @@ void Engine::free_graph_device() {
     out_ready_ = frontier_ = false;
     d_out_ptr_ = d_out_dst_ = d_out_w_ = nullptr;
     d_list_[0] = d_list_[1] = nullptr;
+    d_bits_[0] = d_bits_[1] = d_bits_[2] = nullptr;
     finalized_ = false;
     sell_ready_ = false;
     begun_ = false;
@@ -453,7 +454,15 @@ void Engine::build_sell() {
         while (p2 * 2 <= h) p2 *= 2;
         H = (uint32_t)std::min<uint64_t>(1024, p2);
         T = std::min<uint32_t>(2048, std::max<uint32_t>(256, 2 * H));
+        if (n_parts_ == 1) {   // rows of up to 512 in-edges are spread over lanes: 16 columns at most
+            H = 512;
+            T = std::max<uint32_t>(512, T);
+        }
     }
+    // One partition: columns a lane gathers per work item (sweep_lanes). 16
+    // fill a batch; a small graph takes fewer, so that its items still cover
+    // the chip's ~4,900 resident warps.
+    sweep_cols_ = n_parts_ > 1 ? 0u : total_edges_ >= (1ull << 23) ? 16u : total_edges_ >= (1ull << 21) ? 8u : 4u;
     std::vector<void*> tmp;   // freed when the build ends
     auto talloc = [&](size_t bytes) {
         void* q = nullptr;
@@ -522,7 +531,7 @@ void Engine::build_sell() {
         uint32_t* width = (uint32_t*)talloc(4 * ns + 4);
         uint64_t* off = (uint64_t*)talloc(8 * ns + 8);
         cuda_check(launch_sell_slices(col_ptr, n, rows_out, counts, d_bases, perm, width, off, (uint32_t)ns,
-                                      n_parts_ == 1, stream_), "slices");
+                                      sweep_cols_, stream_), "slices");
         uint64_t sell_size = 0;
         d2h(&sell_size, off + ns, 8);
         // 4. fill
@@ -531,7 +540,7 @@ void Engine::build_sell() {
         part_desc[p] = (SellSlice*)talloc(sizeof(SellSlice) * (ns + 1));
         part_ns[p] = (uint32_t)ns;
         cuda_check(launch_sell_fill(col_ptr, ssrc, sw, perm, width, off, (uint32_t)ns, p, pd_[p].pad_id,
-                                    n_parts_ == 1, sell_src, sell_w, part_desc[p], stream_), "fill slices");
+                                    sweep_cols_, sell_src, sell_w, part_desc[p], stream_), "fill slices");
         // 5. hub rows -> parts of T edges
         uint32_t* hub_list = (uint32_t*)talloc(4 * nh_rows + 4);
         uint32_t* part_off = (uint32_t*)talloc(4 * nh_rows + 4);
@@ -575,16 +584,22 @@ void Engine::build_sell() {
     d_slices_ = (SellSlice*)dalloc(sizeof(SellSlice) * std::max<size_t>(total_slices, 1));
     uint32_t* order_scratch = (uint32_t*)talloc(order_slices_scratch_bytes(n_slices_));
     at = 0;
-    n_zero_slices_ = 0;
     for (uint32_t p = 0; p < n_parts_; ++p) {
         if (part_ns[p])
             cuda_check(launch_order_slices(all + at, part_ns[p], d_slices_ + at, order_scratch, stream_),
                        "order slices");
+        if (n_parts_ == 1) {
+            n_gt8_ = n_gt4_ = n_gt0_ = 0;
+            std::fill(n_lanes_, n_lanes_ + 5, 0u);
+        }
         if (n_parts_ == 1 && part_ns[p]) {
-            // width 0 sorts last: the order's first offset of that bin counts the other slices
-            uint32_t nonzero = 0;
-            d2h(&nonzero, order_scratch, 4);
-            if (nonzero <= part_ns[p]) n_zero_slices_ = part_ns[p] - nonzero;
+            // how many slices each kind of work item takes (sweep.cu)
+            std::vector<uint32_t> wider(16 * sweep_cols_ + 1);
+            d2h(wider.data(), order_slices_starts(order_scratch, part_ns[p]), 4 * wider.size());
+            for (int j = 0; j < 5; ++j) n_lanes_[j] = wider[sweep_cols_ << (4 - j)];
+            n_gt8_ = std::max(wider[8], n_lanes_[4]);
+            n_gt4_ = std::max(wider[4], n_lanes_[4]);
+            n_gt0_ = wider[0];
         }
         at += part_ns[p];
     }
@@ -597,7 +612,8 @@ void Engine::build_sell() {
                                        cudaMemcpyDeviceToDevice, stream_), "gather hub parts");
         at += part_nh[p];
     }
-    d_hub_val_ = (uint32_t*)dalloc(4 * nh1);
+    d_hub_val_ = (unsigned long long*)dalloc(8 * nh1);
+    cuda_check(cudaMemsetAsync(d_hub_val_, 0, 8 * nh1, stream_), "memset");
     d_hub_arrive_ = (uint32_t*)dalloc(4 * nh1);
     cuda_check(cudaMemsetAsync(d_hub_arrive_, 0, 4 * nh1, stream_), "memset");
     cuda_check(cudaStreamSynchronize(stream_), "sell build");
@@ -846,13 +862,20 @@ void Engine::begin(gxp_algo algo, uint32_t source, float damping) {
         // rows without in-edges are never written: both buffers hold their labels
         cuda_check(cudaMemcpyAsync(d_own_[1], d_own_[0], 4ull * V, cudaMemcpyDeviceToDevice, stream_), "copy values");
     }
+    // both value buffers of the min-label algorithms start equal: a push
+    // superstep lowers the next buffer in place, which must hold values no
+    // lower than the current, and a single partition's pull supersteps leave
+    // rows without in-edges alone
+    if (a == Algo::SSSP || a == Algo::CC)
+        cuda_check(cudaMemcpyAsync(d_own_[1], d_own_[0], 4ull * V, cudaMemcpyDeviceToDevice, stream_), "copy values");
     frontier_ = (a == Algo::SSSP || a == Algo::CC) && cfg_.direction != GXP_DIR_PULL &&
                 (uint64_t)V + n_ghost_total_ + (total_edges_ + kItemEdges - 1) / kItemEdges < (1ull << 32);
     if (frontier_) {
         build_out_edges();
-        // both value buffers start equal: the push superstep lowers the next
-        // buffer in place, which must hold values no lower than the current
-        cuda_check(cudaMemcpyAsync(d_own_[1], d_own_[0], 4ull * V, cudaMemcpyDeviceToDevice, stream_), "copy values");
+        if (d_bits_[0]) {
+            const size_t bytes = 4 * (((size_t)V + 31) / 32);
+            for (uint32_t* b : d_bits_) cuda_check(cudaMemsetAsync(b, 0, bytes, stream_), "memset");
+        }
         cur_ = 0;
         step_ = 0;
         seed_frontier(a == Algo::SSSP ? src_int : kInf);   // CC: every label is new
@@ -888,8 +911,8 @@ SellArgs Engine::sell_args() const {
     a.step = step_;
     a.ghost = d_ghost_;
     a.outdeg = d_outdeg_;
-    a.changed_bits = n_parts_ > 1 ? d_changed_ : nullptr;
-    a.hub_val = d_hub_val_;
+    a.changed_bits = d_changed_;
+    a.hub_val = reinterpret_cast<uint32_t*>(d_hub_val_);
     a.hub_arrive = d_hub_arrive_;
     a.err = d_err_;
     a.check_bounds = cfg_.check_bounds;
@@ -897,23 +920,71 @@ SellArgs Engine::sell_args() const {
     a.inv_n = (float)(1.0 / (double)n_vertices_);
     a.ppr_source = ppr_source_;
     a.early_exit = (early_exit_ && algo_ != Algo::PR) ? 1u : 0u;
-    a.n_zero = (algo_ == Algo::PR && n_parts_ == 1) ? n_zero_slices_ : 0u;
     if (frontier_) {   // the kernel picks the direction on the device from the frontier's size
-        a.fc.list_out = d_list_[1];   // non-null: lists on
-        a.fc.direction = cfg_.direction;
-        a.fc.push_div = cfg_.push_div;
-        a.fc.total_edges = total_edges_;
-        a.fc.list_cap = list_cap_;
-        a.fc.err = d_err_;
-        // several partitions: a pull lists its changed vertices only when the
-        // frontier it read was within kListSlack times the push limit (in
-        // vertices, at the average degree); there the list's scattered
-        // out-degree loads cost every pull superstep ~13% (ER 2^24, 8 parts)
-        a.fc.list_max_changed = kAlwaysList;
-        if (n_parts_ > 1 && cfg_.direction == GXP_DIR_AUTO && n_vertices_ > 0) {
+        a.fc = frontier_cfg();
+        // a pull lists its changed vertices only when the frontier it read
+        // was within kListSlack times the push limit (in vertices, at the
+        // average degree); the list's scattered out-degree loads cost every
+        // pull superstep ~13% (ER 2^24, 8 parts)
+        if (cfg_.direction == GXP_DIR_AUTO && n_vertices_ > 0) {
             const double V = (double)n_vertices_, E = (double)total_edges_;
             a.fc.list_max_changed = (uint64_t)(kListSlack * E / ((double)cfg_.push_div * (1.0 + E / V)));
         }
+        a.out_ptr = d_out_ptr_;
+        a.out_dst = d_out_dst_;
+        a.out_w = algo_ == Algo::SSSP ? d_out_w_ : nullptr;
+    }
+    return a;
+}
+
+FrontierCfg Engine::frontier_cfg() const {
+    FrontierCfg f{};
+    f.list_out = d_list_[1];   // non-null: lists on
+    f.direction = cfg_.direction;
+    f.push_div = cfg_.push_div;
+    f.total_edges = total_edges_;
+    f.list_cap = list_cap_;
+    f.err = d_err_;
+    f.list_max_changed = kAlwaysList;
+    return f;
+}
+
+// The same for a single partition.
+SweepArgs Engine::sweep_args() const {
+    SweepArgs a{};
+    a.slices = d_slices_;
+    a.n_slices = n_slices_;
+    a.cols = sweep_cols_;
+    for (int j = 0; j < 5; ++j) a.n_lanes[j] = n_lanes_[j];
+    a.n_gt8 = n_gt8_;
+    a.n_gt4 = n_gt4_;
+    a.n_gt0 = n_gt0_;
+    a.hubs = d_hubs_;
+    a.n_hubs = n_hubs_;
+    a.sell_src = pd_[0].sell_src;
+    a.sell_w = pd_[0].sell_w;
+    a.perm = pd_[0].perm;
+    a.hsrc = pd_[0].hsrc;
+    a.hw = pd_[0].hw;
+    a.n_vertices = (uint32_t)n_vertices_;
+    a.n_hot = sweep_hot_values(n_vertices_, total_edges_, relabeled_);
+    for (int i = 0; i < 2; ++i) {
+        a.own[i] = d_own_[i];
+        a.rank[i] = d_rank_[i];
+        a.lists[i] = d_list_[i];
+    }
+    for (int i = 0; i < 3; ++i) a.bits[i] = d_bits_[i];
+    a.stats = d_stats_;
+    a.outdeg = d_outdeg_;
+    a.hub_val = d_hub_val_;
+    a.hub_arrive = d_hub_arrive_;
+    a.err = d_err_;
+    a.check_bounds = cfg_.check_bounds;
+    a.damping = damping_;
+    a.inv_n = (float)(1.0 / (double)n_vertices_);
+    a.ppr_source = ppr_source_;
+    if (frontier_) {
+        a.fc = frontier_cfg();
         a.out_ptr = d_out_ptr_;
         a.out_dst = d_out_dst_;
         a.out_w = algo_ == Algo::SSSP ? d_out_w_ : nullptr;
@@ -1024,6 +1095,10 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
         l.skip_if_quiet = (early_exit_ && step_ > 0) ? 1u : 0u;
         l.narrow_labels = n_vertices_ <= (1ull << 27) ? 1u : 0u;   // labels are vertex ids
         cuda_check(launch_lp_superstep(l, stream_), "label propagation superstep");
+    } else if (n_parts_ == 1) {
+        RunArgs one{};
+        one.t0 = step_;
+        cuda_check(launch_sweep(algo_, sweep_args(), one, sms_, stream_), "superstep kernel");
     } else {
         const SellArgs a = sell_args();
         cuda_check(launch_superstep_sell(algo_, a, stream_), "superstep kernel");
@@ -1087,20 +1162,28 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
     return st_.last_changed;
 }
 
-// Fold the device-side stats of the supersteps not yet read into st_.
+void Engine::account_step(const StepSum& s) {
+    st_.supersteps++;
+    st_.edges_scanned += s.pushed ? s.push_edges : total_edges_;
+    if (s.pushed) st_.push_supersteps++;
+    st_.last_changed = s.changed;
+    if (algo_ == Algo::PR) {
+        st_.last_dangling = fx_to_double(s.dangling_fx);
+        st_.last_l1_delta = fx_to_double(s.l1_fx);
+    }
+}
+
 // Fold the device-side stats of the supersteps not yet read into st_ (one
 // copy of the stat ring). With stop_at_quiet, stop at the first superstep
 // that changed nothing and roll the step counter back to it (the supersteps
 // enqueued after it ran on a fixed point and changed nothing either); its
 // index is returned, else 0.
-uint64_t Engine::account(bool stop_at_quiet, bool ring_copied) {
+uint64_t Engine::account(bool stop_at_quiet) {
     if (accounted_ == step_) return 0;
-    if (!ring_copied) {
-        cuda_check(cudaStreamSynchronize(stream_), "superstep");
-        ring_host_.resize(kStatRing);
-        cuda_check(cudaMemcpy(ring_host_.data(), d_stats_, sizeof(StepStats) * kStatRing, cudaMemcpyDeviceToHost),
-                   "read stats");
-    }
+    cuda_check(cudaStreamSynchronize(stream_), "superstep");
+    ring_host_.resize(kStatRing);
+    cuda_check(cudaMemcpy(ring_host_.data(), d_stats_, sizeof(StepStats) * kStatRing, cudaMemcpyDeviceToHost),
+               "read stats");
     check_device_error();
     uint64_t quiet = 0;
     for (uint64_t t = accounted_ + 1; t <= step_; ++t) {
@@ -1111,14 +1194,7 @@ uint64_t Engine::account(bool stop_at_quiet, bool ring_copied) {
             dg += s.dangling_fx[i];
             l1 += s.l1_fx[i];
         }
-        st_.supersteps++;
-        st_.edges_scanned += s.pushed ? s.push_edges : total_edges_;
-        if (s.pushed) st_.push_supersteps++;
-        st_.last_changed = ch;
-        if (algo_ == Algo::PR) {
-            st_.last_dangling = fx_to_double(dg);
-            st_.last_l1_delta = fx_to_double(l1);
-        }
+        account_step(StepSum{ch, dg, l1, s.pushed, s.push_edges});
         if (n_parts_ > 1) {
             // every exchange marks its superstep's slot; a missing mark means
             // the caches and upload lists of that superstep were never delivered
@@ -1171,6 +1247,8 @@ void Engine::build_out_edges() {
     d_out_w_ = weighted_ ? (uint32_t*)dalloc(4 * std::max<uint64_t>(E, 1)) : nullptr;
     list_cap_ = (uint64_t)S + (E + kItemEdges - 1) / kItemEdges;
     for (auto& l : d_list_) l = (uint2*)dalloc(sizeof(uint2) * std::max<uint64_t>(list_cap_, 1));
+    if (n_parts_ == 1)
+        for (auto& b : d_bits_) b = (uint32_t*)dalloc(4 * (((size_t)V + 31) / 32));
     std::vector<void*> tmp;
     auto talloc = [&](size_t bytes) -> void* {
         void* q = nullptr;
@@ -1347,56 +1425,6 @@ void Engine::sync_result(uint32_t part, uint32_t* ids, void* vals, uint64_t cap,
     cuda_check(cudaMemcpy(vals, d_gdq_vals_ + base, 4ull * n, cudaMemcpyDefault), "copy gdq values");
 }
 
-// The device-driven loop of the running min-label algorithm: a graph with
-// one WHILE node whose body is the superstep kernel (step read from d_ctl_)
-// followed by the control kernel that advances the step and sets the
-// condition. Built once per algorithm and graph; false if the driver cannot
-// build it (the run then drives the supersteps from the host).
-bool Engine::run_graph_ready() {
-    if (algo_ == Algo::PR || algo_ == Algo::LP || run_graph_failed_) return false;
-    cudaGraphExec_t& ge = run_graph_[algo_ == Algo::SSSP ? 0 : 1];
-    if (ge) return true;
-    if (!h_ctl_) cuda_check(cudaMallocHost(&h_ctl_, 2 * sizeof(RunCtl)), "pinned run control");
-    if (!h_ring_) cuda_check(cudaMallocHost(&h_ring_, sizeof(StepStats) * kStatRing), "pinned stats");
-    if (!d_ctl_) d_ctl_ = (RunCtl*)dalloc(sizeof(RunCtl));
-    cudaStream_t cs = nullptr;
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaGraphCreate(&g, 0);
-    cudaGraphConditionalHandle h = 0;
-    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault);
-    cudaGraphNodeParams np{};
-    np.type = cudaGraphNodeTypeConditional;
-    np.conditional.handle = h;
-    np.conditional.type = cudaGraphCondTypeWhile;
-    np.conditional.size = 1;
-    cudaGraphNode_t node = nullptr;
-    if (e == cudaSuccess) e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &np);
-    if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(cs, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
-                                                            cudaStreamCaptureModeRelaxed);
-    if (e == cudaSuccess) {
-        SellArgs a = sell_args();
-        a.step_dev = &d_ctl_->step;
-        a.early_exit = 0u;   // the loop stops at the first quiet superstep
-        cudaError_t e1 = launch_superstep_sell(algo_, a, cs);
-        cudaError_t e2 = e1 == cudaSuccess ? launch_run_control(d_ctl_, d_stats_, h, cs) : e1;
-        cudaGraph_t body = nullptr;
-        e = cudaStreamEndCapture(cs, &body);
-        if (e == cudaSuccess) e = e2;
-    }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&ge, g, 0);
-    if (g) cudaGraphDestroy(g);
-    if (cs) cudaStreamDestroy(cs);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        if (ge) cudaGraphExecDestroy(ge);
-        ge = nullptr;
-        run_graph_failed_ = true;
-        return false;
-    }
-    return true;
-}
-
 uint32_t Engine::run(gxp_algo algo, uint32_t source, float damping, uint32_t max_steps) {
     TraceRange trace_("gxp run");
     begin(algo, source, damping);
@@ -1404,69 +1432,57 @@ uint32_t Engine::run(gxp_algo algo, uint32_t source, float damping, uint32_t max
     const gxp_merge m = algo_ == Algo::PR ? GXP_MERGE_SUM : algo_ == Algo::LP ? GXP_MERGE_MODE : GXP_MERGE_MIN;
     const gxp_apply ap = algo_ == Algo::PR ? GXP_APPLY_PAGERANK : algo_ == Algo::LP ? GXP_APPLY_SET : GXP_APPLY_MIN;
     uint32_t steps = 0;
+    // SSSP, CC and PageRank on one partition: at most kRunChunk supersteps per
+    // persistent cooperative launch (a grid barrier between supersteps) and
+    // one host read per launch. Its barriers are device waits: a context
+    // whose timeout_ns was set below the default takes a launch per superstep,
+    // which waits for nothing.
+    if (n_parts_ == 1 && algo_ != Algo::LP && cfg_.timeout_ns >= kDefaultTimeoutNs) {
+        const SweepArgs sa = sweep_args();
+        if (!h_run_) cuda_check(cudaHostAlloc(&h_run_, sizeof(RunOut), cudaHostAllocMapped), "pinned run report");
+        if (!d_bar_) {
+            d_bar_ = (GridBar*)dalloc(sizeof(GridBar));
+            cuda_check(cudaMemsetAsync(d_bar_, 0, sizeof(GridBar), stream_), "memset");
+            bar_passed_ = 0;
+        }
+        while (steps < max_steps) {
+            RunArgs r{};
+            r.t0 = step_;
+            r.limit = step_ + std::min<uint32_t>(kRunChunk, max_steps - steps);
+            r.quiet_stop = algo_ != Algo::PR ? 1u : 0u;
+            r.force = faults_.timeout ? 1u : 0u;
+            r.timeout_ns = cfg_.timeout_ns;
+            r.passed = bar_passed_;
+            r.bar = d_bar_;
+            r.out = h_run_;   // mapped: the same address on the device
+            h_run_->step = 0;
+            cuda_check(cudaEventRecord(ev_a_, stream_), "event");
+            cuda_check(launch_sweep(algo_, sa, r, sms_, stream_), "run");
+            ++st_.persistent_launches;
+            cuda_check(cudaEventRecord(ev_b_, stream_), "event");
+            cuda_check(cudaStreamSynchronize(stream_), "run");
+            const uint64_t done = h_run_->step;
+            if (done == 0 || h_run_->err != 0) check_device_error();   // a wait that ran out, a bad index
+            if (done <= r.t0 || done > r.limit) fail(GXP_E_CUDA, "device-driven run lost its step counter");
+            bar_passed_ = h_run_->passed;
+            const uint32_t n_run = (uint32_t)(done - r.t0);
+            for (uint32_t i = 0; i < n_run; ++i) account_step(h_run_->sum[i]);
+            steps += n_run;
+            step_ = accounted_ = done;
+            cur_ = (int)(step_ & 1u);
+            float ms = 0.f;
+            if (cudaEventElapsedTime(&ms, ev_a_, ev_b_) == cudaSuccess)
+                st_.last_superstep_ms = st_.last_kernel_ms = ms / (double)n_run;
+            if (r.quiet_stop && st_.last_changed == 0) return steps;
+        }
+        return steps;
+    }
     if (algo_ == Algo::PR) {
         for (; steps < max_steps; ++steps) superstep(algo, g, m, ap, false);
         account(false);
         return steps;
     }
-    // SSSP / CC on one partition: the loop runs on the device until the first
-    // superstep that changes nothing, at most kRunChunk supersteps per launch
-    // and one host read per launch. A graph whose superstep is a few waves of
-    // CTAs runs all of them in one persistent cooperative kernel (grid
-    // barrier between supersteps); larger ones through a CUDA graph whose
-    // WHILE node repeats superstep + control.
-    const bool one = n_parts_ == 1 && algo_ != Algo::LP;
-    SellArgs la{};
-    if (one) {
-        la = sell_args();
-        la.early_exit = 0u;   // the loop stops at the first quiet superstep
-    }
-    const bool loop = one && sell_loop_fits(algo_, la);
-    if (loop) {
-        if (!h_ctl_) cuda_check(cudaMallocHost(&h_ctl_, 2 * sizeof(RunCtl)), "pinned run control");
-        if (!h_ring_) cuda_check(cudaMallocHost(&h_ring_, sizeof(StepStats) * kStatRing), "pinned stats");
-        if (!d_ctl_) d_ctl_ = (RunCtl*)dalloc(sizeof(RunCtl));
-        if (!d_bar_) d_bar_ = (GridBar*)dalloc(sizeof(GridBar));
-    }
-    if (loop || (one && run_graph_ready())) {
-        const cudaGraphExec_t ge = loop ? nullptr : run_graph_[algo_ == Algo::SSSP ? 0 : 1];
-        while (steps < max_steps) {
-            const uint32_t k = std::min<uint32_t>(kRunChunk, max_steps - steps);
-            h_ctl_[0] = RunCtl{step_, step_ + k, 1u, 0u};
-            before_h2d("run control");
-            cuda_check(cudaMemcpyAsync(d_ctl_, h_ctl_, sizeof(RunCtl), cudaMemcpyHostToDevice, stream_), "run control");
-            if (loop) cuda_check(cudaMemsetAsync(d_bar_, 0, sizeof(GridBar), stream_), "memset");
-            cuda_check(cudaEventRecord(ev_a_, stream_), "event");
-            if (loop) {
-                cuda_check(launch_sell_loop(algo_, la, d_ctl_, d_bar_, cfg_.timeout_ns, faults_.timeout, stream_),
-                           "run loop");
-                ++st_.persistent_launches;
-            } else {
-                cuda_check(cudaGraphLaunch(ge, stream_), "run graph");
-            }
-            cuda_check(cudaEventRecord(ev_b_, stream_), "event");
-            cuda_check(cudaMemcpyAsync(h_ctl_ + 1, d_ctl_, sizeof(RunCtl), cudaMemcpyDeviceToHost, stream_),
-                       "run control");
-            cuda_check(cudaMemcpyAsync(h_ring_, d_stats_, sizeof(StepStats) * kStatRing, cudaMemcpyDeviceToHost,
-                                       stream_), "read stats");
-            cuda_check(cudaStreamSynchronize(stream_), "run");
-            if (loop) check_device_error();   // a grid barrier that ran out of time
-            ring_host_.assign(h_ring_, h_ring_ + kStatRing);
-            const uint64_t done = h_ctl_[1].step;
-            if (done <= step_ || done > step_ + k) fail(GXP_E_CUDA, "device-driven run lost its step counter");
-            steps += (uint32_t)(done - step_);
-            step_ = done;
-            cur_ = (int)(step_ & 1u);
-            const uint64_t n_run = done - accounted_;
-            const uint64_t quiet = account(true, true);
-            float ms = 0.f;
-            if (cudaEventElapsedTime(&ms, ev_a_, ev_b_) == cudaSuccess)
-                st_.last_superstep_ms = st_.last_kernel_ms = ms / (double)n_run;
-            if (quiet) return (uint32_t)quiet;
-        }
-        return steps;
-    }
-    // partitioned graphs: supersteps are enqueued in growing chunks and the
+    // the others: supersteps are enqueued in growing chunks and the
     // host reads their changed counts once per chunk; the run ends at the
     // first superstep that changed nothing (the count includes it) and the
     // ones after a quiet superstep return at once on the device
@@ -1530,14 +1546,10 @@ void Engine::set_values(uint32_t part, const void* in, uint64_t n) {
         cuda_check(cudaMemcpyAsync(d_own_[cur_] + off, in, 4 * cnt, cudaMemcpyDefault, stream_), "copy values");
     }
     cuda_check(launch_init_ghosts(algo_, n_ghost_total_, d_ghost_gid_, d_own_[cur_], d_ghost_, stream_), "refresh caches");
-    if (algo_ == Algo::LP)   // rows without in-edges are read from either buffer
-        cuda_check(cudaMemcpyAsync(d_own_[cur_ ^ 1], d_own_[cur_], 4ull * n_vertices_, cudaMemcpyDeviceToDevice,
-                                   stream_), "copy values");
-    if (frontier_) {   // any value may have moved: every vertex is in the next frontier
-        cuda_check(cudaMemcpyAsync(d_own_[cur_ ^ 1], d_own_[cur_], 4ull * n_vertices_, cudaMemcpyDeviceToDevice,
-                                   stream_), "copy values");
-        seed_frontier(kInf);
-    }
+    // both buffers start equal again (see begin): rows without in-edges are read from either
+    cuda_check(cudaMemcpyAsync(d_own_[cur_ ^ 1], d_own_[cur_], 4ull * n_vertices_, cudaMemcpyDeviceToDevice, stream_),
+               "copy values");
+    if (frontier_) seed_frontier(kInf);   // any value may have moved: every vertex is in the next frontier
     cuda_check(cudaStreamSynchronize(stream_), "set values");
 }
 

@@ -87,8 +87,8 @@ private:
     void build_sell();
     void build_caches();
     uint32_t* upload_u32(const std::vector<uint32_t>& h, size_t n_pad);
-    // ring_copied: ring_host_ already holds the device ring (stream synchronized)
-    uint64_t account(bool stop_at_quiet, bool ring_copied = false);
+    uint64_t account(bool stop_at_quiet);
+    void account_step(const StepSum& s);
     std::vector<StepStats> ring_host_;
     void check_device_error();
     void copy_in(void* dst, const void* src, size_t bytes);   // host or device src -> host dst
@@ -130,8 +130,12 @@ private:
     SellSlice* d_slices_ = nullptr;
     HubPart* d_hubs_ = nullptr;
     uint32_t n_slices_ = 0, n_hubs_ = 0;
-    uint32_t n_zero_slices_ = 0;   // one partition: trailing slices of rows without in-edges
-    uint32_t *d_hub_val_ = nullptr, *d_hub_arrive_ = nullptr;
+    // one partition: columns per lane its slices aim at, and how many slices
+    // are spread over at least 32, 16, 8, 4, 2 lanes, wider than 8, 4, 0 columns
+    uint32_t sweep_cols_ = 0, n_lanes_[5] = {}, n_gt8_ = 0, n_gt4_ = 0, n_gt0_ = 0;
+    uint32_t sms_ = 0;             // multiprocessors of the device
+    unsigned long long* d_hub_val_ = nullptr;   // one partition: tagged partials; several: u32 partials
+    uint32_t* d_hub_arrive_ = nullptr;
     uint32_t* d_outdeg_ = nullptr;
     uint32_t* d_own_[2] = {nullptr, nullptr};
     float* d_rank_[2] = {nullptr, nullptr};
@@ -222,17 +226,15 @@ private:
         uint32_t* d_counts = nullptr;
     } lp_;
     void build_lp();
-    // device-driven runs (min-label algorithms, one partition)
-    static constexpr uint32_t kRunChunk = 32;   // supersteps per graph launch (the stat ring holds 64)
-    cudaGraphExec_t run_graph_[2] = {nullptr, nullptr};   // SSSP, CC
-    bool run_graph_failed_ = false;
-    RunCtl* d_ctl_ = nullptr;
-    GridBar* d_bar_ = nullptr;     // the persistent run's grid barrier
-    RunCtl* h_ctl_ = nullptr;      // pinned: [0] to the device, [1] back
-    StepStats* h_ring_ = nullptr;  // pinned copy of the stat ring
+    // runs of several supersteps per launch (one partition)
+    uint32_t* d_bits_[3] = {nullptr, nullptr, nullptr};   // changed vertices of the pull supersteps (frontier lists)
+    GridBar* d_bar_ = nullptr;     // the run's grid barrier, zero when allocated
+    uint64_t bar_passed_ = 0;      // barriers passed on it
+    RunOut* h_run_ = nullptr;      // pinned: what a launch of a run reports
     std::vector<uint32_t> h_old2new_;   // host copy of the renumbering (source ids)
-    bool run_graph_ready();
     SellArgs sell_args() const;
+    SweepArgs sweep_args() const;
+    FrontierCfg frontier_cfg() const;
     bool early_exit_ = false;      // inside gxp_run: supersteps after a quiet one return at once
     bool auto_tiles_ = false;      // tile / hub sizes chosen from the graph's size
     float damping_ = 0.85f;

@@ -54,28 +54,45 @@ constexpr uint32_t kTailOpen = 2u;
 
 // Sliced-ELL layout of the non-hub rows (SELL-32-sigma): rows are sorted by
 // in-degree inside windows of kSellWindow rows and grouped into slices of 32;
-// a slice stores its rows' in-edges column-major, for a single partition in
-// groups of 4 columns (edges 4g..4g+3 of row slot l at off + 128 g + 4 l, see
-// sell_idx), padded with the partition's padding id.
+// several partitions store a slice's in-edges column-major, a single
+// partition as lane groups (sweep_lanes), padded with the partition's
+// padding id.
 struct SellSlice {
-    uint32_t part;     // partition index
+    uint32_t part;     // partition index; one partition: rows of the slice if they are consecutive
+                       // vertices (first ..), else 0
     uint32_t row0;     // first entry of the slice in the partition's perm array
     uint32_t width;    // edges per row slot (the slice's largest in-degree)
-    uint32_t pad0;
+    uint32_t first;
     uint64_t off;      // first element of the slice in the partition's sell arrays
 };
 constexpr uint32_t kSellPad = 0xFFFFFFFFu;   // empty row slot of a slice (perm)
-// Element of column k, row slot l in a slice's storage. A single partition
-// stores its columns in groups of 4 (g4: a lane reads 4 of its row's sources
-// with one 128-bit load); several partitions column by column (measured
-// faster on their uniform graphs, whose widths the rounding would pad more).
-__host__ __device__ constexpr uint64_t sell_idx(uint32_t k, uint32_t l, bool g4) {
-    return g4 ? 128ull * (k >> 2) + 4ull * l + (k & 3u) : 32ull * k + l;
+// Storage of a slice. `cols` = 0 (several partitions): column by column,
+// element k of row slot r at 32 k + r. Else (one partition) a slice wider
+// than `cols` columns spreads each row over L lanes, L the smallest power of
+// two (at most 32) that brings its columns down to `cols`: the slice is L
+// sub-slices of 32 / L rows, edge k of a row in lane k % L of its lane group
+// and column k / L, and columns are stored in groups of 4, so that a lane
+// reads 4 of its sources with one 128-bit load.
+__host__ __device__ constexpr uint32_t sweep_lanes(uint32_t width, uint32_t cols) {
+    uint32_t l = 1;
+    while (l < 32u && width > cols * l) l *= 2;
+    return l;
 }
-// columns a slice stores: its width, rounded up to a whole group with g4
-__host__ __device__ constexpr uint32_t sell_cols(uint32_t width, bool g4) { return g4 ? (width + 3u) & ~3u : width; }
+// columns a sub-slice stores
+__host__ __device__ constexpr uint32_t sweep_cols(uint32_t width, uint32_t lanes) {
+    return ((width + lanes - 1) / lanes + 3u) & ~3u;
+}
+__host__ __device__ constexpr uint64_t sell_words(uint32_t width, uint32_t cols) {
+    if (!cols) return 32ull * width;
+    const uint32_t l = sweep_lanes(width, cols);
+    return 32ull * l * sweep_cols(width, l);
+}
+// element k of row slot r of a slice stored with L lanes per row, c columns per sub-slice
+__host__ __device__ constexpr uint64_t sweep_idx(uint32_t k, uint32_t r, uint32_t lanes, uint32_t c) {
+    const uint32_t rows = 32u / lanes, col = k / lanes, lane = (r % rows) * lanes + k % lanes;
+    return 32ull * c * (r / rows) + 128ull * (col >> 2) + 4ull * lane + (col & 3u);
+}
 constexpr uint32_t kSellWindow = 65536;      // rows sorted by degree within windows of this size
-constexpr uint32_t kZeroGroup = 4;           // slices of rows without in-edges per warp (PageRank)
 
 // A slice of the in-edges of one hub row (in-degree above the SELL limit),
 // reduced by one warp; the last part of a row to arrive combines all parts.
@@ -100,7 +117,7 @@ struct PartDev {
     uint32_t ghost_base;       // offset of this partition's ghosts in the ghost array
     uint64_t n_edges;
     // sliced-ELL layout (engine path)
-    const uint32_t* sell_src;  // column-major slices, pad_id in empty slots
+    const uint32_t* sell_src;  // slices (sell_words), pad_id in empty slots
     const uint32_t* sell_w;    // weights in the same layout, or nullptr
     const uint32_t* perm;      // slice row slot -> local vertex (kSellPad = empty)
     const uint32_t* hsrc;      // hub rows' in-edges, row after row
@@ -136,9 +153,12 @@ struct StepStats {
     // so a test each CTA of k_sync_pull made for itself would see a moving
     // count and the CTAs could disagree (some copies listed, others not).
     unsigned long long list_copies;
-    // 1: the superstep pulled without listing its changed vertices
-    // (FrontierCfg::list_max_changed), so the next one must pull too
+    // 1: the superstep pulled without listing its changed vertices: with
+    // several partitions (FrontierCfg::list_max_changed) the next one must
+    // pull too; one partition holds them in a bitmap (SweepArgs::bits), which
+    // the next superstep lists if it pushes, reserving list places here
     unsigned long long unlisted;
+    unsigned long long list_cursor;
 };
 __host__ __device__ constexpr unsigned long long list_pack(uint32_t items, uint32_t edges) {
     return ((unsigned long long)items << 32) | edges;
@@ -200,14 +220,14 @@ struct SuperstepArgs {
     uint32_t max_items;          // largest tile (merge items)
 };
 
-// Everything the sliced-ELL superstep kernel touches.
+// Everything the superstep kernel of a partitioned graph touches (sell.cu).
 struct SellArgs {
     const SellSlice* slices;
     uint32_t n_slices;
     const HubPart* hubs;
     uint32_t n_hubs;
     const PartDev* parts;
-    uint32_t n_parts;            // 1: the single-partition kernel (no cached copies, no bitmap)
+    uint32_t n_parts;
     uint32_t n_vertices;         // V: the first cached-copy slot of the push direction
     // superstep t reads value buffer t & 1, stat slot t % kStatRing and
     // frontier list t & 1; it writes buffer / list (t + 1) & 1 and slot t + 1,
@@ -215,9 +235,8 @@ struct SellArgs {
     uint32_t* own[2];
     float* rank[2];
     StepStats* stats;            // [kStatRing]
-    uint2* lists[2];             // frontier lists (min-label algorithms, one partition) or nullptr
-    uint64_t step;               // t, unless
-    const uint64_t* step_dev;    // t lives in device memory (device-driven runs)
+    uint2* lists[2];             // frontier lists (min-label algorithms) or nullptr
+    uint64_t step;               // t
     const uint32_t* ghost;
     const uint32_t* outdeg;
     uint32_t* changed_bits;
@@ -229,17 +248,45 @@ struct SellArgs {
     float inv_n;                 // 1 / N
     uint32_t ppr_source;         // PageRank: kInf; personalized PageRank: the source vertex
     uint32_t early_exit;         // 1: a superstep (t > 0) after a quiet one returns at once
-    // PageRank on one partition: the last n_zero slices (heavy-first order)
-    // hold rows without in-edges; a warp applies kZeroGroup of them at once
-    uint32_t n_zero;
     // SSSP / CC: fc.list_out != nullptr turns the frontier lists on (the
     // kernel points list_in / list_out at lists[]); the out-edge copy is
     // what the push direction reads. Its sources are slots: the V vertices,
-    // then (several partitions) the cached copies, slot V + g for copy g.
+    // then the cached copies, slot V + g for copy g.
     FrontierCfg fc;
     const uint32_t* out_ptr;     // [slots + 1] out-edge offsets, internal ids
     const uint32_t* out_dst;     // [E] destinations (vertices), grouped by source slot
     const uint32_t* out_w;       // [E] weights, or nullptr (CC)
+};
+
+// Everything the superstep kernel of a single-partition graph touches
+// (sweep.cu); buffers, lists and stat slots by superstep as in SellArgs.
+struct SweepArgs {
+    const SellSlice* slices;     // decreasing width
+    uint32_t n_slices;
+    uint32_t cols;               // columns per lane the layout aims at (sweep_lanes): 4, 8 or 16
+    // slices spread over 32, 16, 8, 4, 2 lanes a row end at n_lanes[0..4];
+    // then those wider than 8 columns, 4 and 0
+    uint32_t n_lanes[5], n_gt8, n_gt4, n_gt0;
+    const HubPart* hubs;
+    uint32_t n_hubs;
+    const uint32_t *sell_src, *sell_w, *perm, *hsrc, *hw;   // as in PartDev
+    uint32_t n_vertices;
+    uint32_t n_hot;              // values staged in shared memory: vertices [0, n_hot), a multiple of 4
+    uint32_t* own[2];            // [V + 1]: the identity slot is own[V]
+    float* rank[2];
+    StepStats* stats;
+    uint2* lists[2];
+    uint32_t* bits[3];           // changed vertices of a pull superstep t: bits[t % 3]
+    const uint32_t* outdeg;
+    unsigned long long* hub_val; // [n_hubs] published partials: value bits << 32 | 1, zero between supersteps
+    uint32_t* hub_arrive;        // [n_hubs] arrival counters, indexed by a row's first part, likewise
+    uint32_t* err;
+    uint32_t check_bounds;
+    float damping;
+    float inv_n;
+    uint32_t ppr_source;
+    FrontierCfg fc;
+    const uint32_t *out_ptr, *out_dst, *out_w;
 };
 
 // Arguments of the batched multi-source SSSP superstep kernel (one edge block).
@@ -421,30 +468,38 @@ cudaError_t launch_init_ghosts(Algo a, uint32_t n_ghost_total, const uint32_t* g
 cudaError_t launch_superstep(Algo a, const SuperstepArgs& args, size_t smem_bytes, cudaStream_t s);
 cudaError_t launch_superstep_sell(Algo a, const SellArgs& args, cudaStream_t s);
 
-// Device-driven run: the step counter the superstep kernel reads
-// (SellArgs::step_dev) and the loop's bounds.
-struct RunCtl {
-    uint64_t step;          // supersteps done
-    uint64_t limit;         // the loop stops when step reaches it
-    uint32_t quiet_stop;    // 1: also stop after a superstep that changed nothing
-    uint32_t pad;
-};
-cudaError_t launch_run_control(RunCtl* ctl, const StepStats* ring, cudaGraphConditionalHandle h, cudaStream_t s);
-// Grid barrier state of the persistent run (zeroed before each launch).
+// Grid barrier state of a persistent launch, zero when it starts.
 struct GridBar {
-    uint32_t count;   // CTAs arrived at the current barrier
-    uint32_t gen;     // barriers passed
+    unsigned long long count;   // arrivals so far; top bit: a wait gave up
 };
-// Persistent device-driven run of SSSP / CC on one partition (k_sell_loop):
-// the supersteps of ctl in one cooperative launch of at most one CTA per
-// co-resident slot. Returns cudaErrorNotSupported, launching nothing, when
-// a superstep needs more than kLoopWaves grids of co-resident CTAs (the
-// graph-driven loop then serves); a barrier wait past timeout_ns (or any,
-// with `force`) sets kErrTimeout in args.err and ends the launch.
-constexpr uint32_t kLoopWaves = 2;
-bool sell_loop_fits(Algo a, const SellArgs& args);
-cudaError_t launch_sell_loop(Algo a, const SellArgs& args, RunCtl* ctl, GridBar* bar, uint64_t timeout_ns,
-                             bool force, cudaStream_t s);
+// A superstep's stats, summed over their lanes.
+struct StepSum {
+    unsigned long long changed, dangling_fx, l1_fx, pushed, push_edges;
+};
+constexpr uint32_t kRunChunk = 32;   // supersteps per launch of a run (the stat ring holds 64)
+// What a launch of several supersteps leaves in pinned host memory. The host
+// clears `step` before the launch; a launch that gave up leaves it zero.
+struct RunOut {
+    uint64_t step;          // supersteps done since gxp_begin
+    uint64_t passed;        // grid barriers passed since the counter was zeroed
+    uint32_t err, pad;      // the error word
+    StepSum sum[kRunChunk]; // of the launch's supersteps
+};
+// Supersteps t0, t0 + 1, ... below limit, or until one that changed nothing.
+struct RunArgs {
+    uint64_t t0, limit;
+    uint32_t quiet_stop, force;   // force: every barrier wait gives up (an injected fault)
+    uint64_t timeout_ns;
+    uint64_t passed;        // the barrier counter's value in barriers
+    GridBar* bar;           // nullptr: superstep t0 alone, in a launch that waits for nothing
+    RunOut* out;
+};
+// Supersteps of a single-partition graph (sweep.cu), one CTA on each of the
+// `sms` multiprocessors, in one cooperative launch; a barrier wait past
+// timeout_ns sets kErrTimeout in args.err and ends the launch.
+cudaError_t launch_sweep(Algo a, const SweepArgs& args, const RunArgs& run, uint32_t sms, cudaStream_t s);
+// Values to stage per CTA.
+uint32_t sweep_hot_values(uint64_t n_vertices, uint64_t n_edges, bool by_degree);
 size_t superstep_smem_bytes(Algo a, uint32_t max_items);
 
 cudaError_t launch_sync(const SyncArgs& args, uint32_t max_words, cudaStream_t s);
@@ -547,10 +602,10 @@ cudaError_t launch_sell_windows(const uint32_t* col_ptr, uint32_t n, uint32_t H,
                                 uint32_t* hub_out, uint32_t* nonhub_cnt, uint32_t* hub_cnt, cudaStream_t s);
 cudaError_t launch_sell_slices(const uint32_t* col_ptr, uint32_t n, const uint32_t* rows_out,
                                const uint32_t* nonhub_cnt, const uint32_t* slice_base, uint32_t* perm,
-                               uint32_t* width, uint64_t* off, uint32_t n_slices, bool g4, cudaStream_t s);
+                               uint32_t* width, uint64_t* off, uint32_t n_slices, uint32_t cols, cudaStream_t s);
 cudaError_t launch_sell_fill(const uint32_t* col_ptr, const uint32_t* ssrc, const uint32_t* sw, const uint32_t* perm,
                              const uint32_t* width, const uint64_t* off, uint32_t n_slices, uint32_t part,
-                             uint32_t pad_id, bool g4, uint32_t* sell_src, uint32_t* sell_w, SellSlice* desc,
+                             uint32_t pad_id, uint32_t cols, uint32_t* sell_src, uint32_t* sell_w, SellSlice* desc,
                              cudaStream_t s);
 cudaError_t launch_hub_rows(const uint32_t* col_ptr, uint32_t n, const uint32_t* hub_out, const uint32_t* hub_cnt,
                             const uint32_t* hub_base, uint32_t* hub_list, uint32_t n_hub_rows, uint32_t T,
@@ -558,10 +613,13 @@ cudaError_t launch_hub_rows(const uint32_t* col_ptr, uint32_t n, const uint32_t*
 cudaError_t launch_hub_parts(const uint32_t* col_ptr, const uint32_t* hub_list, const uint32_t* part_off,
                              uint32_t n_hub_rows, uint32_t T, uint32_t part, uint32_t part_base, HubPart* hubs,
                              cudaStream_t s);
-// slices by decreasing width (stable); afterwards scratch[0] holds the number
-// of slices wider than 0 (the first offset of the last bin, width 0)
+// slices by decreasing width (stable); afterwards word b of
+// order_slices_starts(scratch, n) holds the number of slices wider than b
+// (b <= kOrderExact)
+constexpr uint32_t kOrderExact = 1024;
 cudaError_t launch_order_slices(const SellSlice* in, uint32_t n, SellSlice* out, uint32_t* scratch, cudaStream_t s);
 size_t order_slices_scratch_bytes(uint32_t n);
+const uint32_t* order_slices_starts(const uint32_t* scratch, uint32_t n);
 
 // vertex relabelling by decreasing in-degree (sell_build.cu): new2old / old2new
 // and the renumbered offsets rcol[n + 1]; scratch: relabel_scratch_bytes

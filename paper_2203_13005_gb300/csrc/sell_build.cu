@@ -14,11 +14,10 @@
 //     share power-of-two bins), and the list of hub rows (more than H in-edges).
 //  3. k_sell_slices: slices of 32 consecutive sorted rows, their widths and
 //     row slots; k_scan_widths: element offsets of the slices.
-//  4. k_sell_fill: the slice arrays (one warp per slice), columns in groups
-//     of 4 so that a lane reads 4 of its row's sources with one 128-bit load;
-//     the empty slots of rows shorter than their slice (and of the columns
-//     rounding the width up to 4) hold the partition's padding id, whose
-//     value slot always holds the merge's identity.
+//  4. k_sell_fill: the slice arrays (one warp per slice); the empty slots of
+//     rows shorter than their slice (and of the columns rounding the width
+//     up to 4) hold the partition's padding id, whose value slot always
+//     holds the merge's identity.
 //  5. k_hub_rows / k_scan_parts / k_hub_parts: hub rows in id order, split
 //     into parts of T edges.
 //  6. k_order_count / k_order_offsets / k_order_scatter: all partitions'
@@ -33,7 +32,7 @@ namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr uint32_t kSortMax = 2048;     // longest row sorted (shared-memory bitonic)
-constexpr uint32_t kExactBins = 1024;   // in-degrees / widths ordered exactly up to here
+constexpr uint32_t kExactBins = kOrderExact;   // in-degrees / widths ordered exactly up to here
 constexpr uint32_t kBins = kExactBins + 34;   // above: one bin per power of two
 constexpr int kSortWarps = 8;             // warps of a counting-sort CTA
 constexpr uint32_t kSortChunk = kSellWindow / kSortWarps;   // items per warp
@@ -416,10 +415,10 @@ __global__ void k_sell_slices(const uint32_t* col_ptr, const uint32_t* rows_out,
     }
 }
 
-// single CTA: exclusive prefix of a slice's storage, 32 * round_up(width, 4)
-// words (u64), over n slices; out[n] = total
-__global__ void __launch_bounds__(1024) k_scan_widths(const uint32_t* width, uint32_t n, bool g4, uint64_t* out) {
-    auto slice_words = [g4](uint32_t w) { return 32ull * sell_cols(w, g4); };
+// single CTA: exclusive prefix of the slices' storage in words (u64) over n
+// slices; out[n] = total
+__global__ void __launch_bounds__(1024) k_scan_widths(const uint32_t* width, uint32_t n, uint32_t cols, uint64_t* out) {
+    auto slice_words = [cols](uint32_t w) { return sell_words(w, cols); };
     __shared__ unsigned long long part[1024];
     const uint32_t t = threadIdx.x;
     const uint32_t per = (n + 1023) / 1024;
@@ -442,27 +441,56 @@ __global__ void __launch_bounds__(1024) k_scan_widths(const uint32_t* width, uin
     if (t == 1023) out[n] = part[1023];
 }
 
-// one warp per slice: the sources (and weights) in groups of 4 columns, lane
-// l's 4 entries of group g at off + 128 g + 4 l (sell_idx), descriptors
+// one warp per slice: the sources (and weights) as the slice is stored
+// (sell_words: column-major, or lane groups), descriptors. Lane groups are
+// written in storage order: lane l's 4 entries of column group g are one
+// 128-bit store, and its row group's reads of the row are consecutive.
 __global__ void k_sell_fill(const uint32_t* col_ptr, const uint32_t* ssrc, const uint32_t* sw, const uint32_t* perm,
                             const uint32_t* width, const uint64_t* off, uint32_t n_slices, uint32_t part,
-                            uint32_t pad_id, bool g4, uint32_t* sell_src, uint32_t* sell_w, SellSlice* desc) {
+                            uint32_t pad_id, uint32_t cols, uint32_t* sell_src, uint32_t* sell_w, SellSlice* desc) {
     const int lane = threadIdx.x & 31;
     const uint64_t warp0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t s = warp0; s < n_slices; s += n_warps) {
         const uint32_t r = perm[s * 32 + lane];
-        const uint32_t wd = width[s], w4 = sell_cols(wd, g4);
+        const uint32_t wd = width[s];
         const uint64_t o = off[s];
         const uint32_t b = r != kSellPad ? col_ptr[r] : 0u;
         const uint32_t d = r != kSellPad ? col_ptr[r + 1] - b : 0u;
-        for (uint32_t k = 0; k < w4; ++k) {
-            const bool has = k < d;
-            const uint64_t at = o + sell_idx(k, (uint32_t)lane, g4);
-            sell_src[at] = has ? ssrc[b + k] : pad_id;
-            if (sell_w) sell_w[at] = has ? sw[b + k] : 0u;
+        if (!cols) {
+            for (uint32_t k = 0; k < wd; ++k) {
+                const bool has = k < d;
+                const uint64_t at = o + 32ull * k + lane;
+                sell_src[at] = has ? ssrc[b + k] : pad_id;
+                if (sell_w) sell_w[at] = has ? sw[b + k] : 0u;
+            }
+        } else {
+            const uint32_t L = sweep_lanes(wd, cols), rows = 32u / L, c = sweep_cols(wd, L);
+            for (uint32_t sub = 0; sub < L; ++sub) {
+                const int slot = (int)(sub * rows + (uint32_t)lane / L);   // this lane's row
+                const uint32_t rb = __shfl_sync(kFull, b, slot), rd = __shfl_sync(kFull, d, slot);
+                const uint64_t at0 = o + 32ull * c * sub + 4u * lane;   // sweep_idx
+                for (uint32_t g = 0; g < c / 4u; ++g) {
+                    uint32_t x[4], y[4];
+#pragma unroll
+                    for (uint32_t q = 0; q < 4; ++q) {
+                        const uint32_t k = (4u * g + q) * L + (uint32_t)lane % L;
+                        const bool has = k < rd;
+                        x[q] = has ? ssrc[rb + k] : pad_id;
+                        y[q] = (sell_w && has) ? sw[rb + k] : 0u;
+                    }
+                    *reinterpret_cast<uint4*>(sell_src + at0 + 128ull * g) = make_uint4(x[0], x[1], x[2], x[3]);
+                    if (sell_w) *reinterpret_cast<uint4*>(sell_w + at0 + 128ull * g) = make_uint4(y[0], y[1], y[2], y[3]);
+                }
+            }
         }
-        if (lane == 0) desc[s] = SellSlice{part, (uint32_t)(s * 32), wd, 0u, o};
+        if (!cols) {
+            if (lane == 0) desc[s] = SellSlice{part, (uint32_t)(s * 32), wd, 0u, o};
+        } else {   // a renumbered partition's slices mostly hold consecutive vertices, any empty slots last
+            const uint32_t first = __shfl_sync(kFull, r, 0), n = (uint32_t)__popc(__ballot_sync(kFull, r != kSellPad));
+            const bool in_row = __all_sync(kFull, (uint32_t)lane < n ? r == first + (uint32_t)lane : r == kSellPad);
+            if (lane == 0) desc[s] = SellSlice{in_row ? n : 0u, (uint32_t)(s * 32), wd, first, o};
+        }
     }
 }
 
@@ -530,7 +558,7 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_order_count(const SellSlice
 }
 
 // single CTA: per-(chunk, warp) offsets for every bin, bins descending, chunks
-// and warps in order
+// and warps in order; the bins' first offsets follow the table
 __global__ void __launch_bounds__(1024) k_order_offsets(uint32_t* ghist, uint32_t n_warps_total) {
     __shared__ uint32_t tot[kBins];
     for (uint32_t b = threadIdx.x; b < kBins; b += blockDim.x) {
@@ -550,6 +578,7 @@ __global__ void __launch_bounds__(1024) k_order_offsets(uint32_t* ghist, uint32_
     __syncthreads();
     for (uint32_t b = threadIdx.x; b < kBins; b += blockDim.x) {
         uint32_t run = tot[b];
+        ghist[(uint64_t)n_warps_total * kBins + b] = run;
         for (uint32_t w = 0; w < n_warps_total; ++w) {
             const uint32_t c = ghist[(uint64_t)w * kBins + b];
             ghist[(uint64_t)w * kBins + b] = run;
@@ -725,20 +754,20 @@ cudaError_t launch_sell_windows(const uint32_t* col_ptr, uint32_t n, uint32_t H,
 
 cudaError_t launch_sell_slices(const uint32_t* col_ptr, uint32_t n, const uint32_t* rows_out,
                                const uint32_t* nonhub_cnt, const uint32_t* slice_base, uint32_t* perm,
-                               uint32_t* width, uint64_t* off, uint32_t n_slices, bool g4, cudaStream_t s) {
+                               uint32_t* width, uint64_t* off, uint32_t n_slices, uint32_t cols, cudaStream_t s) {
     const uint32_t nw = (n + kSellWindow - 1) / kSellWindow;
     if (nw) k_sell_slices<<<nw, 256, 0, s>>>(col_ptr, rows_out, nonhub_cnt, slice_base, perm, width);
-    k_scan_widths<<<1, 1024, 0, s>>>(width, n_slices, g4, off);
+    k_scan_widths<<<1, 1024, 0, s>>>(width, n_slices, cols, off);
     return cudaGetLastError();
 }
 
 cudaError_t launch_sell_fill(const uint32_t* col_ptr, const uint32_t* ssrc, const uint32_t* sw, const uint32_t* perm,
                              const uint32_t* width, const uint64_t* off, uint32_t n_slices, uint32_t part,
-                             uint32_t pad_id, bool g4, uint32_t* sell_src, uint32_t* sell_w, SellSlice* desc,
+                             uint32_t pad_id, uint32_t cols, uint32_t* sell_src, uint32_t* sell_w, SellSlice* desc,
                              cudaStream_t s) {
     if (n_slices == 0) return cudaSuccess;
     k_sell_fill<<<grid_warps(n_slices, 256), 256, 0, s>>>(col_ptr, ssrc, sw, perm, width, off, n_slices, part,
-                                                          pad_id, g4, sell_src, sell_w, desc);
+                                                          pad_id, cols, sell_src, sell_w, desc);
     return cudaGetLastError();
 }
 
@@ -773,6 +802,11 @@ cudaError_t launch_order_slices(const SellSlice* in, uint32_t n, SellSlice* out,
 size_t order_slices_scratch_bytes(uint32_t n) {
     const uint64_t chunks = (n + kSellWindow - 1) / kSellWindow;
     return 4 * (size_t)(chunks + 1) * kSortWarps * kBins;
+}
+
+const uint32_t* order_slices_starts(const uint32_t* scratch, uint32_t n) {
+    const uint64_t chunks = (n + kSellWindow - 1) / kSellWindow;
+    return scratch + chunks * kSortWarps * kBins;
 }
 
 }  // namespace gxp
