@@ -859,6 +859,12 @@ void Engine::begin(gxp_algo algo, uint32_t source, float damping) {
     // (the packed frontier counter needs lists of fewer than 2^32 items)
     if (a == Algo::LP) {
         build_lp();
+        lp_all_rows_ = true;
+        if (lp_.d_active[0]) {
+            const size_t bytes = 4 * (((size_t)V + 31) / 32);
+            for (uint32_t* b : lp_.d_active) cuda_check(cudaMemsetAsync(b, 0, bytes, stream_), "memset");
+            for (uint32_t* b : lp_.d_changed) cuda_check(cudaMemsetAsync(b, 0, bytes, stream_), "memset");
+        }
         // rows without in-edges are never written: both buffers hold their labels
         cuda_check(cudaMemcpyAsync(d_own_[1], d_own_[0], 4ull * V, cudaMemcpyDeviceToDevice, stream_), "copy values");
     }
@@ -872,6 +878,7 @@ void Engine::begin(gxp_algo algo, uint32_t source, float damping) {
                 (uint64_t)V + n_ghost_total_ + (total_edges_ + kItemEdges - 1) / kItemEdges < (1ull << 32);
     if (frontier_) {
         build_out_edges();
+        build_frontier_lists();
         if (d_bits_[0]) {
             const size_t bytes = 4 * (((size_t)V + 31) / 32);
             for (uint32_t* b : d_bits_) cuda_check(cudaMemsetAsync(b, 0, bytes, stream_), "memset");
@@ -1070,13 +1077,14 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
         LpArgs l{};
         l.parts = lp_.d_parts;
         l.n_parts = n_parts_;
-        l.windows = lp_.d_windows;
-        l.n_windows = lp_.n_windows;
-        l.row_g = lp_.d_row_g;
+        l.slices = lp_.d_slices;
+        l.n_slices = lp_.n_slices;
         l.warp_rows = lp_.d_warp_rows;
         l.n_warp_rows = lp_.n_warp_rows;
         l.chunks = lp_.d_chunks;
         l.n_chunks = lp_.n_chunks;
+        l.big = lp_.d_big;
+        l.n_big = lp_.n_big;
         l.hubs = lp_.d_hubs;
         l.n_hubs = lp_.n_hubs;
         l.segments = lp_.d_segments;
@@ -1093,7 +1101,19 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
         l.stats_out = d_stats_ + (step_ + 1) % kStatRing;
         l.stats_clear = d_stats_ + (step_ + 2) % kStatRing;
         l.skip_if_quiet = (early_exit_ && step_ > 0) ? 1u : 0u;
-        l.narrow_labels = n_vertices_ <= (1ull << 27) ? 1u : 0u;   // labels are vertex ids
+        if (lp_.d_active[0]) {
+            l.active = lp_.d_active[step_ & 1];
+            l.active_next = lp_.d_active[(step_ + 1) & 1];
+            l.changed_bits = lp_.d_changed[step_ % 3];
+            l.changed_next = lp_.d_changed[(step_ + 1) % 3];
+            l.changed_prev = lp_.d_changed[(step_ + 2) % 3];
+            l.all_rows = lp_all_rows_ ? 1u : 0u;
+            l.out_ptr = d_out_ptr_;
+            l.out_dst = d_out_dst_;
+        }
+        lp_all_rows_ = false;
+        l.n_vertices = (uint32_t)n_vertices_;
+        l.n_edges = total_edges_;
         cuda_check(launch_lp_superstep(l, stream_), "label propagation superstep");
     } else if (n_parts_ == 1) {
         RunArgs one{};
@@ -1245,10 +1265,6 @@ void Engine::build_out_edges() {
     d_out_ptr_ = (uint32_t*)dalloc(4 * pad4((size_t)S + 1));
     d_out_dst_ = (uint32_t*)dalloc(4 * std::max<uint64_t>(E, 1));
     d_out_w_ = weighted_ ? (uint32_t*)dalloc(4 * std::max<uint64_t>(E, 1)) : nullptr;
-    list_cap_ = (uint64_t)S + (E + kItemEdges - 1) / kItemEdges;
-    for (auto& l : d_list_) l = (uint2*)dalloc(sizeof(uint2) * std::max<uint64_t>(list_cap_, 1));
-    if (n_parts_ == 1)
-        for (auto& b : d_bits_) b = (uint32_t*)dalloc(4 * (((size_t)V + 31) / 32));
     std::vector<void*> tmp;
     auto talloc = [&](size_t bytes) -> void* {
         void* q = nullptr;
@@ -1290,6 +1306,16 @@ void Engine::build_out_edges() {
     out_ready_ = true;
 }
 
+// The two frontier lists over the out-edge copy, and one partition's bitmaps
+// of changed vertices.
+void Engine::build_frontier_lists() {
+    if (d_list_[0]) return;
+    list_cap_ = (uint64_t)n_slots_ + (total_edges_ + kItemEdges - 1) / kItemEdges;
+    for (auto& l : d_list_) l = (uint2*)dalloc(sizeof(uint2) * std::max<uint64_t>(list_cap_, 1));
+    if (n_parts_ == 1)
+        for (auto& b : d_bits_) b = (uint32_t*)dalloc(4 * ((n_vertices_ + 31) / 32));
+}
+
 // The frontier the next superstep reads: one vertex, or all (kInf) slots.
 // Several partitions start from the slots whose value is finite (every slot
 // for CC; SSSP: the source and its cached copies).
@@ -1308,38 +1334,44 @@ void Engine::seed_frontier(uint32_t source_int) {
                "seed frontier");
 }
 
-// Row lists of label propagation, by in-degree class (host-built once per
-// graph from the partitions' offsets): 1..kLpSmall in-edges (packed into
-// warp windows of adjacent edges, in CSC order), up to kLpChunk, and hub rows
-// cut into chunks of kLpChunk with a hash table each, cut into segments.
+// Row lists of label propagation, by in-degree class: the slices of the rows
+// of up to kLpSmall in-edges are built on the device by the superstep
+// layout's kernels, the longer rows (few) are listed on the host.
 void Engine::build_lp() {
     TraceRange trace_("gxp label-propagation lists");
     if (lp_.ready) return;
     std::vector<LpPart> parts(n_parts_);
-    std::vector<LpRow> chunks, warp_rows;
-    std::vector<LpWindow> windows;
-    std::vector<uint32_t> row_g;
+    std::vector<LpRow> chunks, warp_rows, big;
     std::vector<LpHub> hubs;
     std::vector<LpSegment> segments;
     uint64_t table_slots = 0;
+    std::vector<void*> tmp;
+    auto talloc = [&](size_t bytes) {
+        void* q = nullptr;
+        cuda_check(device_malloc(&q, std::max<size_t>(bytes, 16)), "cudaMalloc");
+        tmp.push_back(q);
+        return q;
+    };
+    struct FreeTmp {
+        std::vector<void*>& v;
+        cudaStream_t s;
+        ~FreeTmp() {
+            cudaStreamSynchronize(s);
+            for (void* q : v) cudaFreeAsync(q, s);   // pool blocks (device_malloc)
+        }
+    } free_tmp{tmp, stream_};
+    auto d2h = [&](void* h, const void* d, size_t bytes) {
+        cuda_check(cudaMemcpyAsync(h, d, bytes, cudaMemcpyDeviceToHost, stream_), "read counts");
+        cuda_check(cudaStreamSynchronize(stream_), "read counts");
+    };
     auto add_row = [&](uint32_t g, uint32_t p, uint32_t e0, uint32_t deg) {
-        if (deg == 0) return;
-        if (deg <= kLpSmall) {
-            // joins the open window if its edges follow on and fit, else opens one
-            LpWindow* w = windows.empty() ? nullptr : &windows.back();
-            const uint32_t wn = w ? (w->n_part & 63u) : 0u;
-            if (!w || (w->n_part >> 6) != p || w->e0 + wn != e0 || wn + deg > 32u) {
-                windows.push_back(LpWindow{e0, (uint32_t)row_g.size(), 0u, p << 6});
-                w = &windows.back();
-            }
-            const uint32_t at = w->n_part & 63u;
-            w->starts |= 1u << at;
-            w->n_part += deg;
-            row_g.push_back(g);
-        } else if (deg <= kLpWarpRow) {
+        if (deg <= kLpSmall) return;   // in the slices
+        if (deg <= kLpWarpRow) {
             warp_rows.push_back(LpRow{g, p, e0, deg, kInf, {0, 0, 0}});
         } else if (deg <= kLpChunk) {
             chunks.push_back(LpRow{g, p, e0, deg, kInf, {0, 0, 0}});
+        } else if (deg <= kLpBig) {
+            big.push_back(LpRow{g, p, e0, deg, kInf, {0, 0, 0}});
         } else {
             uint32_t lg = 1;
             while ((1ull << lg) < 2ull * deg && lg < 32) ++lg;   // 2^32 slots hold any in-degree's labels
@@ -1353,22 +1385,68 @@ void Engine::build_lp() {
                 chunks.push_back(LpRow{g, p, e0 + c, std::min(kLpChunk, deg - c), h, {0, 0, 0}});
         }
     };
+    std::vector<SellSlice*> part_desc(n_parts_);
+    std::vector<uint32_t> part_ns(n_parts_);
+    uint64_t n_slices = 0;
     for (uint32_t p = 0; p < n_parts_; ++p) {
         HostPart& hp = parts_[p];
-        std::vector<uint32_t> cp(hp.n_own + 1);
-        cuda_check(cudaMemcpy(cp.data(), hp.d_col_ptr, 4ull * (hp.n_own + 1), cudaMemcpyDeviceToHost), "row offsets");
-        const uint32_t* src = hp.d_src;
-        if (relabeled_) {   // sources in internal ids, once: no renumbering lookup per edge and superstep
-            uint32_t* rs = (uint32_t*)dalloc(4 * std::max<uint64_t>(hp.n_edges(), 1));
-            cuda_check(launch_permute_u32(d_old2new_, hp.d_src, (uint32_t)hp.n_edges(), rs, false, stream_),
-                       "renumber sources");
-            src = rs;
+        const uint32_t* col = work_[p].col;   // internal row order, as the row-sorted copy
+        const uint32_t n = hp.n_own;
+        // slices of the small rows
+        const uint32_t nw = (n + kSellWindow - 1) / kSellWindow;
+        uint32_t* rows_out = (uint32_t*)talloc(4 * (size_t)n);
+        uint32_t* hub_out = (uint32_t*)talloc(4 * (size_t)n);
+        uint32_t* counts = (uint32_t*)talloc(8 * (size_t)nw + 8);
+        cuda_check(launch_sell_windows(col, n, kLpSmall, rows_out, hub_out, counts, counts + nw, stream_),
+                   "sort windows");
+        std::vector<uint32_t> hc(nw + 1, 0), bases(nw + 1, 0);
+        if (nw) d2h(hc.data(), counts, 4 * (size_t)nw);
+        uint64_t ns = 0;
+        for (uint32_t w = 0; w < nw; ++w) {
+            bases[w] = (uint32_t)ns;
+            ns += (hc[w] + 31) / 32;
         }
-        parts[p] = LpPart{src, hp.v_begin, hp.n_own, hp.ghost_base, 0};
-        for (uint32_t l = 0; l < hp.n_own; ++l) {   // input row order
-            const uint32_t g = relabeled_ ? h_old2new_[l] : hp.v_begin + l;
-            add_row(g, p, cp[l], cp[l + 1] - cp[l]);
+        uint32_t* d_bases = (uint32_t*)talloc(4 * (size_t)nw + 4);
+        if (nw) {
+            before_h2d("upload bases");
+            cuda_check(cudaMemcpyAsync(d_bases, bases.data(), 4 * (size_t)nw, cudaMemcpyHostToDevice, stream_),
+                       "upload bases");
         }
+        uint32_t* perm = (uint32_t*)dalloc(4 * (ns * 32 + 4));
+        uint32_t* width = (uint32_t*)talloc(4 * ns + 4);
+        uint64_t* off = (uint64_t*)talloc(8 * ns + 8);
+        cuda_check(launch_sell_slices(col, n, rows_out, counts, d_bases, perm, width, off, (uint32_t)ns, 0u, stream_),
+                   "slices");
+        uint64_t words = 0;
+        d2h(&words, off + ns, 8);
+        uint32_t* sell = (uint32_t*)dalloc(4 * std::max<uint64_t>(words, 1));
+        part_desc[p] = (SellSlice*)talloc(sizeof(SellSlice) * (ns + 1));
+        cuda_check(launch_sell_fill(col, pd_[p].hsrc, nullptr, perm, width, off, (uint32_t)ns, p, pd_[p].pad_id, 0u,
+                                    sell, nullptr, part_desc[p], stream_), "fill slices");
+        // wide slices first; the rows without in-edges come last and are left out
+        if (ns) {
+            SellSlice* ordered = (SellSlice*)talloc(sizeof(SellSlice) * ns);
+            uint32_t* scratch = (uint32_t*)talloc(order_slices_scratch_bytes((uint32_t)ns));
+            cuda_check(launch_order_slices(part_desc[p], (uint32_t)ns, ordered, scratch, stream_), "order slices");
+            d2h(&part_ns[p], order_slices_starts(scratch, (uint32_t)ns), 4);
+            part_desc[p] = ordered;
+        }
+        n_slices += part_ns[p];
+        parts[p] = LpPart{pd_[p].hsrc, sell, perm, hp.v_begin, n, hp.ghost_base, 0};
+        // the longer rows
+        std::vector<uint32_t> cp((size_t)n + 1);
+        d2h(cp.data(), col, 4ull * (n + 1));
+        for (uint32_t l = 0; l < n; ++l) add_row(hp.v_begin + l, p, cp[l], cp[l + 1] - cp[l]);
+    }
+    if (n_slices > 0xFFFFFFF0ull) fail(GXP_E_INVAL, "graph too large");
+    lp_.n_slices = (uint32_t)n_slices;
+    lp_.d_slices = (SellSlice*)dalloc(sizeof(SellSlice) * std::max<uint64_t>(n_slices, 1));
+    uint64_t at = 0;
+    for (uint32_t p = 0; p < n_parts_; ++p) {
+        if (part_ns[p])
+            cuda_check(cudaMemcpyAsync(lp_.d_slices + at, part_desc[p], sizeof(SellSlice) * part_ns[p],
+                                       cudaMemcpyDeviceToDevice, stream_), "gather slices");
+        at += part_ns[p];
     }
     auto upload = [&](const void* h, size_t bytes) {
         void* d = dalloc(std::max<size_t>(bytes, 16));
@@ -1379,13 +1457,14 @@ void Engine::build_lp() {
         return d;
     };
     lp_.d_parts = (LpPart*)upload(parts.data(), sizeof(LpPart) * parts.size());
-    lp_.d_windows = (LpWindow*)upload(windows.data(), sizeof(LpWindow) * windows.size());
-    lp_.d_row_g = (uint32_t*)upload(row_g.data(), 4 * row_g.size());
     lp_.d_chunks = (LpRow*)upload(chunks.data(), sizeof(LpRow) * chunks.size());
     lp_.d_warp_rows = (LpRow*)upload(warp_rows.data(), sizeof(LpRow) * warp_rows.size());
     lp_.n_warp_rows = (uint32_t)warp_rows.size();
+    // the longest first: a CTA takes one at a time
+    std::stable_sort(big.begin(), big.end(), [](const LpRow& x, const LpRow& y) { return x.n > y.n; });
+    lp_.d_big = (LpRow*)upload(big.data(), sizeof(LpRow) * big.size());
+    lp_.n_big = (uint32_t)big.size();
     lp_.d_hubs = (LpHub*)upload(hubs.data(), sizeof(LpHub) * hubs.size());
-    lp_.n_windows = (uint32_t)windows.size();
     lp_.n_chunks = (uint32_t)chunks.size();
     lp_.n_hubs = (uint32_t)hubs.size();
     lp_.d_segments = (LpSegment*)upload(segments.data(), sizeof(LpSegment) * segments.size());
@@ -1398,6 +1477,19 @@ void Engine::build_lp() {
     lp_.d_counts = (uint32_t*)dalloc(4 * std::max<uint64_t>(table_slots, 1));
     cuda_check(cudaMemsetAsync(lp_.d_keys, 0xFF, 4 * std::max<uint64_t>(table_slots, 1), stream_), "memset");
     cuda_check(cudaMemsetAsync(lp_.d_counts, 0, 4 * std::max<uint64_t>(table_slots, 1), stream_), "memset");
+    // One partition: the out-edge copy that tells which rows a change
+    // reaches. It is an extra: without room for it under mem_budget every
+    // superstep recomputes every row.
+    if (n_parts_ == 1) {
+        const uint64_t V = n_vertices_, E = total_edges_;
+        const uint64_t need = (out_ready_ ? 0 : 4 * pad4(V + 1) + (weighted_ ? 8 : 4) * E) + 5 * 4 * ((V + 31) / 32) + 128;
+        if (!cfg_.mem_budget || graph_bytes_ + need <= cfg_.mem_budget) {
+            build_out_edges();
+            const size_t words = (V + 31) / 32;
+            for (auto& b : lp_.d_active) b = (uint32_t*)dalloc(4 * words);
+            for (auto& b : lp_.d_changed) b = (uint32_t*)dalloc(4 * words);
+        }
+    }
     lp_.ready = true;
 }
 
@@ -1549,6 +1641,7 @@ void Engine::set_values(uint32_t part, const void* in, uint64_t n) {
     // both buffers start equal again (see begin): rows without in-edges are read from either
     cuda_check(cudaMemcpyAsync(d_own_[cur_ ^ 1], d_own_[cur_], 4ull * n_vertices_, cudaMemcpyDeviceToDevice, stream_),
                "copy values");
+    lp_all_rows_ = true;
     if (frontier_) seed_frontier(kInf);   // any value may have moved: every vertex is in the next frontier
     cuda_check(cudaStreamSynchronize(stream_), "set values");
 }

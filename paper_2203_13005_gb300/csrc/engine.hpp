@@ -207,24 +207,29 @@ private:
     uint64_t list_cap_ = 0;
     uint32_t n_slots_ = 0;         // push sources: the vertices, then (several partitions) the cached copies
     void build_out_edges();
+    void build_frontier_lists();
     void seed_frontier(uint32_t source_int);
-    // label propagation: rows by in-degree class, hub hash tables
+    // label propagation: rows by in-degree class, hub hash tables, and for one
+    // partition the bitmaps of rows to recompute (see LpArgs::active)
     struct LpLists {
         bool ready = false;
         LpPart* d_parts = nullptr;
-        LpWindow* d_windows = nullptr;
-        uint32_t* d_row_g = nullptr;
+        SellSlice* d_slices = nullptr;
         LpRow* d_chunks = nullptr;
         LpRow* d_warp_rows = nullptr;
-        uint32_t n_warp_rows = 0;
+        LpRow* d_big = nullptr;
+        uint32_t n_warp_rows = 0, n_big = 0;
         LpHub* d_hubs = nullptr;
         LpSegment* d_segments = nullptr;
         unsigned long long* d_hub_best = nullptr;
         uint32_t* d_seg_used = nullptr;
-        uint32_t n_windows = 0, n_chunks = 0, n_hubs = 0, n_segments = 0;
+        uint32_t n_slices = 0, n_chunks = 0, n_hubs = 0, n_segments = 0;
         uint32_t* d_keys = nullptr;
         uint32_t* d_counts = nullptr;
+        uint32_t* d_active[2] = {nullptr, nullptr};
+        uint32_t* d_changed[3] = {nullptr, nullptr, nullptr};
     } lp_;
+    bool lp_all_rows_ = true;      // the next LP superstep recomputes every row
     void build_lp();
     // runs of several supersteps per launch (one partition)
     uint32_t* d_bits_[3] = {nullptr, nullptr, nullptr};   // changed vertices of the pull supersteps (frontier lists)

@@ -340,19 +340,22 @@ struct PprArgs {
     uint64_t finish_mask;            // slots whose last superstep this is
 };
 
-// Mode-label propagation (lp.cu). Rows are listed by in-degree class:
-// 1..32 in-edges (packed into warp windows), up to kLpWarpRow (a warp per
-// row) and up to kLpChunk (a CTA per row), both counting in shared-memory
-// hash tables, more (a hub: chunks of kLpChunk
-// counted the same way and added into a global hash table of its own, which
-// segments of kLpSegment slots then reduce). Rows without in-edges keep their
-// labels and are not listed.
+// Mode-label propagation (lp.cu). Rows by in-degree class: up to kLpSmall in
+// 32-row slices, a row per lane; up to kLpWarpRow a warp per row and up to
+// kLpChunk a CTA per row, counting labels in shared-memory hash tables; up
+// to kLpBig a large CTA per row, in passes over the labels' hash range; more
+// (a hub): chunks of kLpChunk counted the same way and added into a global
+// hash table of the hub's own, which segments of kLpSegment slots then
+// reduce. Rows without in-edges keep their labels and are not listed.
 constexpr uint32_t kLpSmall = 32;
-constexpr uint32_t kLpWarpRow = 256;   // rows up to this many in-edges: a warp each
+constexpr uint32_t kLpWarpRow = 256;
 constexpr uint32_t kLpChunk = 2048;
+constexpr uint32_t kLpBig = 65536;
 constexpr uint32_t kLpSegment = 4096;
 struct LpPart {                 // where a row's in-edges and their labels are
-    const uint32_t* src;        // CSC sources as local ids (a renumbered partition's, renumbered once)
+    const uint32_t* src;        // row-sorted CSC sources as local ids
+    const uint32_t* sell;       // slices of the small rows, column-major
+    const uint32_t* perm;       // their row slots -> local vertices
     uint32_t v_begin, n_own, ghost_base, pad;
 };
 struct LpRow {                  // a row, or a chunk of a hub row
@@ -362,15 +365,6 @@ struct LpRow {                  // a row, or a chunk of a hub row
     uint32_t n;                 // in-edges
     uint32_t hub;               // hub index for a hub chunk, else kInf
     uint32_t pad[3];
-};
-// Consecutive rows of 1..32 in-edges whose edges are adjacent, packed into
-// one warp's 32 lanes: lane k reads edge e0 + k; bit k of `starts` marks
-// the lanes where a row begins (the rows' value indices are row_g[first ..]).
-struct LpWindow {
-    uint32_t e0;
-    uint32_t first;
-    uint32_t starts;
-    uint32_t n_part;            // edges (low 6 bits) | partition << 6
 };
 struct LpHub {
     uint32_t g;
@@ -387,13 +381,14 @@ struct LpSegment {              // kLpSegment slots (or fewer) of one hub's tabl
 struct LpArgs {
     const LpPart* parts;
     uint32_t n_parts;           // 1: no cached copies (sources are indices into own_cur)
-    const LpWindow* windows;    // rows of 1..kLpSmall in-edges
-    uint32_t n_windows;
-    const uint32_t* row_g;      // their value indices
+    const SellSlice* slices;    // rows of 1..kLpSmall in-edges, by partition, wide slices first
+    uint32_t n_slices;
     const LpRow* warp_rows;     // kLpSmall < in-edges <= kLpWarpRow
     uint32_t n_warp_rows;
     const LpRow* chunks;        // kLpWarpRow < in-edges <= kLpChunk (hub = kInf), and hub chunks
     uint32_t n_chunks;
+    const LpRow* big;           // kLpChunk < in-edges <= kLpBig
+    uint32_t n_big;
     const LpHub* hubs;
     uint32_t n_hubs;
     const LpSegment* segments;  // the hub tables cut into segments
@@ -405,12 +400,24 @@ struct LpArgs {
     const uint32_t* own_cur;
     uint32_t* own_nxt;
     const uint32_t* ghost;
-    uint32_t* changed_bits;     // partitions: bitmap of changed vertices, or nullptr
+    uint32_t* changed_bits;     // bitmap of the vertices this superstep changes, or nullptr
     const StepStats* stats_in;
     StepStats* stats_out;
     StepStats* stats_clear;
     uint32_t skip_if_quiet;     // 1: return at once if the previous superstep changed nothing
-    uint32_t narrow_labels;     // 1: labels < 2^27 (32-bit (row, label) keys suffice)
+    // One partition with an out-edge copy: a row none of whose in-neighbours
+    // changed in the previous superstep keeps its label, so when the changed
+    // vertices have few out-edges only their out-neighbours (and they
+    // themselves, to bring the other buffer up to date) are recomputed.
+    // nullptr: every row is recomputed.
+    uint32_t* active;           // bitmap of the rows to recompute
+    uint32_t* active_next;      // cleared for the next superstep, with changed_next
+    uint32_t* changed_next;
+    const uint32_t* changed_prev;   // the previous superstep's changed vertices
+    uint32_t all_rows;          // 1: recompute every row (first superstep, values set)
+    uint32_t n_vertices;
+    uint64_t n_edges;
+    const uint32_t *out_ptr, *out_dst;
 };
 cudaError_t launch_lp_superstep(const LpArgs& a, cudaStream_t s);
 

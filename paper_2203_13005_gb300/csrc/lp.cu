@@ -4,24 +4,32 @@
 // label) and MSGApply = take it. Jacobi order: labels are read from the
 // previous superstep's buffer and written to the other one.
 //
-//  * rows with 1..32 in-edges: packed (in input order, edges adjacent) into
-//    windows of at most 32 edges, one per warp step: each lane loads one
-//    edge's label (coalesced), __match_any_sync on (row, label) gives every
-//    label's count in its row, and two reductions over the row's lanes
-//    (largest count, then smallest label with it) give the row's mode. No
-//    sort (sorting each row in its lane cost about 2,000 instructions per 32
-//    rows, every lane waiting on the longest row);
-//  * rows with 33..256 in-edges: a warp per row, 257..2048: a CTA per row;
-//    both count the labels in a shared-memory hash table (2^k >= 2 in-degree
-//    slots, open addressing; equal labels of a warp added once) and reduce
-//    (count, -label) over it (sorting each row with a bitonic network in a
-//    CTA, up to 78 barriers a row, ran 3x slower on R-MAT);
+//  * rows with 1..32 in-edges: slices of 32 rows, a row per lane. The lane
+//    gathers its row's labels (a coalesced load of sources per column), sorts
+//    them in registers with an odd-even merge network of the slice's width
+//    and scans the runs: about 15 instructions per edge of 32 rows, so the
+//    gathers set the pace. (Windows of 32 adjacent edges, one per lane, with
+//    __match_any_sync per window were bound by that instruction: ER 2^20 in 8
+//    partitions 169 us a superstep.)
+//  * rows with 33..256 in-edges: a warp per row, 257..2048: a CTA per row,
+//    up to 65,536: a CTA of 1,024 threads per row. All count the labels in a
+//    shared-memory hash table (open addressing; a slot is taken by one
+//    compare-and-swap, which also counts the label's first occurrence; a
+//    warp's lanes that carry its first lane's label, once labels settle most
+//    of them, count as one) and reduce (count, -label) over it. The largest
+//    class makes several passes, each over the labels of one range of a
+//    second hash, so that a 16,384-slot table holds them;
 //  * hub rows (more in-edges): each chunk of 2048 is counted the same way
 //    and its counts are added into the hub's global hash table; segments of
 //    4096 slots that a label entered this superstep, spread over all CTAs,
-//    reduce the tables into a 64-bit maximum per hub and empty them (once
-//    labels settle, most segments stay empty and are skipped), and a thread
-//    per hub applies.
+//    reduce the tables into a 64-bit maximum per hub and empty them, and a
+//    thread per hub applies.
+//
+// One partition: a row whose in-neighbours all kept their labels keeps its
+// own, so once few labels change k_lp_mark marks the rows a change reaches
+// (the changed vertices' out-neighbours) and the kernels skip the others.
+// On R-MAT 20 (33.5 M edges) twelve of fifteen supersteps change a few
+// hundred labels.
 #include "frontier.cuh"
 
 #include <algorithm>
@@ -33,19 +41,13 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kLpBlock = 256;
 constexpr int kLpWarps = kLpBlock / 32;
 constexpr int kGatherUnroll = 4;
+constexpr int kBigBlock = 1024;
+constexpr uint32_t kBigSlots = 16384;      // 128 KB of keys and counts
+constexpr uint32_t kBigPerPass = 8192;     // labels a pass aims at
 
 // the label of in-edge source s of partition P (previous superstep)
 __device__ __forceinline__ uint32_t lp_label(const LpArgs& a, const LpPart& P, uint32_t s) {
     return s < P.n_own ? __ldg(a.own_cur + P.v_begin + s) : __ldg(a.ghost + P.ghost_base + (s - P.n_own));
-}
-
-// MSGApply: returns whether the label changed
-__device__ __forceinline__ bool lp_apply(const LpArgs& a, uint32_t g, uint32_t label) {
-    const uint32_t old = a.own_cur[g];
-    a.own_nxt[g] = label;
-    if (label == old) return false;
-    if (a.changed_bits) atomicOr(a.changed_bits + (g >> 5), 1u << (g & 31u));
-    return true;
 }
 
 // a min-label superstep after a quiet one changes nothing: the same holds
@@ -58,8 +60,40 @@ __device__ __forceinline__ bool lp_quiet(const LpArgs& a, int lane) {
     return c == 0ull;
 }
 
-__device__ __forceinline__ void lp_count(const LpArgs& a, uint32_t n_changed, uint64_t slot) {
-    if (n_changed) atomicAdd(&a.stats_out->changed[slot % kStatLanes], (unsigned long long)n_changed);
+// Whether only the marked rows are recomputed (the same in every thread of
+// the superstep's kernels): the vertices changed by the previous superstep
+// have at most an eighth of the edges. Marking costs an atomic per out-edge,
+// a recomputed row several instructions per in-edge; the eighth is the push
+// direction's line.
+__device__ __forceinline__ bool lp_sparse(const LpArgs& a) {
+    return a.active != nullptr && !a.all_rows && (a.stats_in->list_ne & 0xFFFFFFFFull) * 8ull <= a.n_edges;
+}
+
+__device__ __forceinline__ bool lp_marked(const LpArgs& a, uint32_t g) {
+    return (__ldg(a.active + (g >> 5)) >> (g & 31u)) & 1u;
+}
+
+// what a thread adds up: changed rows and the out-edges of their vertices
+struct LpAcc {
+    uint32_t changed = 0, edges = 0;
+};
+
+// MSGApply
+__device__ __forceinline__ void lp_apply(const LpArgs& a, uint32_t g, uint32_t label, LpAcc& acc) {
+    const uint32_t old = a.own_cur[g];
+    a.own_nxt[g] = label;
+    if (label == old) return;
+    ++acc.changed;
+    if (a.active) acc.edges += __ldg(a.out_ptr + g + 1) - __ldg(a.out_ptr + g);
+    if (a.changed_bits) atomicOr(a.changed_bits + (g >> 5), 1u << (g & 31u));
+}
+
+// a warp's sums into the superstep's stats
+__device__ __forceinline__ void lp_count(const LpArgs& a, const LpAcc& acc, int lane, uint64_t slot) {
+    const uint32_t c = __reduce_add_sync(kFull, acc.changed), e = __reduce_add_sync(kFull, acc.edges);
+    if (lane != 0 || c == 0u) return;
+    atomicAdd(&a.stats_out->changed[slot % kStatLanes], (unsigned long long)c);
+    if (e) atomicAdd(&a.stats_out->list_ne, (unsigned long long)e);
 }
 
 // (count, -label) as one key: the larger key is the more frequent label,
@@ -68,12 +102,87 @@ __device__ __forceinline__ unsigned long long mode_key(uint32_t count, uint32_t 
     return ((unsigned long long)count << 32) | (unsigned long long)(~label);
 }
 
-constexpr int kWinUnroll = 4;   // windows a warp has in flight
+// Start of a superstep (one partition): the bitmaps of the next superstep
+// cleared and, when few labels changed, the rows those changes reach marked.
+// A warp takes 32 vertices and walks the out-edges of the changed ones.
+__global__ void __launch_bounds__(kLpBlock) k_lp_mark(const LpArgs a) {
+    const int lane = threadIdx.x & 31;
+    if (lp_quiet(a, lane)) return;
+    const uint32_t words = (a.n_vertices + 31u) / 32u;
+    for (uint32_t i = blockIdx.x * kLpBlock + threadIdx.x; i < words; i += gridDim.x * kLpBlock) {
+        a.active_next[i] = 0u;
+        a.changed_next[i] = 0u;
+    }
+    if (!lp_sparse(a)) return;
+    const uint32_t n_warps = gridDim.x * kLpWarps;
+    for (uint32_t w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < words; w += n_warps) {
+        const uint32_t bits = __ldg(a.changed_prev + w);
+        if (bits == 0u) continue;
+        if (lane == 0) atomicOr(a.active + w, bits);   // their other buffer is brought up to date
+        for (uint32_t b = bits; b; b &= b - 1u) {
+            const uint32_t v = w * 32u + (uint32_t)(__ffs(b) - 1);
+            const uint32_t e1 = __ldg(a.out_ptr + v + 1);
+            for (uint32_t e = __ldg(a.out_ptr + v) + (uint32_t)lane; e < e1; e += 32u) {
+                const uint32_t d = __ldg(a.out_dst + e);
+                atomicOr(a.active + (d >> 5), 1u << (d & 31u));
+            }
+        }
+    }
+}
+
+// Ascending sort of N registers: Batcher's odd-even merge sorting network
+// (K. E. Batcher, Sorting networks and their applications, 1968), one
+// template instance per comparator distance K of merge size P, so that every
+// index is a constant. Entries known to be kInf at the end cost nothing:
+// min(x, kInf) folds away.
+template <int N, int P, int K>
+__device__ __forceinline__ void sort_step(uint32_t (&x)[N]) {
+#pragma unroll
+    for (int t = K % P; t < N - K; ++t) {
+        if ((t - K % P) % (2 * K) < K && t / (2 * P) == (t + K) / (2 * P)) {
+            const uint32_t lo = min(x[t], x[t + K]), hi = max(x[t], x[t + K]);
+            x[t] = lo;
+            x[t + K] = hi;
+        }
+    }
+    if constexpr (K > 1) sort_step<N, P, K / 2>(x);
+    else if constexpr (2 * P < N) sort_step<N, 2 * P, 2 * P>(x);
+}
+
+// One slice of at most W columns: lane l's row.
+template <bool kOnePart, int W>
+__device__ __forceinline__ void lp_slice(const LpArgs& a, const LpPart& P, const SellSlice& sl, uint32_t row, bool want,
+                                         int lane, LpAcc& acc) {
+    constexpr int N = W <= 4 ? 4 : W <= 8 ? 8 : W <= 16 ? 16 : 32;   // the network's size
+    const uint32_t* col = P.sell + sl.off + lane;
+    uint32_t x[N];
+#pragma unroll
+    for (int k = 0; k < W; ++k) x[k] = (uint32_t)k < sl.width ? __ldcs(col + 32 * k) : kInf;
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+        if constexpr (kOnePart) x[k] = (uint32_t)k < sl.width ? __ldg(a.own_cur + x[k]) : kInf;   // padding: the identity slot
+        else x[k] = (uint32_t)k < sl.width ? lp_label(a, P, x[k]) : kInf;
+    }
+#pragma unroll
+    for (int k = W; k < N; ++k) x[k] = kInf;
+    sort_step<N, 1, 1>(x);
+    // runs of equal labels, ascending: the first longest one is the mode
+    uint32_t best = 1u, mode = x[0], run = 1u;
+#pragma unroll
+    for (int k = 1; k < W; ++k) {
+        run = x[k] == x[k - 1] ? run + 1u : 1u;
+        if (run > best && x[k] != kInf) {
+            best = run;
+            mode = x[k];
+        }
+    }
+    if (want && mode != kInf) lp_apply(a, P.v_begin + row, mode, acc);   // (a row without in-edges keeps its label)
+}
 
 // kOnePart: one partition (no cached copies): every source is a local
-// index into the label array, read without the partition descriptor
+// index into the label array
 template <bool kOnePart>
-__global__ void __launch_bounds__(kLpBlock) k_lp_windows(const LpArgs a) {
+__global__ void __launch_bounds__(kLpBlock) k_lp_slices(const LpArgs a) {
     const int lane = threadIdx.x & 31;
     if (blockIdx.x == 0 && a.stats_clear != nullptr) {
         // zero the ring slot two supersteps ahead (never read or written by this one)
@@ -81,78 +190,37 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_windows(const LpArgs a) {
         for (uint32_t i = threadIdx.x; i < sizeof(StepStats) / 8; i += kLpBlock) z[i] = 0ull;
     }
     if (lp_quiet(a, lane)) return;
+    const bool sparse = kOnePart && lp_sparse(a);
     const uint64_t w0 = ((uint64_t)blockIdx.x * kLpBlock + threadIdx.x) >> 5;
     const uint64_t nw = ((uint64_t)gridDim.x * kLpBlock) >> 5;
-    const uint32_t upto = lane == 31 ? 0xFFFFFFFFu : (2u << lane) - 1u;   // lanes 0..lane
-    uint32_t n_changed = 0;
-    for (uint64_t wb = w0 * kWinUnroll; wb < a.n_windows; wb += nw * kWinUnroll) {
-        // loads of kWinUnroll windows issued together: descriptor, then the
-        // edge's source and the row's value index, then the label and the
-        // row's old label
-        LpWindow W[kWinUnroll];
-        const LpPart* P[kWinUnroll];
-        uint32_t src[kWinUnroll], g[kWinUnroll], label[kWinUnroll], old[kWinUnroll];
-        bool has[kWinUnroll], lead[kWinUnroll];
-#pragma unroll
-        for (int q = 0; q < kWinUnroll; ++q) {
-            const bool live = wb + q < a.n_windows;
-            W[q] = live ? a.windows[wb + q] : LpWindow{0u, 0u, 0u, 0u};
-            P[q] = a.parts + (W[q].n_part >> 6);
-            has[q] = (uint32_t)lane < (W[q].n_part & 63u);
-            lead[q] = has[q] && ((W[q].starts >> lane) & 1u);
+    LpAcc acc;
+    for (uint64_t i = w0; i < a.n_slices; i += nw) {
+        const SellSlice sl = a.slices[i];
+        const LpPart P = a.parts[kOnePart ? 0 : sl.part];
+        const uint32_t row = __ldg(P.perm + sl.row0 + lane);
+        bool want = row != kSellPad;
+        if (sparse) {
+            want = want && lp_marked(a, row);
+            if (!__any_sync(kFull, want)) continue;
         }
-        const uint32_t* src0 = kOnePart ? a.parts[0].src : nullptr;
-#pragma unroll
-        for (int q = 0; q < kWinUnroll; ++q) {
-            src[q] = has[q] ? __ldg((kOnePart ? src0 : P[q]->src) + W[q].e0 + lane) : 0u;
-            g[q] = lead[q] ? __ldg(a.row_g + W[q].first + (uint32_t)__popc(W[q].starts & upto) - 1u) : 0u;
-        }
-#pragma unroll
-        for (int q = 0; q < kWinUnroll; ++q) {
-            if constexpr (kOnePart) label[q] = has[q] ? __ldg(a.own_cur + src[q]) : 0u;
-            else label[q] = has[q] ? lp_label(a, *P[q], src[q]) : 0u;
-            old[q] = lead[q] ? a.own_cur[g[q]] : 0u;
-        }
-#pragma unroll
-        for (int q = 0; q < kWinUnroll; ++q) {
-            // the lanes of this lane's row: [first, end) of the window
-            const uint32_t total = W[q].n_part & 63u;
-            const uint32_t mine = W[q].starts & upto;
-            const uint32_t first = mine ? 31u - (uint32_t)__clz(mine) : 0u;
-            const uint32_t above = W[q].starts & ~upto;
-            const uint32_t end = above ? (uint32_t)(__ffs(above) - 1) : total;
-            const uint32_t row_lanes = (end >= 32u ? 0xFFFFFFFFu : (1u << end) - 1u) & ~((1u << first) - 1u);
-            const unsigned act = __ballot_sync(kFull, has[q]);
-            if (has[q]) {
-                // lanes of the row carrying the same label: the label's count in the row
-                unsigned grp;
-                if (a.narrow_labels)
-                    grp = __match_any_sync(act, (first << 27) | label[q]);
-                else
-                    grp = __match_any_sync(act, ((unsigned long long)first << 32) | label[q]);
-                const uint32_t c = (uint32_t)__popc(grp);
-                // the row's largest count, then the smallest label with it
-                const uint32_t cmax = __reduce_max_sync(row_lanes, c);
-                const uint32_t mode = __reduce_min_sync(row_lanes, c == cmax ? label[q] : kInf);
-                if (lead[q]) {
-                    a.own_nxt[g[q]] = mode;
-                    if (mode != old[q]) {
-                        ++n_changed;
-                        if (a.changed_bits) atomicOr(a.changed_bits + (g[q] >> 5), 1u << (g[q] & 31u));
-                    }
-                }
-            }
+        switch ((sl.width + 3u) / 4u) {
+            case 1: lp_slice<kOnePart, 4>(a, P, sl, row, want, lane, acc); break;
+            case 2: lp_slice<kOnePart, 8>(a, P, sl, row, want, lane, acc); break;
+            case 3: lp_slice<kOnePart, 12>(a, P, sl, row, want, lane, acc); break;
+            case 4: lp_slice<kOnePart, 16>(a, P, sl, row, want, lane, acc); break;
+            case 5: lp_slice<kOnePart, 20>(a, P, sl, row, want, lane, acc); break;
+            case 6: lp_slice<kOnePart, 24>(a, P, sl, row, want, lane, acc); break;
+            case 7: lp_slice<kOnePart, 28>(a, P, sl, row, want, lane, acc); break;
+            default: lp_slice<kOnePart, 32>(a, P, sl, row, want, lane, acc); break;
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) n_changed += __shfl_xor_sync(kFull, n_changed, o);
-    if (lane == 0) lp_count(a, n_changed, w0);
+    lp_count(a, acc, lane, w0);
 }
 
-// add `count` occurrences of `label` to a hash table of 2^log2_size slots
-// (open addressing with linear probing; a table of 2^k >= 2 n slots, or 2^32,
-// has a free slot for every distinct label, so one is always found). Works
-// on global and on shared memory tables.
+// add `count` occurrences of `label` to a hub's global hash table of
+// 2^log2_size slots (open addressing with linear probing; a table of 2^k >= 2
+// n slots, or 2^32, has a free slot for every distinct label, so one is
+// always found)
 __device__ __forceinline__ uint32_t lp_table_add(uint32_t* keys, uint32_t* counts, uint32_t log2_size,
                                                  uint32_t label, uint32_t count) {
     const uint32_t mask = log2_size >= 32u ? 0xFFFFFFFFu : (1u << log2_size) - 1u;
@@ -168,6 +236,35 @@ __device__ __forceinline__ uint32_t lp_table_add(uint32_t* keys, uint32_t* count
     return 0u;
 }
 
+// Add a warp's labels (where `has`) to a shared-memory table of 2^log2_size
+// slots. A slot's count is its label's occurrences less one, so a label
+// that occurs once costs the compare-and-swap alone. Returns false for a lane
+// whose label found no slot (a full table). All 32 lanes must call it.
+__device__ __forceinline__ bool lp_warp_add(uint32_t* keys, uint32_t* more, uint32_t log2_size, uint32_t label, bool has,
+                                            int lane) {
+    const unsigned act = __ballot_sync(kFull, has);
+    if (act == 0u) return true;
+    // lanes that carry the first lane's label count as one
+    const int first = __ffs(act) - 1;
+    const uint32_t l0 = __shfl_sync(kFull, label, first);
+    const unsigned same = __ballot_sync(kFull, has && label == l0);
+    if (!has || (label == l0 && lane != first)) return true;
+    const uint32_t c = lane == first ? (uint32_t)__popc(same) : 1u;
+    const uint32_t mask = (1u << log2_size) - 1u;
+    uint32_t slot = (label * 0x9E3779B1u) >> (32u - log2_size);
+    for (uint32_t probe = 0; probe <= mask; ++probe) {
+        const uint32_t k = atomicCAS(keys + slot, kInf, label);
+        if (k == kInf || k == label) {
+            const uint32_t add = k == kInf ? c - 1u : c;
+            if (add) atomicAdd(more + slot, add);
+            return true;
+        }
+        slot = (slot + 1u) & mask;
+    }
+    return false;
+}
+
+template <int kThreads>
 __device__ __forceinline__ unsigned long long block_max(unsigned long long v, unsigned long long* s_red) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -175,8 +272,22 @@ __device__ __forceinline__ unsigned long long block_max(unsigned long long v, un
     if (lane == 0) s_red[warp] = v;
     __syncthreads();
     unsigned long long b = 0ull;
-    for (int w = 0; w < kLpWarps; ++w) b = max(b, s_red[w]);
+    for (int w = 0; w < kThreads / 32; ++w) b = max(b, s_red[w]);
     return b;
+}
+
+// Which of a CTA's next kThreads rows (first, first + step, ... below n) are
+// wanted, a thread asking for each: a superstep that recomputes few rows then
+// costs a look at 32 of them where one row after another would be a chain of
+// two loads each. Every thread gets the bits; returns whether there are any.
+template <int kThreads>
+__device__ __forceinline__ bool lp_wanted(const LpArgs& a, const LpRow* rows, uint64_t first, uint64_t step, uint64_t n,
+                                          bool sparse, uint32_t* s_want) {
+    const uint64_t mine = first + (uint64_t)threadIdx.x * step;
+    const bool want = mine < n && (!sparse || lp_marked(a, __ldg(&rows[mine].g)));
+    const unsigned b = __ballot_sync(kFull, want);
+    if ((threadIdx.x & 31) == 0) s_want[threadIdx.x >> 5] = b;
+    return __syncthreads_or(want) != 0;
 }
 
 // Rows of 33..256 in-edges, a warp each (8 rows in flight per CTA): the
@@ -184,21 +295,26 @@ __device__ __forceinline__ unsigned long long block_max(unsigned long long v, un
 // 2n slots, at most 512), takes the largest (count, -label) over the table
 // with a warp reduction and empties it.
 __global__ void __launch_bounds__(kLpBlock) k_lp_warp_rows(const LpArgs a) {
-    __shared__ uint32_t t_key[kLpWarps][2 * kLpWarpRow], t_cnt[kLpWarps][2 * kLpWarpRow];
+    __shared__ uint32_t t_key[kLpWarps][2 * kLpWarpRow], t_more[kLpWarps][2 * kLpWarpRow];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lp_quiet(a, lane)) return;
-    uint32_t* keys = t_key[warp];
-    uint32_t* cnts = t_cnt[warp];
+    const bool sparse = lp_sparse(a);
+    uint32_t* keys = t_key[warp];   // a warp's own table: no other warp waits for it
+    uint32_t* more = t_more[warp];
     for (uint32_t i = (uint32_t)lane; i < 2 * kLpWarpRow; i += 32u) {
         keys[i] = kInf;
-        cnts[i] = 0u;
+        more[i] = 0u;
     }
     __syncwarp();
     const uint64_t w0 = ((uint64_t)blockIdx.x * kLpBlock + threadIdx.x) >> 5;
     const uint64_t nw = ((uint64_t)gridDim.x * kLpBlock) >> 5;
-    uint32_t n_changed = 0;
-    for (uint64_t ri = w0; ri < a.n_warp_rows; ri += nw) {
-        const LpRow r = a.warp_rows[ri];
+    LpAcc acc;
+    // the warp's next 32 rows, w0, w0 + nw, ...: lane j asks whether row j is wanted
+    for (uint64_t r0 = w0; r0 < a.n_warp_rows; r0 += 32u * nw) {
+    const uint64_t mine = r0 + (uint64_t)lane * nw;
+    const bool want = mine < a.n_warp_rows && (!sparse || lp_marked(a, __ldg(&a.warp_rows[mine].g)));
+    for (unsigned todo = __ballot_sync(kFull, want); todo; todo &= todo - 1u) {
+        const LpRow r = a.warp_rows[r0 + (uint64_t)(__ffs(todo) - 1) * nw];
         const LpPart P = a.parts[r.part];
         const uint32_t n = r.n;
         uint32_t lg = 1;
@@ -216,49 +332,53 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_warp_rows(const LpArgs a) {
                 lab[q] = i < n ? lp_label(a, P, sv[q]) : 0u;
             }
 #pragma unroll
-            for (int q = 0; q < kGatherUnroll; ++q) {
-                const bool has = i0 + 32u * q + (uint32_t)lane < n;
-                const unsigned act = __ballot_sync(kFull, has);
-                if (has) {
-                    const unsigned grp = __match_any_sync(act, lab[q]);
-                    if (lane == __ffs(grp) - 1) lp_table_add(keys, cnts, lg, lab[q], (uint32_t)__popc(grp));
-                }
-            }
+            for (int q = 0; q < kGatherUnroll; ++q)   // (a table of 2n slots never fills)
+                lp_warp_add(keys, more, lg, lab[q], i0 + 32u * q + (uint32_t)lane < n, lane);
         }
         __syncwarp();
         unsigned long long best = 0ull;
         for (uint32_t i = (uint32_t)lane; i < (1u << lg); i += 32u) {
             const uint32_t k = keys[i];
             if (k != kInf) {
-                best = max(best, mode_key(cnts[i], k));
+                best = max(best, mode_key(more[i] + 1u, k));
                 keys[i] = kInf;
-                cnts[i] = 0u;
+                more[i] = 0u;
             }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(kFull, best, o));
-        if (lane == 0 && lp_apply(a, r.g, ~(uint32_t)best)) ++n_changed;
+        if (lane == 0) lp_apply(a, r.g, ~(uint32_t)best, acc);
         __syncwarp();
     }
-    if (lane == 0) lp_count(a, n_changed, w0);
+    }
+    lp_count(a, acc, lane, w0);
 }
 
 // Rows of 257..2048 in-edges (hub = kInf) and chunks of 2048 of hub rows: the
 // CTA counts the labels in a shared-memory hash table (2^k >= 2n slots),
 // then takes the mode (a row) or adds its counts into the hub's table.
 __global__ void __launch_bounds__(kLpBlock) k_lp_rows(const LpArgs a) {
-    __shared__ uint32_t t_key[2 * kLpChunk], t_cnt[2 * kLpChunk];
+    __shared__ uint32_t t_key[2 * kLpChunk], t_more[2 * kLpChunk];
     __shared__ unsigned long long s_red[kLpWarps];
+    __shared__ uint32_t s_want[kLpWarps];
     const int tid = threadIdx.x, lane = tid & 31;
     if (lp_quiet(a, lane)) return;
-    for (uint32_t i = (uint32_t)tid; i < 2 * kLpChunk; i += kLpBlock) {
-        t_key[i] = kInf;
-        t_cnt[i] = 0u;
+    const bool sparse = lp_sparse(a);
+    bool empty = false;   // the table is set up
+    LpAcc acc;
+    for (uint64_t c0 = blockIdx.x; c0 < a.n_chunks; c0 += (uint64_t)gridDim.x * kLpBlock) {
+    if (!lp_wanted<kLpBlock>(a, a.chunks, c0, gridDim.x, a.n_chunks, sparse, s_want)) continue;
+    if (!empty) {
+        for (uint32_t i = (uint32_t)tid; i < 2 * kLpChunk; i += kLpBlock) {
+            t_key[i] = kInf;
+            t_more[i] = 0u;
+        }
+        empty = true;
+        __syncthreads();
     }
-    __syncthreads();
-    uint32_t n_changed = 0;
-    for (uint64_t c = blockIdx.x; c < a.n_chunks; c += gridDim.x) {
-        const LpRow r = a.chunks[c];
+    for (int wd = 0; wd < kLpWarps; ++wd)
+    for (unsigned todo = s_want[wd]; todo; todo &= todo - 1u) {
+        const LpRow r = a.chunks[c0 + (uint64_t)(32 * wd + __ffs(todo) - 1) * gridDim.x];
         const LpPart P = a.parts[r.part];
         const uint32_t n = r.n;
         uint32_t lg = 1;
@@ -276,17 +396,9 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_rows(const LpArgs a) {
                 const uint32_t i = i0 + (uint32_t)q * kLpBlock + (uint32_t)tid;
                 lab[q] = i < n ? lp_label(a, P, sv[q]) : 0u;
             }
-            // lanes with the same label add once (labels repeat as they settle:
-            // one slot's atomics would otherwise serialize)
 #pragma unroll
-            for (int q = 0; q < kGatherUnroll; ++q) {
-                const bool has = i0 + (uint32_t)q * kLpBlock + (uint32_t)tid < n;
-                const unsigned act = __ballot_sync(kFull, has);
-                if (has) {
-                    const unsigned grp = __match_any_sync(act, lab[q]);
-                    if (lane == __ffs(grp) - 1) lp_table_add(t_key, t_cnt, lg, lab[q], (uint32_t)__popc(grp));
-                }
-            }
+            for (int q = 0; q < kGatherUnroll; ++q)
+                lp_warp_add(t_key, t_more, lg, lab[q], i0 + (uint32_t)q * kLpBlock + (uint32_t)tid < n, lane);
         }
         __syncthreads();
         // read the counts and empty the table for the next row
@@ -294,7 +406,7 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_rows(const LpArgs a) {
         for (uint32_t i = (uint32_t)tid; i < size; i += kLpBlock) {
             const uint32_t k = t_key[i];
             if (k != kInf) {
-                const uint32_t cnt = t_cnt[i];
+                const uint32_t cnt = t_more[i] + 1u;
                 if (r.hub == kInf) {
                     best = max(best, mode_key(cnt, k));
                 } else {
@@ -303,16 +415,99 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_rows(const LpArgs a) {
                     a.seg_used[H.seg0 + slot / kLpSegment] = 1u;   // same value from every writer
                 }
                 t_key[i] = kInf;
-                t_cnt[i] = 0u;
+                t_more[i] = 0u;
             }
         }
         if (r.hub == kInf) {
-            best = block_max(best, s_red);
-            if (tid == 0 && lp_apply(a, r.g, ~(uint32_t)best)) ++n_changed;
+            best = block_max<kLpBlock>(best, s_red);
+            if (tid == 0) lp_apply(a, r.g, ~(uint32_t)best, acc);
         }
         __syncthreads();   // the table and s_red are reused by the next row
     }
-    if (tid == 0) lp_count(a, n_changed, blockIdx.x);
+    __syncthreads();   // s_want is read
+    }
+    if (tid < 32) lp_count(a, acc, lane, blockIdx.x);
+}
+
+// Rows of 2049..65,536 in-edges, a large CTA each: `passes` sweeps over the
+// row, pass p counting the labels whose second hash falls in its range. A
+// pass whose labels do not fit the table (they are as many as it aims at up
+// to the hash's spread) starts the row again with twice as many passes.
+__global__ void __launch_bounds__(kBigBlock) k_lp_big(const LpArgs a) {
+    extern __shared__ uint32_t s_table[];
+    uint32_t* t_key = s_table;
+    uint32_t* t_more = s_table + kBigSlots;
+    __shared__ unsigned long long s_red[kBigBlock / 32];
+    __shared__ uint32_t s_want[kBigBlock / 32];
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (lp_quiet(a, lane)) return;
+    const bool sparse = lp_sparse(a);
+    bool empty = false;   // the table is set up
+    LpAcc acc;
+    for (uint64_t c0 = blockIdx.x; c0 < a.n_big; c0 += (uint64_t)gridDim.x * kBigBlock) {
+    if (!lp_wanted<kBigBlock>(a, a.big, c0, gridDim.x, a.n_big, sparse, s_want)) continue;
+    if (!empty) {
+        for (uint32_t i = (uint32_t)tid; i < kBigSlots; i += kBigBlock) {
+            t_key[i] = kInf;
+            t_more[i] = 0u;
+        }
+        empty = true;
+        __syncthreads();
+    }
+    for (int wd = 0; wd < kBigBlock / 32; ++wd)
+    for (unsigned todo = s_want[wd]; todo; todo &= todo - 1u) {
+        const LpRow r = a.big[c0 + (uint64_t)(32 * wd + __ffs(todo) - 1) * gridDim.x];
+        const LpPart P = a.parts[r.part];
+        const uint32_t n = r.n;
+        uint32_t passes = (n + kBigPerPass - 1) / kBigPerPass;
+        uint32_t lg = 12;
+        while (lg < 14u && (1u << lg) < 2u * min(n, kBigPerPass)) ++lg;
+        const uint32_t size = 1u << lg;
+        unsigned long long best = 0ull;
+        for (uint32_t p = 0; p < passes; ++p) {
+            bool ok = true;
+            for (uint32_t i0 = 0; i0 < n; i0 += (uint32_t)kBigBlock * kGatherUnroll) {
+                uint32_t sv[kGatherUnroll], lab[kGatherUnroll];
+#pragma unroll
+                for (int q = 0; q < kGatherUnroll; ++q) {
+                    const uint32_t i = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid;
+                    sv[q] = i < n ? __ldg(P.src + r.e0 + i) : 0u;
+                }
+#pragma unroll
+                for (int q = 0; q < kGatherUnroll; ++q) {
+                    const uint32_t i = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid;
+                    lab[q] = i < n ? lp_label(a, P, sv[q]) : 0u;
+                }
+#pragma unroll
+                for (int q = 0; q < kGatherUnroll; ++q) {
+                    const bool mine = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid < n &&
+                                      __umulhi(lab[q] * 0x85EBCA6Bu, passes) == p;
+                    ok &= lp_warp_add(t_key, t_more, lg, lab[q], mine, lane);
+                }
+            }
+            ok = __syncthreads_and(ok);
+            for (uint32_t i = (uint32_t)tid; i < size; i += kBigBlock) {
+                const uint32_t k = t_key[i];
+                if (k != kInf) {
+                    if (ok) best = max(best, mode_key(t_more[i] + 1u, k));
+                    t_key[i] = kInf;
+                    t_more[i] = 0u;
+                }
+            }
+            __syncthreads();
+            if (!ok) {   // again, with smaller passes (labels are distinct under the hash: this ends)
+                passes = min(2u * passes, 1u << 30);
+                best = 0ull;
+                p = 0xFFFFFFFFu;   // ++ -> 0
+            }
+        }
+        best = block_max<kBigBlock>(best, s_red);
+        if (tid == 0) lp_apply(a, r.g, ~(uint32_t)best, acc);
+        __syncthreads();   // s_red is reused by the next row
+    }
+    __syncthreads();   // s_want is read
+    }
+    if (tid < 32) lp_count(a, acc, lane, blockIdx.x + 31u);
 }
 
 // hub tables, a segment per CTA: the best (count, -label) of the segment
@@ -335,7 +530,7 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_segments(const LpArgs a) {
                 counts[i] = 0u;
             }
         }
-        best = block_max(best, s_red);
+        best = block_max<kLpBlock>(best, s_red);
         if (tid == 0) {
             if (best) atomicMax(a.hub_best + S.hub, best);
             a.seg_used[sg] = 0u;
@@ -344,32 +539,39 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_segments(const LpArgs a) {
     }
 }
 
-// a thread per hub: apply the mode its segments agreed on
+// a thread per hub: apply the mode its segments agreed on (none: the hub
+// was not recomputed)
 __global__ void k_lp_hubs(const LpArgs a) {
     const int lane = threadIdx.x & 31;
     if (lp_quiet(a, lane)) return;
-    uint32_t n_changed = 0;
+    LpAcc acc;
     for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < a.n_hubs; h += gridDim.x * blockDim.x) {
         const unsigned long long best = a.hub_best[h];
+        if (best == 0ull) continue;
         a.hub_best[h] = 0ull;
-        if (lp_apply(a, a.hubs[h].g, ~(uint32_t)best)) ++n_changed;
+        lp_apply(a, a.hubs[h].g, ~(uint32_t)best, acc);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) n_changed += __shfl_xor_sync(kFull, n_changed, o);
-    if (lane == 0) lp_count(a, n_changed, blockIdx.x * 8u + (threadIdx.x >> 5) + 17u);
+    lp_count(a, acc, lane, blockIdx.x * 8u + (threadIdx.x >> 5) + 17u);
 }
 
 }  // namespace
 
 cudaError_t launch_lp_superstep(const LpArgs& a, cudaStream_t s) {
-    const uint32_t g_win =
-        (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((a.n_windows + 8 * kWinUnroll - 1) / (8 * kWinUnroll),
-                                                           152ull * 16));
-    if (a.n_parts == 1) k_lp_windows<true><<<g_win, kLpBlock, 0, s>>>(a);   // also clears the stat slot
-    else k_lp_windows<false><<<g_win, kLpBlock, 0, s>>>(a);                 // two supersteps ahead
+    if (a.active)
+        k_lp_mark<<<(uint32_t)std::min<uint64_t>((a.n_vertices / 32u + 8u) / 8u, 152ull * 8), kLpBlock, 0, s>>>(a);
+    const uint32_t g_slices =
+        (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((a.n_slices + 7ull) / 8, 152ull * 64));
+    if (a.n_parts == 1) k_lp_slices<true><<<g_slices, kLpBlock, 0, s>>>(a);   // also clears the stat slot
+    else k_lp_slices<false><<<g_slices, kLpBlock, 0, s>>>(a);                 // two supersteps ahead
+    if (a.n_big) {
+        const int smem = 8 * (int)kBigSlots;
+        const cudaError_t e = cudaFuncSetAttribute(k_lp_big, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        k_lp_big<<<(uint32_t)std::min<uint64_t>(a.n_big, 152ull), kBigBlock, smem, s>>>(a);
+    }
+    if (a.n_chunks) k_lp_rows<<<(uint32_t)std::min<uint64_t>(a.n_chunks, 152ull * 6), kLpBlock, 0, s>>>(a);
     if (a.n_warp_rows)
-        k_lp_warp_rows<<<(uint32_t)std::min<uint64_t>((a.n_warp_rows + 7) / 8, 152ull * 8), kLpBlock, 0, s>>>(a);
-    if (a.n_chunks) k_lp_rows<<<(uint32_t)std::min<uint64_t>(a.n_chunks, 152ull * 4), kLpBlock, 0, s>>>(a);
+        k_lp_warp_rows<<<(uint32_t)std::min<uint64_t>((a.n_warp_rows + 7) / 8, 152ull * 6), kLpBlock, 0, s>>>(a);
     if (a.n_segments)
         k_lp_segments<<<(uint32_t)std::min<uint64_t>(a.n_segments, 152ull * 8), kLpBlock, 0, s>>>(a);
     if (a.n_hubs) k_lp_hubs<<<(uint32_t)std::min<uint64_t>((a.n_hubs + 255) / 256, 152ull * 4), 256, 0, s>>>(a);
