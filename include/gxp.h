@@ -540,7 +540,7 @@ GXP_API gxp_status gxp_block_size_model(double k1, double k2, double k3, double 
  * partition's CSC that lives in the caller's device memory, computing d_next
  * from d_cur exactly as gxp_superstep does. It calls no cudaMalloc, cudaFree
  * or allocating library routine. Its scratch is a fixed file-scope device
- * array of about 6.8 MB that every GPU loading libgxp.so holds until the
+ * array of about 5.8 MB that every GPU loading libgxp.so holds until the
  * process exits; it limits the input to 4 * n_vertices + n_edges <= 2^28
  * (larger inputs return GXP_E_INVAL).
  *
@@ -562,13 +562,13 @@ GXP_API gxp_status gxp_block_size_model(double k1, double k2, double k3, double 
  * device); make that first call before any stream capture. Every call clears
  * the parts of the scratch that must start at zero, but all calls share the
  * one array: calls that overlap on the GPU race and give wrong results.
- * Before any edge block is cut, a kernel checks the CSC on the device (the
- * call waits for it): offsets that do not run from 0 to n_edges without
- * decreasing return GXP_E_INVAL, a source id >= n_vertices GXP_E_BOUNDS, and
- * nothing else runs. The kernel's bounded waits on its bulk copies return
- * GXP_E_TIMEOUT when they run out (GXP_FAULT=timeout makes every wait give
- * up at once, to test that path); a warp that gives up first waits for its
- * own copies in flight.
+ * A kernel checks the CSC on the device first: offsets that do not run from 0
+ * to n_edges without decreasing return GXP_E_INVAL, a source id >= n_vertices
+ * GXP_E_BOUNDS, and the superstep kernel after it stages and writes nothing
+ * then. That kernel's bounded waits on its bulk copies return GXP_E_TIMEOUT
+ * when they run out (GXP_FAULT=timeout makes every wait give up at once, to
+ * test that path); a warp that gives up first waits for its own copies in
+ * flight.
  * Errors: GXP_E_INVAL (sizes, null, misaligned or overlapping pointers,
  * input beyond the scratch limit, CSC offsets out of order),
  * GXP_E_UNSUPPORTED (other algorithms), GXP_E_BOUNDS (a source id out of

@@ -1,6 +1,4 @@
 // Load-time and per-superstep helper kernels:
-//  * edge-block (tile) construction over a partition's CSC — the paired edge
-//    and vertex blocks of Section II-B, with hub vertices split;
 //  * out-degrees (PageRank's MSGGen divides by them);
 //  * initial vertex values and cache (ghost) fills;
 //  * synchronization caching and skipping between partitions (Section
@@ -15,81 +13,6 @@ namespace gxp {
 namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
-
-// -------------------------------------------------------------- tiles
-
-// Merge-path position of a cut (vertex ends consumed i, edges consumed j): a
-// vertex end weighs kVertexCost items, an edge one.
-__device__ __forceinline__ uint64_t cut_pos(uint64_t c) {
-    return (c >> 32) * kVertexCost + (c & 0xFFFFFFFFull);
-}
-
-// Cut k of the merged sequence (vertex ends + edges) at weighted position k*T,
-// clamped before the end of the vertex it falls in and snapped back to the
-// start of that vertex unless it is a hub (in-degree > H). Packed as
-// (vertex << 32 | edge).
-__global__ void k_cuts(const uint32_t* __restrict__ col_ptr, uint32_t n, uint32_t n_edges,
-                       uint32_t T, uint32_t H, uint32_t nt, uint64_t* __restrict__ cuts) {
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > nt) return;
-    const uint64_t total = (uint64_t)n * kVertexCost + n_edges;
-    const uint64_t D = min((uint64_t)k * T, total);
-    // largest i in [0, n] with i*cost + col_ptr[i] <= D
-    uint32_t lo = 0, hi = n;
-    while (lo < hi) {
-        const uint32_t mid = lo + (hi - lo + 1u) / 2u;
-        if ((uint64_t)mid * kVertexCost + col_ptr[mid] <= D) lo = mid;
-        else hi = mid - 1u;
-    }
-    const uint32_t i = lo;
-    uint64_t j = D - (uint64_t)i * kVertexCost;
-    if (i < n) {
-        if (j > col_ptr[i + 1]) j = col_ptr[i + 1];   // inside vertex i's end item: cut before it
-        if (j > col_ptr[i] && col_ptr[i + 1] - col_ptr[i] <= H) j = col_ptr[i];
-    }
-    cuts[k] = ((uint64_t)i << 32) | j;
-}
-
-__device__ uint32_t upper_bound_cut(const uint64_t* cuts, uint32_t nt, uint64_t p) {
-    // first k in [0, nt] with cut_pos(cuts[k]) > p (nt + 1 if none)
-    uint32_t lo = 0, hi = nt + 1u;
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (cut_pos(cuts[mid]) > p) hi = mid;
-        else lo = mid + 1u;
-    }
-    return lo;
-}
-
-__global__ void k_tiles(const uint32_t* __restrict__ col_ptr, uint32_t n, const uint64_t* __restrict__ cuts,
-                        uint32_t nt, uint32_t part, uint32_t tile_base, Tile* __restrict__ tiles) {
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nt) return;
-    const uint32_t i0 = (uint32_t)(cuts[k] >> 32), j0 = (uint32_t)cuts[k];
-    const uint32_t i1 = (uint32_t)(cuts[k + 1] >> 32), j1 = (uint32_t)cuts[k + 1];
-    const bool head = i0 < n && j0 > col_ptr[i0];
-    const bool tail = i1 < n && j1 > col_ptr[i1];
-    Tile t;
-    t.v0 = i0;
-    t.nv = i1 - i0 + (tail ? 1u : 0u);
-    t.e0 = j0;
-    t.ne = j1 - j0;
-    t.part = part;
-    t.flags = (head ? kHeadOpen : 0u) | (tail ? kTailOpen : 0u);
-    t.hub_t0 = kInf;
-    t.nparts = 0;
-    if (t.nv == 0u && t.ne == 0u) t.flags = 0u;
-    if (head) {
-        const uint64_t p_first = (uint64_t)i0 * kVertexCost + col_ptr[i0];
-        t.hub_t0 = tile_base + upper_bound_cut(cuts, nt, p_first) - 1u;
-    }
-    if (tail && !(head && t.nv == 1u)) {
-        const uint64_t p_end = (uint64_t)i1 * kVertexCost + col_ptr[i1 + 1];
-        const uint32_t t1 = upper_bound_cut(cuts, nt, p_end) - 1u;
-        t.nparts = t1 - k + 1u;
-    }
-    tiles[k] = t;
-}
 
 // ----------------------------------------------------------- out-degree
 
@@ -429,21 +352,6 @@ __global__ void k_sync_pull(const SyncArgs a) {
 }
 
 }  // namespace
-
-uint32_t tile_count(uint32_t n_own, uint64_t n_edges, uint32_t tile_items) {
-    const uint64_t items = (uint64_t)n_own * kVertexCost + n_edges;
-    return (uint32_t)((items + tile_items - 1) / tile_items);
-}
-
-cudaError_t launch_build_tiles(const uint32_t* col_ptr, uint32_t n_own, uint32_t n_edges,
-                               uint32_t tile_items, uint32_t hub_items, uint32_t part,
-                               uint32_t tile_base, uint32_t nt, Tile* tiles, uint64_t* cuts,
-                               cudaStream_t s) {
-    if (nt == 0) return cudaSuccess;
-    k_cuts<<<(nt + 1 + 255) / 256, 256, 0, s>>>(col_ptr, n_own, n_edges, tile_items, hub_items, nt, cuts);
-    k_tiles<<<(nt + 255) / 256, 256, 0, s>>>(col_ptr, n_own, cuts, nt, part, tile_base, tiles);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_outdeg(const PartDev& p, const uint32_t* src, const uint32_t* ghost_gid,
                           uint32_t* outdeg, cudaStream_t s) {

@@ -192,31 +192,21 @@ constexpr uint32_t kListSlack = 4;
 
 
 
-// Everything the superstep kernel touches.
+// Everything the tile superstep kernel touches (superstep.cu: SSSP or CC over
+// one CSC in the caller's memory).
 struct SuperstepArgs {
     const Tile* tiles;
-    const PartDev* parts;
+    PartDev part;
     uint32_t n_tiles;
-    const uint32_t* own_cur;     // [V] current values (u32 or f32 bits), global id order;
-                                 // own_cur, rank_cur and outdeg are padded to a multiple of 4
+    const uint32_t* own_cur;     // [V] current values, padded to a multiple of 4
     uint32_t* own_nxt;           // [V] next values
-    const uint32_t* ghost;       // [sum of n_ghost] cached remote values
-    const float* rank_cur;       // PageRank ranks [V] (fp32)
-    float* rank_nxt;
-    const uint32_t* outdeg;      // [V] global out-degree (PageRank)
-    uint32_t* changed_bits;      // [ceil(V/32)] or nullptr
     uint32_t* part_head;         // [n_tiles] partials of rows split across tiles (value bits)
     uint32_t* part_tail;         // [n_tiles]
     uint32_t* hub_cnt;           // [n_tiles] arrival counters (self-resetting)
-    StepStats* stats_in;         // slot of the current state (PageRank: its dangling mass)
-    StepStats* stats_out;        // slot the superstep accumulates into
-    StepStats* stats_clear;      // slot zeroed for the superstep after next
-    uint32_t* err;               // device error word
+    unsigned long long* changed; // [kStatLanes] changed vertices
+    uint32_t* err;               // device error word; the kernel does nothing when it is set at its start
     uint64_t timeout_ns;         // limit of any device-side wait
     uint32_t force_timeout;      // injected fault: every wait gives up at once (then drains)
-    uint32_t check_bounds;
-    float damping;
-    double inv_n;                // 1 / N
     uint32_t max_items;          // largest tile (merge items)
 };
 
@@ -450,12 +440,6 @@ struct SyncArgs {
 };
 
 // ------------------------------------------------------------ launchers
-cudaError_t launch_build_tiles(const uint32_t* d_col_ptr, uint32_t n_own, uint32_t n_edges,
-                               uint32_t tile_items, uint32_t hub_items, uint32_t part,
-                               uint32_t tile_base, uint32_t n_tiles, Tile* d_tiles,
-                               uint64_t* d_scratch_cuts, cudaStream_t s);
-uint32_t tile_count(uint32_t n_own, uint64_t n_edges, uint32_t tile_items);
-
 cudaError_t launch_outdeg(const PartDev& p, const uint32_t* d_src, const uint32_t* d_ghost_gid,
                           uint32_t* d_outdeg, cudaStream_t s);
 cudaError_t launch_csc_import(const uint64_t* cp64, uint32_t n, uint64_t n_edges, uint32_t* cp32,
@@ -472,7 +456,7 @@ cudaError_t launch_identity_slots(uint32_t* a, uint32_t* b, uint32_t* c, uint32_
 cudaError_t launch_init_ghosts(Algo a, uint32_t n_ghost_total, const uint32_t* ghost_gid_all,
                                const uint32_t* own_cur, uint32_t* ghost, cudaStream_t s);
 
-cudaError_t launch_superstep(Algo a, const SuperstepArgs& args, size_t smem_bytes, cudaStream_t s);
+cudaError_t launch_superstep(Algo a, const SuperstepArgs& args, uint32_t sms, cudaStream_t s);
 cudaError_t launch_superstep_sell(Algo a, const SellArgs& args, cudaStream_t s);
 
 // Grid barrier state of a persistent launch, zero when it starts.
@@ -507,7 +491,6 @@ struct RunArgs {
 cudaError_t launch_sweep(Algo a, const SweepArgs& args, const RunArgs& run, uint32_t sms, cudaStream_t s);
 // Values to stage per CTA.
 uint32_t sweep_hot_values(uint64_t n_vertices, uint64_t n_edges, bool by_degree);
-size_t superstep_smem_bytes(Algo a, uint32_t max_items);
 
 cudaError_t launch_sync(const SyncArgs& args, uint32_t max_words, cudaStream_t s);
 

@@ -8,7 +8,7 @@
 // tiles and owns a private ring of two shared-memory stages. For tile t+2 one
 // lane issues cp.async.bulk copies of the tile's col_ptr slice (the
 // vertex-edge mapping table), its source ids (+ weights) and the apply-side
-// vertex slices (old value, or rank and out-degree), completing on the
+// vertex slice (old values), completing on the
 // stage's mbarrier, while the warp computes tile t:
 //   MSGGen   lanes read staged source ids lane-consecutively and gather the
 //            sources' values with independent loads in flight; each message
@@ -21,8 +21,8 @@
 //            writing coalesced, and __ballot_sync builds the changed bitmap.
 // A row split across tiles (a hub, in-degree > hub_items) publishes one
 // partial per tile; the last tile to arrive combines them in tile order.
-// Every sum runs in a fixed order, so fp32 PageRank is deterministic; its
-// global sums (dangling mass, L1 delta) are exact 64-bit fixed point.
+// Used by gxp_superstep_min_noalloc (noalloc.cu), which checks the CSC and
+// cuts the tiles.
 #include <algorithm>
 
 #include "gxp_internal.hpp"
@@ -108,7 +108,6 @@ template <Algo A> struct Traits;
 template <> struct Traits<Algo::SSSP> {
     using T = uint32_t;
     static constexpr bool kWeighted = true;
-    static constexpr bool kRank = false;
     static constexpr int kUnroll = 8;   // gathers in flight per lane
     __device__ static T ident() { return kInf; }
     __device__ static T combine(T a, T b) { return min(a, b); }
@@ -126,26 +125,12 @@ template <> struct Traits<Algo::SSSP> {
 template <> struct Traits<Algo::CC> {
     using T = uint32_t;
     static constexpr bool kWeighted = false;
-    static constexpr bool kRank = false;
     static constexpr int kUnroll = 16;
     __device__ static T ident() { return kInf; }
     __device__ static T combine(T a, T b) { return min(a, b); }
     __device__ static T from_bits(uint32_t x) { return x; }
     __device__ static uint32_t to_bits(T x) { return x; }
     __device__ static T gen(uint32_t lu, uint32_t) { return lu; }
-};
-
-template <> struct Traits<Algo::PR> {
-    using T = float;
-    static constexpr bool kWeighted = false;
-    static constexpr bool kRank = true;
-    static constexpr int kUnroll = 16;
-    __device__ static T ident() { return 0.0f; }
-    __device__ static T combine(T a, T b) { return a + b; }
-    __device__ static T from_bits(uint32_t x) { return __uint_as_float(x); }
-    __device__ static uint32_t to_bits(T x) { return __float_as_uint(x); }
-    // The message array already holds r[u] / outdeg(u) (written by Apply).
-    __device__ static T gen(uint32_t cu, uint32_t) { return __uint_as_float(cu); }
 };
 
 // Merge-path split of a tile: the merged sequence interleaves the tile's
@@ -184,7 +169,7 @@ __host__ __device__ inline Geometry geometry(Algo a, uint32_t max_items) {
     const uint32_t cost = max_items + kVertexCost;
     g.vm = ((cost / kVertexCost + 1u + 8u) + 3u) & ~3u;   // col_ptr slice / vertex slices
     g.em = ((cost + 8u) + 3u) & ~3u;                      // source ids (then messages), weights
-    const uint32_t arrays_v = a == Algo::PR ? 3u : 2u;    // col + (rank, outdeg) | (old value)
+    const uint32_t arrays_v = 2u;                         // col + old value
     const uint32_t arrays_e = a == Algo::SSSP ? 2u : 1u;  // src (+ w)
     g.stage_words = arrays_v * g.vm + arrays_e * g.em;
     g.warp_words = kStages * g.stage_words;
@@ -192,7 +177,7 @@ __host__ __device__ inline Geometry geometry(Algo a, uint32_t max_items) {
 }
 
 template <Algo A>
-__global__ void __launch_bounds__(kBlock) k_superstep(const SuperstepArgs args) {
+__global__ void __launch_bounds__(kBlock, 8) k_superstep(const SuperstepArgs args) {
     using Tr = Traits<A>;
     using T = typename Tr::T;
     constexpr int kU = Tr::kUnroll;
@@ -200,8 +185,9 @@ __global__ void __launch_bounds__(kBlock) k_superstep(const SuperstepArgs args) 
     extern __shared__ __align__(128) uint32_t smem[];
     __shared__ uint64_t s_bar[kWarps][kStages];
     __shared__ Tile s_tile[kWarps][kStages];
-    __shared__ unsigned long long s_acc[3];
+    __shared__ unsigned long long s_changed;
     __shared__ uint32_t s_done;
+    if (__ldcg(args.err)) return;   // the CSC did not pass its checks: nothing is staged or written
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t nwarps = blockDim.x >> 5;   // 1..kWarps, chosen at launch to fit shared memory
@@ -210,39 +196,21 @@ __global__ void __launch_bounds__(kBlock) k_superstep(const SuperstepArgs args) 
                       (uint32_t)warp * geo.warp_words;
     auto st_col = [&](int s) { return wbase + (uint32_t)s * geo.stage_words; };
     auto st_vx = [&](int s) { return wbase + (uint32_t)s * geo.stage_words + geo.vm; };   // old value | rank
-    auto st_od = [&](int s) { return wbase + (uint32_t)s * geo.stage_words + 2u * geo.vm; };   // out-degree (PR)
-    auto st_src = [&](int s) {
-        return wbase + (uint32_t)s * geo.stage_words + (Tr::kRank ? 3u : 2u) * geo.vm;
-    };
+    auto st_src = [&](int s) { return wbase + (uint32_t)s * geo.stage_words + 2u * geo.vm; };
     auto st_w = [&](int s) { return st_src(s) + geo.em; };
 
-    if (blockIdx.x == 0 && args.stats_clear != nullptr) {
-        // zero the ring slot two supersteps ahead (never read or written by this one)
-        unsigned long long* z = reinterpret_cast<unsigned long long*>(args.stats_clear);
-        for (uint32_t i = tid; i < sizeof(StepStats) / 8; i += blockDim.x) z[i] = 0ull;
-    }
     if (tid == 0) {
-        s_acc[0] = s_acc[1] = s_acc[2] = 0ull;
+        s_changed = 0ull;
         s_done = 0u;
     }
     if (lane == 0) {
         for (int s = 0; s < kStages; ++s) mbar_init(&s_bar[warp][s], 1u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    float base = 0.0f;
-    if constexpr (A == Algo::PR) {
-        // base term (1-d)/N + d*D/N from the exact dangling-mass sum of the current ranks
-        unsigned long long sd = args.stats_in->dangling_fx[lane] + args.stats_in->dangling_fx[lane + 32];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sd += __shfl_xor_sync(kFull, sd, o);
-        const double d = (double)args.damping;
-        base = (float)((1.0 - d) * args.inv_n + d * fx_to_double(sd) * args.inv_n);
-    }
-    __syncthreads();   // barriers, s_acc, s_done initialised
-    const float damping = args.damping;
+    __syncthreads();   // barriers, s_changed, s_done initialised
 
     uint32_t n_changed = 0;
-    unsigned long long l1 = 0ull, dang = 0ull;
+    const PartDev& P = args.part;
 
     // this warp's contiguous range of tiles
     const uint64_t gw = (uint64_t)blockIdx.x * nwarps + (uint32_t)warp;
@@ -277,13 +245,12 @@ __global__ void __launch_bounds__(kBlock) k_superstep(const SuperstepArgs args) 
         const Tile d = desc_of(t);
         if (lane == 0) {
             s_tile[warp][s] = d;
-            const PartDev P = args.parts[d.part];
             const uint32_t g0 = P.v_begin + d.v0;
             const uint32_t c_lo = d.v0 & ~3u, c_hi = round4(d.v0 + d.nv + 1u);
             const uint32_t e_lo = d.e0 & ~3u, e_hi = round4(d.e0 + d.ne);
             const uint32_t g_lo = g0 & ~3u, g_hi = round4(g0 + d.nv);
             const uint32_t bc = (c_hi - c_lo) * 4u, be = (e_hi - e_lo) * 4u, bg = (g_hi - g_lo) * 4u;
-            const uint32_t total = bc + be * (Tr::kWeighted ? 2u : 1u) + bg * (Tr::kRank ? 2u : 1u);
+            const uint32_t total = bc + be * (Tr::kWeighted ? 2u : 1u) + bg;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive_expect_tx(&s_bar[warp][s], total);
             bulk_g2s(st_col(s), P.col_ptr + c_lo, bc, &s_bar[warp][s]);   // bc >= 16
@@ -291,14 +258,7 @@ __global__ void __launch_bounds__(kBlock) k_superstep(const SuperstepArgs args) 
                 bulk_g2s(st_src(s), P.src + e_lo, be, &s_bar[warp][s]);
                 if (Tr::kWeighted) bulk_g2s(st_w(s), P.w + e_lo, be, &s_bar[warp][s]);
             }
-            if (bg) {
-                if constexpr (Tr::kRank) {
-                    bulk_g2s(st_vx(s), args.rank_cur + g_lo, bg, &s_bar[warp][s]);
-                    bulk_g2s(st_od(s), args.outdeg + g_lo, bg, &s_bar[warp][s]);
-                } else {
-                    bulk_g2s(st_vx(s), args.own_cur + g_lo, bg, &s_bar[warp][s]);
-                }
-            }
+            if (bg) bulk_g2s(st_vx(s), args.own_cur + g_lo, bg, &s_bar[warp][s]);
         }
     };
 
@@ -327,7 +287,6 @@ __global__ void __launch_bounds__(kBlock) k_superstep(const SuperstepArgs args) 
             break;
         }
         const Tile tile = s_tile[warp][s];
-        const PartDev P = args.parts[tile.part];
         const bool head_open = (tile.flags & kHeadOpen) != 0;
         const bool tail_open = (tile.flags & kTailOpen) != 0;
         const uint32_t nv = tile.nv, ne = tile.ne, e0 = tile.e0;
@@ -339,13 +298,9 @@ __global__ void __launch_bounds__(kBlock) k_superstep(const SuperstepArgs args) 
         uint32_t* s_msg = st_src(s) + (e0 & 3u);
         const uint32_t* s_w = st_w(s) + (e0 & 3u);
         const uint32_t* s_vx = st_vx(s) + (g0 & 3u);
-        const uint32_t* s_od = st_od(s) + (g0 & 3u);
 
         // ---- MSGGen: messages overwrite the staged source ids
         {
-            const uint32_t n_local = P.n_own + P.n_ghost;
-            const uint32_t* own = args.own_cur + P.v_begin;
-            const uint32_t* ghost = args.ghost + P.ghost_base;
             for (uint32_t jb = 0; jb < ne; jb += 32u * kU) {
                 uint32_t x[kU];
                 bool valid[kU];
@@ -356,10 +311,10 @@ __global__ void __launch_bounds__(kBlock) k_superstep(const SuperstepArgs args) 
                     valid[q] = false;
                     if (j < ne) {
                         const uint32_t u = s_msg[j];
-                        if (args.check_bounds && u >= n_local) {
+                        if (u >= P.n_own) {
                             atomicOr(args.err, kErrBounds);
                         } else {
-                            x[q] = __ldg(u < P.n_own ? own + u : ghost + (u - P.n_own));
+                            x[q] = __ldg(args.own_cur + u);
                             valid[q] = true;
                         }
                     }
@@ -420,25 +375,10 @@ __global__ void __launch_bounds__(kBlock) k_superstep(const SuperstepArgs args) 
         // ---- MSGApply of row rr (staged old values) with merged message m
         auto apply = [&](uint32_t rr, T m) -> bool {
             const uint32_t gid = g0 + rr;
-            if constexpr (A == Algo::PR) {
-                const float rn = fmaf(damping, m, base);
-                const float ro = __uint_as_float(s_vx[rr]);
-                const uint32_t od = s_od[rr];
-                args.rank_nxt[gid] = rn;
-                const float c = od ? __fdiv_rn(rn, (float)od) : 0.0f;
-                const uint32_t cb = __float_as_uint(c);
-                args.own_nxt[gid] = cb;
-                const unsigned long long fn = fx_of(rn), fo = fx_of(ro);
-                l1 += fn > fo ? fn - fo : fo - fn;
-                if (od == 0u) dang += fn;
-                // message changes are tracked only when a bitmap is wanted (partitions)
-                return args.changed_bits != nullptr && cb != args.own_cur[gid];
-            } else {
-                const uint32_t old = s_vx[rr];
-                const uint32_t nw = min(old, (uint32_t)m);
-                args.own_nxt[gid] = nw;
-                return nw != old;
-            }
+            const uint32_t old = s_vx[rr];
+            const uint32_t nw = min(old, (uint32_t)m);
+            args.own_nxt[gid] = nw;
+            return nw != old;
         };
 
         // rows split across tiles: publish a partial; the last tile of the row
@@ -475,10 +415,7 @@ __global__ void __launch_bounds__(kBlock) k_superstep(const SuperstepArgs args) 
                 tot = warp_combine_all<Tr>(tot);
                 if (lane == 0) {
                     args.hub_cnt[t0] = 0u;   // ready for the next superstep
-                    if (apply(vrow, tot)) {
-                        ++n_changed;
-                        if (args.changed_bits) atomicOr(&args.changed_bits[(g0 + vrow) >> 5], 1u << ((g0 + vrow) & 31u));
-                    }
+                    if (apply(vrow, tot)) ++n_changed;
                 }
             }
         }
@@ -488,43 +425,21 @@ __global__ void __launch_bounds__(kBlock) k_superstep(const SuperstepArgs args) 
             const uint32_t rr = rb + (uint32_t)lane;
             const bool ch = rr < n_ends && apply(rr, Tr::from_bits(s_col[rr + 1]));
             const unsigned mask = __ballot_sync(kFull, ch);
-            if (lane == 0 && mask) {
-                n_changed += __popc(mask);
-                if (args.changed_bits) {
-                    const uint32_t g = g0 + rb;
-                    const uint32_t wd = g >> 5, sh = g & 31u;
-                    atomicOr(&args.changed_bits[wd], mask << sh);
-                    if (sh && (mask >> (32u - sh))) atomicOr(&args.changed_bits[wd + 1u], mask >> (32u - sh));
-                }
-            }
+            if (lane == 0) n_changed += __popc(mask);
         }
         __syncwarp();   // stage s is refilled next
         if (tix + kStages < t_end) issue(tix + kStages, s);
     }
 
     // warp totals -> CTA totals in shared memory; the last warp flushes them
-    unsigned long long c64 = n_changed;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        c64 += __shfl_xor_sync(kFull, c64, o);
-        if constexpr (A == Algo::PR) {
-            l1 += __shfl_xor_sync(kFull, l1, o);
-            dang += __shfl_xor_sync(kFull, dang, o);
-        }
-    }
+    const unsigned long long c64 = __reduce_add_sync(kFull, n_changed);
     if (lane == 0) {
-        if (c64) atomicAdd(&s_acc[0], c64);
-        if (l1) atomicAdd(&s_acc[1], l1);
-        if (dang) atomicAdd(&s_acc[2], dang);
+        if (c64) atomicAdd(&s_changed, c64);
         __threadfence_block();
         if (atomicAdd(&s_done, 1u) == nwarps - 1u) {
             __threadfence_block();
-            const unsigned long long a = atomicAdd(&s_acc[0], 0ull), b = atomicAdd(&s_acc[1], 0ull),
-                                     c = atomicAdd(&s_acc[2], 0ull);
-            const uint32_t ln = blockIdx.x % kStatLanes;
-            if (a) atomicAdd(&args.stats_out->changed[ln], a);
-            if (b) atomicAdd(&args.stats_out->l1_fx[ln], b);
-            if (c) atomicAdd(&args.stats_out->dangling_fx[ln], c);
+            const unsigned long long a = atomicAdd(&s_changed, 0ull);
+            if (a) atomicAdd(&args.changed[blockIdx.x % kStatLanes], a);
         }
     }
 }
@@ -541,44 +456,29 @@ static uint32_t warps_per_cta(Algo a, uint32_t max_items) {
     return (uint32_t)std::min<size_t>(std::max<size_t>(nw, 0), kWarps);
 }
 
-size_t superstep_smem_bytes(Algo a, uint32_t max_items) {
-    return (size_t)geometry(a, max_items).warp_words * warps_per_cta(a, max_items) * sizeof(uint32_t) + 128;
-}
-
 template <Algo A>
-static cudaError_t launch_persistent(const SuperstepArgs& args, cudaStream_t s) {
+static cudaError_t launch_tiles(const SuperstepArgs& args, uint32_t sms, cudaStream_t s) {
     const uint32_t nw = warps_per_cta(A, args.max_items);
     if (nw == 0) return cudaErrorInvalidValue;   // a single warp's stages exceed shared memory
-    const size_t smem = superstep_smem_bytes(A, args.max_items);
+    const size_t smem = (size_t)geometry(A, args.max_items).warp_words * nw * sizeof(uint32_t) + 128;
     cudaError_t e = cudaFuncSetAttribute(k_superstep<A>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    // SM count and occupancy of the current device, queried per launch (host
-    // threads may drive different GPUs; the queries cost microseconds)
-    int dev = 0, n_sm = 0, blocks = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_superstep<A>, (int)(32 * nw), smem)) !=
-        cudaSuccess)
-        return e;
-    const uint64_t blocks_max = (uint64_t)n_sm * (uint64_t)(blocks > 0 ? blocks : 1);
-    const uint64_t blocks_needed = ((uint64_t)args.n_tiles + nw - 1) / nw;
-    const uint32_t grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(blocks_max, blocks_needed));
+    // as many CTAs as their stages and their registers (64 a thread) let stay
+    // on the SMs; no CTA waits for another
+    const uint64_t per_sm = std::max<uint64_t>(1, std::min<uint64_t>(kSmemLimit / (smem + 1024 + 512), 1024 / (32 * nw)));
+    const uint64_t needed = ((uint64_t)args.n_tiles + nw - 1) / nw;
+    const uint32_t grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(sms * per_sm, needed));
     k_superstep<A><<<grid, 32 * nw, smem, s>>>(args);
     return cudaGetLastError();
 }
 
-cudaError_t launch_superstep(Algo a, const SuperstepArgs& args, size_t, cudaStream_t s) {
-    if (args.n_tiles == 0) {
-        // nothing to compute, but the stat slot two supersteps ahead must still be cleared
-        if (args.stats_clear) return cudaMemsetAsync(args.stats_clear, 0, sizeof(StepStats), s);
-        return cudaSuccess;
-    }
+cudaError_t launch_superstep(Algo a, const SuperstepArgs& args, uint32_t sms, cudaStream_t s) {
+    if (args.n_tiles == 0) return cudaSuccess;
     switch (a) {
-        case Algo::SSSP: return launch_persistent<Algo::SSSP>(args, s);
-        case Algo::CC: return launch_persistent<Algo::CC>(args, s);
-        case Algo::PR: return launch_persistent<Algo::PR>(args, s);
+        case Algo::SSSP: return launch_tiles<Algo::SSSP>(args, sms, s);
+        case Algo::CC: return launch_tiles<Algo::CC>(args, sms, s);
+        default: return cudaErrorInvalidValue;
     }
-    return cudaErrorInvalidValue;
 }
 
 }  // namespace gxp
