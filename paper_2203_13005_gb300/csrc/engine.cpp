@@ -158,7 +158,7 @@ void Engine::free_graph_device() {
     d_own_[0] = d_own_[1] = nullptr;
     d_rank_[0] = d_rank_[1] = nullptr;
     d_ghost_ = d_ghost_gid_ = nullptr;
-    d_changed_ = d_boundary_ = nullptr;
+    d_changed_[0] = d_changed_[1] = d_boundary_ = nullptr;
     d_gdq_ids_ = d_gdq_vals_ = nullptr;
     d_gdq_base_ = nullptr;
     d_block_counts_ = d_block_offsets_ = d_part_counts_ = nullptr;
@@ -766,7 +766,7 @@ void Engine::build_caches() {
     }
     if (gdq_total > 0xFFFFFFF0ull) fail(GXP_E_INVAL, "global data queue too large");
     d_boundary_ = (uint32_t*)dalloc(4 * words);
-    d_changed_ = (uint32_t*)dalloc(4 * words);
+    for (auto& c : d_changed_) c = (uint32_t*)dalloc(4 * words);
     d_gdq_ids_ = (uint32_t*)dalloc(4 * std::max<uint64_t>(gdq_total, 1));
     d_gdq_vals_ = (uint32_t*)dalloc(4 * std::max<uint64_t>(gdq_total, 1));
     d_gdq_base_ = (uint64_t*)dalloc(8 * n_parts_);
@@ -776,14 +776,14 @@ void Engine::build_caches() {
     d_block_counts_ = (uint32_t*)dalloc(4 * (size_t)n_parts_ * sync_blocks_x_);
     d_block_offsets_ = (uint32_t*)dalloc(4 * (size_t)n_parts_ * sync_blocks_x_);
     d_part_counts_ = (uint32_t*)dalloc(4 * n_parts_);
-    d_done_ctr_ = (uint32_t*)dalloc(4);
+    d_done_ctr_ = (uint32_t*)dalloc(4 * n_parts_);
     before_h2d("upload");
     cuda_check(cudaMemcpyAsync(d_boundary_, bbits.data(), 4 * words, cudaMemcpyHostToDevice, stream_), "upload");
     before_h2d("upload");
     cuda_check(cudaMemcpyAsync(d_gdq_base_, gb.data(), 8 * n_parts_, cudaMemcpyHostToDevice, stream_), "upload");
-    cuda_check(cudaMemsetAsync(d_changed_, 0, 4 * words, stream_), "memset");
+    for (uint32_t* c : d_changed_) cuda_check(cudaMemsetAsync(c, 0, 4 * words, stream_), "memset");
     cuda_check(cudaMemsetAsync(d_part_counts_, 0, 4 * n_parts_, stream_), "memset");
-    cuda_check(cudaMemsetAsync(d_done_ctr_, 0, 4, stream_), "memset");
+    cuda_check(cudaMemsetAsync(d_done_ctr_, 0, 4 * n_parts_, stream_), "memset");
     // caching under a budget: the LRU state of every copy (lru.cu); the
     // cache starts empty at every gxp_begin
     lru_ = Lru{};
@@ -853,7 +853,8 @@ void Engine::begin(gxp_algo algo, uint32_t source, float damping) {
     cuda_check(launch_identity_slots(d_own_[0] + V, d_own_[1] + V, d_ghost_ + n_ghost_total_,
                                      a == Algo::PR ? 0u : kInf, stream_),
                "identity slots");
-    if (d_changed_) cuda_check(cudaMemsetAsync(d_changed_, 0, 4 * (((size_t)V + 31) / 32 + 2), stream_), "memset");
+    for (uint32_t* c : d_changed_)
+        if (c) cuda_check(cudaMemsetAsync(c, 0, 4 * (((size_t)V + 31) / 32 + 2), stream_), "memset");
     cur_ = 0;
     lru_reset(a == Algo::SSSP || personalized ? src_int : kInf);
     // (the packed frontier counter needs lists of fewer than 2^32 items)
@@ -918,7 +919,9 @@ SellArgs Engine::sell_args() const {
     a.step = step_;
     a.ghost = d_ghost_;
     a.outdeg = d_outdeg_;
-    a.changed_bits = d_changed_;
+    a.changed_bits = d_changed_[step_ & 1];
+    a.changed_next = d_changed_[(step_ + 1) & 1];
+    a.boundary_bits = d_boundary_;
     a.hub_val = reinterpret_cast<uint32_t*>(d_hub_val_);
     a.hub_arrive = d_hub_arrive_;
     a.err = d_err_;
@@ -1096,7 +1099,11 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
         l.own_cur = d_own_[cur_];
         l.own_nxt = d_own_[nx];
         l.ghost = d_ghost_;
-        l.changed_bits = n_parts_ > 1 ? d_changed_ : nullptr;
+        if (n_parts_ > 1) {
+            l.changed_bits = d_changed_[step_ & 1];
+            l.changed_next = d_changed_[(step_ + 1) & 1];
+            l.boundary_bits = d_boundary_;
+        }
         l.stats_in = d_stats_ + step_ % kStatRing;
         l.stats_out = d_stats_ + (step_ + 1) % kStatRing;
         l.stats_clear = d_stats_ + (step_ + 2) % kStatRing;
@@ -1128,7 +1135,8 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
         SyncArgs s{};
         s.parts = d_parts_;
         s.n_parts = n_parts_;
-        s.changed_bits = d_changed_;
+        s.changed_bits = d_changed_[step_ & 1];
+        s.queue = queue_ ? 1u : 0u;
         s.boundary_bits = d_boundary_;
         s.own_val = d_own_[nx];
         s.ghost_gid = d_ghost_gid_;
@@ -1169,11 +1177,10 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
                 LruArgs la = lru_args(d_stats_ + (step_ + 2) % kStatRing,
                                       maybe_quiet ? d_stats_ + step_ % kStatRing : nullptr);
                 la.own_val = d_own_[nx];
-                la.frontier_bits = d_changed_;
+                la.frontier_bits = d_changed_[step_ & 1];
                 cuda_check(launch_lru_boundary(la, lru_.max_per_part, stream_), "cache update");
             }
         }
-        cuda_check(cudaMemsetAsync(d_changed_, 0, 4 * (((size_t)n_vertices_ + 31) / 32 + 2), stream_), "memset");
     }
     cuda_check(cudaEventRecord(ev_b_, stream_), "event");
     cur_ = nx;
@@ -1569,8 +1576,18 @@ uint32_t Engine::run(gxp_algo algo, uint32_t source, float damping, uint32_t max
         }
         return steps;
     }
+    struct Guard {
+        bool &early_exit, &queue;
+        ~Guard() {
+            early_exit = false;
+            queue = true;
+        }
+    } guard{early_exit_, queue_};
     if (algo_ == Algo::PR) {
-        for (; steps < max_steps; ++steps) superstep(algo, g, m, ap, false);
+        for (; steps < max_steps; ++steps) {
+            queue_ = steps + 1 == max_steps;
+            superstep(algo, g, m, ap, false);
+        }
         account(false);
         return steps;
     }
@@ -1579,14 +1596,13 @@ uint32_t Engine::run(gxp_algo algo, uint32_t source, float damping, uint32_t max
     // first superstep that changed nothing (the count includes it) and the
     // ones after a quiet superstep return at once on the device
     uint32_t chunk = 4;
-    struct EarlyExit {
-        bool& f;
-        ~EarlyExit() { f = false; }
-    } guard{early_exit_};
     early_exit_ = true;
     while (steps < max_steps) {
         const uint32_t k = std::min<uint32_t>(chunk, max_steps - steps);
-        for (uint32_t i = 0; i < k; ++i) superstep(algo, g, m, ap, false);
+        for (uint32_t i = 0; i < k; ++i) {
+            queue_ = steps + i + 1 == max_steps;   // (a run that ends earlier ends on an empty queue)
+            superstep(algo, g, m, ap, false);
+        }
         const uint64_t quiet = account(true);
         if (quiet) return (uint32_t)quiet;
         steps += k;

@@ -142,7 +142,8 @@ private:
     uint32_t* d_ghost_ = nullptr;
     uint32_t* d_ghost_gid_ = nullptr;
     uint32_t n_ghost_total_ = 0;
-    uint32_t *d_changed_ = nullptr, *d_boundary_ = nullptr;
+    uint32_t* d_changed_[2] = {nullptr, nullptr};   // superstep t marks its changed vertices in [t & 1]
+    uint32_t* d_boundary_ = nullptr;
     uint32_t *d_gdq_ids_ = nullptr, *d_gdq_vals_ = nullptr;
     uint64_t* d_gdq_base_ = nullptr;
     uint32_t *d_block_counts_ = nullptr, *d_block_offsets_ = nullptr, *d_part_counts_ = nullptr;
@@ -241,6 +242,9 @@ private:
     SweepArgs sweep_args() const;
     FrontierCfg frontier_cfg() const;
     bool early_exit_ = false;      // inside gxp_run: supersteps after a quiet one return at once
+    // inside gxp_run the global data queue is written by the last superstep
+    // alone: the run's others overwrite it before gxp_sync could be called
+    bool queue_ = true;
     bool auto_tiles_ = false;      // tile / hub sizes chosen from the graph's size
     float damping_ = 0.85f;
     int cur_ = 0;

@@ -110,9 +110,9 @@ __device__ __forceinline__ uint32_t push_message(uint32_t du, uint32_t w) {
 // vertex slots only. Every edge belongs to exactly one slot, and every
 // destination is a vertex of the partition holding the edge, so each
 // partition's push writes only its own values. A destination that joins the
-// next frontier also gets its changed bit (changed_bits, several partitions),
-// from which the exchange uploads it; its cached copies join the next
-// frontier when the exchange delivers them (k_sync_pull).
+// next frontier also gets its changed bit, from which the exchange uploads
+// it, and counts in n_boundary if another partition caches it; its cached
+// copies join the next frontier when the exchange delivers them (k_sync_pull).
 // Values stay double-buffered, so this is the same Jacobi superstep as the
 // pull direction (same values, same changed set):
 //  * sources' values come from the previous superstep's buffer, which
@@ -134,8 +134,8 @@ __device__ __forceinline__ uint32_t push_superstep(const FrontierCfg& f, const u
                                                    const uint32_t* out_dst, const uint32_t* out_w,
                                                    const uint32_t* own_cur, uint32_t* own_nxt,
                                                    const uint32_t* ghost, uint32_t n_own_total,
-                                                   uint32_t* changed_bits,
-                                                   const StepStats* stats_in, StepStats* stats_out,
+                                                   uint32_t* changed_bits, const uint32_t* boundary_bits,
+                                                   uint32_t& n_boundary, const StepStats* stats_in, StepStats* stats_out,
                                                    uint64_t warp0, uint64_t n_warps, int lane) {
     const unsigned long long ne = stats_in->list_ne;
     const unsigned long long n_items = min(ne >> 32, (unsigned long long)f.list_cap);
@@ -179,7 +179,8 @@ __device__ __forceinline__ uint32_t push_superstep(const FrontierCfg& f, const u
                 if (m < nv && m < cv) app = atomicMin(own_nxt + v, m) >= cv;
                 if (app) {
                     deg = __ldg(out_ptr + v + 1) - __ldg(out_ptr + v);
-                    if (changed_bits) atomicOr(changed_bits + (v >> 5), 1u << (v & 31u));
+                    atomicOr(changed_bits + (v >> 5), 1u << (v & 31u));
+                    n_boundary += (__ldg(boundary_bits + (v >> 5)) >> (v & 31u)) & 1u;
                 }
             }
             n_changed += (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, app));

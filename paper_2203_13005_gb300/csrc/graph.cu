@@ -155,11 +155,39 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t* s_warp
     return warp_off + incl - x;
 }
 
-// Count changed ∩ boundary per block; the last block to finish turns the
-// counts into per-block offsets and decides whether the exchange is skipped.
+// Whether the exchange is skipped (Section III-B3) and whether it lists the
+// changed copies, from the counts the superstep left: the changed boundary
+// vertices are counted where they change, so this is one warp's sum rather
+// than a pass over the bitmaps (9.8 us a superstep of 3 M vertices).
+__global__ void __launch_bounds__(32) k_sync_decide(const SyncArgs a) {
+    const int lane = threadIdx.x;
+    StepStats* st = a.stats_out;
+    unsigned long long grand = __ldcg(&st->boundary[lane]) + __ldcg(&st->boundary[lane + 32]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) grand += __shfl_xor_sync(kFull, grand, o);
+    if (lane != 0) return;
+    st->boundary_changed = grand;
+    st->skipped = grand == 0 ? 1ull : 0ull;
+    st->exchanged = 1ull;
+    // the next superstep pulls anyway when its frontier would be too much
+    // work to push: its own vertices' items and out-edges, plus at least
+    // one item per changed boundary vertex for the copies that would join
+    // (each has a copy somewhere); then the copies are not listed. Nor
+    // are they when the superstep did not list its own vertices.
+    bool list = a.fc.list_out != nullptr && __ldcg(&st->unlisted) == 0ull;
+    if (list && a.fc.direction == GXP_DIR_AUTO) {
+        const unsigned long long ne = __ldcg(&st->list_ne);
+        list = ((ne >> 32) + (ne & 0xFFFFFFFFull) + grand) * (unsigned long long)a.fc.push_div <= a.fc.total_edges;
+    }
+    st->list_copies = list ? 1ull : 0ull;
+}
+
+// Changed ∩ boundary per block of bitmap words; the last block of a
+// partition turns its counts into offsets in the partition's queue.
 __global__ void __launch_bounds__(kSyncBlock) k_sync_count(const SyncArgs a) {
     __shared__ uint32_t s_warp[kSyncBlock / 32];
     __shared__ bool s_last;
+    if (a.stats_out->skipped) return;   // uniform
     const uint32_t p = blockIdx.y;
     const PartDev P = a.parts[p];
     const uint32_t v_lo = P.v_begin, v_hi = P.v_begin + P.n_own;
@@ -172,43 +200,23 @@ __global__ void __launch_bounds__(kSyncBlock) k_sync_count(const SyncArgs a) {
     if (threadIdx.x == 0) {
         a.block_counts[p * a.blocks_x + blockIdx.x] = total;
         __threadfence();
-        const uint32_t ticket = atomicAdd(a.done_ctr, 1u);
-        s_last = ticket == gridDim.x * gridDim.y - 1u;
+        s_last = atomicAdd(a.done_ctr + p, 1u) == gridDim.x - 1u;
     }
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    unsigned long long grand = 0;
-    for (uint32_t q = 0; q < a.n_parts; ++q) {
-        uint32_t run = 0;
-        for (uint32_t b0 = 0; b0 < a.blocks_x; b0 += kSyncBlock) {
-            const uint32_t b = b0 + threadIdx.x;
-            const uint32_t x = b < a.blocks_x ? __ldcg(&a.block_counts[q * a.blocks_x + b]) : 0u;
-            uint32_t tot;
-            const uint32_t ex = block_excl_scan(x, s_warp, tot);
-            if (b < a.blocks_x) a.block_offsets[q * a.blocks_x + b] = run + ex;
-            run += tot;
-        }
-        if (threadIdx.x == 0) a.part_counts[q] = run;
-        grand += run;
+    uint32_t run = 0;
+    for (uint32_t b0 = 0; b0 < a.blocks_x; b0 += kSyncBlock) {
+        const uint32_t b = b0 + threadIdx.x;
+        const uint32_t x = b < a.blocks_x ? __ldcg(&a.block_counts[p * a.blocks_x + b]) : 0u;
+        uint32_t tot;
+        const uint32_t ex = block_excl_scan(x, s_warp, tot);
+        if (b < a.blocks_x) a.block_offsets[p * a.blocks_x + b] = run + ex;
+        run += tot;
     }
     if (threadIdx.x == 0) {
-        a.stats_out->boundary_changed = grand;
-        a.stats_out->skipped = grand == 0 ? 1ull : 0ull;
-        a.stats_out->exchanged = 1ull;
-        // the next superstep pulls anyway when its frontier would be too much
-        // work to push: its own vertices' items and out-edges, plus at least
-        // one item per changed boundary vertex for the copies that would join
-        // (each has a copy somewhere); then the copies are not listed. Nor
-        // are they when the superstep did not list its own vertices.
-        bool list = a.fc.list_out != nullptr && __ldcg(&a.stats_out->unlisted) == 0ull;
-        if (list && a.fc.direction == GXP_DIR_AUTO) {
-            const unsigned long long ne = __ldcg(&a.stats_out->list_ne);
-            list = ((ne >> 32) + (ne & 0xFFFFFFFFull) + grand) * (unsigned long long)a.fc.push_div <=
-                   a.fc.total_edges;
-        }
-        a.stats_out->list_copies = list ? 1ull : 0ull;
-        *a.done_ctr = 0u;
+        a.part_counts[p] = run;
+        a.done_ctr[p] = 0u;
     }
 }
 
@@ -259,7 +267,7 @@ __global__ void __launch_bounds__(kSyncBlock) k_sync_write(const SyncArgs a) {
 // holds it relaxes its in-edges from that vertex if the next superstep pushes.
 __global__ void k_sync_pull(const SyncArgs a) {
     if (a.stats_out->skipped) return;   // uniform: Section III-B3 skip
-    const bool list = a.stats_out->list_copies != 0ull;   // decided by k_sync_count for every CTA
+    const bool list = a.stats_out->list_copies != 0ull;   // decided by k_sync_decide for every CTA
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto pull = [&](uint32_t g) -> bool {   // copy g takes its owner's new value if it changed
         const uint32_t gid = a.ghost_gid[g];
@@ -401,9 +409,12 @@ cudaError_t launch_init_ghosts(Algo, uint32_t n_ghost, const uint32_t* gid, cons
 
 cudaError_t launch_sync(const SyncArgs& a, uint32_t, cudaStream_t s) {
     if (a.n_parts == 0 || a.blocks_x == 0) return cudaSuccess;
-    dim3 grid(a.blocks_x, a.n_parts);
-    k_sync_count<<<grid, kSyncBlock, 0, s>>>(a);
-    k_sync_write<<<grid, kSyncBlock, 0, s>>>(a);
+    k_sync_decide<<<1, 32, 0, s>>>(a);
+    if (a.queue) {
+        dim3 grid(a.blocks_x, a.n_parts);
+        k_sync_count<<<grid, kSyncBlock, 0, s>>>(a);
+        k_sync_write<<<grid, kSyncBlock, 0, s>>>(a);
+    }
     if (a.n_pull)
         k_sync_pull<<<std::min<uint32_t>((a.n_pull + 255) / 256, 152u * 16), 256, 0, s>>>(a);
     return cudaGetLastError();

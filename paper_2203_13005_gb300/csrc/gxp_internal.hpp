@@ -136,6 +136,7 @@ struct StepStats {
     unsigned long long changed[kStatLanes];
     unsigned long long dangling_fx[kStatLanes];   // sum of fx(r) over out-degree-0 vertices
     unsigned long long l1_fx[kStatLanes];         // sum |fx(r_new) - fx(r_old)|
+    unsigned long long boundary[kStatLanes];      // partitions: changed boundary vertices
     unsigned long long boundary_changed;          // pairs uploaded by the sync (all partitions)
     unsigned long long skipped;                   // 1 if the exchange was skipped
     // frontier of the next superstep (min-label algorithms, single partition):
@@ -148,7 +149,7 @@ struct StepStats {
                                                   // partitions ran (skipped or not)
     unsigned long long downloads;                 // copies the superstep used that were not cached
     // 1: the exchange lists the changed cached copies in the next frontier.
-    // Decided once by k_sync_count from the own vertices' appends and the
+    // Decided once by k_sync_decide from the own vertices' appends and the
     // changed boundary vertices: the copies' appends then advance list_ne,
     // so a test each CTA of k_sync_pull made for itself would see a moving
     // count and the CTAs could disagree (some copies listed, others not).
@@ -229,7 +230,9 @@ struct SellArgs {
     uint64_t step;               // t
     const uint32_t* ghost;
     const uint32_t* outdeg;
-    uint32_t* changed_bits;
+    uint32_t* changed_bits;      // bitmap of the vertices this superstep changes
+    uint32_t* changed_next;      // the next superstep's, cleared by this one
+    const uint32_t* boundary_bits;   // vertices another partition caches
     uint32_t* hub_val;           // [n_hubs] published partials (value bits)
     uint32_t* hub_arrive;        // [n_hubs] arrival counters, indexed by a row's first part
     uint32_t* err;
@@ -401,8 +404,9 @@ struct LpArgs {
     // themselves, to bring the other buffer up to date) are recomputed.
     // nullptr: every row is recomputed.
     uint32_t* active;           // bitmap of the rows to recompute
-    uint32_t* active_next;      // cleared for the next superstep, with changed_next
-    uint32_t* changed_next;
+    uint32_t* active_next;      // cleared for the next superstep
+    uint32_t* changed_next;     // the next superstep's changed_bits, cleared by this one
+    const uint32_t* boundary_bits;  // partitions: vertices another one caches
     const uint32_t* changed_prev;   // the previous superstep's changed vertices
     uint32_t all_rows;          // 1: recompute every row (first superstep, values set)
     uint32_t n_vertices;
@@ -429,7 +433,8 @@ struct SyncArgs {
     uint32_t* block_counts;           // [n_parts * blocks_x]
     uint32_t* block_offsets;          // [n_parts * blocks_x]
     uint32_t* part_counts;            // [n_parts]
-    uint32_t* done_ctr;               // arrival counter of the count kernel
+    uint32_t* done_ctr;               // [n_parts] arrival counters of the count kernel
+    uint32_t queue;                   // 1: write the global data queue (gxp_sync returns it)
     uint32_t blocks_x;
     StepStats* stats_out;
     // frontier lists on (push direction possible): every cached copy whose

@@ -75,7 +75,7 @@ __device__ __forceinline__ bool lp_marked(const LpArgs& a, uint32_t g) {
 
 // what a thread adds up: changed rows and the out-edges of their vertices
 struct LpAcc {
-    uint32_t changed = 0, edges = 0;
+    uint32_t changed = 0, edges = 0, boundary = 0;
 };
 
 // MSGApply
@@ -86,14 +86,17 @@ __device__ __forceinline__ void lp_apply(const LpArgs& a, uint32_t g, uint32_t l
     ++acc.changed;
     if (a.active) acc.edges += __ldg(a.out_ptr + g + 1) - __ldg(a.out_ptr + g);
     if (a.changed_bits) atomicOr(a.changed_bits + (g >> 5), 1u << (g & 31u));
+    if (a.boundary_bits) acc.boundary += (__ldg(a.boundary_bits + (g >> 5)) >> (g & 31u)) & 1u;
 }
 
 // a warp's sums into the superstep's stats
 __device__ __forceinline__ void lp_count(const LpArgs& a, const LpAcc& acc, int lane, uint64_t slot) {
-    const uint32_t c = __reduce_add_sync(kFull, acc.changed), e = __reduce_add_sync(kFull, acc.edges);
+    const uint32_t c = __reduce_add_sync(kFull, acc.changed), e = __reduce_add_sync(kFull, acc.edges),
+                   b = __reduce_add_sync(kFull, acc.boundary);
     if (lane != 0 || c == 0u) return;
     atomicAdd(&a.stats_out->changed[slot % kStatLanes], (unsigned long long)c);
     if (e) atomicAdd(&a.stats_out->list_ne, (unsigned long long)e);
+    if (b) atomicAdd(&a.stats_out->boundary[slot % kStatLanes], (unsigned long long)b);
 }
 
 // (count, -label) as one key: the larger key is the more frequent label,
@@ -189,6 +192,10 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_slices(const LpArgs a) {
         unsigned long long* z = reinterpret_cast<unsigned long long*>(a.stats_clear);
         for (uint32_t i = threadIdx.x; i < sizeof(StepStats) / 8; i += kLpBlock) z[i] = 0ull;
     }
+    if (!kOnePart)   // (one partition: k_lp_mark)
+        for (uint64_t i = (uint64_t)blockIdx.x * kLpBlock + threadIdx.x; i <= a.n_vertices / 32u;
+             i += (uint64_t)gridDim.x * kLpBlock)
+            a.changed_next[i] = 0u;
     if (lp_quiet(a, lane)) return;
     const bool sparse = kOnePart && lp_sparse(a);
     const uint64_t w0 = ((uint64_t)blockIdx.x * kLpBlock + threadIdx.x) >> 5;

@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kSellBlock, Tune<A>::kMinBlocks) k_sell(const 
     constexpr int kU = Tune<A>::kUnroll;
     const uint64_t t = a.step;
     const uint32_t vb = blockIdx.x;
-    __shared__ unsigned long long s_acc[3];
+    __shared__ unsigned long long s_acc[4];
     __shared__ uint32_t s_done;
     __shared__ uint32_t s_ftot[kSellWarps], s_fedges[kSellWarps];   // frontier items, out-edges per warp
     __shared__ unsigned long long s_fbase;
@@ -83,9 +83,11 @@ __global__ void __launch_bounds__(kSellBlock, Tune<A>::kMinBlocks) k_sell(const 
         unsigned long long* z = reinterpret_cast<unsigned long long*>(a.stats + (t + 2) % kStatRing);
         for (uint32_t i = tid; i < sizeof(StepStats) / 8; i += kSellBlock) z[i] = 0ull;
     }
+    for (uint64_t i = (uint64_t)vb * kSellBlock + tid; i <= a.n_vertices / 32u; i += (uint64_t)gridDim.x * kSellBlock)
+        a.changed_next[i] = 0u;
     __shared__ bool s_quiet, s_list;
     if (tid == 0) {
-        s_acc[0] = s_acc[1] = s_acc[2] = 0ull;
+        s_acc[0] = s_acc[1] = s_acc[2] = s_acc[3] = 0ull;
         s_done = 0u;
         s_quiet = false;
         s_list = true;
@@ -116,7 +118,7 @@ __global__ void __launch_bounds__(kSellBlock, Tune<A>::kMinBlocks) k_sell(const 
     if (s_quiet) return;   // same for every thread of the grid
     const float damping = a.damping;
 
-    uint32_t n_changed = 0;
+    uint32_t n_changed = 0, n_boundary = 0;
     unsigned long long l1 = 0ull, dang = 0ull;
 
     // MSGApply of local vertex v of partition P with merged message m
@@ -160,7 +162,7 @@ __global__ void __launch_bounds__(kSellBlock, Tune<A>::kMinBlocks) k_sell(const 
     if constexpr (A != Algo::PR) {
         if (push_chosen(fc, stats_in)) {   // same choice in every thread of the grid
             const uint32_t c = push_superstep<Op::kWeighted>(fc, a.out_ptr, a.out_dst, a.out_w, own_cur, own_nxt,
-                                                             a.ghost, a.n_vertices, a.changed_bits, stats_in,
+                                                             a.ghost, a.n_vertices, a.changed_bits, a.boundary_bits, n_boundary, stats_in,
                                                              stats_out, gw, (uint64_t)gridDim.x * kSellWarps, lane);
             if (lane == 0) n_changed += c;
             pushed = true;
@@ -218,10 +220,9 @@ __global__ void __launch_bounds__(kSellBlock, Tune<A>::kMinBlocks) k_sell(const 
         const bool ch = do_apply && lane == 0 && apply(P, hp.v, total);
         if (ch) {
             ++n_changed;
-            if (a.changed_bits) {
-                const uint32_t g = P.v_begin + hp.v;
-                atomicOr(&a.changed_bits[g >> 5], 1u << (g & 31u));
-            }
+            const uint32_t g = P.v_begin + hp.v;
+            atomicOr(&a.changed_bits[g >> 5], 1u << (g & 31u));
+            n_boundary += (__ldg(a.boundary_bits + (g >> 5)) >> (g & 31u)) & 1u;
         }
         if constexpr (A != Algo::PR) {
             if (ch && fc.list_out) {   // the vertex joins the next frontier
@@ -268,12 +269,15 @@ __global__ void __launch_bounds__(kSellBlock, Tune<A>::kMinBlocks) k_sell(const 
                 f_v = P.v_begin + row;
             }
         }
-        if (ch && a.changed_bits) {
+        if (ch) {
             // one atomic per bitmap word touched by this warp
             const uint32_t g = P.v_begin + row;
             const unsigned grp = __match_any_sync(chm, g >> 5);
             const unsigned bits = __reduce_or_sync(grp, 1u << (g & 31u));
-            if ((uint32_t)lane == (uint32_t)(__ffs(grp) - 1)) atomicOr(&a.changed_bits[g >> 5], bits);
+            if ((uint32_t)lane == (uint32_t)(__ffs(grp) - 1)) {
+                atomicOr(&a.changed_bits[g >> 5], bits);
+                n_boundary += (uint32_t)__popc(bits & __ldg(a.boundary_bits + (g >> 5)));
+            }
         }
     }
 
@@ -307,7 +311,7 @@ __global__ void __launch_bounds__(kSellBlock, Tune<A>::kMinBlocks) k_sell(const 
     }
 
     // warp totals -> CTA totals in shared memory; the last warp flushes them
-    const unsigned long long c64 = __reduce_add_sync(kFull, n_changed);
+    const unsigned long long c64 = __reduce_add_sync(kFull, n_changed), b64 = __reduce_add_sync(kFull, n_boundary);
     if constexpr (A == Algo::PR) {
         l1 = warp_sum_u62(l1);
         dang = warp_sum_u62(dang);
@@ -316,15 +320,17 @@ __global__ void __launch_bounds__(kSellBlock, Tune<A>::kMinBlocks) k_sell(const 
         if (c64) atomicAdd(&s_acc[0], c64);
         if (l1) atomicAdd(&s_acc[1], l1);
         if (dang) atomicAdd(&s_acc[2], dang);
+        if (b64) atomicAdd(&s_acc[3], b64);
         __threadfence_block();
         if (atomicAdd(&s_done, 1u) == (uint32_t)kSellWarps - 1u) {
             __threadfence_block();
             const unsigned long long x0 = atomicAdd(&s_acc[0], 0ull), x1 = atomicAdd(&s_acc[1], 0ull),
-                                     x2 = atomicAdd(&s_acc[2], 0ull);
+                                     x2 = atomicAdd(&s_acc[2], 0ull), x3 = atomicAdd(&s_acc[3], 0ull);
             const uint32_t ln = vb % kStatLanes;
             if (x0) atomicAdd(&stats_out->changed[ln], x0);
             if (x1) atomicAdd(&stats_out->l1_fx[ln], x1);
             if (x2) atomicAdd(&stats_out->dangling_fx[ln], x2);
+            if (x3) atomicAdd(&stats_out->boundary[ln], x3);
         }
     }
 }
