@@ -87,6 +87,7 @@ Engine::~Engine() {
     if (ev_b_) cudaEventDestroy(ev_b_);
     if (ev_k_) cudaEventDestroy(ev_k_);
     if (h_run_) cudaFreeHost(h_run_);
+    if (h_steps_) cudaFreeHost(h_steps_);
     if (stream_) cudaStreamSynchronize(stream_);   // the frees above
     if (pool_) cudaMemPoolDestroy(pool_);
     if (own_stream_) cudaStreamDestroy(own_stream_);
@@ -164,6 +165,8 @@ void Engine::free_graph_device() {
     d_block_counts_ = d_block_offsets_ = d_part_counts_ = nullptr;
     d_done_ctr_ = nullptr;
     d_stats_ = nullptr;
+    d_n_dangling_ = nullptr;
+    seed_all_ne_ = 0;
     d_err_ = nullptr;
     for (auto& hp : parts_)
         if (!hp.on_device) hp.d_col_ptr = hp.d_src = hp.d_w = nullptr;
@@ -186,6 +189,7 @@ void Engine::copy_in(void* dst, const void* src, size_t bytes) {
 }
 
 void Engine::check_device_error() {
+    err_unread_ = false;
     uint32_t err = 0;
     if (d_err_) cuda_check(cudaMemcpy(&err, d_err_, 4, cudaMemcpyDeviceToHost), "read error word");
     if (err & kErrTimeout) fail(GXP_E_TIMEOUT, "a device-side wait exceeded timeout_ns");
@@ -719,6 +723,8 @@ void Engine::finalize() {
     if (relabeled_)
         cuda_check(launch_permute_u32(outdeg_in, d_old2new_, V, d_outdeg_, true, stream_), "out-degrees");
 
+    d_n_dangling_ = (unsigned long long*)dalloc(8);
+    cuda_check(launch_count_dangling(d_outdeg_, V, d_n_dangling_, stream_), "out-degrees");
     for (int b = 0; b < 2; ++b) {
         d_own_[b] = (uint32_t*)dalloc(4 * pad4(V));
         d_rank_[b] = (float*)dalloc(4 * pad4(V));
@@ -841,53 +847,75 @@ void Engine::begin(gxp_algo algo, uint32_t source, float damping) {
     if (!sell_ready_) build_sell();
     const uint32_t V = (uint32_t)n_vertices_;
     begun_ = false;   // until the state below is complete
-    cuda_check(cudaMemsetAsync(d_stats_, 0, sizeof(StepStats) * kStatRing, stream_), "memset");
     uint32_t src_int = source;   // the source in internal ids
     if (relabeled_ && (a == Algo::SSSP || personalized)) src_int = h_old2new_[source];
     const uint32_t ppr_source = personalized ? src_int : kInf;
-    cuda_check(launch_init_values(a, ppr_source, V, src_int, d_own_[0], d_rank_[0], d_outdeg_, d_stats_,
-                                  relabeled_ ? d_new2old_ : nullptr, stream_),
-               "init values");
-    cuda_check(launch_init_ghosts(a, n_ghost_total_, d_ghost_gid_, d_own_[0], d_ghost_, stream_), "init caches");
-    // the identity slots empty SELL slots read: 0 (sums) or INF (minima)
-    cuda_check(launch_identity_slots(d_own_[0] + V, d_own_[1] + V, d_ghost_ + n_ghost_total_,
-                                     a == Algo::PR ? 0u : kInf, stream_),
-               "identity slots");
-    for (uint32_t* c : d_changed_)
-        if (c) cuda_check(cudaMemsetAsync(c, 0, 4 * (((size_t)V + 31) / 32 + 2), stream_), "memset");
-    cur_ = 0;
-    lru_reset(a == Algo::SSSP || personalized ? src_int : kInf);
+    if (a == Algo::LP) build_lp();
     // (the packed frontier counter needs lists of fewer than 2^32 items)
-    if (a == Algo::LP) {
-        build_lp();
-        lp_all_rows_ = true;
-        if (lp_.d_active[0]) {
-            const size_t bytes = 4 * (((size_t)V + 31) / 32);
-            for (uint32_t* b : lp_.d_active) cuda_check(cudaMemsetAsync(b, 0, bytes, stream_), "memset");
-            for (uint32_t* b : lp_.d_changed) cuda_check(cudaMemsetAsync(b, 0, bytes, stream_), "memset");
-        }
-        // rows without in-edges are never written: both buffers hold their labels
-        cuda_check(cudaMemcpyAsync(d_own_[1], d_own_[0], 4ull * V, cudaMemcpyDeviceToDevice, stream_), "copy values");
-    }
-    // both value buffers of the min-label algorithms start equal: a push
-    // superstep lowers the next buffer in place, which must hold values no
-    // lower than the current, and a single partition's pull supersteps leave
-    // rows without in-edges alone
-    if (a == Algo::SSSP || a == Algo::CC)
-        cuda_check(cudaMemcpyAsync(d_own_[1], d_own_[0], 4ull * V, cudaMemcpyDeviceToDevice, stream_), "copy values");
     frontier_ = (a == Algo::SSSP || a == Algo::CC) && cfg_.direction != GXP_DIR_PULL &&
                 (uint64_t)V + n_ghost_total_ + (total_edges_ + kItemEdges - 1) / kItemEdges < (1ull << 32);
     if (frontier_) {
         build_out_edges();
         build_frontier_lists();
-        if (d_bits_[0]) {
-            const size_t bytes = 4 * (((size_t)V + 31) / 32);
-            for (uint32_t* b : d_bits_) cuda_check(cudaMemsetAsync(b, 0, bytes, stream_), "memset");
-        }
-        cur_ = 0;
-        step_ = 0;
-        seed_frontier(a == Algo::SSSP ? src_int : kInf);   // CC: every label is new
     }
+    cur_ = 0;
+    step_ = 0;
+    lp_all_rows_ = true;
+    err_unread_ = true;
+    // One pass writes the initial state. Both value buffers of the min-label
+    // algorithms and of LP start equal: a push superstep lowers the next
+    // buffer in place, which must hold values no lower than the current, and
+    // pull and LP supersteps may leave rows without in-edges alone.
+    BeginArgs ba{};
+    ba.algo = a;
+    ba.n = V;
+    ba.n_ghost = n_ghost_total_;
+    ba.source = a == Algo::SSSP || personalized ? src_int : kInf;
+    ba.r0 = (float)(1.0 / (double)n_vertices_);
+    ba.own[0] = d_own_[0];
+    ba.own[1] = d_own_[1];
+    ba.rank = d_rank_[0];
+    ba.outdeg = d_outdeg_;
+    ba.label_of = relabeled_ ? d_new2old_ : nullptr;
+    ba.ghost_gid = d_ghost_gid_;
+    ba.ghost = d_ghost_;
+    ba.identity = a == Algo::PR ? 0u : kInf;
+    ba.stats = d_stats_;
+    ba.n_dangling = d_n_dangling_;
+    int nc = 0;
+    auto clear = [&](uint32_t* b) {
+        if (b) ba.clear[nc++] = b;
+    };
+    if (n_parts_ > 1) {
+        clear(d_changed_[0]);
+        clear(d_changed_[1]);
+    } else if (a == Algo::LP) {
+        for (uint32_t* b : lp_.d_active) clear(b);
+        for (uint32_t* b : lp_.d_changed) clear(b);
+    } else if (frontier_) {
+        for (uint32_t* b : d_bits_) clear(b);
+    }
+    ba.seed = kInf;
+    if (frontier_) {
+        ba.out_ptr = d_out_ptr_;
+        ba.fc = frontier_cfg();
+        ba.fc.list_out = d_list_[0];
+        if (n_parts_ == 1 && a == Algo::SSSP) ba.seed = src_int;
+        else if (a == Algo::CC && cfg_.direction == GXP_DIR_AUTO) ba.list_ne = seed_all_ne_;
+    }
+    cuda_check(launch_begin(ba, stream_), "initial state");
+    if (frontier_ && ba.seed == kInf && !ba.list_ne) {
+        // several partitions' SSSP starts from the source and its cached
+        // copies, a forced push from a list of every slot; a CC run in auto
+        // direction needs the count of all slots alone, the same every time
+        seed_frontier(a == Algo::SSSP ? src_int : kInf);
+        if (a == Algo::CC && cfg_.direction == GXP_DIR_AUTO) {
+            cuda_check(cudaMemcpyAsync(&seed_all_ne_, &d_stats_[0].list_ne, 8, cudaMemcpyDeviceToHost, stream_),
+                       "frontier size");
+            cuda_check(cudaStreamSynchronize(stream_), "frontier size");
+        }
+    }
+    lru_reset(a == Algo::SSSP || personalized ? src_int : kInf);
     algo_ = a;
     ppr_source_ = ppr_source;
     source_ = source;
@@ -1075,7 +1103,9 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
                     (algo_ == Algo::LP && g == GXP_GEN_LABEL && m == GXP_MERGE_MODE && ap == GXP_APPLY_SET);
     if (!ok) fail(GXP_E_UNSUPPORTED, "unsupported (msggen, merge, apply) template for this algorithm");
     const int nx = cur_ ^ 1;
-    cuda_check(cudaEventRecord(ev_a_, stream_), "event");
+    err_unread_ = true;
+    if (!h_steps_) cuda_check(cudaHostAlloc(&h_steps_, sizeof(StepReport), cudaHostAllocMapped), "pinned reports");
+    if (timed_) cuda_check(cudaEventRecord(ev_a_, stream_), "event");
     if (algo_ == Algo::LP) {
         LpArgs l{};
         l.parts = lp_.d_parts;
@@ -1130,9 +1160,14 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
         const SellArgs a = sell_args();
         cuda_check(launch_superstep_sell(algo_, a, stream_), "superstep kernel");
     }
-    cuda_check(cudaEventRecord(ev_k_, stream_), "event");
+    if (timed_) cuda_check(cudaEventRecord(ev_k_, stream_), "event");
     if (n_parts_ > 1) {
         SyncArgs s{};
+        s.report = &h_steps_->sum[(step_ + 1) % kStatRing];   // mapped: the same address on the device
+        s.err = d_err_;
+        s.report_err = &h_steps_->err;
+        s.max_words = max_words_;
+        *s.report = StepSum{};   // read by the host only after the exchange has written it
         s.parts = d_parts_;
         s.n_parts = n_parts_;
         s.changed_bits = d_changed_[step_ & 1];
@@ -1182,7 +1217,7 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
             }
         }
     }
-    cuda_check(cudaEventRecord(ev_b_, stream_), "event");
+    if (timed_) cuda_check(cudaEventRecord(ev_b_, stream_), "event");
     cur_ = nx;
     ++step_;
     if (want || step_ - accounted_ >= 32) account(false);
@@ -1207,21 +1242,16 @@ void Engine::account_step(const StepSum& s) {
 // index is returned, else 0.
 uint64_t Engine::account(bool stop_at_quiet) {
     if (accounted_ == step_) return 0;
+    // several partitions report as they go; one partition's sums are taken here
+    if (n_parts_ == 1)
+        cuda_check(launch_step_sums(d_stats_, accounted_ + 1, step_, d_err_, h_steps_, stream_), "superstep sums");
     cuda_check(cudaStreamSynchronize(stream_), "superstep");
-    ring_host_.resize(kStatRing);
-    cuda_check(cudaMemcpy(ring_host_.data(), d_stats_, sizeof(StepStats) * kStatRing, cudaMemcpyDeviceToHost),
-               "read stats");
-    check_device_error();
+    err_unread_ = n_parts_ > 1;   // the last exchange's kernels run after its report
+    if (h_steps_->err) check_device_error();
     uint64_t quiet = 0;
     for (uint64_t t = accounted_ + 1; t <= step_; ++t) {
-        const StepStats& s = ring_host_[t % kStatRing];
-        unsigned long long ch = 0, dg = 0, l1 = 0;
-        for (int i = 0; i < kStatLanes; ++i) {
-            ch += s.changed[i];
-            dg += s.dangling_fx[i];
-            l1 += s.l1_fx[i];
-        }
-        account_step(StepSum{ch, dg, l1, s.pushed, s.push_edges});
+        const StepSum& s = h_steps_->sum[t % kStatRing];
+        account_step(s);
         if (n_parts_ > 1) {
             // every exchange marks its superstep's slot; a missing mark means
             // the caches and upload lists of that superstep were never delivered
@@ -1234,6 +1264,7 @@ uint64_t Engine::account(bool stop_at_quiet) {
             if (s.skipped) st_.syncs_skipped++;
             else st_.syncs_done++;
         }
+        const unsigned long long ch = s.changed;
         if (stop_at_quiet && ch == 0) {
             quiet = t;
             break;
@@ -1510,8 +1541,7 @@ void Engine::sync_result(uint32_t part, uint32_t* ids, void* vals, uint64_t cap,
         if (skipped) *skipped = 1;
         return;
     }
-    StepStats s;
-    cuda_check(cudaMemcpy(&s, d_stats_ + (step_ % kStatRing), sizeof(s), cudaMemcpyDeviceToHost), "read stats");
+    const StepSum& s = h_steps_->sum[step_ % kStatRing];
     uint32_t n = 0;
     if (!s.skipped) cuda_check(cudaMemcpy(&n, d_part_counts_ + part, 4, cudaMemcpyDeviceToHost), "read count");
     *n_out = n;
@@ -1561,6 +1591,7 @@ uint32_t Engine::run(gxp_algo algo, uint32_t source, float damping, uint32_t max
             cuda_check(cudaEventRecord(ev_b_, stream_), "event");
             cuda_check(cudaStreamSynchronize(stream_), "run");
             const uint64_t done = h_run_->step;
+            err_unread_ = false;
             if (done == 0 || h_run_->err != 0) check_device_error();   // a wait that ran out, a bad index
             if (done <= r.t0 || done > r.limit) fail(GXP_E_CUDA, "device-driven run lost its step counter");
             bar_passed_ = h_run_->passed;
@@ -1577,15 +1608,15 @@ uint32_t Engine::run(gxp_algo algo, uint32_t source, float damping, uint32_t max
         return steps;
     }
     struct Guard {
-        bool &early_exit, &queue;
+        bool &early_exit, &queue, &timed;
         ~Guard() {
             early_exit = false;
-            queue = true;
+            queue = timed = true;
         }
-    } guard{early_exit_, queue_};
+    } guard{early_exit_, queue_, timed_};
     if (algo_ == Algo::PR) {
         for (; steps < max_steps; ++steps) {
-            queue_ = steps + 1 == max_steps;
+            queue_ = timed_ = steps + 1 == max_steps;
             superstep(algo, g, m, ap, false);
         }
         account(false);
@@ -1601,6 +1632,7 @@ uint32_t Engine::run(gxp_algo algo, uint32_t source, float damping, uint32_t max
         const uint32_t k = std::min<uint32_t>(chunk, max_steps - steps);
         for (uint32_t i = 0; i < k; ++i) {
             queue_ = steps + i + 1 == max_steps;   // (a run that ends earlier ends on an empty queue)
+            timed_ = i + 1 == k;
             superstep(algo, g, m, ap, false);
         }
         const uint64_t quiet = account(true);
@@ -1622,14 +1654,18 @@ void Engine::get_values(uint32_t part, void* out, uint64_t n) {
     }
     if (n != cnt) fail(GXP_E_INVAL, "n must equal the number of vertices requested");
     const void* src = algo_ == Algo::PR ? (const void*)(d_rank_[cur_] + off) : (const void*)(d_own_[cur_] + off);
-    if (relabeled_) {   // internal order -> input ids
-        cuda_check(launch_permute_u32((const uint32_t*)src, d_old2new_, (uint32_t)cnt, d_perm_tmp_, false, stream_),
-                   "map values");
-        src = d_perm_tmp_;
+    if (relabeled_) {   // internal order -> input ids, straight into the caller's array if it is this device's
+        cudaPointerAttributes at{};
+        const bool direct = cudaPointerGetAttributes(&at, out) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
+                            at.device == device_ && ((uintptr_t)out & 3u) == 0;
+        if (!direct) cudaGetLastError();
+        uint32_t* to = direct ? (uint32_t*)out : d_perm_tmp_;
+        cuda_check(launch_permute_u32((const uint32_t*)src, d_old2new_, (uint32_t)cnt, to, false, stream_), "map values");
+        src = to;
     }
-    cuda_check(cudaMemcpyAsync(out, src, 4 * cnt, cudaMemcpyDefault, stream_), "copy values");
+    if (src != out) cuda_check(cudaMemcpyAsync(out, src, 4 * cnt, cudaMemcpyDefault, stream_), "copy values");
     cuda_check(cudaStreamSynchronize(stream_), "copy values");
-    check_device_error();
+    if (err_unread_) check_device_error();
 }
 
 void Engine::set_values(uint32_t part, const void* in, uint64_t n) {

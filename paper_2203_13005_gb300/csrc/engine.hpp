@@ -89,8 +89,8 @@ private:
     uint32_t* upload_u32(const std::vector<uint32_t>& h, size_t n_pad);
     uint64_t account(bool stop_at_quiet);
     void account_step(const StepSum& s);
-    std::vector<StepStats> ring_host_;
     void check_device_error();
+    bool err_unread_ = false;   // kernels that may set the error word ran since it was last read
     void copy_in(void* dst, const void* src, size_t bytes);   // host or device src -> host dst
     void load_csc_device(HostPart& hp, uint64_t n_edges, const void* col_ptr, const uint32_t* src,
                          const uint32_t* weights);
@@ -161,6 +161,7 @@ private:
     void lru_reset(uint32_t source_int);
     uint32_t sync_blocks_x_ = 0, max_words_ = 0;
     StepStats* d_stats_ = nullptr;
+    unsigned long long* d_n_dangling_ = nullptr;   // vertices without out-edges
     uint32_t* d_err_ = nullptr;
     bool weighted_ = false;
 
@@ -206,6 +207,7 @@ private:
     uint32_t* d_out_w_ = nullptr;
     uint2* d_list_[2] = {nullptr, nullptr};
     uint64_t list_cap_ = 0;
+    unsigned long long seed_all_ne_ = 0;   // the frontier count of all slots (a CC run's start), once known
     uint32_t n_slots_ = 0;         // push sources: the vertices, then (several partitions) the cached copies
     void build_out_edges();
     void build_frontier_lists();
@@ -237,6 +239,8 @@ private:
     GridBar* d_bar_ = nullptr;     // the run's grid barrier, zero when allocated
     uint64_t bar_passed_ = 0;      // barriers passed on it
     RunOut* h_run_ = nullptr;      // pinned: what a launch of a run reports
+    StepReport* h_steps_ = nullptr;   // pinned: what other supersteps report
+    bool timed_ = true;            // the coming superstep records its events (inside gxp_run: a chunk's last)
     std::vector<uint32_t> h_old2new_;   // host copy of the renumbering (source ids)
     SellArgs sell_args() const;
     SweepArgs sweep_args() const;

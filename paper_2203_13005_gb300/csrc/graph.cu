@@ -79,35 +79,70 @@ __global__ void k_csc_import(const uint64_t* __restrict__ cp64, uint32_t n, uint
 // ------------------------------------------------------- initial values
 
 
-__global__ void k_init_values(int algo, uint32_t ppr_source, uint32_t n, uint32_t source, uint32_t* own,
-                              float* rank, const uint32_t* outdeg, StepStats* st, const uint32_t* label_of) {
-    unsigned long long dang = 0;
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        if (algo == (int)Algo::SSSP) {
-            own[v] = (v == source) ? 0u : kInf;
-        } else if (algo == (int)Algo::CC || algo == (int)Algo::LP) {
-            own[v] = label_of ? label_of[v] : v;   // CC / LP labels are input ids
-        } else {
-            // PageRank: r_0 = 1/N everywhere; personalized PageRank: r_0 = e_source
-            const float r0 = ppr_source == kInf ? (float)(1.0 / (double)n) : (v == ppr_source ? 1.0f : 0.0f);
-            rank[v] = r0;
-            const uint32_t od = outdeg[v];
-            own[v] = __float_as_uint(od ? __fdiv_rn(r0, (float)od) : 0.0f);
-            if (od == 0u) dang += fx_of(r0);
-        }
+// The initial state of a run (BeginArgs) in one launch: a run used to take
+// nine operations (~35 us of enqueueing) to set it up.
+__global__ void __launch_bounds__(256) k_begin(const BeginArgs a) {
+    const uint32_t t0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    const bool pr = a.algo == Algo::PR, personalized = pr && a.source != kInf;
+    auto rank0 = [&](uint32_t v) { return personalized ? (v == a.source ? 1.0f : 0.0f) : a.r0; };
+    // the value other vertices gather of vertex v
+    auto value = [&](uint32_t v) -> uint32_t {
+        if (a.algo == Algo::SSSP) return v == a.source ? 0u : kInf;
+        if (!pr) return a.label_of ? a.label_of[v] : v;   // CC / LP labels are input ids
+        const uint32_t od = a.outdeg[v];
+        return __float_as_uint(od ? __fdiv_rn(rank0(v), (float)od) : 0.0f);
+    };
+    for (uint64_t v = t0; v < a.n; v += stride) {
+        const uint32_t x = value((uint32_t)v);
+        a.own[0][v] = x;
+        if (pr) a.rank[v] = rank0((uint32_t)v);
+        else a.own[1][v] = x;
     }
-    if (algo == (int)Algo::PR) {
+    for (uint64_t g = t0; g < a.n_ghost; g += stride) a.ghost[g] = value(a.ghost_gid[g]);
+    const uint32_t words = (a.n + 31u) / 32u;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) dang += __shfl_xor_sync(kFull, dang, o);
-        if ((threadIdx.x & 31) == 0 && dang)
-            atomicAdd(&st->dangling_fx[(blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32) % kStatLanes], dang);
+    for (int k = 0; k < 5; ++k)
+        if (a.clear[k])
+            for (uint32_t i = t0; i < words; i += stride) a.clear[k][i] = 0u;
+    for (uint32_t slot = blockIdx.x; slot < (uint32_t)kStatRing; slot += gridDim.x) {
+        unsigned long long* z = reinterpret_cast<unsigned long long*>(a.stats + slot);
+        for (uint32_t i = threadIdx.x; i < sizeof(StepStats) / 8; i += blockDim.x) z[i] = 0ull;
+    }
+    if (blockIdx.x != 0) return;
+    __syncthreads();   // slot 0 is block 0's
+    if (a.seed != kInf) {
+        const uint32_t deg = a.out_ptr[a.seed + 1] - a.out_ptr[a.seed], items = frontier_items(deg);
+        for (uint32_t k = threadIdx.x; k < items; k += blockDim.x) {
+            if (k < a.fc.list_cap) a.fc.list_out[k] = make_uint2(a.seed, k);
+            else atomicOr(a.fc.err, kErrBounds);
+        }
+        if (threadIdx.x == 0) a.stats->list_ne = list_pack(items, deg);
+    } else if (threadIdx.x == 0) {
+        a.stats->list_ne = a.list_ne;
+    }
+    if (threadIdx.x == 0) {
+        // the identity slots that empty SELL slots read
+        a.own[0][a.n] = a.identity;
+        a.own[1][a.n] = a.identity;
+        a.ghost[a.n_ghost] = a.identity;
+        if (pr)   // every dangling vertex starts with the same rank: an exact multiple
+            a.stats->dangling_fx[0] = personalized ? (a.outdeg[a.source] ? 0ull : fx_of(1.0f))
+                                                   : *a.n_dangling * fx_of(a.r0);
     }
 }
 
-__global__ void k_identity_slots(uint32_t* a, uint32_t* b, uint32_t* c, uint32_t v) {
-    *a = v;
-    *b = v;
-    *c = v;
+__global__ void __launch_bounds__(256) k_count_dangling(const uint32_t* __restrict__ outdeg, uint32_t n,
+                                                        unsigned long long* out) {
+    uint32_t c = 0;
+    for (uint64_t v = blockIdx.x * 256ull + threadIdx.x; v < n; v += gridDim.x * 256ull) c += outdeg[v] == 0u;
+    c = __reduce_add_sync(kFull, c);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, (unsigned long long)c);
+}
+
+__global__ void __launch_bounds__(32) k_step_sums(const StepStats* ring, uint64_t first, const uint32_t* err,
+                                                  StepReport* out) {
+    const uint64_t slot = (first + blockIdx.x) % kStatRing;
+    report_step(ring + slot, &out->sum[slot], err, &out->err);
 }
 
 __global__ void k_init_ghosts(uint32_t n_ghost, const uint32_t* __restrict__ gid,
@@ -129,6 +164,7 @@ __device__ __forceinline__ uint32_t range_mask(uint32_t w, uint32_t v_lo, uint32
 
 constexpr int kSyncBlock = 256;
 
+template <int kThreads = kSyncBlock>
 __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t* s_warp, uint32_t& total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t incl = x;
@@ -140,17 +176,17 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t* s_warp
     if (lane == 31) s_warp[warp] = incl;
     __syncthreads();
     if (warp == 0) {
-        uint32_t v = lane < kSyncBlock / 32 ? s_warp[lane] : 0u;
+        uint32_t v = lane < kThreads / 32 ? s_warp[lane] : 0u;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t y = __shfl_up_sync(kFull, v, o);
             if (lane >= o) v += y;
         }
-        if (lane < kSyncBlock / 32) s_warp[lane] = v;
+        if (lane < kThreads / 32) s_warp[lane] = v;
     }
     __syncthreads();
     const uint32_t warp_off = warp ? s_warp[warp - 1] : 0u;
-    total = s_warp[kSyncBlock / 32 - 1];
+    total = s_warp[kThreads / 32 - 1];
     __syncthreads();
     return warp_off + incl - x;
 }
@@ -158,29 +194,38 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t* s_warp
 // Whether the exchange is skipped (Section III-B3) and whether it lists the
 // changed copies, from the counts the superstep left: the changed boundary
 // vertices are counted where they change, so this is one warp's sum rather
-// than a pass over the bitmaps (9.8 us a superstep of 3 M vertices).
-__global__ void __launch_bounds__(32) k_sync_decide(const SyncArgs a) {
-    const int lane = threadIdx.x;
-    StepStats* st = a.stats_out;
+// than a pass over the bitmaps (9.8 us a superstep of 3 M vertices). Also
+// reports the superstep's sums to the host.
+__device__ __forceinline__ unsigned long long boundary_total(const StepStats* st) {   // by one warp
+    const int lane = threadIdx.x & 31;
     unsigned long long grand = __ldcg(&st->boundary[lane]) + __ldcg(&st->boundary[lane + 32]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) grand += __shfl_xor_sync(kFull, grand, o);
-    if (lane != 0) return;
-    st->boundary_changed = grand;
-    st->skipped = grand == 0 ? 1ull : 0ull;
-    st->exchanged = 1ull;
-    // the next superstep pulls anyway when its frontier would be too much
-    // work to push: its own vertices' items and out-edges, plus at least
-    // one item per changed boundary vertex for the copies that would join
-    // (each has a copy somewhere); then the copies are not listed. Nor
-    // are they when the superstep did not list its own vertices.
-    bool list = a.fc.list_out != nullptr && __ldcg(&st->unlisted) == 0ull;
-    if (list && a.fc.direction == GXP_DIR_AUTO) {
-        const unsigned long long ne = __ldcg(&st->list_ne);
-        list = ((ne >> 32) + (ne & 0xFFFFFFFFull) + grand) * (unsigned long long)a.fc.push_div <= a.fc.total_edges;
-    }
-    st->list_copies = list ? 1ull : 0ull;
+    return grand;
 }
+__device__ __forceinline__ void sync_decide(const SyncArgs& a) {   // by one warp
+    StepStats* st = a.stats_out;
+    const unsigned long long grand = boundary_total(st);
+    if ((threadIdx.x & 31) == 0) {
+        st->boundary_changed = grand;
+        st->skipped = grand == 0 ? 1ull : 0ull;
+        st->exchanged = 1ull;
+        // the next superstep pulls anyway when its frontier would be too much
+        // work to push: its own vertices' items and out-edges, plus at least
+        // one item per changed boundary vertex for the copies that would join
+        // (each has a copy somewhere); then the copies are not listed. Nor
+        // are they when the superstep did not list its own vertices.
+        bool list = a.fc.list_out != nullptr && __ldcg(&st->unlisted) == 0ull;
+        if (list && a.fc.direction == GXP_DIR_AUTO) {
+            const unsigned long long ne = __ldcg(&st->list_ne);
+            list = ((ne >> 32) + (ne & 0xFFFFFFFFull) + grand) * (unsigned long long)a.fc.push_div <= a.fc.total_edges;
+        }
+        st->list_copies = list ? 1ull : 0ull;
+    }
+    __syncwarp();
+    report_step(st, a.report, a.err, a.report_err);
+}
+__global__ void __launch_bounds__(32) k_sync_decide(const SyncArgs a) { sync_decide(a); }
 
 // Changed ∩ boundary per block of bitmap words; the last block of a
 // partition turns its counts into offsets in the partition's queue.
@@ -220,22 +265,9 @@ __global__ void __launch_bounds__(kSyncBlock) k_sync_count(const SyncArgs a) {
     }
 }
 
-// Write each partition's global data queue (ascending ids): the changed
-// boundary vertices with their new values.
-__global__ void __launch_bounds__(kSyncBlock) k_sync_write(const SyncArgs a) {
-    __shared__ uint32_t s_warp[kSyncBlock / 32];
-    if (a.stats_out->skipped) return;   // uniform: Section III-B3 skip
-    const uint32_t p = blockIdx.y;
-    const PartDev P = a.parts[p];
-    const uint32_t v_lo = P.v_begin, v_hi = P.v_begin + P.n_own;
-    const uint32_t w_lo = v_lo >> 5, w_hi = (v_hi + 31u) >> 5;
-    const uint32_t w = w_lo + blockIdx.x * kSyncBlock + threadIdx.x;
-    uint32_t bits = 0;
-    if (P.n_own && w < w_hi) bits = a.changed_bits[w] & a.boundary_bits[w] & range_mask(w, v_lo, v_hi);
-    uint32_t total;
-    uint32_t pos = block_excl_scan(__popc(bits), s_warp, total);
-    if (P.n_own == 0 || blockIdx.x * kSyncBlock >= w_hi - w_lo) return;
-    pos += a.block_offsets[p * a.blocks_x + blockIdx.x] + (uint32_t)a.gdq_base[p];
+// The pairs of a warp's 32 words (each lane's `bits` of word w) at positions
+// pos of each lane.
+__device__ __forceinline__ void write_queue(const SyncArgs& a, uint32_t bits, uint32_t pos, uint32_t w) {
     // A warp writes its 32 words' pairs one word at a time, lane l taking the
     // word's bit l: the word's vertices are 32 consecutive ids, so the value
     // load is one 128-byte line and the pairs land at consecutive positions
@@ -255,6 +287,52 @@ __global__ void __launch_bounds__(kSyncBlock) k_sync_write(const SyncArgs a) {
             a.gdq_vals[at] = a.own_val[gid];
         }
     }
+}
+
+// Write each partition's global data queue (ascending ids): the changed
+// boundary vertices with their new values.
+__global__ void __launch_bounds__(kSyncBlock) k_sync_write(const SyncArgs a) {
+    __shared__ uint32_t s_warp[kSyncBlock / 32];
+    if (a.stats_out->skipped) return;   // uniform: Section III-B3 skip
+    const uint32_t p = blockIdx.y;
+    const PartDev P = a.parts[p];
+    const uint32_t v_lo = P.v_begin, v_hi = P.v_begin + P.n_own;
+    const uint32_t w_lo = v_lo >> 5, w_hi = (v_hi + 31u) >> 5;
+    const uint32_t w = w_lo + blockIdx.x * kSyncBlock + threadIdx.x;
+    uint32_t bits = 0;
+    if (P.n_own && w < w_hi) bits = a.changed_bits[w] & a.boundary_bits[w] & range_mask(w, v_lo, v_hi);
+    uint32_t total;
+    uint32_t pos = block_excl_scan(__popc(bits), s_warp, total);
+    if (P.n_own == 0 || blockIdx.x * kSyncBlock >= w_hi - w_lo) return;
+    pos += a.block_offsets[p * a.blocks_x + blockIdx.x] + (uint32_t)a.gdq_base[p];
+    write_queue(a, bits, pos, w);
+}
+
+// The decision and the queues in one launch, a CTA per partition that scans
+// its words 1,024 at a time: for partitions of at most kQueueWords words,
+// where a launch costs more than the scan (partitions of 65,536 vertices:
+// decide + count + write 7 us, this 4).
+constexpr int kQueueBlock = 1024;
+constexpr uint32_t kQueueWords = 4096;
+__global__ void __launch_bounds__(kQueueBlock) k_sync_queue(const SyncArgs a) {
+    __shared__ uint32_t s_warp[kQueueBlock / 32];
+    const uint32_t p = blockIdx.x;
+    const bool none = boundary_total(a.stats_out) == 0ull;   // every warp sums
+    if (p == 0 && threadIdx.x < 32) sync_decide(a);
+    if (none) return;   // uniform: Section III-B3 skip
+    const PartDev P = a.parts[p];
+    const uint32_t v_lo = P.v_begin, v_hi = P.v_begin + P.n_own;
+    const uint32_t w_lo = v_lo >> 5, w_hi = P.n_own ? (v_hi + 31u) >> 5 : w_lo;
+    uint32_t run = 0;
+    for (uint32_t w0 = w_lo; w0 < w_hi; w0 += kQueueBlock) {
+        const uint32_t w = w0 + threadIdx.x;
+        const uint32_t bits = w < w_hi ? a.changed_bits[w] & a.boundary_bits[w] & range_mask(w, v_lo, v_hi) : 0u;
+        uint32_t total;
+        const uint32_t pos = block_excl_scan<kQueueBlock>((uint32_t)__popc(bits), s_warp, total);
+        write_queue(a, bits, run + pos + (uint32_t)a.gdq_base[p], w);
+        run += total;
+    }
+    if (threadIdx.x == 0) a.part_counts[p] = run;
 }
 
 // Caching (Section III-B): every cached copy of an uploaded vertex takes its
@@ -386,16 +464,24 @@ cudaError_t launch_csc_import(const uint64_t* cp64, uint32_t n, uint64_t n_edges
     return cudaGetLastError();
 }
 
-cudaError_t launch_init_values(Algo a, uint32_t ppr_source, uint32_t n, uint32_t source, uint32_t* own, float* rank,
-                               const uint32_t* outdeg, StepStats* st, const uint32_t* label_of, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    const uint32_t blocks = std::min<uint32_t>((n + 255) / 256, 152u * 8);
-    k_init_values<<<blocks, 256, 0, s>>>((int)a, ppr_source, n, source, own, rank, outdeg, st, label_of);
+cudaError_t launch_begin(const BeginArgs& a, cudaStream_t s) {
+    const uint64_t items = std::max<uint64_t>(a.n, a.n_ghost);
+    const uint32_t blocks = (uint32_t)std::min<uint64_t>((items + 255) / 256, 152u * 8);
+    k_begin<<<blocks, 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_identity_slots(uint32_t* a, uint32_t* b, uint32_t* c, uint32_t v, cudaStream_t s) {
-    k_identity_slots<<<1, 1, 0, s>>>(a, b, c, v);
+cudaError_t launch_count_dangling(const uint32_t* outdeg, uint32_t n, unsigned long long* out, cudaStream_t s) {
+    const cudaError_t e = cudaMemsetAsync(out, 0, 8, s);
+    if (e != cudaSuccess) return e;
+    k_count_dangling<<<std::min<uint32_t>((n + 255) / 256, 152u * 8), 256, 0, s>>>(outdeg, n, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_step_sums(const StepStats* ring, uint64_t first, uint64_t last, const uint32_t* err, StepReport* out,
+                             cudaStream_t s) {
+    if (last < first || last - first >= (uint64_t)kStatRing) return cudaErrorInvalidValue;
+    k_step_sums<<<(unsigned)(last - first + 1), 32, 0, s>>>(ring, first, err, out);
     return cudaGetLastError();
 }
 
@@ -409,8 +495,12 @@ cudaError_t launch_init_ghosts(Algo, uint32_t n_ghost, const uint32_t* gid, cons
 
 cudaError_t launch_sync(const SyncArgs& a, uint32_t, cudaStream_t s) {
     if (a.n_parts == 0 || a.blocks_x == 0) return cudaSuccess;
-    k_sync_decide<<<1, 32, 0, s>>>(a);
-    if (a.queue) {
+    if (a.queue && a.max_words <= kQueueWords) {
+        k_sync_queue<<<a.n_parts, kQueueBlock, 0, s>>>(a);
+    } else {
+        k_sync_decide<<<1, 32, 0, s>>>(a);
+    }
+    if (a.queue && a.max_words > kQueueWords) {
         dim3 grid(a.blocks_x, a.n_parts);
         k_sync_count<<<grid, kSyncBlock, 0, s>>>(a);
         k_sync_write<<<grid, kSyncBlock, 0, s>>>(a);

@@ -161,6 +161,37 @@ struct StepStats {
     unsigned long long unlisted;
     unsigned long long list_cursor;
 };
+// A superstep's stats, summed over their lanes.
+struct StepSum {
+    unsigned long long changed, dangling_fx, l1_fx, pushed, push_edges;
+    unsigned long long boundary_changed, skipped, exchanged, downloads;   // several partitions
+};
+// What supersteps leave in pinned host memory, by ring slot: written by the
+// exchange's decision (several partitions) or by launch_step_sums (one) and
+// read once the stream is synchronized, in place of a copy of the ring.
+struct StepReport {
+    StepSum sum[kStatRing];
+    uint32_t err, pad;      // the error word
+};
+#ifdef __CUDACC__
+// by one warp
+__device__ __forceinline__ void report_step(const StepStats* st, StepSum* out, const uint32_t* err, uint32_t* err_out) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long c = __ldcg(&st->changed[lane]) + __ldcg(&st->changed[lane + 32]);
+    unsigned long long d = __ldcg(&st->dangling_fx[lane]) + __ldcg(&st->dangling_fx[lane + 32]);
+    unsigned long long l = __ldcg(&st->l1_fx[lane]) + __ldcg(&st->l1_fx[lane + 32]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
+        d += __shfl_xor_sync(0xFFFFFFFFu, d, o);
+        l += __shfl_xor_sync(0xFFFFFFFFu, l, o);
+    }
+    if (lane != 0) return;
+    *out = StepSum{c, d, l, __ldcg(&st->pushed), __ldcg(&st->push_edges), __ldcg(&st->boundary_changed),
+                   __ldcg(&st->skipped), __ldcg(&st->exchanged), __ldcg(&st->downloads)};
+    *err_out = __ldcg(err);
+}
+#endif
 __host__ __device__ constexpr unsigned long long list_pack(uint32_t items, uint32_t edges) {
     return ((unsigned long long)items << 32) | edges;
 }
@@ -435,6 +466,10 @@ struct SyncArgs {
     uint32_t* part_counts;            // [n_parts]
     uint32_t* done_ctr;               // [n_parts] arrival counters of the count kernel
     uint32_t queue;                   // 1: write the global data queue (gxp_sync returns it)
+    uint32_t max_words;               // bitmap words of the largest partition
+    StepSum* report;                  // pinned host memory: the superstep's sums
+    const uint32_t* err;
+    uint32_t* report_err;
     uint32_t blocks_x;
     StepStats* stats_out;
     // frontier lists on (push direction possible): every cached copy whose
@@ -454,10 +489,35 @@ cudaError_t launch_csc_import(const uint64_t* cp64, uint32_t n, uint64_t n_edges
 cudaError_t launch_validate_csc(const uint32_t* d_col_ptr, uint32_t n_own, const uint32_t* d_src,
                                 uint64_t n_edges, uint32_t n_local, uint32_t* d_err, cudaStream_t s);
 
-cudaError_t launch_init_values(Algo a, uint32_t ppr_source, uint32_t n_vertices, uint32_t source,
-                               uint32_t* own_cur, float* rank_cur, const uint32_t* outdeg,
-                               StepStats* stats0, const uint32_t* label_of, cudaStream_t s);
-cudaError_t launch_identity_slots(uint32_t* a, uint32_t* b, uint32_t* c, uint32_t v, cudaStream_t s);   // *a = *b = *c = v
+// The initial state of a run, in one pass: values (both buffers of the
+// min-label algorithms and LP; PageRank's ranks and messages), cached copies,
+// identity slots, stat ring, bitmaps, and the seed of the frontier.
+struct BeginArgs {
+    Algo algo;
+    uint32_t n, n_ghost;
+    uint32_t source;             // SSSP: the source; PPR: likewise; else kInf
+    float r0;                    // PageRank's 1 / N
+    uint32_t* own[2];
+    float* rank;
+    const uint32_t* outdeg;
+    const uint32_t* label_of;    // CC / LP: input ids of renumbered vertices, or nullptr
+    const uint32_t* ghost_gid;
+    uint32_t* ghost;
+    uint32_t identity;           // of the merge
+    StepStats* stats;            // [kStatRing]
+    const unsigned long long* n_dangling;   // vertices without out-edges
+    uint32_t* clear[5];          // bitmaps of the vertices, or nullptr
+    uint32_t seed;               // vertex whose items are the first frontier, or kInf
+    const uint32_t* out_ptr;
+    FrontierCfg fc;              // list_out: the list the seed goes to
+    unsigned long long list_ne;  // the first frontier's count, when no vertex is seeded
+};
+cudaError_t launch_begin(const BeginArgs& a, cudaStream_t s);
+// *out = vertices without out-edges
+cudaError_t launch_count_dangling(const uint32_t* outdeg, uint32_t n, unsigned long long* out, cudaStream_t s);
+// report sums of supersteps first .. last (one partition), and the error word
+cudaError_t launch_step_sums(const StepStats* ring, uint64_t first, uint64_t last, const uint32_t* err, StepReport* out,
+                             cudaStream_t s);
 cudaError_t launch_init_ghosts(Algo a, uint32_t n_ghost_total, const uint32_t* ghost_gid_all,
                                const uint32_t* own_cur, uint32_t* ghost, cudaStream_t s);
 
@@ -467,10 +527,6 @@ cudaError_t launch_superstep_sell(Algo a, const SellArgs& args, cudaStream_t s);
 // Grid barrier state of a persistent launch, zero when it starts.
 struct GridBar {
     unsigned long long count;   // arrivals so far; top bit: a wait gave up
-};
-// A superstep's stats, summed over their lanes.
-struct StepSum {
-    unsigned long long changed, dangling_fx, l1_fx, pushed, push_edges;
 };
 constexpr uint32_t kRunChunk = 32;   // supersteps per launch of a run (the stat ring holds 64)
 // What a launch of several supersteps leaves in pinned host memory. The host

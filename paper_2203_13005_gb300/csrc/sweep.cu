@@ -773,15 +773,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_sweep(const SweepArgs a, const 
             const uint64_t mine = run.t0 + (uint32_t)warp;
             if (mine < t) {
                 const StepStats* st = a.stats + (mine + 1) % kStatRing;
-                const unsigned long long c = warp_sum_u62(__ldcg(&st->changed[lane]) + __ldcg(&st->changed[lane + 32]));
-                const unsigned long long d =
-                    warp_sum_u62(__ldcg(&st->dangling_fx[lane]) + __ldcg(&st->dangling_fx[lane + 32]));
-                const unsigned long long l = warp_sum_u62(__ldcg(&st->l1_fx[lane]) + __ldcg(&st->l1_fx[lane + 32]));
-                if (lane == 0) run.out->sum[warp] = StepSum{c, d, l, __ldcg(&st->pushed), __ldcg(&st->push_edges)};
+                report_step(st, &run.out->sum[warp], a.err, &run.out->err);
             }
             if (tid == 0) {
                 run.out->passed = passed;
-                run.out->err = __ldcg(a.err);
                 run.out->step = t;
             }
         }
