@@ -28,6 +28,15 @@ void destroy_graph(cudaGraphExec_t& g) {
 
 }  // namespace
 
+std::vector<uint4> units_longest_first(const std::vector<uint4>& units) {
+    std::vector<uint64_t> at(kUnitEdges + 2, 0);
+    for (const uint4& u : units) ++at[kUnitEdges - u.z + 1];
+    for (uint32_t k = 0; k <= kUnitEdges; ++k) at[k + 1] += at[k];
+    std::vector<uint4> sorted(units.size());
+    for (const uint4& u : units) sorted[at[kUnitEdges - u.z]++] = u;
+    return sorted;
+}
+
 void Engine::free_batch() {
     Batch& b = batch_;
     if (b.s_h2d) cudaStreamSynchronize(b.s_h2d);
@@ -74,13 +83,8 @@ void Engine::prepare_batch(bool streamed) {
         uint32_t wmax = 0;
         for (uint32_t x : hp.w) wmax = std::max(wmax, x);
         b.packed = packable(V, wmax);
+        b.no_sat = V * (uint64_t)wmax < 0xFFFFFFFFull ? 1u : 0u;   // a path has fewer than V edges
         b.esize = b.packed ? 4u : 8u;
-        b.d_units = (uint4*)dalloc(sizeof(uint4) * std::max<size_t>(b.units.size(), 1));
-        if (!b.units.empty()) {
-            before_h2d("upload units");
-            cuda_check(cudaMemcpy(b.d_units, b.units.data(), sizeof(uint4) * b.units.size(), cudaMemcpyHostToDevice),
-                       "upload units");
-        }
         b.d_dist = (uint32_t*)dalloc(sizeof(uint32_t) * 64 * V);
         const size_t words = (V + 31) / 32 + 1;
         b.d_frontier[0] = (uint32_t*)dalloc(4 * words);
@@ -100,6 +104,18 @@ void Engine::prepare_batch(bool streamed) {
         cuda_check(cudaEventCreate(&b.ev_t1), "event");
         b.ready = true;
     }
+    // units in destination order for streamed edge blocks, longest first for
+    // resident edges
+    auto upload_units = [&](const std::vector<uint4>& u) {
+        uint4* d = (uint4*)dalloc(sizeof(uint4) * std::max<size_t>(u.size(), 1));
+        if (!u.empty()) {
+            before_h2d("upload units");
+            cuda_check(cudaMemcpy(d, u.data(), sizeof(uint4) * u.size(), cudaMemcpyHostToDevice), "upload units");
+        }
+        return d;
+    };
+    if (streamed && !b.d_units) b.d_units = upload_units(b.units);
+    if (!streamed && !b.d_units_long) b.d_units_long = upload_units(units_longest_first(b.units));
     auto fill = [&](void* dst, bool packed) {
         if (packed) {
             uint32_t* d = static_cast<uint32_t*>(dst);
@@ -154,9 +170,11 @@ void Engine::superstep_batch(const std::vector<uint64_t>& cuts, bool streamed, b
     if (!dry) cuda_check(cudaMemsetAsync(fr_next, 0, 4 * words, stream_), "memset");
     cuda_check(cudaMemsetAsync(b.d_changed, 0, 8 * std::max<size_t>(nb, 1), stream_), "memset");
     MsArgs a{};
-    a.units = b.d_units;
+    a.units = streamed ? b.d_units : b.d_units_long;
     a.packed = streamed && b.packed;
     a.dist = b.d_dist;
+    a.no_sat = b.no_sat;
+    a.idle_mask = dry ? 0ull : b.idle_mask;   // the tuner times full rows, whatever this call asks for
     a.frontier_cur = fr_cur;
     a.frontier_next = fr_next;
     a.active = dry ? nullptr : b.d_active;
@@ -245,6 +263,7 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
     const bool pipelined = !streamed || opts.pipelined != 0;
     prepare_batch(streamed);
     Batch& b = batch_;
+    b.idle_mask = n_src == 64 ? 0ull : ~0ull << n_src;   // the slots without a source are not computed
     const uint64_t E = b.unit_edge.back(), V = n_vertices_;
     const uint64_t words = (V + 31) / 32 + 1;
     gxp_batch_report r{};
@@ -318,6 +337,7 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
             a.edges = b.d_ring[0];
             a.edge_base = 0;
             a.dist = b.d_dist;
+            a.no_sat = b.no_sat;
             a.frontier_cur = b.d_frontier[0];
             a.frontier_next = b.d_frontier[1];
             a.changed = b.d_changed;
@@ -415,7 +435,7 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
     // CUDA graphs of one superstep, one per frontier parity
     const bool use_graph = opts.use_graph != 0;
     if (use_graph && (!b.graph[0] || b.graph_block_edges != block_edges || b.graph_streamed != streamed ||
-                      b.graph_pipelined != pipelined)) {
+                      b.graph_pipelined != pipelined || b.graph_idle != b.idle_mask)) {
         destroy_graph(b.graph[0]);
         destroy_graph(b.graph[1]);
         cuda_check(cudaStreamSynchronize(stream_), "sync");
@@ -431,6 +451,7 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
         b.graph_block_edges = block_edges;
         b.graph_streamed = streamed;
         b.graph_pipelined = pipelined;
+        b.graph_idle = b.idle_mask;
     }
 
     cuda_check(cudaMemsetAsync(b.d_active, 0, 8, stream_), "memset");
@@ -445,13 +466,15 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
         cuda_check(cudaMemsetAsync(b.d_loop_changed, 0, 8 * 4, stream_), "memset");
         cuda_check(cudaMemsetAsync(b.d_bar, 0, sizeof(GridBar), stream_), "memset");
         MsArgs a{};
-        a.units = b.d_units;
+        a.units = b.d_units_long;
         a.u_begin = 0;
         a.u_end = b.units.size();
         a.edges = b.d_edges;
         a.packed = 0;
         a.edge_base = 0;
         a.dist = b.d_dist;
+        a.no_sat = b.no_sat;
+        a.idle_mask = b.idle_mask;
         a.active = b.d_active;
         cuda_check(cudaEventRecord(b.ev_t0, stream_), "event");
         const cudaError_t e = launch_msssp_loop(a, b.d_frontier, b.d_loop_changed, words, max_steps, b.d_bar,

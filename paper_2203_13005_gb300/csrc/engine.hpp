@@ -170,12 +170,15 @@ private:
         bool ready = false, resident = false, pinned_ready = false;
         std::vector<uint4> units;          // {dst, first edge, edges, split}
         std::vector<uint64_t> unit_edge;   // first edge of each unit, + total at the end
-        uint4* d_units = nullptr;
+        uint4* d_units = nullptr;          // as units, for streamed blocks
+        uint4* d_units_long = nullptr;     // longest first, for resident edges
         void* h_edges = nullptr;           // pinned streamed edges, destination order (esize bytes each)
         void* d_edges = nullptr;           // resident copy, (source, weight) uint2
         void* d_ring[3] = {nullptr, nullptr, nullptr};
         uint32_t esize = 8;                // streamed edge: 8 = (source, weight) uint2, 4 = packed uint32
         bool packed = false;
+        uint32_t no_sat = 0;
+        uint64_t idle_mask = 0, graph_idle = 0;   // slots without a source: of this call, of the captured graphs
         uint64_t ring_edges = 0;
         uint32_t* d_dist = nullptr;        // [V][64]
         uint32_t* d_frontier[3] = {nullptr, nullptr, nullptr};   // [2]: the persistent run's third bitmap

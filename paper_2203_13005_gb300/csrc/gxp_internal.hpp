@@ -8,6 +8,7 @@
 #include <cstdint>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "gxp.h"
@@ -320,6 +321,11 @@ constexpr uint32_t kPackSrcBits = 24;
 inline bool packable(uint64_t n_vertices, uint32_t max_weight) {
     return n_vertices <= (1ull << kPackSrcBits) && max_weight < 256u;
 }
+// Work units (edges in .z, at most kUnitEdges) longest first, stably: dealt
+// out round robin, every warp then gets about as many edges (in destination
+// order the warps' shares of R-MAT 20 spread by tens of percent and a
+// superstep waited for the longest).
+std::vector<uint4> units_longest_first(const std::vector<uint4>& units);
 struct MsArgs {
     const uint4* units;          // {dst, first edge (global), edges, split-row flag}
     uint64_t u_begin, u_end;     // this block's units
@@ -334,7 +340,19 @@ struct MsArgs {
     unsigned long long* active;  // nullable: running count of in-edges whose source was in the frontier
     uint32_t* slot_improved;     // nullable: [2] bit s of word 0 / s - 32 of word 1 = slot s improved
     uint64_t idle_mask;          // slots to skip (no query in them); 0 = compute all 64
+    uint32_t no_sat;             // 1: n_vertices x the largest weight is below 2^32 - 1, no sum saturates
 };
+
+// f(integral_constant<int, lanes>) with the lanes of four slots each that hold
+// the slots in use (the highest of `busy` decides): 16 for 64 slots down to 1
+template <class F>
+inline cudaError_t with_slot_lanes(uint64_t busy, F f) {
+    if (busy >> 32) return f(std::integral_constant<int, 16>{});
+    if (busy >> 16) return f(std::integral_constant<int, 8>{});
+    if (busy >> 8) return f(std::integral_constant<int, 4>{});
+    if (busy >> 4) return f(std::integral_constant<int, 2>{});
+    return f(std::integral_constant<int, 1>{});
+}
 
 // Finished query slots whose columns are copied out as result vectors.
 struct GatherList {
@@ -346,7 +364,7 @@ struct GatherList {
 // Arguments of the personalized-PageRank superstep over 64 query slots
 // (serving). Matrices are [V][64] fp32, one 256-byte row per vertex.
 struct PprArgs {
-    const uint4* units;              // {dst, first edge, edges, partial index + 1 | 0}
+    const uint4* units;              // {dst, first edge, edges, partial index + 1 | 0}, longest first
     uint64_t n_units;                // covers every vertex (empty rows too)
     const uint32_t* src;             // source id of each edge, destination order
     const uint2* split_rows;         // [n_split_rows + 1] {row, first partial}; last .y = n_partials

@@ -9,10 +9,12 @@
 //        r_{t+1} = d * A^T D^-1 r_t + ((1 - d) + d * D_t) e_s
 //    (Jacobi; D_t = rank mass on dangling vertices, returned to the source s
 //    together with the teleport), with fp32 messages c = r * (1 / outdeg)
-//    and exact fixed-point dangling sums per slot. Lane l of a warp holds
-//    slots 2l and 2l+1; lanes whose slots are both idle skip every load and
-//    store.
-//      k_ppr_units   one warp per work unit (<= 256 in-edges of one vertex):
+//    and exact fixed-point dangling sums per slot. A lane holds four slots
+//    (128-bit loads), so LG lanes hold a row: 16 for 64 slots, fewer when
+//    only the first slots hold queries; a warp works on 32 / LG units at once,
+//    each summed in its own edge order, so a slot's result does not depend
+//    on LG.
+//      k_ppr_units   LG lanes per work unit (<= 256 in-edges of one vertex):
 //                    sums the sources' message rows in edge order; a vertex
 //                    held by one unit is applied at once, a vertex split
 //                    over several units leaves one partial row per unit;
@@ -30,7 +32,7 @@ namespace {
 
 constexpr int kSvBlock = 256;
 constexpr int kSvWarps = kSvBlock / 32;
-constexpr int kSvUnroll = 8;
+constexpr int kSvUnroll = 4;   // message rows in flight per lane
 constexpr int kTileRows = 64;   // rows per transpose tile
 
 uint32_t grid_for(uint64_t items, uint64_t per_block) {
@@ -56,8 +58,8 @@ namespace {
 // (kInf for an idle slot) and (1 - d) + d * D_t, D_t from the exact
 // fixed-point sum of the slot's dangling mass.
 struct PprSlots {
-    float2 d[32], add[32];
-    uint2 src[32];
+    float4 d[16], add[16];
+    uint4 src[16];
     unsigned long long dang[64];   // this block's dangling mass of r_{t+1}
     uint32_t warps_done;
 
@@ -78,18 +80,28 @@ struct PprSlots {
 
     // MSGApply of vertex v (1 / out-degree inv, 0 if dangling) for lane l's
     // slots with merged sum: r = d * sum, plus the source term at the slot's
-    // source; message r * inv; ranks only in a slot's last superstep
-    __device__ void apply(const PprArgs& a, uint32_t v, float inv, float2 sum, int l) {
-        const float2 dl = d[l], al = add[l];
-        const uint2 sl = src[l];
-        float2 r = make_float2(dl.x * sum.x, dl.y * sum.y);
-        if (v == sl.x) r.x += al.x;
-        if (v == sl.y) r.y += al.y;
-        reinterpret_cast<float2*>(a.msg_nxt)[(uint64_t)v * 32u + l] = make_float2(r.x * inv, r.y * inv);
-        if ((a.finish_mask >> (2 * l)) & 3ull) reinterpret_cast<float2*>(a.rank)[(uint64_t)v * 32u + l] = r;
+    // source; message r * inv; ranks only in a slot's last superstep. Rounded
+    // operation by operation, so that every lane grouping gives the same bits.
+    __device__ void apply(const PprArgs& a, uint32_t v, float inv, float4 sum, uint32_t l) {
+        const float4 dl = d[l];
+        const uint4 sl = src[l];
+        float4 r = make_float4(__fmul_rn(dl.x, sum.x), __fmul_rn(dl.y, sum.y), __fmul_rn(dl.z, sum.z),
+                               __fmul_rn(dl.w, sum.w));
+        if (v == sl.x || v == sl.y || v == sl.z || v == sl.w) {
+            const float4 al = add[l];
+            if (v == sl.x) r.x = __fadd_rn(r.x, al.x);
+            if (v == sl.y) r.y = __fadd_rn(r.y, al.y);
+            if (v == sl.z) r.z = __fadd_rn(r.z, al.z);
+            if (v == sl.w) r.w = __fadd_rn(r.w, al.w);
+        }
+        reinterpret_cast<float4*>(a.msg_nxt)[(uint64_t)v * 16u + l] =
+            make_float4(r.x * inv, r.y * inv, r.z * inv, r.w * inv);
+        if ((a.finish_mask >> (4 * l)) & 15ull) reinterpret_cast<float4*>(a.rank)[(uint64_t)v * 16u + l] = r;
         if (inv == 0.0f) {
-            atomicAdd(&dang[2 * l], fx_of(r.x));
-            atomicAdd(&dang[2 * l + 1], fx_of(r.y));
+            if (r.x != 0.0f) atomicAdd(&dang[4 * l], fx_of(r.x));
+            if (r.y != 0.0f) atomicAdd(&dang[4 * l + 1], fx_of(r.y));
+            if (r.z != 0.0f) atomicAdd(&dang[4 * l + 2], fx_of(r.z));
+            if (r.w != 0.0f) atomicAdd(&dang[4 * l + 3], fx_of(r.w));
         }
     }
 
@@ -112,66 +124,86 @@ struct PprSlots {
     }
 };
 
-// One warp per work unit, lane l holding slots 2l and 2l+1 (idle pairs skip
-// every load and store). kSvUnroll source ids are read at a time (each a
-// broadcast load), then their kSvUnroll message rows (256 bytes each) are in
-// flight together; the sum runs in edge order. Per-slot constants live in
-// shared memory so that 32 registers suffice and 64 warps fit on an SM.
-__global__ void __launch_bounds__(kSvBlock, 8) k_ppr_units(const PprArgs a) {
+// LG lanes per work unit, 32 / LG units per warp (neighbours in the units'
+// order, which have about the same length); lanes without a busy slot skip
+// every load and store. kSvUnroll source ids are read at a time (a broadcast
+// load within the lane group), then their message rows are in flight
+// together; the sum runs in edge order. What bounds it: the L2 bandwidth of
+// the rows with all slots in use, instruction issue with few. 32 queries on
+// each of three graphs (8.4, 2.1 and 0.5 M edges, ~22 supersteps each): 10.9 ms
+// in this kernel with a unit per warp and two slots a lane whatever the slots
+// in use, 4.8 ms so (4 rows in flight and 6 CTAs an SM; 8 rows and 3 / 4 CTAs
+// 5.2 / 4.5 ms, 4 rows and 8 CTAs 5.5 ms, the whole burst 13.8 / 13.9 / 12.6
+// against 12.8 ms).
+template <int LG>
+__global__ void __launch_bounds__(kSvBlock, 6) k_ppr_units(const PprArgs a) {
+    constexpr uint32_t kPer = 32 / LG;
     __shared__ PprSlots sl;
     sl.init(a);
-    const int lane = threadIdx.x & 31;
-    const bool live = (a.active_mask >> (2 * lane)) & 3ull;
-    const float2* msg = reinterpret_cast<const float2*>(a.msg_cur);
+    const uint32_t lane = threadIdx.x & 31u, l = lane % LG, sub = lane / LG;
+    const bool live = (a.active_mask >> (4 * l)) & 15ull;
+    const float4* msg = reinterpret_cast<const float4*>(a.msg_cur);
     const uint64_t warp0 = ((uint64_t)blockIdx.x * kSvBlock + threadIdx.x) >> 5;
     const uint64_t n_warps = ((uint64_t)gridDim.x * kSvBlock) >> 5;
-    for (uint64_t k = warp0; k < a.n_units; k += n_warps) {
-        const uint4 un = a.units[k];   // dst, first edge, edges, partial + 1 | 0
+    for (uint64_t k0 = warp0 * kPer; k0 < a.n_units; k0 += n_warps * kPer) {
+        const bool has = k0 + sub < a.n_units;
+        const uint4 un = has ? a.units[k0 + sub] : make_uint4(0u, 0u, 0u, 0u);   // dst, first edge, edges, partial + 1 | 0
         const float inv = __ldg(a.inv_outdeg + un.x);
         const uint32_t* e = a.src + un.y;
-        float2 acc = make_float2(0.0f, 0.0f);
+        float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         for (uint32_t i = 0; i < un.z; i += kSvUnroll) {
             uint32_t u[kSvUnroll];
 #pragma unroll
             for (int q = 0; q < kSvUnroll; ++q) u[q] = i + q < un.z ? __ldg(e + i + q) : kInf;
-            float2 m[kSvUnroll];
+            float4 m[kSvUnroll];
 #pragma unroll
             for (int q = 0; q < kSvUnroll; ++q)
-                m[q] = (u[q] != kInf && live) ? msg[(uint64_t)u[q] * 32u + lane] : make_float2(0.0f, 0.0f);
+                m[q] = (u[q] != kInf && live) ? msg[(uint64_t)u[q] * 16u + l] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-            for (int q = 0; q < kSvUnroll; ++q)
-                if (u[q] != kInf) {
-                    acc.x += m[q].x;
-                    acc.y += m[q].y;
-                }
+            for (int q = 0; q < kSvUnroll; ++q) {   // (an absent edge adds zero)
+                acc.x += m[q].x;
+                acc.y += m[q].y;
+                acc.z += m[q].z;
+                acc.w += m[q].w;
+            }
         }
-        if (!live) continue;
-        if (un.w) reinterpret_cast<float2*>(a.partial)[(uint64_t)(un.w - 1u) * 32u + lane] = acc;
-        else sl.apply(a, un.x, inv, acc, lane);
+        if (!live || !has) continue;
+        if (un.w) reinterpret_cast<float4*>(a.partial)[(uint64_t)(un.w - 1u) * 16u + l] = acc;
+        else sl.apply(a, un.x, inv, acc, l);
     }
     sl.flush(a.dang_next);
 }
 
-// One warp per vertex split over several units: adds its partial rows in
-// unit order and applies.
-__global__ void __launch_bounds__(kSvBlock, 8) k_ppr_split(const PprArgs a) {
+// LG lanes per vertex split over several units: its partial rows added in
+// unit order (eight in flight), applied.
+template <int LG>
+__global__ void __launch_bounds__(kSvBlock, 4) k_ppr_split(const PprArgs a) {
+    constexpr uint32_t kPer = 32 / LG;
     __shared__ PprSlots sl;
     sl.init(a);
-    const int lane = threadIdx.x & 31;
-    const bool live = (a.active_mask >> (2 * lane)) & 3ull;
-    const float2* part = reinterpret_cast<const float2*>(a.partial);
+    const uint32_t lane = threadIdx.x & 31u, l = lane % LG, sub = lane / LG;
+    const bool live = (a.active_mask >> (4 * l)) & 15ull;
+    const float4* part = reinterpret_cast<const float4*>(a.partial);
     const uint32_t warp0 = (blockIdx.x * kSvBlock + threadIdx.x) >> 5;
     const uint32_t n_warps = (gridDim.x * kSvBlock) >> 5;
-    for (uint32_t r = warp0; r < a.n_split_rows && live; r += n_warps) {
+    for (uint64_t r = (uint64_t)warp0 * kPer + sub; r < a.n_split_rows && live; r += (uint64_t)n_warps * kPer) {
         const uint2 sr = a.split_rows[r];   // {vertex, first partial}
         const uint32_t end = a.split_rows[r + 1].y;
-        float2 acc = make_float2(0.0f, 0.0f);
-        for (uint32_t p = sr.y; p < end; ++p) {   // unit order
-            const float2 x = part[(uint64_t)p * 32u + lane];
-            acc.x += x.x;
-            acc.y += x.y;
+        float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        for (uint32_t p = sr.y; p < end; p += 8u) {   // unit order
+            float4 x[8];
+#pragma unroll
+            for (uint32_t q = 0; q < 8; ++q)
+                x[q] = p + q < end ? part[(uint64_t)(p + q) * 16u + l] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+            for (uint32_t q = 0; q < 8; ++q) {
+                acc.x += x[q].x;
+                acc.y += x[q].y;
+                acc.z += x[q].z;
+                acc.w += x[q].w;
+            }
         }
-        sl.apply(a, sr.x, __ldg(a.inv_outdeg + sr.x), acc, lane);
+        sl.apply(a, sr.x, __ldg(a.inv_outdeg + sr.x), acc, l);
     }
     sl.flush(a.dang_next);
 }
@@ -244,9 +276,14 @@ __global__ void __launch_bounds__(kSvBlock) k_gather_columns(const uint32_t* mat
 }  // namespace
 
 cudaError_t launch_ppr_superstep(const PprArgs& a, cudaStream_t s) {
-    k_ppr_units<<<serve_grid(a.n_units), kSvBlock, 0, s>>>(a);
-    if (a.n_split_rows) k_ppr_split<<<serve_grid(a.n_split_rows), kSvBlock, 0, s>>>(a);
-    return cudaGetLastError();
+    return with_slot_lanes(a.active_mask, [&](auto lanes) {
+        constexpr int LG = decltype(lanes)::value;
+        constexpr uint64_t kPer = 32 / LG;
+        k_ppr_units<LG><<<serve_grid((a.n_units + kPer - 1) / kPer), kSvBlock, 0, s>>>(a);
+        if (a.n_split_rows)
+            k_ppr_split<LG><<<serve_grid((a.n_split_rows + kPer - 1) / kPer), kSvBlock, 0, s>>>(a);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_ppr_slots_init(float* msg_cur, const float* inv_outdeg, uint64_t n, uint64_t mask,

@@ -161,6 +161,10 @@ uint32_t Server::add_graph(uint64_t n, uint64_t m, const uint32_t* src_in, const
         }
     }
     if (partials >= 0xFFFFFFFFull) fail(GXP_E_INVAL, "too many split rows");
+    // longest first: units that share a warp have about the same length, and
+    // the long ones do not come last
+    all = units_longest_first(all);
+    nz = units_longest_first(nz);
     split.push_back(make_uint2(kInf, (uint32_t)partials));   // sentinel: end of the last split row
 
     auto G = std::make_unique<ServedGraph>();
@@ -179,6 +183,9 @@ uint32_t Server::add_graph(uint64_t n, uint64_t m, const uint32_t* src_in, const
     G->d_units_all = (uint4*)up(all.data(), sizeof(uint4) * all.size());
     G->d_units_nz = (uint4*)up(nz.data(), sizeof(uint4) * nz.size());
     G->packed = packed;
+    uint32_t wmax = 1;
+    for (uint64_t e = 0; w && e < m; ++e) wmax = std::max(wmax, w[e]);
+    G->no_sat = n * (uint64_t)wmax < 0xFFFFFFFFull ? 1u : 0u;   // a path has fewer than n edges
     G->d_edges = packed ? up(epacked.data(), 4 * m) : up(edges.data(), sizeof(uint2) * m);
     G->d_src = (uint32_t*)up(esrc.data(), 4 * m);
     std::vector<float> inv(n);
@@ -438,6 +445,7 @@ void Server::lane_step(Lane& L, ServedGraph& G, uint64_t admit) {
         a.changed = L.d_changed;
         a.slot_improved = L.d_improved;
         a.idle_mask = ~L.busy;
+        a.no_sat = G.no_sat;
         cuda_check(launch_msssp(a, false, serve_grid(G.n_units_nz), st), "sssp superstep");
         cuda_check(cudaMemsetAsync(L.d_frontier[L.cur], 0, 4 * ((G.n + 31) / 32 + 1), st), "memset");
         cuda_check(cudaMemcpyAsync(L.h_improved, L.d_improved, 8, cudaMemcpyDeviceToHost, st), "read flags");
