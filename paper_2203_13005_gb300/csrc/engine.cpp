@@ -90,18 +90,20 @@ Engine::~Engine() {
     if (h_steps_) cudaFreeHost(h_steps_);
     if (stream_) cudaStreamSynchronize(stream_);   // the frees above
     if (pool_) cudaMemPoolDestroy(pool_);
+    if (load_stream_) cudaStreamDestroy(load_stream_);
     if (own_stream_) cudaStreamDestroy(own_stream_);
 }
 
 // Device memory comes from the context's own memory pool, which keeps what
 // is freed for reuse (release threshold: never), so reloading a graph of the
 // same size maps no new pages: a first load pays cudaMalloc's page mapping,
-// later ones take the pool's blocks at once. The allocation is made complete
-// (the stream synchronized) before it returns, so any stream may use it, and
+// later ones take the pool's blocks at once. With `wait` the allocation is
+// made complete (the stream synchronized) before it returns, so any stream may
+// use it; without, it is ordered on stream_. And
 // frees are ordered after the context stream's work; every free happens once
 // the buffer's users are done, as it did with cudaFree. When the pool cannot
 // grow, it is trimmed and the allocation tried once more.
-cudaError_t Engine::device_malloc(void** p, size_t bytes) {
+cudaError_t Engine::device_malloc(void** p, size_t bytes, bool wait) {
     ++n_allocs_;
     if (faults_.alloc_at == n_allocs_) return cudaErrorMemoryAllocation;   // injected fault
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool_, stream_);
@@ -111,7 +113,7 @@ cudaError_t Engine::device_malloc(void** p, size_t bytes) {
         cudaMemPoolTrimTo(pool_, 0);
         e = cudaMallocFromPoolAsync(p, bytes, pool_, stream_);
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream_);
+    if (e == cudaSuccess && wait) e = cudaStreamSynchronize(stream_);
     return e;
 }
 
@@ -126,11 +128,17 @@ void Engine::before_h2d(const char* what) {
 }
 
 void* Engine::dalloc(size_t bytes) {
+    void* p = dalloc_ordered(bytes);
+    cuda_check(cudaStreamSynchronize(stream_), "cudaMalloc");
+    return p;
+}
+
+void* Engine::dalloc_ordered(size_t bytes) {
     bytes = std::max<size_t>(bytes, 16);
     if (cfg_.mem_budget && graph_bytes_ + bytes > cfg_.mem_budget)
         fail(GXP_E_NOMEM, "allocation exceeds the context's mem_budget");
     void* p = nullptr;
-    cuda_check(device_malloc(&p, bytes), "cudaMalloc");
+    cuda_check(device_malloc(&p, bytes, false), "cudaMalloc");
     graph_allocs_.push_back(p);
     graph_bytes_ += bytes;
     return p;
@@ -142,6 +150,7 @@ void Engine::free_graph_device() {
     d_bar_ = nullptr;
     bar_passed_ = 0;
     h_old2new_.clear();
+    n_lookups_ = 0;
     lp_ = LpLists{};
     lru_ = Lru{};
     for (void* p : graph_allocs_) device_free(p);
@@ -350,7 +359,7 @@ void Engine::load_csc_device(HostPart& hp, uint64_t E, const void* cp_in, const 
         void* q = nullptr;
         if (cfg_.mem_budget && graph_bytes_ + bytes > cfg_.mem_budget)
             fail(GXP_E_NOMEM, "allocation exceeds the context's mem_budget");
-        cuda_check(device_malloc(&q, std::max<size_t>(bytes, 16)), "cudaMalloc");
+        cuda_check(device_malloc(&q, std::max<size_t>(bytes, 16), false), "cudaMalloc");
         return q;
     };
     uint64_t* cp64 = nullptr;
@@ -360,25 +369,43 @@ void Engine::load_csc_device(HostPart& hp, uint64_t E, const void* cp_in, const 
         hp.d_src = (uint32_t*)own(4 * pad4(E));
         if (w_in) hp.d_w = (uint32_t*)own(4 * pad4(E));
         hp.on_device = true;
+        hp.d_outdeg = (uint32_t*)own(4 * std::max<size_t>(n, 1));
         cp64 = (uint64_t*)own(8 * ((size_t)n + 1));
         flag = (uint32_t*)own(4);
+        cuda_check(cudaMemsetAsync(hp.d_outdeg, 0, 4ull * n, stream_), "memset");
         cuda_check(cudaMemsetAsync(flag, 0, 4, stream_), "memset");
         cuda_check(cudaMemsetAsync(hp.d_col_ptr, 0, 4 * pad4(n + 1), stream_), "memset");
         cuda_check(cudaMemsetAsync(hp.d_src + E, 0, 4 * (pad4(E) - E), stream_), "memset");
         before_h2d("copy col_ptr");
         cuda_check(cudaMemcpyAsync(cp64, cp_in, 8 * ((size_t)n + 1), cudaMemcpyDefault, stream_), "copy col_ptr");
+        cuda_check(launch_csc_offsets(cp64, n, E, hp.d_col_ptr, flag, stream_), "check CSC");
+        // The sources are copied in chunks on a stream of their own; while the
+        // next one travels, the chunk that arrived is checked and its out-degrees
+        // are counted.
         if (E) {
             before_h2d("copy sources");
-            cuda_check(cudaMemcpyAsync(hp.d_src, src_in, 4 * E, cudaMemcpyDefault, stream_), "copy sources");
+            if (!load_stream_) cuda_check(cudaStreamCreateWithFlags(&load_stream_, cudaStreamNonBlocking), "stream");
+            const uint64_t chunk = std::max<uint64_t>(1ull << 21, ((E + 7) / 8 + 3) & ~3ull);
+            cuda_check(cudaEventRecord(ev_k_, stream_), "event");   // the buffers exist
+            cuda_check(cudaStreamWaitEvent(load_stream_, ev_k_, 0), "wait");
+            for (uint64_t e0 = 0; e0 < E; e0 += chunk) {
+                const uint64_t ne = std::min(chunk, E - e0);
+                cuda_check(cudaMemcpyAsync(hp.d_src + e0, src_in + e0, 4 * ne, cudaMemcpyDefault, load_stream_),
+                           "copy sources");
+                cuda_check(cudaEventRecord(ev_k_, load_stream_), "event");
+                cuda_check(cudaStreamWaitEvent(stream_, ev_k_, 0), "wait");
+                cuda_check(launch_csc_sources(hp.d_src + e0, ne, n, hp.d_outdeg, flag, stream_), "check CSC");
+            }
         }
         if (w_in) {
             cuda_check(cudaMemsetAsync(hp.d_w + E, 0, 4 * (pad4(E) - E), stream_), "memset");
             if (E) {
-                before_h2d("copy weights");
-                cuda_check(cudaMemcpyAsync(hp.d_w, w_in, 4 * E, cudaMemcpyDefault, stream_), "copy weights");
+                before_h2d("copy weights");   // (after the sources: the copies share the link)
+                cuda_check(cudaMemcpyAsync(hp.d_w, w_in, 4 * E, cudaMemcpyDefault, load_stream_), "copy weights");
+                cuda_check(cudaEventRecord(ev_k_, load_stream_), "event");
+                cuda_check(cudaStreamWaitEvent(stream_, ev_k_, 0), "wait");
             }
         }
-        cuda_check(launch_csc_import(cp64, n, E, hp.d_col_ptr, hp.d_src, n, flag, stream_), "check CSC");
         uint32_t bad = 0;
         cuda_check(cudaMemcpyAsync(&bad, flag, 4, cudaMemcpyDeviceToHost, stream_), "read check");
         cuda_check(cudaStreamSynchronize(stream_), "check CSC");
@@ -389,6 +416,7 @@ void Engine::load_csc_device(HostPart& hp, uint64_t E, const void* cp_in, const 
         if (bad & 1u) fail(GXP_E_INVAL, "CSC col_ptr must run from 0 to n_edges, non-decreasing");
         if (bad & 2u) fail(GXP_E_INVAL, "source id out of range");
     } catch (...) {
+        if (load_stream_) cudaStreamSynchronize(load_stream_);   // copies into the buffers released below
         if (cp64) device_free(cp64);
         if (flag) device_free(flag);
         release_part(hp);
@@ -405,7 +433,8 @@ void Engine::release_part(HostPart& hp) {
         device_free(hp.d_col_ptr);
         device_free(hp.d_src);
         if (hp.d_w) device_free(hp.d_w);
-        hp.d_col_ptr = hp.d_src = hp.d_w = nullptr;
+        if (hp.d_outdeg) device_free(hp.d_outdeg);
+        hp.d_col_ptr = hp.d_src = hp.d_w = hp.d_outdeg = nullptr;
         hp.on_device = false;
         hp.dev_edges = 0;
         hp.dev_weighted = false;
@@ -427,7 +456,7 @@ void Engine::ensure_host(HostPart& hp) {
 }
 
 uint32_t* Engine::upload_u32(const std::vector<uint32_t>& h, size_t n_pad) {
-    uint32_t* d = (uint32_t*)dalloc(4 * std::max<size_t>(n_pad, 1));
+    uint32_t* d = (uint32_t*)dalloc_ordered(4 * std::max<size_t>(n_pad, 1));
     cuda_check(cudaMemsetAsync(d, 0, 4 * std::max<size_t>(n_pad, 1), stream_), "memset");
     if (!h.empty()) {
         before_h2d("upload");
@@ -467,10 +496,14 @@ void Engine::build_sell() {
     // fill a batch; a small graph takes fewer, so that its items still cover
     // the chip's ~4,900 resident warps.
     sweep_cols_ = n_parts_ > 1 ? 0u : total_edges_ >= (1ull << 23) ? 16u : total_edges_ >= (1ull << 21) ? 8u : 4u;
+    if (n_parts_ == 1 && relabeled_ && H <= kOrderExact) {
+        build_sell_sorted(H, T);
+        return;
+    }
     std::vector<void*> tmp;   // freed when the build ends
     auto talloc = [&](size_t bytes) {
         void* q = nullptr;
-        cuda_check(device_malloc(&q, std::max<size_t>(bytes, 16)), "cudaMalloc");
+        cuda_check(device_malloc(&q, std::max<size_t>(bytes, 16), false), "cudaMalloc");
         tmp.push_back(q);
         return q;
     };
@@ -499,8 +532,8 @@ void Engine::build_sell() {
         const uint64_t E = hp.n_edges();
         // 1. rows sorted by (source, weight); the sorted copy also serves the hub parts
         const uint32_t* col_ptr = work_[p].col;   // offsets of the rows the build writes
-        uint32_t* ssrc = (uint32_t*)dalloc(4 * pad4(E));
-        uint32_t* sw = weighted ? (uint32_t*)dalloc(4 * pad4(E)) : nullptr;
+        uint32_t* ssrc = (uint32_t*)dalloc_ordered(4 * pad4(E));
+        uint32_t* sw = weighted ? (uint32_t*)dalloc_ordered(4 * pad4(E)) : nullptr;
         uint2* big = (uint2*)talloc(8 * ((size_t)n + E / 2048 + 1));
         uint32_t* cnt = (uint32_t*)talloc(4);
         cuda_check(launch_sort_rows(col_ptr, n, work_[p].in, pd_[p].n_own + pd_[p].n_ghost, ssrc, sw, big, cnt,
@@ -531,7 +564,7 @@ void Engine::build_sell() {
                        "upload bases");
         }
         // 3. slices and their offsets
-        uint32_t* perm = (uint32_t*)dalloc(4 * pad4(ns * 32));
+        uint32_t* perm = (uint32_t*)dalloc_ordered(4 * pad4(ns * 32));
         uint32_t* width = (uint32_t*)talloc(4 * ns + 4);
         uint64_t* off = (uint64_t*)talloc(8 * ns + 8);
         cuda_check(launch_sell_slices(col_ptr, n, rows_out, counts, d_bases, perm, width, off, (uint32_t)ns,
@@ -539,8 +572,8 @@ void Engine::build_sell() {
         uint64_t sell_size = 0;
         d2h(&sell_size, off + ns, 8);
         // 4. fill
-        uint32_t* sell_src = (uint32_t*)dalloc(4 * pad4(sell_size));
-        uint32_t* sell_w = weighted ? (uint32_t*)dalloc(4 * pad4(sell_size)) : nullptr;
+        uint32_t* sell_src = (uint32_t*)dalloc_ordered(4 * pad4(sell_size));
+        uint32_t* sell_w = weighted ? (uint32_t*)dalloc_ordered(4 * pad4(sell_size)) : nullptr;
         part_desc[p] = (SellSlice*)talloc(sizeof(SellSlice) * (ns + 1));
         part_ns[p] = (uint32_t)ns;
         cuda_check(launch_sell_fill(col_ptr, ssrc, sw, perm, width, off, (uint32_t)ns, p, pd_[p].pad_id,
@@ -585,7 +618,7 @@ void Engine::build_sell() {
     // it gathers at any moment are that partition's own vertices and cached
     // copies (tens of MB, L2-resident) rather than every partition's copies
     // at once.
-    d_slices_ = (SellSlice*)dalloc(sizeof(SellSlice) * std::max<size_t>(total_slices, 1));
+    d_slices_ = (SellSlice*)dalloc_ordered(sizeof(SellSlice) * std::max<size_t>(total_slices, 1));
     uint32_t* order_scratch = (uint32_t*)talloc(order_slices_scratch_bytes(n_slices_));
     at = 0;
     for (uint32_t p = 0; p < n_parts_; ++p) {
@@ -608,7 +641,7 @@ void Engine::build_sell() {
         at += part_ns[p];
     }
     const size_t nh1 = std::max<size_t>(total_hubs, 1);
-    d_hubs_ = (HubPart*)dalloc(sizeof(HubPart) * nh1);
+    d_hubs_ = (HubPart*)dalloc_ordered(sizeof(HubPart) * nh1);
     at = 0;
     for (uint32_t p = 0; p < n_parts_; ++p) {
         if (part_nh[p])
@@ -616,10 +649,91 @@ void Engine::build_sell() {
                                        cudaMemcpyDeviceToDevice, stream_), "gather hub parts");
         at += part_nh[p];
     }
-    d_hub_val_ = (unsigned long long*)dalloc(8 * nh1);
+    d_hub_val_ = (unsigned long long*)dalloc_ordered(8 * nh1);
     cuda_check(cudaMemsetAsync(d_hub_val_, 0, 8 * nh1, stream_), "memset");
-    d_hub_arrive_ = (uint32_t*)dalloc(4 * nh1);
+    d_hub_arrive_ = (uint32_t*)dalloc_ordered(4 * nh1);
     cuda_check(cudaMemsetAsync(d_hub_arrive_, 0, 4 * nh1, stream_), "memset");
+    cuda_check(cudaStreamSynchronize(stream_), "sell build");
+    check_device_error();
+    sell_ready_ = true;
+}
+
+// The layout of a renumbered partition: its vertices are in order of
+// decreasing in-degree, exactly up to kOrderExact >= H, so the hub rows come
+// first, the slices are its other rows 32 by 32, heavy first as they stand,
+// and the host knows from the counts of in_degree_above_ how wide each slice
+// is and where it starts.
+void Engine::build_sell_sorted(uint32_t H, uint32_t T) {
+    HostPart& hp = parts_[0];
+    const uint32_t n = hp.n_own, C = sweep_cols_;
+    const uint64_t E = hp.n_edges();
+    const bool weighted = hp.weighted();
+    const uint32_t* col = work_[0].col;
+    const std::vector<uint32_t>& above = in_degree_above_;
+    const uint32_t nh = above[H];   // hub rows
+    const uint64_t ns = ((uint64_t)n - nh + 31) / 32;
+    // slices wider than b columns: those whose first row has more in-edges
+    auto wider = [&](uint64_t b) -> uint32_t {
+        return b >= H ? 0u : (uint32_t)(((uint64_t)above[b] - nh + 31) / 32);
+    };
+    // at[w] + s * sell_words(w): where slice s starts if it is w wide
+    std::vector<uint64_t> at(H + 1, 0);
+    uint64_t words = 0;
+    for (uint32_t w = H; w >= 1; --w) {
+        const uint64_t s0 = wider(w), s1 = wider(w - 1), per = sell_words(w, C);
+        at[w] = words - s0 * per;   // (modulo 2^64)
+        words += (s1 - s0) * per;
+    }
+    std::vector<void*> tmp;
+    auto talloc = [&](size_t bytes) {
+        void* q = nullptr;
+        cuda_check(device_malloc(&q, std::max<size_t>(bytes, 16), false), "cudaMalloc");
+        tmp.push_back(q);
+        return q;
+    };
+    struct FreeTmp {
+        std::vector<void*>& v;
+        cudaStream_t s;
+        ~FreeTmp() {
+            cudaStreamSynchronize(s);
+            for (void* q : v) cudaFreeAsync(q, s);   // pool blocks (device_malloc)
+        }
+    } free_tmp{tmp, stream_};
+    // (the hub rows' parts are counted first: the host waits for the count)
+    uint32_t* part_off = (uint32_t*)talloc(4 * (size_t)nh + 4);
+    cuda_check(launch_hub_offsets(col, nh, T, part_off, stream_), "hub rows");
+    uint32_t n_parts = 0;
+    cuda_check(cudaMemcpyAsync(&n_parts, part_off + nh, 4, cudaMemcpyDeviceToHost, stream_), "read counts");
+    uint32_t* ssrc = (uint32_t*)dalloc_ordered(4 * pad4(E));
+    uint32_t* sw = weighted ? (uint32_t*)dalloc_ordered(4 * pad4(E)) : nullptr;
+    cuda_check(launch_renumber_rows(col, n, work_[0].in, E, ssrc, sw, stream_), "renumber rows");
+    uint64_t* d_at = (uint64_t*)talloc(8 * at.size());
+    before_h2d("upload slice starts");
+    cuda_check(cudaMemcpyAsync(d_at, at.data(), 8 * at.size(), cudaMemcpyHostToDevice, stream_), "upload slice starts");
+    uint32_t* sell_src = (uint32_t*)dalloc_ordered(4 * pad4(words));
+    uint32_t* sell_w = weighted ? (uint32_t*)dalloc_ordered(4 * pad4(words)) : nullptr;
+    n_slices_ = (uint32_t)ns;
+    d_slices_ = (SellSlice*)dalloc_ordered(sizeof(SellSlice) * std::max<uint64_t>(ns, 1));
+    cuda_check(launch_sell_fill_sorted(col, ssrc, sw, n, nh, d_at, (uint32_t)ns, C, sell_src, sell_w, d_slices_, stream_),
+               "fill slices");
+    if (n_parts > 0xFFFFFFF0u) fail(GXP_E_INVAL, "too many hub parts");
+    n_hubs_ = n_parts;
+    const size_t nh1 = std::max<size_t>(n_parts, 1);
+    d_hubs_ = (HubPart*)dalloc_ordered(sizeof(HubPart) * nh1);
+    cuda_check(launch_hub_parts(col, nullptr, part_off, nh, T, 0u, 0u, d_hubs_, stream_), "hub parts");
+    d_hub_val_ = (unsigned long long*)dalloc_ordered(8 * nh1);
+    cuda_check(cudaMemsetAsync(d_hub_val_, 0, 8 * nh1, stream_), "memset");
+    d_hub_arrive_ = (uint32_t*)dalloc_ordered(4 * nh1);
+    cuda_check(cudaMemsetAsync(d_hub_arrive_, 0, 4 * nh1, stream_), "memset");
+    pd_[0].sell_src = sell_src;
+    pd_[0].sell_w = sell_w;
+    pd_[0].perm = nullptr;   // every slice's rows are consecutive
+    pd_[0].hsrc = ssrc;
+    pd_[0].hw = sw;
+    for (int j = 0; j < 5; ++j) n_lanes_[j] = wider((uint64_t)C << (4 - j));
+    n_gt8_ = std::max(wider(8), n_lanes_[4]);
+    n_gt4_ = std::max(wider(4), n_lanes_[4]);
+    n_gt0_ = wider(0);
     cuda_check(cudaStreamSynchronize(stream_), "sell build");
     check_device_error();
     sell_ready_ = true;
@@ -674,14 +788,20 @@ void Engine::finalize() {
     relabeled_ = false;
     if (n_parts_ == 1 && !cfg_.keep_ids && V > 1) {
         HostPart& hp = parts_[0];
-        d_new2old_ = (uint32_t*)dalloc(4 * pad4(V));
-        d_old2new_ = (uint32_t*)dalloc(4 * pad4(V));
-        d_perm_tmp_ = (uint32_t*)dalloc(4 * pad4(V));
-        uint32_t* rcol = (uint32_t*)dalloc(4 * pad4(V + 1));
+        d_new2old_ = (uint32_t*)dalloc_ordered(4 * pad4(V));
+        d_old2new_ = (uint32_t*)dalloc_ordered(4 * pad4(V));
+        d_perm_tmp_ = (uint32_t*)dalloc_ordered(4 * pad4(V));
+        uint32_t* rcol = (uint32_t*)dalloc_ordered(4 * pad4(V + 1));
         cuda_check(cudaMemsetAsync(rcol, 0, 4 * pad4(V + 1), stream_), "memset");
         void* scratch = nullptr;
-        cudaError_t e = device_malloc(&scratch, relabel_scratch_bytes(V));
-        if (e == cudaSuccess) e = launch_relabel(hp.d_col_ptr, V, d_new2old_, d_old2new_, rcol, (uint32_t*)scratch, stream_);
+        const uint32_t* starts = nullptr;
+        in_degree_above_.resize(kOrderExact + 1);
+        cudaError_t e = device_malloc(&scratch, relabel_scratch_bytes(V), false);
+        if (e == cudaSuccess)
+            e = launch_relabel(hp.d_col_ptr, V, d_new2old_, d_old2new_, rcol, (uint32_t*)scratch, &starts, stream_);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(in_degree_above_.data(), starts, 4 * in_degree_above_.size(), cudaMemcpyDeviceToHost,
+                                stream_);
         cudaError_t e2 = cudaStreamSynchronize(stream_);
         if (scratch) device_free(scratch);
         cuda_check(e, "relabel");
@@ -690,19 +810,16 @@ void Engine::finalize() {
         work_[0].in.row_map = d_new2old_;
         work_[0].in.src_map = d_old2new_;
         relabeled_ = true;
-        // host copy of the map: sources are renumbered without a device round trip
-        h_old2new_.resize(V);
-        cuda_check(cudaMemcpy(h_old2new_.data(), d_old2new_, 4ull * V, cudaMemcpyDeviceToHost), "relabel map");
     }
-    d_parts_ = (PartDev*)dalloc(sizeof(PartDev) * n_parts_);
+    d_parts_ = (PartDev*)dalloc_ordered(sizeof(PartDev) * n_parts_);
     before_h2d("upload");
     cuda_check(cudaMemcpyAsync(d_parts_, pd_.data(), sizeof(PartDev) * n_parts_, cudaMemcpyHostToDevice, stream_),
                "upload parts");
     sell_ready_ = false;
     const std::vector<PartDev>& pd = pd_;
 
-    d_ghost_gid_ = (uint32_t*)dalloc(4 * (size_t)std::max<uint32_t>(n_ghost_total_, 1));
-    d_ghost_ = (uint32_t*)dalloc(4 * pad4((size_t)n_ghost_total_ + 1));   // + the identity slot
+    d_ghost_gid_ = (uint32_t*)dalloc_ordered(4 * (size_t)std::max<uint32_t>(n_ghost_total_, 1));
+    d_ghost_ = (uint32_t*)dalloc_ordered(4 * pad4((size_t)n_ghost_total_ + 1));   // + the identity slot
     for (auto& hp : parts_)
         if (!hp.ghost_gid.empty()) {
             before_h2d("upload ghost ids");
@@ -713,26 +830,32 @@ void Engine::finalize() {
 
     // out-degrees over all partitions' edges
     // vertex arrays are padded so 16-byte-aligned bulk copies of any slice stay inside
-    d_outdeg_ = (uint32_t*)dalloc(4 * pad4(V));
+    d_outdeg_ = (uint32_t*)dalloc_ordered(4 * pad4(V));
     cuda_check(cudaMemsetAsync(d_outdeg_, 0, 4 * pad4(V), stream_), "memset");
+    const uint32_t* counted = parts_[0].on_device ? parts_[0].d_outdeg : nullptr;   // at the load, in input ids
     uint32_t* outdeg_in = relabeled_ ? d_perm_tmp_ : d_outdeg_;   // input ids, then renumbered
-    if (relabeled_) cuda_check(cudaMemsetAsync(outdeg_in, 0, 4 * pad4(V), stream_), "memset");
-    for (uint32_t p = 0; p < n_parts_; ++p)
-        cuda_check(launch_outdeg(pd[p], parts_[p].d_src, d_ghost_gid_ + parts_[p].ghost_base, outdeg_in, stream_),
-                   "out-degrees");
+    if (!counted) {
+        if (relabeled_) cuda_check(cudaMemsetAsync(outdeg_in, 0, 4 * pad4(V), stream_), "memset");
+        for (uint32_t p = 0; p < n_parts_; ++p)
+            cuda_check(launch_outdeg(pd[p], parts_[p].d_src, d_ghost_gid_ + parts_[p].ghost_base, outdeg_in, stream_),
+                       "out-degrees");
+    }
     if (relabeled_)
-        cuda_check(launch_permute_u32(outdeg_in, d_old2new_, V, d_outdeg_, true, stream_), "out-degrees");
+        cuda_check(launch_permute_u32(counted ? counted : outdeg_in, d_old2new_, V, d_outdeg_, true, stream_),
+                   "out-degrees");
+    else if (counted)
+        cuda_check(cudaMemcpyAsync(d_outdeg_, counted, 4ull * V, cudaMemcpyDeviceToDevice, stream_), "out-degrees");
 
-    d_n_dangling_ = (unsigned long long*)dalloc(8);
+    d_n_dangling_ = (unsigned long long*)dalloc_ordered(8);
     cuda_check(launch_count_dangling(d_outdeg_, V, d_n_dangling_, stream_), "out-degrees");
     for (int b = 0; b < 2; ++b) {
-        d_own_[b] = (uint32_t*)dalloc(4 * pad4(V));
-        d_rank_[b] = (float*)dalloc(4 * pad4(V));
+        d_own_[b] = (uint32_t*)dalloc_ordered(4 * pad4(V));
+        d_rank_[b] = (float*)dalloc_ordered(4 * pad4(V));
         cuda_check(cudaMemsetAsync(d_own_[b], 0, 4 * pad4(V), stream_), "memset");
         cuda_check(cudaMemsetAsync(d_rank_[b], 0, 4 * pad4(V), stream_), "memset");
     }
-    d_stats_ = (StepStats*)dalloc(sizeof(StepStats) * kStatRing);
-    d_err_ = (uint32_t*)dalloc(4);
+    d_stats_ = (StepStats*)dalloc_ordered(sizeof(StepStats) * kStatRing);
+    d_err_ = (uint32_t*)dalloc_ordered(4);
     cuda_check(cudaMemsetAsync(d_err_, 0, 4, stream_), "memset");
     if (cfg_.check_bounds)
         for (uint32_t p = 0; p < n_parts_; ++p)
@@ -771,18 +894,18 @@ void Engine::build_caches() {
         max_words_ = std::max(max_words_, hp.n_own ? wh - wl : 0u);
     }
     if (gdq_total > 0xFFFFFFF0ull) fail(GXP_E_INVAL, "global data queue too large");
-    d_boundary_ = (uint32_t*)dalloc(4 * words);
-    for (auto& c : d_changed_) c = (uint32_t*)dalloc(4 * words);
-    d_gdq_ids_ = (uint32_t*)dalloc(4 * std::max<uint64_t>(gdq_total, 1));
-    d_gdq_vals_ = (uint32_t*)dalloc(4 * std::max<uint64_t>(gdq_total, 1));
-    d_gdq_base_ = (uint64_t*)dalloc(8 * n_parts_);
+    d_boundary_ = (uint32_t*)dalloc_ordered(4 * words);
+    for (auto& c : d_changed_) c = (uint32_t*)dalloc_ordered(4 * words);
+    d_gdq_ids_ = (uint32_t*)dalloc_ordered(4 * std::max<uint64_t>(gdq_total, 1));
+    d_gdq_vals_ = (uint32_t*)dalloc_ordered(4 * std::max<uint64_t>(gdq_total, 1));
+    d_gdq_base_ = (uint64_t*)dalloc_ordered(8 * n_parts_);
     std::vector<uint64_t> gb(n_parts_);
     for (uint32_t p = 0; p < n_parts_; ++p) gb[p] = parts_[p].gdq_base;
     sync_blocks_x_ = std::max<uint32_t>((max_words_ + 255) / 256, 1);
-    d_block_counts_ = (uint32_t*)dalloc(4 * (size_t)n_parts_ * sync_blocks_x_);
-    d_block_offsets_ = (uint32_t*)dalloc(4 * (size_t)n_parts_ * sync_blocks_x_);
-    d_part_counts_ = (uint32_t*)dalloc(4 * n_parts_);
-    d_done_ctr_ = (uint32_t*)dalloc(4 * n_parts_);
+    d_block_counts_ = (uint32_t*)dalloc_ordered(4 * (size_t)n_parts_ * sync_blocks_x_);
+    d_block_offsets_ = (uint32_t*)dalloc_ordered(4 * (size_t)n_parts_ * sync_blocks_x_);
+    d_part_counts_ = (uint32_t*)dalloc_ordered(4 * n_parts_);
+    d_done_ctr_ = (uint32_t*)dalloc_ordered(4 * n_parts_);
     before_h2d("upload");
     cuda_check(cudaMemcpyAsync(d_boundary_, bbits.data(), 4 * words, cudaMemcpyHostToDevice, stream_), "upload");
     before_h2d("upload");
@@ -808,13 +931,13 @@ void Engine::build_caches() {
         const size_t G = n_ghost_total_;
         lru_.d_base = upload_u32(base, base.size());
         lru_.d_reads = upload_u32(reads, G);
-        lru_.d_weight = (uint32_t*)dalloc(4 * G);
-        lru_.d_flags = (uint8_t*)dalloc(G);
-        lru_.d_hist = (uint32_t*)dalloc(4ull * kLruBins * n_parts_);
-        lru_.d_part = (LruPart*)dalloc(sizeof(LruPart) * n_parts_);
-        lru_.d_tie = (uint32_t*)dalloc(4 * G);
-        lru_.d_tie_scan = (uint32_t*)dalloc(4 * (G + 1));
-        lru_.d_scratch = (uint32_t*)dalloc(4 * ((G + 2047) / 2048 + 1));
+        lru_.d_weight = (uint32_t*)dalloc_ordered(4 * G);
+        lru_.d_flags = (uint8_t*)dalloc_ordered(G);
+        lru_.d_hist = (uint32_t*)dalloc_ordered(4ull * kLruBins * n_parts_);
+        lru_.d_part = (LruPart*)dalloc_ordered(sizeof(LruPart) * n_parts_);
+        lru_.d_tie = (uint32_t*)dalloc_ordered(4 * G);
+        lru_.d_tie_scan = (uint32_t*)dalloc_ordered(4 * (G + 1));
+        lru_.d_scratch = (uint32_t*)dalloc_ordered(4 * ((G + 2047) / 2048 + 1));
         cuda_check(cudaMemsetAsync(lru_.d_hist, 0, 4ull * kLruBins * n_parts_, stream_), "memset");
         cuda_check(cudaMemsetAsync(lru_.d_part, 0, sizeof(LruPart) * n_parts_, stream_), "memset");
     }
@@ -835,6 +958,25 @@ static Algo to_algo(gxp_algo a) {
     }
 }
 
+// The first few sources are looked up on the device, one word each; a
+// context that keeps asking copies the map (a load that runs PageRank or CC
+// never pays for the copy).
+uint32_t Engine::internal_id(uint32_t v) {
+    if (h_old2new_.empty() && ++n_lookups_ < kLookups) {
+        uint32_t x = 0;
+        cuda_check(cudaMemcpyAsync(&x, d_old2new_ + v, 4, cudaMemcpyDeviceToHost, stream_), "relabel map");
+        cuda_check(cudaStreamSynchronize(stream_), "relabel map");
+        return x;
+    }
+    if (h_old2new_.empty()) {
+        h_old2new_.resize(n_vertices_);
+        cuda_check(cudaMemcpyAsync(h_old2new_.data(), d_old2new_, 4ull * n_vertices_, cudaMemcpyDeviceToHost, stream_),
+                   "relabel map");
+        cuda_check(cudaStreamSynchronize(stream_), "relabel map");
+    }
+    return h_old2new_[v];
+}
+
 void Engine::begin(gxp_algo algo, uint32_t source, float damping) {
     TraceRange trace_("gxp begin");
     if (!have_graph_) fail(GXP_E_STATE, "no graph");
@@ -848,7 +990,7 @@ void Engine::begin(gxp_algo algo, uint32_t source, float damping) {
     const uint32_t V = (uint32_t)n_vertices_;
     begun_ = false;   // until the state below is complete
     uint32_t src_int = source;   // the source in internal ids
-    if (relabeled_ && (a == Algo::SSSP || personalized)) src_int = h_old2new_[source];
+    if (relabeled_ && (a == Algo::SSSP || personalized)) src_int = internal_id(source);
     const uint32_t ppr_source = personalized ? src_int : kInf;
     if (a == Algo::LP) build_lp();
     // (the packed frontier counter needs lists of fewer than 2^32 items)
@@ -1300,13 +1442,13 @@ void Engine::build_out_edges() {
     const uint32_t S = V + n_ghost_total_;   // slots
     if ((uint64_t)V + n_ghost_total_ >= 0xFFFFFFF0ull) fail(GXP_E_INVAL, "too many vertices and cached copies");
     n_slots_ = S;
-    d_out_ptr_ = (uint32_t*)dalloc(4 * pad4((size_t)S + 1));
-    d_out_dst_ = (uint32_t*)dalloc(4 * std::max<uint64_t>(E, 1));
-    d_out_w_ = weighted_ ? (uint32_t*)dalloc(4 * std::max<uint64_t>(E, 1)) : nullptr;
+    d_out_ptr_ = (uint32_t*)dalloc_ordered(4 * pad4((size_t)S + 1));
+    d_out_dst_ = (uint32_t*)dalloc_ordered(4 * std::max<uint64_t>(E, 1));
+    d_out_w_ = weighted_ ? (uint32_t*)dalloc_ordered(4 * std::max<uint64_t>(E, 1)) : nullptr;
     std::vector<void*> tmp;
     auto talloc = [&](size_t bytes) -> void* {
         void* q = nullptr;
-        cuda_check(device_malloc(&q, std::max<size_t>(bytes, 16)), "cudaMalloc");
+        cuda_check(device_malloc(&q, std::max<size_t>(bytes, 16), false), "cudaMalloc");
         tmp.push_back(q);
         return q;
     };
@@ -1349,9 +1491,9 @@ void Engine::build_out_edges() {
 void Engine::build_frontier_lists() {
     if (d_list_[0]) return;
     list_cap_ = (uint64_t)n_slots_ + (total_edges_ + kItemEdges - 1) / kItemEdges;
-    for (auto& l : d_list_) l = (uint2*)dalloc(sizeof(uint2) * std::max<uint64_t>(list_cap_, 1));
+    for (auto& l : d_list_) l = (uint2*)dalloc_ordered(sizeof(uint2) * std::max<uint64_t>(list_cap_, 1));
     if (n_parts_ == 1)
-        for (auto& b : d_bits_) b = (uint32_t*)dalloc(4 * ((n_vertices_ + 31) / 32));
+        for (auto& b : d_bits_) b = (uint32_t*)dalloc_ordered(4 * ((n_vertices_ + 31) / 32));
 }
 
 // The frontier the next superstep reads: one vertex, or all (kInf) slots.

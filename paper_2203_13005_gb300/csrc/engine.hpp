@@ -38,6 +38,7 @@ struct HostPart {
     // device arrays above belong to the partition and the host vectors stay
     // empty until something needs them (ensure_host)
     bool on_device = false;
+    uint32_t* d_outdeg = nullptr;   // out-degrees in input ids, counted as the sources arrive
     uint64_t dev_edges = 0;
     bool dev_weighted = false;
 
@@ -73,10 +74,14 @@ public:
     uint64_t n_vertices() const { return n_vertices_; }
 
 private:
+    // dalloc: usable from any stream when it returns. dalloc_ordered: from
+    // stream_ alone until the caller has synchronized it, with no wait (the
+    // build's allocations each waited for the kernels before them: ~500 us a load)
     void* dalloc(size_t bytes);
+    void* dalloc_ordered(size_t bytes);
     // every device allocation and host-to-device copy of the context goes
     // through these, so that an injected fault can fail the n-th one
-    cudaError_t device_malloc(void** p, size_t bytes);
+    cudaError_t device_malloc(void** p, size_t bytes, bool wait = true);
     void device_free(void* p);
     cudaMemPool_t pool_ = nullptr;   // the context's device memory (device_malloc)
     void before_h2d(const char* what);
@@ -105,6 +110,7 @@ private:
     int device_;
     gxp_config cfg_;
     cudaStream_t own_stream_ = nullptr, stream_ = nullptr;
+    cudaStream_t load_stream_ = nullptr;   // a load's copies, next to the checks of what has arrived
     cudaEvent_t ev_a_ = nullptr, ev_b_ = nullptr, ev_k_ = nullptr;   // superstep start, end, kernel end
 
     // graph
@@ -244,7 +250,12 @@ private:
     RunOut* h_run_ = nullptr;      // pinned: what a launch of a run reports
     StepReport* h_steps_ = nullptr;   // pinned: what other supersteps report
     bool timed_ = true;            // the coming superstep records its events (inside gxp_run: a chunk's last)
-    std::vector<uint32_t> h_old2new_;   // host copy of the renumbering (source ids)
+    std::vector<uint32_t> h_old2new_;   // host copy of the renumbering, made at the kLookups-th source
+    static constexpr uint32_t kLookups = 8;
+    uint32_t n_lookups_ = 0;
+    uint32_t internal_id(uint32_t v);   // of input vertex v
+    std::vector<uint32_t> in_degree_above_;   // renumbered: vertices of in-degree above b, b = 0 .. kOrderExact
+    void build_sell_sorted(uint32_t H, uint32_t T);
     SellArgs sell_args() const;
     SweepArgs sweep_args() const;
     FrontierCfg frontier_cfg() const;

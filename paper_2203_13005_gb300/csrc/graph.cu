@@ -20,29 +20,45 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // block: atomics on one address serialize, and power-law generators that do
 // not permute ids (R-MAT) put their hubs at the lowest ids (the hottest
 // R-MAT 22 source has ~160K out-edges, which took ~1 ms of global atomics).
+// 16.8 M edges of a million-vertex R-MAT graph take 191 us read one source a
+// thread and 214 us read four: the reads do not bound it. A single partition's
+// CSC is therefore counted chunk by chunk behind its copy from the host (189 us
+// in eight chunks, next to 363 us of copies).
 constexpr uint32_t kOutdegHot = 8192;
 
+// kCheck: ids of n_local and above are not counted but reported (bit 1 of err).
+template <bool kCheck>
 __global__ void __launch_bounds__(256) k_outdeg(const uint32_t* __restrict__ src, uint64_t n_edges, uint32_t n_own,
                                                 uint32_t v_begin, const uint32_t* __restrict__ ghost_gid,
-                                                uint32_t* __restrict__ outdeg) {
+                                                uint32_t* __restrict__ outdeg, uint32_t* err) {
     __shared__ uint32_t hot[kOutdegHot];
     for (uint32_t i = threadIdx.x; i < kOutdegHot; i += blockDim.x) hot[i] = 0u;
     __syncthreads();
-    for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < n_edges;
-         e += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t u = src[e];
-        const uint32_t g = u < n_own ? v_begin + u : ghost_gid[u - n_own];
-        if (g < kOutdegHot) {
-            atomicAdd(&hot[g], 1u);
-        } else {
-            // one atomic per distinct source among the active lanes
-            const unsigned act = __activemask();
-            const unsigned peers = __match_any_sync(act, g);
-            if ((threadIdx.x & 31) == (unsigned)(__ffs(peers) - 1)) atomicAdd(&outdeg[g], (uint32_t)__popc(peers));
+    bool bad = false;
+    auto count = [&](uint32_t u) {
+        if (kCheck && u >= n_own) {
+            bad = true;
+            return;
         }
+        const uint32_t g = u < n_own ? v_begin + u : ghost_gid[u - n_own];
+        if (g < kOutdegHot) atomicAdd(&hot[g], 1u);
+        else atomicAdd(&outdeg[g], 1u);
+    };
+    // four sources a load (src is 16-byte aligned)
+    const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
+    const uint4* src4 = reinterpret_cast<const uint4*>(src);
+    for (uint64_t e = t0; e < n_edges / 4u; e += stride) {
+        const uint4 u = __ldg(src4 + e);
+        count(u.x);
+        count(u.y);
+        count(u.z);
+        count(u.w);
     }
+    for (uint64_t e = (n_edges & ~3ull) + t0; e < n_edges; e += stride) count(src[e]);
+    if (kCheck && bad) atomicOr(err, 2u);
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < kOutdegHot; i += blockDim.x)
+    const uint32_t n_hot = kCheck ? min(kOutdegHot, n_own) : kOutdegHot;
+    for (uint32_t i = threadIdx.x; i < n_hot; i += blockDim.x)
         if (hot[i]) atomicAdd(&outdeg[i], hot[i]);
 }
 
@@ -58,22 +74,17 @@ __global__ void k_validate(const uint32_t* __restrict__ col_ptr, uint32_t n_own,
         atomicOr(err, kErrInput);
 }
 
-// CSC imported as given: col_ptr (u64) -> u32 with its checks (bit 0 of
-// err: not running from 0 to n_edges or decreasing), sources < n_local (bit 1)
-__global__ void k_csc_import(const uint64_t* __restrict__ cp64, uint32_t n, uint64_t n_edges,
-                             uint32_t* __restrict__ cp32, const uint32_t* __restrict__ src, uint32_t n_local,
-                             uint32_t* err) {
+// offsets imported as given: col_ptr (u64) -> u32 with its checks (bit 0 of
+// err: not running from 0 to n_edges or decreasing)
+__global__ void k_csc_offsets(const uint64_t* __restrict__ cp64, uint32_t n, uint64_t n_edges,
+                              uint32_t* __restrict__ cp32, uint32_t* err) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    for (uint64_t v = t0; v <= n; v += stride) {
+    for (uint64_t v = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; v <= n; v += stride) {
         const uint64_t c = cp64[v];
         const bool bad = c > n_edges || (v == 0 && c != 0) || (v == n && c != n_edges) || (v < n && cp64[v + 1] < c);
         if (bad) atomicOr(err, 1u);
         cp32[v] = (uint32_t)c;
     }
-    bool oob = false;
-    for (uint64_t e = t0; e < n_edges; e += stride) oob |= src[e] >= n_local;
-    if (__any_sync(0xFFFFFFFFu, oob) && (threadIdx.x & 31) == 0) atomicOr(err, 2u);
 }
 
 // ------------------------------------------------------- initial values
@@ -444,7 +455,7 @@ cudaError_t launch_outdeg(const PartDev& p, const uint32_t* src, const uint32_t*
     if (p.n_edges == 0) return cudaSuccess;
     // a few blocks per SM: each flushes its shared counters once
     const uint64_t blocks = std::min<uint64_t>((p.n_edges + 255) / 256, 152ull * 4);
-    k_outdeg<<<(unsigned)blocks, 256, 0, s>>>(src, p.n_edges, p.n_own, p.v_begin, ghost_gid, outdeg);
+    k_outdeg<false><<<(unsigned)blocks, 256, 0, s>>>(src, p.n_edges, p.n_own, p.v_begin, ghost_gid, outdeg, nullptr);
     return cudaGetLastError();
 }
 
@@ -456,11 +467,18 @@ cudaError_t launch_validate_csc(const uint32_t* col_ptr, uint32_t n_own, const u
     return cudaGetLastError();
 }
 
-cudaError_t launch_csc_import(const uint64_t* cp64, uint32_t n, uint64_t n_edges, uint32_t* cp32,
-                              const uint32_t* src, uint32_t n_local, uint32_t* err, cudaStream_t s) {
-    const uint64_t work = std::max<uint64_t>((uint64_t)n + 1, n_edges);
-    const uint64_t blocks = std::min<uint64_t>((work + 255) / 256, 152ull * 16);
-    k_csc_import<<<(unsigned)blocks, 256, 0, s>>>(cp64, n, n_edges, cp32, src, n_local, err);
+cudaError_t launch_csc_offsets(const uint64_t* cp64, uint32_t n, uint64_t n_edges, uint32_t* cp32, uint32_t* err,
+                               cudaStream_t s) {
+    k_csc_offsets<<<(unsigned)std::min<uint64_t>(((uint64_t)n + 256) / 256, 152ull * 16), 256, 0, s>>>(cp64, n, n_edges,
+                                                                                                       cp32, err);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_csc_sources(const uint32_t* src, uint64_t n_edges, uint32_t n_local, uint32_t* outdeg, uint32_t* err,
+                               cudaStream_t s) {
+    if (n_edges == 0) return cudaSuccess;
+    const uint64_t blocks = std::min<uint64_t>((n_edges + 255) / 256, 152ull * 4);
+    k_outdeg<true><<<(unsigned)blocks, 256, 0, s>>>(src, n_edges, n_local, 0u, nullptr, outdeg, err);
     return cudaGetLastError();
 }
 

@@ -500,8 +500,13 @@ struct SyncArgs {
 // ------------------------------------------------------------ launchers
 cudaError_t launch_outdeg(const PartDev& p, const uint32_t* d_src, const uint32_t* d_ghost_gid,
                           uint32_t* d_outdeg, cudaStream_t s);
-cudaError_t launch_csc_import(const uint64_t* cp64, uint32_t n, uint64_t n_edges, uint32_t* cp32,
-                              const uint32_t* src, uint32_t n_local, uint32_t* err, cudaStream_t s);
+// A CSC as loaded: the offsets checked (bit 0 of *err: not running from 0 to
+// n_edges, non-decreasing) and narrowed to 32 bits; the sources checked (bit 1:
+// >= n_local) and counted into outdeg[n_local] (zeroed by the caller)
+cudaError_t launch_csc_offsets(const uint64_t* cp64, uint32_t n, uint64_t n_edges, uint32_t* cp32, uint32_t* err,
+                               cudaStream_t s);
+cudaError_t launch_csc_sources(const uint32_t* src, uint64_t n_edges, uint32_t n_local, uint32_t* outdeg, uint32_t* err,
+                               cudaStream_t s);
 // sources >= n_local set kErrBounds; offsets that do not run from 0 to n_edges
 // without decreasing set kErrInput
 cudaError_t launch_validate_csc(const uint32_t* d_col_ptr, uint32_t n_own, const uint32_t* d_src,
@@ -667,6 +672,10 @@ struct RowSource {
 cudaError_t launch_sort_rows(const uint32_t* col_ptr, uint32_t n, const RowSource& in, uint32_t n_src,
                              uint32_t* ssrc, uint32_t* sw, uint2* scratch_runs, uint32_t* scratch_cnt,
                              cudaStream_t s);   // scratch_runs: n + n_edges / 2048 + 1 entries
+// rows of col_ptr (in.row_map and in.src_map set, rows without in-edges last) as
+// loaded, sources renumbered
+cudaError_t launch_renumber_rows(const uint32_t* col_ptr, uint32_t n, const RowSource& in, uint64_t n_edges,
+                                 uint32_t* ssrc, uint32_t* sw, cudaStream_t s);
 cudaError_t launch_sell_windows(const uint32_t* col_ptr, uint32_t n, uint32_t H, uint32_t* rows_out,
                                 uint32_t* hub_out, uint32_t* nonhub_cnt, uint32_t* hub_cnt, cudaStream_t s);
 cudaError_t launch_sell_slices(const uint32_t* col_ptr, uint32_t n, const uint32_t* rows_out,
@@ -676,12 +685,20 @@ cudaError_t launch_sell_fill(const uint32_t* col_ptr, const uint32_t* ssrc, cons
                              const uint32_t* width, const uint64_t* off, uint32_t n_slices, uint32_t part,
                              uint32_t pad_id, uint32_t cols, uint32_t* sell_src, uint32_t* sell_w, SellSlice* desc,
                              cudaStream_t s);
+// a renumbered partition's slices: rows first_row .. n_rows - 1, in order of
+// decreasing in-degree (at[w] + s * sell_words(w) is slice s's start if it is w wide)
+cudaError_t launch_sell_fill_sorted(const uint32_t* col_ptr, const uint32_t* ssrc, const uint32_t* sw, uint32_t n_rows,
+                                    uint32_t first_row, const uint64_t* at, uint32_t n_slices, uint32_t cols,
+                                    uint32_t* sell_src, uint32_t* sell_w, SellSlice* desc, cudaStream_t s);
+// exclusive prefix of the parts of hub rows 0 .. n_hub_rows - 1, and their total
+cudaError_t launch_hub_offsets(const uint32_t* col_ptr, uint32_t n_hub_rows, uint32_t T, uint32_t* part_off,
+                               cudaStream_t s);
 cudaError_t launch_hub_rows(const uint32_t* col_ptr, uint32_t n, const uint32_t* hub_out, const uint32_t* hub_cnt,
                             const uint32_t* hub_base, uint32_t* hub_list, uint32_t n_hub_rows, uint32_t T,
                             uint32_t* part_off, cudaStream_t s);
 cudaError_t launch_hub_parts(const uint32_t* col_ptr, const uint32_t* hub_list, const uint32_t* part_off,
                              uint32_t n_hub_rows, uint32_t T, uint32_t part, uint32_t part_base, HubPart* hubs,
-                             cudaStream_t s);
+                             cudaStream_t s);   // hub_list nullptr: rows 0 .. n_hub_rows - 1
 // slices by decreasing width (stable); afterwards word b of
 // order_slices_starts(scratch, n) holds the number of slices wider than b
 // (b <= kOrderExact)
@@ -691,10 +708,12 @@ size_t order_slices_scratch_bytes(uint32_t n);
 const uint32_t* order_slices_starts(const uint32_t* scratch, uint32_t n);
 
 // vertex relabelling by decreasing in-degree (sell_build.cu): new2old / old2new
-// and the renumbered offsets rcol[n + 1]; scratch: relabel_scratch_bytes
+// and the renumbered offsets rcol[n + 1]; scratch: relabel_scratch_bytes.
+// *starts (in scratch): word b is the number of vertices of in-degree above b
+// (b <= kOrderExact)
 size_t relabel_scratch_bytes(uint32_t n);
 cudaError_t launch_relabel(const uint32_t* col_ptr, uint32_t n, uint32_t* new2old, uint32_t* old2new, uint32_t* rcol,
-                           uint32_t* scratch, cudaStream_t s);
+                           uint32_t* scratch, const uint32_t** starts, cudaStream_t s);
 // out[v] = in[map[v]] (gather) or out[map[v]] = in[v] (scatter)
 cudaError_t launch_permute_u32(const uint32_t* in, const uint32_t* map, uint32_t n, uint32_t* out, bool scatter,
                                cudaStream_t s);

@@ -1,6 +1,9 @@
 // Device-side build of the sliced-ELL layout of one partition (the edge
 // blocks of Section II-B, in the form the superstep kernel reads):
 //
+// One partition with renumbered vertices skips most of it (k_renumber_rows,
+// k_sell_fill_sorted): its rows are in order of in-degree already. Otherwise:
+//
 //  1. k_sort_rows_warp / k_sort_rows_block: each row's in-edges sorted by
 //     source, so the k-th sources of a slice's rows fall in similar id
 //     ranges. Rows of up to 32 / 256 edges are bitonic-sorted in a warp's
@@ -274,6 +277,69 @@ __global__ void __launch_bounds__(kRadixWarps * 32) k_sort_rows_block(const uint
     }
 }
 
+// A renumbered partition's rows, in the order of their in-edges as loaded:
+// edge e of the result (row r, offsets col_ptr) is in's edge of row row_map[r]
+// with its source renumbered. A CTA takes kRowChunk consecutive edges: the
+// rows they belong to (rows without in-edges come last, so at most that many)
+// are found by a 32-ary search and their offsets kept in shared memory.
+// The rows are not sorted by source: one partition's superstep kernel gains
+// nothing from it (traced, unsorted / sorted: PageRank R-MAT 22 3,045 / 3,051
+// us a run, SSSP R-MAT 22 973 / 1,020 us), and the two sort kernels took 691 us
+// of a load of 16.8 M edges; this one takes 89 us (unweighted; 12 bytes an
+// edge, so 2.3 TB/s).
+constexpr uint32_t kRowChunk = 2048;
+__device__ __forceinline__ uint32_t row_of_edge(const uint32_t* __restrict__ col_ptr, uint32_t n, uint32_t e) {   // by one warp
+    // the last row r < n with col_ptr[r] <= e
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t lo = 0, hi = n - 1u;
+    while (lo < hi) {
+        const uint32_t step = (hi - lo + 31u) / 32u;
+        const uint32_t at = (uint32_t)min((uint64_t)lo + (uint64_t)(lane + 1u) * step, (uint64_t)hi);
+        const uint32_t c = (uint32_t)__popc(__ballot_sync(kFull, __ldg(col_ptr + at) <= e));
+        const uint64_t nlo = (uint64_t)lo + (uint64_t)c * step, nhi = nlo + step - 1u;
+        if (c == 32u) {
+            lo = hi;
+        } else {
+            hi = (uint32_t)min(nhi, (uint64_t)hi);
+            lo = (uint32_t)min(nlo, (uint64_t)hi);
+        }
+    }
+    return lo;
+}
+template <bool kW>
+__global__ void __launch_bounds__(256) k_renumber_rows(const uint32_t* __restrict__ col_ptr, uint32_t n, const RowSource in,
+                                                       uint32_t n_edges, uint32_t* __restrict__ ssrc,
+                                                       uint32_t* __restrict__ sw) {
+    __shared__ uint32_t s_off[kRowChunk + 1], s_delta[kRowChunk];   // a row's first edge; its input edge less that
+    __shared__ uint32_t s_row[2];
+    const uint32_t e0 = blockIdx.x * kRowChunk, ne = min(kRowChunk, n_edges - e0);
+    const uint32_t warp = threadIdx.x >> 5;
+    if (warp < 2) {
+        const uint32_t r = row_of_edge(col_ptr, n, warp ? e0 + ne - 1u : e0);
+        if ((threadIdx.x & 31) == 0) s_row[warp] = r;
+    }
+    __syncthreads();
+    const uint32_t r0 = s_row[0], nr = min(s_row[1] - r0 + 1u, kRowChunk);
+    for (uint32_t k = threadIdx.x; k < nr; k += 256u) {
+        const uint32_t c = col_ptr[r0 + k];
+        s_off[k] = c;
+        s_delta[k] = in.col_ptr[in.row_map[r0 + k]] - c;
+    }
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < ne; j += 256u) {
+        const uint32_t e = e0 + j;
+        uint32_t lo = 0, hi = nr - 1u;
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi + 1u) >> 1;
+            if (s_off[mid] <= e) lo = mid;
+            else hi = mid - 1u;
+        }
+        const uint32_t i = e + s_delta[lo];
+        ssrc[e] = __ldg(in.src_map + __ldcs(in.src + i));
+        if (kW) sw[e] = __ldcs(in.w + i);
+    }
+}
+
 __device__ __forceinline__ uint32_t deg_bin(uint32_t d) {
     return d <= kExactBins ? d : kExactBins + (31u - (uint32_t)__clz(d));
 }
@@ -441,10 +507,34 @@ __global__ void __launch_bounds__(1024) k_scan_widths(const uint32_t* width, uin
     if (t == 1023) out[n] = part[1023];
 }
 
+// A slice stored as lane groups at o (sell_words), its rows' in-edges [b, b +
+// d) one per lane, written in storage order: lane l's 4 entries of column
+// group g are one 128-bit store, and its row group's reads are consecutive.
+__device__ __forceinline__ void fill_lane_groups(const uint32_t* ssrc, const uint32_t* sw, uint32_t b, uint32_t d,
+                                                 uint32_t wd, uint32_t cols, uint64_t o, uint32_t pad_id,
+                                                 uint32_t* sell_src, uint32_t* sell_w, int lane) {
+    const uint32_t L = sweep_lanes(wd, cols), rows = 32u / L, c = sweep_cols(wd, L);
+    for (uint32_t sub = 0; sub < L; ++sub) {
+        const int slot = (int)(sub * rows + (uint32_t)lane / L);   // this lane's row
+        const uint32_t rb = __shfl_sync(kFull, b, slot), rd = __shfl_sync(kFull, d, slot);
+        const uint64_t at0 = o + 32ull * c * sub + 4u * lane;   // sweep_idx
+        for (uint32_t g = 0; g < c / 4u; ++g) {
+            uint32_t x[4], y[4];
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q) {
+                const uint32_t k = (4u * g + q) * L + (uint32_t)lane % L;
+                const bool has = k < rd;
+                x[q] = has ? ssrc[rb + k] : pad_id;
+                y[q] = (sell_w && has) ? sw[rb + k] : 0u;
+            }
+            *reinterpret_cast<uint4*>(sell_src + at0 + 128ull * g) = make_uint4(x[0], x[1], x[2], x[3]);
+            if (sell_w) *reinterpret_cast<uint4*>(sell_w + at0 + 128ull * g) = make_uint4(y[0], y[1], y[2], y[3]);
+        }
+    }
+}
+
 // one warp per slice: the sources (and weights) as the slice is stored
-// (sell_words: column-major, or lane groups), descriptors. Lane groups are
-// written in storage order: lane l's 4 entries of column group g are one
-// 128-bit store, and its row group's reads of the row are consecutive.
+// (sell_words: column-major, or lane groups), descriptors
 __global__ void k_sell_fill(const uint32_t* col_ptr, const uint32_t* ssrc, const uint32_t* sw, const uint32_t* perm,
                             const uint32_t* width, const uint64_t* off, uint32_t n_slices, uint32_t part,
                             uint32_t pad_id, uint32_t cols, uint32_t* sell_src, uint32_t* sell_w, SellSlice* desc) {
@@ -464,33 +554,36 @@ __global__ void k_sell_fill(const uint32_t* col_ptr, const uint32_t* ssrc, const
                 sell_src[at] = has ? ssrc[b + k] : pad_id;
                 if (sell_w) sell_w[at] = has ? sw[b + k] : 0u;
             }
-        } else {
-            const uint32_t L = sweep_lanes(wd, cols), rows = 32u / L, c = sweep_cols(wd, L);
-            for (uint32_t sub = 0; sub < L; ++sub) {
-                const int slot = (int)(sub * rows + (uint32_t)lane / L);   // this lane's row
-                const uint32_t rb = __shfl_sync(kFull, b, slot), rd = __shfl_sync(kFull, d, slot);
-                const uint64_t at0 = o + 32ull * c * sub + 4u * lane;   // sweep_idx
-                for (uint32_t g = 0; g < c / 4u; ++g) {
-                    uint32_t x[4], y[4];
-#pragma unroll
-                    for (uint32_t q = 0; q < 4; ++q) {
-                        const uint32_t k = (4u * g + q) * L + (uint32_t)lane % L;
-                        const bool has = k < rd;
-                        x[q] = has ? ssrc[rb + k] : pad_id;
-                        y[q] = (sell_w && has) ? sw[rb + k] : 0u;
-                    }
-                    *reinterpret_cast<uint4*>(sell_src + at0 + 128ull * g) = make_uint4(x[0], x[1], x[2], x[3]);
-                    if (sell_w) *reinterpret_cast<uint4*>(sell_w + at0 + 128ull * g) = make_uint4(y[0], y[1], y[2], y[3]);
-                }
-            }
-        }
-        if (!cols) {
             if (lane == 0) desc[s] = SellSlice{part, (uint32_t)(s * 32), wd, 0u, o};
-        } else {   // a renumbered partition's slices mostly hold consecutive vertices, any empty slots last
+        } else {
+            fill_lane_groups(ssrc, sw, b, d, wd, cols, o, pad_id, sell_src, sell_w, lane);
+            // (empty slots come last)
             const uint32_t first = __shfl_sync(kFull, r, 0), n = (uint32_t)__popc(__ballot_sync(kFull, r != kSellPad));
             const bool in_row = __all_sync(kFull, (uint32_t)lane < n ? r == first + (uint32_t)lane : r == kSellPad);
             if (lane == 0) desc[s] = SellSlice{in_row ? n : 0u, (uint32_t)(s * 32), wd, first, o};
         }
+    }
+}
+
+// The slices of a renumbered partition, whose rows from `first_row` on are in
+// order of decreasing in-degree: slice s holds rows first_row + 32 s .., is as
+// wide as its first row and starts at at[width] + s * sell_words(width),
+// which the host derives from the in-degree counts. No window sort, row
+// slots, width scan or slice order (at 1 M vertices those took 510 us).
+__global__ void k_sell_fill_sorted(const uint32_t* col_ptr, const uint32_t* ssrc, const uint32_t* sw, uint32_t n_rows,
+                                   uint32_t first_row, const uint64_t* at, uint32_t n_slices, uint32_t cols,
+                                   uint32_t* sell_src, uint32_t* sell_w, SellSlice* desc) {
+    const int lane = threadIdx.x & 31;
+    const uint64_t warp0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t n_warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    for (uint64_t s = warp0; s < n_slices; s += n_warps) {
+        const uint32_t first = first_row + (uint32_t)(32u * s), n = min(32u, n_rows - first);
+        const bool has = (uint32_t)lane < n;
+        const uint32_t b = has ? col_ptr[first + lane] : 0u, d = has ? col_ptr[first + lane + 1] - b : 0u;
+        const uint32_t wd = __shfl_sync(kFull, d, 0);
+        const uint64_t o = at[wd] + s * sell_words(wd, cols);
+        if (wd) fill_lane_groups(ssrc, sw, b, d, wd, cols, o, n_rows, sell_src, sell_w, lane);   // padding id: n_rows
+        if (lane == 0) desc[s] = SellSlice{n, 0u, wd, first, o};
     }
 }
 
@@ -501,7 +594,8 @@ __global__ void k_hub_rows(const uint32_t* hub_out, const uint32_t* hub_cnt, con
     for (uint32_t i = threadIdx.x; i < cnt; i += blockDim.x) hub_list[base + i] = hub_out[w0 + i];
 }
 
-// single CTA: exclusive prefix of the parts of each hub row; out[n] = total
+// single CTA: exclusive prefix of the parts of each hub row (hub_list, or rows
+// 0 .. n - 1 of a renumbered partition); out[n] = total
 __global__ void __launch_bounds__(1024) k_scan_parts(const uint32_t* col_ptr, const uint32_t* hub_list, uint32_t n,
                                                      uint32_t T, uint32_t* out) {
     __shared__ uint32_t part[1024];
@@ -509,7 +603,7 @@ __global__ void __launch_bounds__(1024) k_scan_parts(const uint32_t* col_ptr, co
     const uint32_t per = (n + 1023) / 1024;
     const uint32_t a = min(n, t * per), b = min(n, a + per);
     auto parts = [&](uint32_t h) {
-        const uint32_t v = hub_list[h];
+        const uint32_t v = hub_list ? hub_list[h] : h;
         const uint32_t d = col_ptr[v + 1] - col_ptr[v];
         return (d + T - 1) / T;
     };
@@ -533,11 +627,13 @@ __global__ void __launch_bounds__(1024) k_scan_parts(const uint32_t* col_ptr, co
 
 __global__ void k_hub_parts(const uint32_t* col_ptr, const uint32_t* hub_list, const uint32_t* part_off, uint32_t n,
                             uint32_t T, uint32_t part, uint32_t part_base, HubPart* hubs) {
-    for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < n; h += gridDim.x * blockDim.x) {
-        const uint32_t v = hub_list[h];
+    // a warp per row: the longest have hundreds of parts
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t h = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; h < n; h += (gridDim.x * blockDim.x) >> 5) {
+        const uint32_t v = hub_list ? hub_list[h] : h;
         const uint32_t b = col_ptr[v], d = col_ptr[v + 1] - b;
         const uint32_t np = (d + T - 1) / T, local = part_off[h], t0 = part_base + local;
-        for (uint32_t k = 0; k < np; ++k)   // this partition's array; t0 indexes all partitions' parts
+        for (uint32_t k = lane; k < np; k += 32u)   // this partition's array; t0 indexes all partitions' parts
             hubs[local + k] = HubPart{v, part, b + k * T, min(T, d - k * T), t0, np, {0u, 0u}};
     }
 }
@@ -602,37 +698,112 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_order_scatter(const SellSli
 // the most gathered values share cache lines (exact up to kExactBins, by
 // power of two above)
 
+//
+// A CTA per kRelChunk vertices (at 65,536, the windows' size, a graph of a
+// million vertices kept 16 SMs busy: scatter 119 us, now 35): per-chunk bin
+// counts, a warp per bin scanning them over the chunks, the bins' starts, and
+// a scatter whose warps recount their own shares in shared memory. The
+// scatter writes the inverse map and the new vertices' in-degrees too.
+constexpr uint32_t kRelChunk = 8192;
+constexpr uint32_t kRelShare = kRelChunk / kSortWarps;
+
 __global__ void __launch_bounds__(kSortWarps * 32) k_vdeg_count(const uint32_t* col_ptr, uint32_t n,
                                                                 uint32_t* ghist) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __shared__ uint32_t hist[kSortWarps][kBins];
-    for (uint32_t i = threadIdx.x; i < kSortWarps * kBins; i += blockDim.x) (&hist[0][0])[i] = 0u;
+    __shared__ uint32_t hist[kBins];
+    for (uint32_t i = threadIdx.x; i < kBins; i += blockDim.x) hist[i] = 0u;
     __syncthreads();
-    const uint32_t c0 = min(n, blockIdx.x * kSellWindow + warp * kSortChunk), c1 = min(n, c0 + kSortChunk);
-    for (uint32_t v = c0 + lane; v < c1; v += 32) atomicAdd(&hist[warp][deg_bin(col_ptr[v + 1] - col_ptr[v])], 1u);
+    const uint32_t c0 = blockIdx.x * kRelChunk, c1 = (uint32_t)min((uint64_t)n, (uint64_t)c0 + kRelChunk);
+    for (uint32_t v = c0 + threadIdx.x; v < c1; v += blockDim.x) {
+        // most vertices share a few low bins: one add per bin and warp
+        const uint32_t b = deg_bin(col_ptr[v + 1] - col_ptr[v]);
+        const unsigned act = __activemask(), peers = __match_any_sync(act, b);
+        if ((threadIdx.x & 31) == (unsigned)(__ffs(peers) - 1)) atomicAdd(&hist[b], (uint32_t)__popc(peers));
+    }
     __syncthreads();
-    uint32_t* g = ghist + (uint64_t)blockIdx.x * kSortWarps * kBins;
-    for (uint32_t i = threadIdx.x; i < kSortWarps * kBins; i += blockDim.x) g[i] = (&hist[0][0])[i];
+    for (uint32_t i = threadIdx.x; i < kBins; i += blockDim.x) ghist[(uint64_t)blockIdx.x * kBins + i] = hist[i];
+}
+
+// a warp per bin: exclusive prefix over the chunks, total into tot[bin]
+__global__ void __launch_bounds__(256) k_bin_prefix(uint32_t* ghist, uint32_t chunks, uint32_t* tot) {
+    const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (b >= kBins) return;
+    uint32_t run = 0;
+    for (uint32_t c0 = 0; c0 < chunks; c0 += 32) {
+        const uint32_t c = c0 + lane;
+        const uint32_t x = c < chunks ? ghist[(uint64_t)c * kBins + b] : 0u;
+        uint32_t incl = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (c < chunks) ghist[(uint64_t)c * kBins + b] = run + incl - x;
+        run += __shfl_sync(kFull, incl, 31);
+    }
+    if (lane == 0) tot[b] = run;
+}
+
+// one warp: tot[b] -> the number of vertices in bins above b
+__global__ void __launch_bounds__(32) k_bin_starts(uint32_t* tot) {
+    const int lane = threadIdx.x;
+    constexpr int kChunk = (int)((kBins + 31) / 32);
+    const int hi = (int)kBins - 1 - lane * kChunk;   // lane l takes a chunk of bins, descending
+    uint32_t x[kChunk], sum = 0;
+#pragma unroll
+    for (int i = 0; i < kChunk; ++i) x[i] = hi - i >= 0 ? tot[hi - i] : 0u;
+#pragma unroll
+    for (int i = 0; i < kChunk; ++i) sum += x[i];
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += t;
+    }
+    uint32_t run = incl - sum;
+#pragma unroll
+    for (int i = 0; i < kChunk; ++i) {
+        if (hi - i >= 0) tot[hi - i] = run;
+        run += x[i];
+    }
 }
 
 __global__ void __launch_bounds__(kSortWarps * 32) k_vdeg_scatter(const uint32_t* col_ptr, uint32_t n,
-                                                                  uint32_t* ghist, uint32_t* new2old) {
-    const int warp = threadIdx.x >> 5;
-    const uint32_t c0 = min(n, blockIdx.x * kSellWindow + warp * kSortChunk), c1 = min(n, c0 + kSortChunk);
-    uint32_t* offs = ghist + ((uint64_t)blockIdx.x * kSortWarps + warp) * kBins;
-    warp_scatter(
-        c0, c1, offs, [&](uint32_t v) { return deg_bin(col_ptr[v + 1] - col_ptr[v]); },
-        [&](uint32_t v, uint32_t pos) { new2old[pos] = v; });
-}
-
-// old2new = inverse of new2old; rdeg[i] = in-degree of new vertex i
-__global__ void k_invert(const uint32_t* col_ptr, const uint32_t* new2old, uint32_t n, uint32_t* old2new,
-                         uint32_t* rdeg) {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const uint32_t v = new2old[i];
-        old2new[v] = i;
-        rdeg[i] = col_ptr[v + 1] - col_ptr[v];
+                                                                  const uint32_t* ghist, const uint32_t* starts,
+                                                                  uint32_t* new2old, uint32_t* old2new, uint32_t* rdeg) {
+    __shared__ uint32_t hist[kSortWarps][kBins];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (uint32_t i = threadIdx.x; i < kSortWarps * kBins; i += blockDim.x) (&hist[0][0])[i] = 0u;
+    __syncthreads();
+    const uint64_t base = (uint64_t)blockIdx.x * kRelChunk + (uint64_t)warp * kRelShare;
+    const uint32_t c0 = (uint32_t)min((uint64_t)n, base), c1 = (uint32_t)min((uint64_t)n, base + kRelShare);
+    auto bin_of = [&](uint32_t v) { return deg_bin(col_ptr[v + 1] - col_ptr[v]); };
+    for (uint32_t v0 = c0; v0 < c1; v0 += 32) {
+        const uint32_t v = v0 + lane;
+        const bool ok = v < c1;
+        const uint32_t b = ok ? bin_of(v) : 0u;
+        const unsigned act = __ballot_sync(kFull, ok);
+        if (ok) {
+            const unsigned peers = __match_any_sync(act, b);
+            if (lane == __ffs(peers) - 1) hist[warp][b] += (uint32_t)__popc(peers);
+        }
+        __syncwarp();
     }
+    __syncthreads();
+    for (uint32_t b = threadIdx.x; b < kBins; b += blockDim.x) {
+        uint32_t run = starts[b] + ghist[(uint64_t)blockIdx.x * kBins + b];
+        for (int w = 0; w < kSortWarps; ++w) {
+            const uint32_t c = hist[w][b];
+            hist[w][b] = run;
+            run += c;
+        }
+    }
+    __syncthreads();
+    warp_scatter(c0, c1, hist[warp], bin_of, [&](uint32_t v, uint32_t pos) {
+        new2old[pos] = v;
+        old2new[v] = pos;
+        rdeg[pos] = col_ptr[v + 1] - col_ptr[v];
+    });
 }
 
 // three-phase exclusive scan of u32 counts: x[0..n) -> out[0..n], out[n] = total
@@ -744,6 +915,15 @@ cudaError_t launch_sort_rows(const uint32_t* col_ptr, uint32_t n, const RowSourc
     return cudaGetLastError();
 }
 
+cudaError_t launch_renumber_rows(const uint32_t* col_ptr, uint32_t n, const RowSource& in, uint64_t n_edges,
+                                 uint32_t* ssrc, uint32_t* sw, cudaStream_t s) {
+    if (n_edges == 0) return cudaSuccess;
+    const uint32_t grid = (uint32_t)((n_edges + kRowChunk - 1) / kRowChunk);
+    if (in.w) k_renumber_rows<true><<<grid, 256, 0, s>>>(col_ptr, n, in, (uint32_t)n_edges, ssrc, sw);
+    else k_renumber_rows<false><<<grid, 256, 0, s>>>(col_ptr, n, in, (uint32_t)n_edges, ssrc, sw);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_sell_windows(const uint32_t* col_ptr, uint32_t n, uint32_t H, uint32_t* rows_out,
                                 uint32_t* hub_out, uint32_t* nonhub_cnt, uint32_t* hub_cnt, cudaStream_t s) {
     const uint32_t nw = (n + kSellWindow - 1) / kSellWindow;
@@ -771,6 +951,21 @@ cudaError_t launch_sell_fill(const uint32_t* col_ptr, const uint32_t* ssrc, cons
     return cudaGetLastError();
 }
 
+cudaError_t launch_sell_fill_sorted(const uint32_t* col_ptr, const uint32_t* ssrc, const uint32_t* sw, uint32_t n_rows,
+                                    uint32_t first_row, const uint64_t* at, uint32_t n_slices, uint32_t cols,
+                                    uint32_t* sell_src, uint32_t* sell_w, SellSlice* desc, cudaStream_t s) {
+    if (n_slices == 0) return cudaSuccess;
+    k_sell_fill_sorted<<<grid_warps(n_slices, 256), 256, 0, s>>>(col_ptr, ssrc, sw, n_rows, first_row, at, n_slices,
+                                                                 cols, sell_src, sell_w, desc);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_hub_offsets(const uint32_t* col_ptr, uint32_t n_hub_rows, uint32_t T, uint32_t* part_off,
+                               cudaStream_t s) {
+    k_scan_parts<<<1, 1024, 0, s>>>(col_ptr, nullptr, n_hub_rows, T, part_off);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_hub_rows(const uint32_t* col_ptr, uint32_t n, const uint32_t* hub_out, const uint32_t* hub_cnt,
                             const uint32_t* hub_base, uint32_t* hub_list, uint32_t n_hub_rows, uint32_t T,
                             uint32_t* part_off, cudaStream_t s) {
@@ -784,7 +979,7 @@ cudaError_t launch_hub_parts(const uint32_t* col_ptr, const uint32_t* hub_list, 
                              uint32_t n_hub_rows, uint32_t T, uint32_t part, uint32_t part_base, HubPart* hubs,
                              cudaStream_t s) {
     if (n_hub_rows == 0) return cudaSuccess;
-    k_hub_parts<<<(n_hub_rows + 255) / 256, 256, 0, s>>>(col_ptr, hub_list, part_off, n_hub_rows, T, part, part_base,
+    k_hub_parts<<<grid_warps(n_hub_rows, 256), 256, 0, s>>>(col_ptr, hub_list, part_off, n_hub_rows, T, part, part_base,
                                                          hubs);
     return cudaGetLastError();
 }
@@ -814,27 +1009,28 @@ const uint32_t* order_slices_starts(const uint32_t* scratch, uint32_t n) {
 namespace gxp {
 
 size_t relabel_scratch_bytes(uint32_t n) {
-    const uint64_t chunks = (n + kSellWindow - 1) / kSellWindow;
+    const uint64_t chunks = (n + kRelChunk - 1) / kRelChunk;
     const uint64_t scan_blocks = (n + kScanChunk - 1) / kScanChunk;
-    return 4 * ((size_t)(chunks + 1) * kSortWarps * kBins + (size_t)scan_blocks + 1 + (size_t)n + 1);
+    return 4 * ((size_t)(chunks + 1) * kBins + (size_t)scan_blocks + 1 + (size_t)n + 1);
 }
 
 cudaError_t launch_relabel(const uint32_t* col_ptr, uint32_t n, uint32_t* new2old, uint32_t* old2new, uint32_t* rcol,
-                           uint32_t* scratch, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    const uint32_t chunks = (n + kSellWindow - 1) / kSellWindow;
+                           uint32_t* scratch, const uint32_t** starts, cudaStream_t s) {
+    if (n == 0) return cudaErrorInvalidValue;
+    const uint32_t chunks = (n + kRelChunk - 1) / kRelChunk;
     const uint32_t scan_blocks = (n + kScanChunk - 1) / kScanChunk;
     uint32_t* ghist = scratch;
-    uint32_t* sums = ghist + (size_t)(chunks + 1) * kSortWarps * kBins;
+    uint32_t* tot = ghist + (size_t)chunks * kBins;
+    uint32_t* sums = tot + kBins;
     uint32_t* rdeg = sums + scan_blocks + 1;
     k_vdeg_count<<<chunks, kSortWarps * 32, 0, s>>>(col_ptr, n, ghist);
-    k_order_offsets<<<1, 1024, 0, s>>>(ghist, chunks * kSortWarps);
-    k_vdeg_scatter<<<chunks, kSortWarps * 32, 0, s>>>(col_ptr, n, ghist, new2old);
-    const uint32_t g = std::min<uint32_t>((n + 255) / 256, 152u * 16);
-    k_invert<<<g, 256, 0, s>>>(col_ptr, new2old, n, old2new, rdeg);
+    k_bin_prefix<<<(kBins + 7) / 8, 256, 0, s>>>(ghist, chunks, tot);
+    k_bin_starts<<<1, 32, 0, s>>>(tot);
+    k_vdeg_scatter<<<chunks, kSortWarps * 32, 0, s>>>(col_ptr, n, ghist, tot, new2old, old2new, rdeg);
     k_scan_sums<<<scan_blocks, 256, 0, s>>>(rdeg, n, sums);
     k_scan_top<<<1, 1024, 0, s>>>(sums, scan_blocks);
     k_scan_apply<<<scan_blocks, 256, 0, s>>>(rdeg, n, sums, rcol);
+    *starts = tot;
     return cudaGetLastError();
 }
 
