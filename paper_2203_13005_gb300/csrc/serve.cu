@@ -33,6 +33,16 @@ namespace {
 constexpr int kSvBlock = 256;
 constexpr int kSvWarps = kSvBlock / 32;
 constexpr int kSvUnroll = 4;   // message rows in flight per lane
+constexpr int kSvDeep = 8;     // and where few warps share the chip
+// The lines between them, from bursts of n R-MAT vertices, 12 n edges:
+//  * up to kDeepWarps warps a superstep, 8 rows in flight and the next ids read
+//    ahead (3 CTAs an SM): 32 queries, n = 2^16, 17 K warps 3,152 us against
+//    3,310, n = 2^17, 35 K warps 3,860 / 3,897, n = 2^18 5,114 / 4,659.
+//  * lane groups are widened until a superstep has kFullWarps warps (16 an SM):
+//    a query alone, n = 2^14: 754 us against 840; 32 an SM 738, 64 an SM 733,
+//    but 32 queries, n = 2^15, 2,795 / 2,956 / 3,100 us.
+constexpr uint64_t kDeepWarps = 152ull * 160;
+constexpr uint64_t kFullWarps = 152ull * 16;
 constexpr int kTileRows = 64;   // rows per transpose tile
 
 uint32_t grid_for(uint64_t items, uint64_t per_block) {
@@ -126,24 +136,32 @@ struct PprSlots {
 
 // LG lanes per work unit, 32 / LG units per warp (neighbours in the units'
 // order, which have about the same length); lanes without a busy slot skip
-// every load and store. kSvUnroll source ids are read at a time (a broadcast
-// load within the lane group), then their message rows are in flight
-// together; the sum runs in edge order. What bounds it: the L2 bandwidth of
-// the rows with all slots in use, instruction issue with few. 32 queries on
+// every load and store. U source ids are read at a time (a broadcast load
+// within the lane group), then their message rows are in flight together; the
+// sum runs in edge order. What bounds it: the L2 bandwidth of the rows with all
+// slots in use; on small graphs the chain of a unit's 256 edges (a query alone
+// on 2^14 vertices: 33 us a launch with a unit a warp and 8 rows in flight,
+// 64 us with 4 rows and 32 units a warp). 32 queries on
 // each of three graphs (8.4, 2.1 and 0.5 M edges, ~22 supersteps each): 10.9 ms
 // in this kernel with a unit per warp and two slots a lane whatever the slots
 // in use, 4.8 ms so (4 rows in flight and 6 CTAs an SM; 8 rows and 3 / 4 CTAs
 // 5.2 / 4.5 ms, 4 rows and 8 CTAs 5.5 ms, the whole burst 13.8 / 13.9 / 12.6
 // against 12.8 ms).
-template <int LG>
-__global__ void __launch_bounds__(kSvBlock, 6) k_ppr_units(const PprArgs a) {
+template <int LG, int U, int kCtas>
+__global__ void __launch_bounds__(kSvBlock, kCtas) k_ppr_units(const PprArgs a) {
     constexpr uint32_t kPer = 32 / LG;
     __shared__ PprSlots sl;
     sl.init(a);
     const uint32_t lane = threadIdx.x & 31u, l = lane % LG, sub = lane / LG;
     const bool live = (a.active_mask >> (4 * l)) & 15ull;
     const float4* msg = reinterpret_cast<const float4*>(a.msg_cur);
-    const uint64_t warp0 = ((uint64_t)blockIdx.x * kSvBlock + threadIdx.x) >> 5;
+    // With up to four slots a warp holds many units and the longest are few
+    // warps: those go to a CTA each (a query alone, n = 2^19 R-MAT vertices:
+    // 3,100 us against 3,516). With more slots neighbouring units stay together
+    // (32 queries there: 6,437 us against 7,692).
+    const uint32_t warp = threadIdx.x >> 5;
+    const uint64_t warp0 = a.active_mask >> 4 ? (uint64_t)blockIdx.x * kSvWarps + warp
+                                              : (uint64_t)warp * gridDim.x + blockIdx.x;
     const uint64_t n_warps = ((uint64_t)gridDim.x * kSvBlock) >> 5;
     for (uint64_t k0 = warp0 * kPer; k0 < a.n_units; k0 += n_warps * kPer) {
         const bool has = k0 + sub < a.n_units;
@@ -151,21 +169,28 @@ __global__ void __launch_bounds__(kSvBlock, 6) k_ppr_units(const PprArgs a) {
         const float inv = __ldg(a.inv_outdeg + un.x);
         const uint32_t* e = a.src + un.y;
         float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        for (uint32_t i = 0; i < un.z; i += kSvUnroll) {
-            uint32_t u[kSvUnroll];
+        uint32_t u[U], next[U];
 #pragma unroll
-            for (int q = 0; q < kSvUnroll; ++q) u[q] = i + q < un.z ? __ldg(e + i + q) : kInf;
-            float4 m[kSvUnroll];
+        for (int q = 0; q < U; ++q) u[q] = q < un.z ? __ldg(e + q) : kInf;
+        for (uint32_t i = 0; i < un.z; i += U) {
+            if (U > kSvUnroll) {   // the next ids on their way with these rows
 #pragma unroll
-            for (int q = 0; q < kSvUnroll; ++q)
+                for (int q = 0; q < U; ++q) next[q] = i + U + q < un.z ? __ldg(e + i + U + q) : kInf;
+            }
+            float4 m[U];
+#pragma unroll
+            for (int q = 0; q < U; ++q)
                 m[q] = (u[q] != kInf && live) ? msg[(uint64_t)u[q] * 16u + l] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-            for (int q = 0; q < kSvUnroll; ++q) {   // (an absent edge adds zero)
+            for (int q = 0; q < U; ++q) {   // (an absent edge adds zero)
                 acc.x += m[q].x;
                 acc.y += m[q].y;
                 acc.z += m[q].z;
                 acc.w += m[q].w;
             }
+#pragma unroll
+            for (int q = 0; q < U; ++q)
+                u[q] = U > kSvUnroll ? next[q] : (i + U + q < un.z ? __ldg(e + i + U + q) : kInf);
         }
         if (!live || !has) continue;
         if (un.w) reinterpret_cast<float4*>(a.partial)[(uint64_t)(un.w - 1u) * 16u + l] = acc;
@@ -276,10 +301,15 @@ __global__ void __launch_bounds__(kSvBlock) k_gather_columns(const uint32_t* mat
 }  // namespace
 
 cudaError_t launch_ppr_superstep(const PprArgs& a, cudaStream_t s) {
-    return with_slot_lanes(a.active_mask, [&](auto lanes) {
+    uint64_t lanes_mask = a.active_mask;   // (LG lanes for the highest set slot)
+    for (uint32_t lg = 1; lg < 16u; lg *= 2)
+        if (a.n_units * lg < 32u * kFullWarps) lanes_mask |= 1ull << (4u * lg);
+    return with_slot_lanes(lanes_mask, [&](auto lanes) {
         constexpr int LG = decltype(lanes)::value;
         constexpr uint64_t kPer = 32 / LG;
-        k_ppr_units<LG><<<serve_grid((a.n_units + kPer - 1) / kPer), kSvBlock, 0, s>>>(a);
+        const uint64_t warps = (a.n_units + kPer - 1) / kPer;
+        if (warps <= kDeepWarps) k_ppr_units<LG, kSvDeep, 3><<<serve_grid(warps), kSvBlock, 0, s>>>(a);
+        else k_ppr_units<LG, kSvUnroll, 6><<<serve_grid(warps), kSvBlock, 0, s>>>(a);
         if (a.n_split_rows)
             k_ppr_split<LG><<<serve_grid((a.n_split_rows + kPer - 1) / kPer), kSvBlock, 0, s>>>(a);
         return cudaGetLastError();
