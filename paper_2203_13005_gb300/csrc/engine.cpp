@@ -1250,6 +1250,7 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
     if (timed_) cuda_check(cudaEventRecord(ev_a_, stream_), "event");
     if (algo_ == Algo::LP) {
         LpArgs l{};
+        l.n_ghost = n_ghost_total_;
         l.parts = lp_.d_parts;
         l.n_parts = n_parts_;
         l.slices = lp_.d_slices;

@@ -441,6 +441,7 @@ struct LpArgs {
     uint32_t* seg_used;             // [n_segments] 1 once a label took a slot of the segment; cleared after use
     const uint32_t* own_cur;
     uint32_t* own_nxt;
+    uint32_t n_ghost;                // all partitions' copies
     const uint32_t* ghost;
     uint32_t* changed_bits;     // bitmap of the vertices this superstep changes, or nullptr
     const StepStats* stats_in;

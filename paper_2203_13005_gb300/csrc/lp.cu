@@ -566,8 +566,17 @@ __global__ void k_lp_hubs(const LpArgs a) {
 cudaError_t launch_lp_superstep(const LpArgs& a, cudaStream_t s) {
     if (a.active)
         k_lp_mark<<<(uint32_t)std::min<uint64_t>((a.n_vertices / 32u + 8u) / 8u, 152ull * 8), kLpBlock, 0, s>>>(a);
-    const uint32_t g_slices =
-        (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((a.n_slices + 7ull) / 8, 152ull * 64));
+    // The slices run partition after partition, wide ones first. Where labels
+    // and copies do not fit L2 (129 MB) only a grid of a warp per slice keeps
+    // to that order, so that one partition's copies are gathered from at a
+    // time; where they fit, 4 CTAs an SM stride over the slices. ER graphs in 8
+    // partitions, m = 16 n, a run of 14 or 15 supersteps, a warp per slice / 4
+    // CTAs an SM: n = 2^24 (537 MB) 19.6 / 26.1 ms, 2^23 (268 MB) 9.4 / 9.7 ms,
+    // 2^22 (134 MB) 4.9 / 4.7 ms; one partition of 2^24 (67 MB) 15.8 / 13.5 ms.
+    // (64 CTAs an SM, each striding over every partition: 59.5 ms at 2^24.)
+    const bool in_order = 4ull * ((uint64_t)a.n_vertices + a.n_ghost) > (160ull << 20);
+    const uint32_t g_slices = (uint32_t)std::max<uint64_t>(
+        1, std::min<uint64_t>((a.n_slices + 7ull) / 8, in_order ? 1ull << 24 : 152ull * 4));
     if (a.n_parts == 1) k_lp_slices<true><<<g_slices, kLpBlock, 0, s>>>(a);   // also clears the stat slot
     else k_lp_slices<false><<<g_slices, kLpBlock, 0, s>>>(a);                 // two supersteps ahead
     if (a.n_big) {
