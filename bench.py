@@ -649,7 +649,7 @@ def run_lp(args):
         "sync_pairs": st["sync_pairs"],
         "roofline": {"bound": "hbm", "achieved": bytes_step / (k_us * 1e-6) / 1e9, "peak": peaks["hbm_gbs"],
                      "unit": "GB/s", "frac": bytes_step / (k_us * 1e-6) / 1e9 / peaks["hbm_gbs"], "traffic": None,
-                     "peak_source": peaks["source"], "kernel": "k_lp_small + k_lp_chunks + k_lp_hubs (+ sync)",
+                     "peak_source": peaks["source"], "kernel": "k_lp_slices, row and hub kernels (+ sync)",
                      "avg_superstep_us": k_us, "algorithmic_bytes_per_superstep": bytes_step},
         "clocks": clk.summary(),
     }
