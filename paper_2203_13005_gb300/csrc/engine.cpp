@@ -365,10 +365,10 @@ void Engine::load_csc_device(HostPart& hp, uint64_t E, const void* cp_in, const 
     uint64_t* cp64 = nullptr;
     uint32_t* flag = nullptr;
     try {
+        hp.on_device = true;   // (what follows belongs to the partition, also if it fails)
         hp.d_col_ptr = (uint32_t*)own(4 * pad4(n + 1));
         hp.d_src = (uint32_t*)own(4 * pad4(E));
         if (w_in) hp.d_w = (uint32_t*)own(4 * pad4(E));
-        hp.on_device = true;
         hp.d_outdeg = (uint32_t*)own(4 * std::max<size_t>(n, 1));
         cp64 = (uint64_t*)own(8 * ((size_t)n + 1));
         flag = (uint32_t*)own(4);
@@ -427,6 +427,8 @@ void Engine::load_csc_device(HostPart& hp, uint64_t E, const void* cp_in, const 
     hp.loaded = true;
 }
 
+// Forget a partition's edges, on the device and on the host: host copies that
+// outlived them would pass for copies of the edges loaded next (ensure_host).
 void Engine::release_part(HostPart& hp) {
     if (hp.on_device) {
         if (stream_) cudaStreamSynchronize(stream_);
@@ -438,8 +440,12 @@ void Engine::release_part(HostPart& hp) {
         hp.on_device = false;
         hp.dev_edges = 0;
         hp.dev_weighted = false;
-        hp.loaded = false;
     }
+    hp.col_ptr = {};
+    hp.src = {};
+    hp.w = {};
+    hp.ghost_gid = {};
+    hp.loaded = false;
 }
 
 // Host copies of a device-loaded partition, for the paths that work on the host.
