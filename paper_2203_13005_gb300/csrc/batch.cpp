@@ -41,8 +41,7 @@ void Engine::free_batch() {
     Batch& b = batch_;
     if (b.s_h2d) cudaStreamSynchronize(b.s_h2d);
     if (b.s_d2h) cudaStreamSynchronize(b.s_d2h);
-    destroy_graph(b.graph[0]);
-    destroy_graph(b.graph[1]);
+    drop_batch_graphs();
     if (b.h_edges) cudaFreeHost(b.h_edges);
     if (b.h_changed) cudaFreeHost(b.h_changed);
     for (int i = 0; i < 3; ++i) {
@@ -138,6 +137,32 @@ void Engine::prepare_batch(bool streamed) {
         before_h2d("upload");
         cuda_check(cudaMemcpy(b.d_edges, tmp.data(), 8 * E, cudaMemcpyHostToDevice), "upload edges");
         b.resident = true;
+    }
+}
+
+void Engine::drop_batch_graphs() {
+    for (auto& g : batch_.graph) destroy_graph(g);
+}
+
+// Ring slots of `ring` edges and counters for `blocks` blocks. The captured
+// graphs hold the addresses of both, so they go when either is replaced.
+void Engine::reserve_batch(uint64_t ring, size_t blocks) {
+    Batch& b = batch_;
+    if (ring > b.ring_edges || blocks > b.max_blocks) {
+        cuda_check(cudaStreamSynchronize(stream_), "sync");
+        drop_batch_graphs();
+    }
+    if (ring > b.ring_edges) {
+        for (int i = 0; i < 3; ++i) b.d_ring[i] = dalloc((size_t)b.esize * ring);
+        b.ring_edges = ring;
+    }
+    if (blocks > b.max_blocks) {
+        b.max_blocks = 0;   // until both exist
+        b.d_changed = (unsigned long long*)dalloc(8 * blocks);
+        if (b.h_changed) cudaFreeHost(b.h_changed);
+        b.h_changed = nullptr;
+        cuda_check(cudaHostAlloc((void**)&b.h_changed, 8 * blocks, cudaHostAllocDefault), "pinned counters");
+        b.max_blocks = blocks;
     }
 }
 
@@ -273,18 +298,6 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
     uint64_t block_edges = E;
     if (streamed) {
         const uint64_t sample = std::min<uint64_t>(std::max<uint64_t>(E, 1), 1ull << 24);
-        auto ensure = [&](uint64_t ring, size_t blocks) {
-            if (ring > b.ring_edges) {
-                for (int i = 0; i < 3; ++i) b.d_ring[i] = dalloc((size_t)b.esize * ring);
-                b.ring_edges = ring;
-            }
-            if (blocks > b.max_blocks) {
-                b.d_changed = (unsigned long long*)dalloc(8 * blocks);
-                if (b.h_changed) cudaFreeHost(b.h_changed);
-                cuda_check(cudaHostAlloc((void**)&b.h_changed, 8 * blocks, cudaHostAllocDefault), "pinned counters");
-                b.max_blocks = blocks;
-            }
-        };
         // the tune cache's key: the graph's shape, the streamed edge size and the GPU
         std::string tune_key;
         gxp_tune_record cached{};
@@ -310,7 +323,7 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
             r.tune_from_cache = 1;
             block_edges = (uint64_t)cached.block_edges;
         } else {
-            ensure(sample + kUnitEdges, 64);
+            reserve_batch(sample + kUnitEdges, 64);
             // k1: download cost per edge (pinned H2D)
             cudaEvent_t t0 = b.ev_t0, t1 = b.ev_t1;
             float best = 1e30f;
@@ -354,7 +367,7 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
             }
             r.k2 = best / (double)std::max<uint64_t>(e_s, 1);
             // a: fixed cost of a block (copy + launch + upload) from 32 near-empty blocks
-            ensure(sample + kUnitEdges, 64);
+            reserve_batch(sample + kUnitEdges, 64);
             {
                 std::vector<uint64_t> tiny{0};
                 for (uint64_t i = 1; i <= 32 && i <= b.units.size(); ++i) tiny.push_back(i);
@@ -391,7 +404,7 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
                 const auto cc = block_cuts(c);
                 uint64_t mx = 0;
                 for (size_t i = 0; i + 1 < cc.size(); ++i) mx = std::max<uint64_t>(mx, b.unit_edge[cc[i + 1]] - b.unit_edge[cc[i]]);
-                ensure(mx, cc.size());
+                reserve_batch(mx, cc.size());
                 const double t = time_pipeline(c, true, true, 2);
                 if (t < best_t) {
                     best_t = t;
@@ -407,22 +420,11 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
         }
     }
     const auto cuts = streamed ? block_cuts(block_edges) : std::vector<uint64_t>{0, b.units.size()};
-    if (streamed) {
-        uint64_t mx = 0;
-        for (size_t i = 0; i + 1 < cuts.size(); ++i) mx = std::max<uint64_t>(mx, b.unit_edge[cuts[i + 1]] - b.unit_edge[cuts[i]]);
-        if (mx > b.ring_edges) {
-            for (int i = 0; i < 3; ++i) b.d_ring[i] = dalloc((size_t)b.esize * mx);
-            b.ring_edges = mx;
-        }
-    }
+    uint64_t largest = 0;
+    for (size_t i = 0; streamed && i + 1 < cuts.size(); ++i)
+        largest = std::max<uint64_t>(largest, b.unit_edge[cuts[i + 1]] - b.unit_edge[cuts[i]]);
+    reserve_batch(largest, std::max<size_t>(cuts.size() - 1, 1));
     if (!b.d_active) b.d_active = (unsigned long long*)dalloc(8);
-    if (cuts.size() - 1 > b.max_blocks || !b.d_changed) {
-        const size_t nb = std::max<size_t>(cuts.size() - 1, 1);
-        b.d_changed = (unsigned long long*)dalloc(8 * nb);
-        if (b.h_changed) cudaFreeHost(b.h_changed);
-        cuda_check(cudaHostAlloc((void**)&b.h_changed, 8 * nb, cudaHostAllocDefault), "pinned counters");
-        b.max_blocks = nb;
-    }
     r.block_edges = block_edges;
     r.blocks = (uint32_t)(cuts.size() - 1);
 
@@ -434,11 +436,10 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
 
     // CUDA graphs of one superstep, one per frontier parity
     const bool use_graph = opts.use_graph != 0;
-    if (use_graph && (!b.graph[0] || b.graph_block_edges != block_edges || b.graph_streamed != streamed ||
+    if (use_graph && (!b.graph[1] || b.graph_block_edges != block_edges || b.graph_streamed != streamed ||
                       b.graph_pipelined != pipelined || b.graph_idle != b.idle_mask)) {
-        destroy_graph(b.graph[0]);
-        destroy_graph(b.graph[1]);
         cuda_check(cudaStreamSynchronize(stream_), "sync");
+        drop_batch_graphs();
         for (int par = 0; par < 2; ++par) {
             cudaGraph_t g = nullptr;
             cuda_check(cudaStreamBeginCapture(stream_, cudaStreamCaptureModeThreadLocal), "begin capture");

@@ -102,6 +102,8 @@ private:
     void release_part(HostPart& hp);
     void ensure_host(HostPart& hp);
     void prepare_batch(bool streamed);
+    void reserve_batch(uint64_t ring, size_t blocks);
+    void drop_batch_graphs();
     void free_batch();
     double time_pipeline(uint64_t block_edges, bool pipelined, bool dry, int reps);
     void superstep_batch(const std::vector<uint64_t>& cuts, bool streamed, bool pipelined, bool dry, int parity);
