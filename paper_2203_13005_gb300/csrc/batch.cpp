@@ -141,7 +141,8 @@ void Engine::prepare_batch(bool streamed) {
 }
 
 void Engine::drop_batch_graphs() {
-    for (auto& g : batch_.graph) destroy_graph(g);
+    for (auto& pair : batch_.graph)
+        for (auto& g : pair) destroy_graph(g);
 }
 
 // Ring slots of `ring` edges and counters for `blocks` blocks. The captured
@@ -288,7 +289,14 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
     const bool pipelined = !streamed || opts.pipelined != 0;
     prepare_batch(streamed);
     Batch& b = batch_;
-    b.idle_mask = n_src == 64 ? 0ull : ~0ull << n_src;   // the slots without a source are not computed
+    // Slots past the lane groups that hold the sources (with_slot_lanes) are
+    // not computed; those within have no source, stay INF and never improve.
+    // So calls with other numbers of sources share five masks, and five pairs
+    // of captured graphs.
+    uint32_t cls = 0;
+    while (n_src > 4u << cls) ++cls;
+    b.idle_mask = cls == 4 ? 0ull : ~0ull << (4u << cls);
+    cudaGraphExec_t* const graph = b.graph[cls];
     const uint64_t E = b.unit_edge.back(), V = n_vertices_;
     const uint64_t words = (V + 31) / 32 + 1;
     gxp_batch_report r{};
@@ -436,23 +444,24 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
 
     // CUDA graphs of one superstep, one per frontier parity
     const bool use_graph = opts.use_graph != 0;
-    if (use_graph && (!b.graph[1] || b.graph_block_edges != block_edges || b.graph_streamed != streamed ||
-                      b.graph_pipelined != pipelined || b.graph_idle != b.idle_mask)) {
+    if (use_graph && (!graph[1] || b.graph_block_edges != block_edges || b.graph_streamed != streamed ||
+                      b.graph_pipelined != pipelined)) {
         cuda_check(cudaStreamSynchronize(stream_), "sync");
-        drop_batch_graphs();
+        if (b.graph_block_edges != block_edges || b.graph_streamed != streamed || b.graph_pipelined != pipelined)
+            drop_batch_graphs();
+        for (int par = 0; par < 2; ++par) destroy_graph(graph[par]);   // one of them only, after an error
         for (int par = 0; par < 2; ++par) {
             cudaGraph_t g = nullptr;
             cuda_check(cudaStreamBeginCapture(stream_, cudaStreamCaptureModeThreadLocal), "begin capture");
             superstep_batch(cuts, streamed, pipelined, false, par);
             cuda_check(cudaStreamEndCapture(stream_, &g), "end capture");
-            cudaError_t e = cudaGraphInstantiate(&b.graph[par], g, 0);
+            cudaError_t e = cudaGraphInstantiate(&graph[par], g, 0);
             cudaGraphDestroy(g);
             cuda_check(e, "instantiate");
         }
         b.graph_block_edges = block_edges;
         b.graph_streamed = streamed;
         b.graph_pipelined = pipelined;
-        b.graph_idle = b.idle_mask;
     }
 
     cuda_check(cudaMemsetAsync(b.d_active, 0, 8, stream_), "memset");
@@ -491,7 +500,7 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
     int parity = 0;
     uint32_t steps = 0;
     while (!persistent && steps < max_steps) {
-        if (use_graph) cuda_check(cudaGraphLaunch(b.graph[parity], stream_), "graph launch");
+        if (use_graph) cuda_check(cudaGraphLaunch(graph[parity], stream_), "graph launch");
         else superstep_batch(cuts, streamed, pipelined, false, parity);
         cuda_check(cudaStreamSynchronize(stream_), "superstep");
         unsigned long long changed = 0;

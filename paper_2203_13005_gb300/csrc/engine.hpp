@@ -186,7 +186,7 @@ private:
         uint32_t esize = 8;                // streamed edge: 8 = (source, weight) uint2, 4 = packed uint32
         bool packed = false;
         uint32_t no_sat = 0;
-        uint64_t idle_mask = 0, graph_idle = 0;   // slots without a source: of this call, of the captured graphs
+        uint64_t idle_mask = 0;            // slots this call leaves out
         uint64_t ring_edges = 0;
         uint32_t* d_dist = nullptr;        // [V][64]
         uint32_t* d_frontier[3] = {nullptr, nullptr, nullptr};   // [2]: the persistent run's third bitmap
@@ -200,7 +200,7 @@ private:
         size_t max_blocks = 0;
         cudaStream_t s_h2d = nullptr, s_d2h = nullptr;
         cudaEvent_t ev_loaded[3] = {}, ev_free[3] = {}, ev_t0 = nullptr, ev_t1 = nullptr;
-        cudaGraphExec_t graph[2] = {nullptr, nullptr};
+        cudaGraphExec_t graph[5][2] = {};   // by lane groups in use (4, 8 .. 64 slots) and frontier parity
         uint64_t graph_block_edges = 0;
         bool graph_streamed = false, graph_pipelined = false;
     } batch_;

@@ -27,6 +27,7 @@ def graph():
     [(500, True, True, 64), (20_000, False, True, 64), (500, True, True, 64)],    # a larger ring in between
     [(9000, True, True, 64), (0, True, True, 64), (9000, True, True, 64)],        # the tuner in between
     [(9000, True, True, 64), (0, False, False, 64), (300, True, True, 64), (9000, True, True, 64)],
+    [(2000, True, True, k) for k in (1, 4, 5, 8, 33, 64, 9, 32, 17, 16, 3, 64)],  # a graph per lane grouping, kept
 ])
 def test_buffers_replaced_between_graph_runs(gpu, graph, calls):
     n, src, dst, w, sources, refs = graph
