@@ -1494,13 +1494,19 @@ void Engine::build_out_edges() {
 }
 
 // The two frontier lists over the out-edge copy, and one partition's bitmaps
-// of changed vertices.
+// of changed vertices: all of them or, when an allocation fails, none (a
+// later call on the same graph tries again).
 void Engine::build_frontier_lists() {
     if (d_list_[0]) return;
-    list_cap_ = (uint64_t)n_slots_ + (total_edges_ + kItemEdges - 1) / kItemEdges;
-    for (auto& l : d_list_) l = (uint2*)dalloc_ordered(sizeof(uint2) * std::max<uint64_t>(list_cap_, 1));
+    const uint64_t cap = (uint64_t)n_slots_ + (total_edges_ + kItemEdges - 1) / kItemEdges;
+    uint2* lists[2];
+    uint32_t* bits[3] = {};
+    for (auto& l : lists) l = (uint2*)dalloc_ordered(sizeof(uint2) * std::max<uint64_t>(cap, 1));
     if (n_parts_ == 1)
-        for (auto& b : d_bits_) b = (uint32_t*)dalloc_ordered(4 * ((n_vertices_ + 31) / 32));
+        for (auto& b : bits) b = (uint32_t*)dalloc_ordered(4 * ((n_vertices_ + 31) / 32));
+    list_cap_ = cap;
+    std::copy(lists, lists + 2, d_list_);
+    std::copy(bits, bits + 3, d_bits_);
 }
 
 // The frontier the next superstep reads: one vertex, or all (kInf) slots.

@@ -1,0 +1,55 @@
+"""An allocation fails in the middle of a call's first use of a loaded graph
+(an injected out-of-memory): the call returns GXP_E_NOMEM, and the same call
+again, on the graph as loaded, completes whatever was left unbuilt. Every
+allocation of the call is failed in turn."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2203_13005_gb300 import gxp
+
+pytestmark = pytest.mark.gpu
+
+N, M = 2000, 12_000
+
+
+@pytest.fixture(scope="module")
+def graph():
+    rng = np.random.default_rng(11)
+    src, dst = rng.integers(0, N, M).astype(np.uint32), rng.integers(0, N, M).astype(np.uint32)
+    return src, dst, rng.integers(1, 100, M).astype(np.uint32)
+
+
+def _every_allocation(graph, call, parts, direction, least):
+    src, dst, w = graph
+    hit = 0
+    for at in range(1, 200):
+        with gxp.Context(0, fault=gxp.GXP_FAULT_ALLOC, fault_at=at, direction=direction) as c:
+            c.create_graph(N, parts)
+            try:
+                c.load_coo(src, dst, w)
+            except gxp.GxpError:
+                continue   # the load's allocations: its own tests
+            try:
+                call(c)
+            except gxp.GxpError as e:
+                assert e.code == gxp.GXP_E_NOMEM, at
+                hit += 1
+                call(c)    # again, nothing loaded anew
+                continue
+        break
+    assert hit >= least
+
+
+@pytest.mark.parametrize("direction", [gxp.GXP_DIR_AUTO, gxp.GXP_DIR_PUSH])
+@pytest.mark.parametrize("parts", [1, 3])
+@pytest.mark.parametrize("algo", [gxp.GXP_ALGO_SSSP, gxp.GXP_ALGO_CC])
+def test_run_again(gpu, graph, algo, parts, direction):
+    src, dst, w = graph
+    ref, steps, _ = oracle.sssp(N, src, dst, w, 3) if algo == gxp.GXP_ALGO_SSSP else oracle.cc(N, src, dst)
+
+    def call(c):
+        assert c.run(algo, source=3) == steps
+        assert np.array_equal(c.values(), ref)
+
+    _every_allocation(graph, call, parts, direction, 10)
