@@ -1679,8 +1679,10 @@ void Engine::build_lp() {
         if (!cfg_.mem_budget || graph_bytes_ + need <= cfg_.mem_budget) {
             build_out_edges();
             const size_t words = (V + 31) / 32;
-            for (auto& b : lp_.d_active) b = (uint32_t*)dalloc(4 * words);
-            for (auto& b : lp_.d_changed) b = (uint32_t*)dalloc(4 * words);
+            uint32_t* bits[5];   // all of them or none, as superstep() takes them
+            for (auto& b : bits) b = (uint32_t*)dalloc(4 * words);
+            std::copy(bits, bits + 2, lp_.d_active);
+            std::copy(bits + 2, bits + 5, lp_.d_changed);
         }
     }
     lp_.ready = true;

@@ -53,3 +53,15 @@ def test_run_again(gpu, graph, algo, parts, direction):
         assert np.array_equal(c.values(), ref)
 
     _every_allocation(graph, call, parts, direction, 10)
+
+
+@pytest.mark.parametrize("parts", [1, 3])
+def test_label_propagation_again(gpu, graph, parts):
+    src, dst, _ = graph
+    ref, steps, _ = oracle.lp(N, src, dst)
+
+    def call(c):
+        assert c.run(gxp.GXP_ALGO_LP, max_steps=15) == steps
+        assert np.array_equal(c.values(), ref)
+
+    _every_allocation(graph, call, parts, gxp.GXP_DIR_AUTO, 10)
