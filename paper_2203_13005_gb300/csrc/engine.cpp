@@ -144,6 +144,23 @@ void* Engine::dalloc_ordered(size_t bytes) {
     return p;
 }
 
+// What `make` allocates for the graph, or nothing if it runs out of memory.
+template <class F> bool Engine::if_it_fits(F make) {
+    const size_t n = graph_allocs_.size();
+    const uint64_t bytes = graph_bytes_;
+    try {
+        make();
+        return true;
+    } catch (const Error& e) {
+        if (e.code != GXP_E_NOMEM) throw;
+    }
+    cuda_check(cudaStreamSynchronize(stream_), "sync");
+    for (size_t i = n; i < graph_allocs_.size(); ++i) device_free(graph_allocs_[i]);
+    graph_allocs_.resize(n);
+    graph_bytes_ = bytes;
+    return false;
+}
+
 void Engine::free_graph_device() {
     if (stream_) cudaStreamSynchronize(stream_);
     free_batch();   // graphs and pinned buffers that refer to the device buffers below
@@ -1671,19 +1688,21 @@ void Engine::build_lp() {
     cuda_check(cudaMemsetAsync(lp_.d_keys, 0xFF, 4 * std::max<uint64_t>(table_slots, 1), stream_), "memset");
     cuda_check(cudaMemsetAsync(lp_.d_counts, 0, 4 * std::max<uint64_t>(table_slots, 1), stream_), "memset");
     // One partition: the out-edge copy that tells which rows a change
-    // reaches. It is an extra: without room for it under mem_budget every
-    // superstep recomputes every row.
+    // reaches. It is an extra: without room for it, under mem_budget or on the
+    // device, every superstep recomputes every row.
     if (n_parts_ == 1) {
         const uint64_t V = n_vertices_, E = total_edges_;
         const uint64_t need = (out_ready_ ? 0 : 4 * pad4(V + 1) + (weighted_ ? 8 : 4) * E) + 5 * 4 * ((V + 31) / 32) + 128;
-        if (!cfg_.mem_budget || graph_bytes_ + need <= cfg_.mem_budget) {
-            build_out_edges();
+        const bool room = !cfg_.mem_budget || graph_bytes_ + need <= cfg_.mem_budget;
+        if (room && !out_ready_ && !if_it_fits([&] { build_out_edges(); }))
+            d_out_ptr_ = d_out_dst_ = d_out_w_ = nullptr;
+        if (room && out_ready_) if_it_fits([&] {
             const size_t words = (V + 31) / 32;
             uint32_t* bits[5];   // all of them or none, as superstep() takes them
             for (auto& b : bits) b = (uint32_t*)dalloc(4 * words);
             std::copy(bits, bits + 2, lp_.d_active);
             std::copy(bits + 2, bits + 5, lp_.d_changed);
-        }
+        });
     }
     lp_.ready = true;
 }

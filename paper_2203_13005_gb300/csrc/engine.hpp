@@ -79,6 +79,7 @@ private:
     // build's allocations each waited for the kernels before them: ~500 us a load)
     void* dalloc(size_t bytes);
     void* dalloc_ordered(size_t bytes);
+    template <class F> bool if_it_fits(F make);
     // every device allocation and host-to-device copy of the context goes
     // through these, so that an injected fault can fail the n-th one
     cudaError_t device_malloc(void** p, size_t bytes, bool wait = true);

@@ -65,3 +65,42 @@ def test_label_propagation_again(gpu, graph, parts):
         assert np.array_equal(c.values(), ref)
 
     _every_allocation(graph, call, parts, gxp.GXP_DIR_AUTO, 10)
+
+
+def test_label_propagation_without_its_extras(gpu, graph):
+    """One partition's out-edge copy and bitmaps are extras of label
+    propagation: an allocation of theirs that fails fails no call. So the calls
+    that fail are those of a context whose budget never has room for them."""
+    src, dst, _ = graph
+    ref, steps, _ = oracle.lp(N, src, dst)
+    cc_ref, _, _ = oracle.cc(N, src, dst)
+
+    def failing(mem_budget):
+        hit = []
+        for at in range(1, 100):
+            with gxp.Context(0, fault=gxp.GXP_FAULT_ALLOC, fault_at=at, mem_budget=mem_budget) as c:
+                c.create_graph(N, 1)
+                try:
+                    c.load_coo(src, dst)
+                    assert c.run(gxp.GXP_ALGO_LP, max_steps=15) == steps
+                except gxp.GxpError as e:
+                    assert e.code == gxp.GXP_E_NOMEM
+                    hit.append(at)
+                    continue
+                assert np.array_equal(c.values(), ref)
+                if mem_budget > 32 << 20:   # builds its own out-edge copy, whatever became of that one
+                    try:
+                        c.run(gxp.GXP_ALGO_CC)
+                    except gxp.GxpError as e:
+                        assert e.code == gxp.GXP_E_NOMEM
+                        c.run(gxp.GXP_ALGO_CC)
+                    assert np.array_equal(c.values(), cc_ref)
+        return hit
+
+    with gxp.Context(0) as c:
+        c.create_graph(N, 1)
+        c.load_coo(src, dst)
+        c.run(gxp.GXP_ALGO_LP, max_steps=15)
+        used = c.stats()["device_bytes"]
+    # (the first has room for everything; the second for all but the extras)
+    assert failing(64 << 20) == failing(used - 4 * M)
