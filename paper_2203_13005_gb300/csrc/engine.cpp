@@ -1020,7 +1020,7 @@ void Engine::begin(gxp_algo algo, uint32_t source, float damping) {
     frontier_ = (a == Algo::SSSP || a == Algo::CC) && cfg_.direction != GXP_DIR_PULL &&
                 (uint64_t)V + n_ghost_total_ + (total_edges_ + kItemEdges - 1) / kItemEdges < (1ull << 32);
     if (frontier_) {
-        build_out_edges();
+        build_out_edges(a == Algo::SSSP || !out_ready_);
         build_frontier_lists();
     }
     cur_ = 0;
@@ -1458,17 +1458,22 @@ uint64_t Engine::account(bool stop_at_quiet) {
 // out-edges into their own partition) then every partition's cached copies
 // (that partition's in-edges from the copied vertex), built from a CSC over
 // global rows with slot sources (temporary).
-void Engine::build_out_edges() {
+// Label propagation reads no weights: a copy it made without them is built
+// again, with them, by the first SSSP run.
+void Engine::build_out_edges(bool weights) {
     TraceRange trace_("gxp out-edge build");
-    if (out_ready_) return;
+    weights = weights && weighted_;
+    if (out_ready_ && (!weights || d_out_w_)) return;
     const uint32_t V = (uint32_t)n_vertices_;
     const uint64_t E = total_edges_;
     const uint32_t S = V + n_ghost_total_;   // slots
     if ((uint64_t)V + n_ghost_total_ >= 0xFFFFFFF0ull) fail(GXP_E_INVAL, "too many vertices and cached copies");
     n_slots_ = S;
-    d_out_ptr_ = (uint32_t*)dalloc_ordered(4 * pad4((size_t)S + 1));
-    d_out_dst_ = (uint32_t*)dalloc_ordered(4 * std::max<uint64_t>(E, 1));
-    d_out_w_ = weighted_ ? (uint32_t*)dalloc_ordered(4 * std::max<uint64_t>(E, 1)) : nullptr;
+    if (!out_ready_) {
+        d_out_ptr_ = (uint32_t*)dalloc_ordered(4 * pad4((size_t)S + 1));
+        d_out_dst_ = (uint32_t*)dalloc_ordered(4 * std::max<uint64_t>(E, 1));
+    }
+    uint32_t* out_w = weights ? (uint32_t*)dalloc_ordered(4 * std::max<uint64_t>(E, 1)) : nullptr;
     std::vector<void*> tmp;
     auto talloc = [&](size_t bytes) -> void* {
         void* q = nullptr;
@@ -1489,7 +1494,7 @@ void Engine::build_out_edges() {
     if (n_parts_ > 1) {
         uint32_t* ucol = (uint32_t*)talloc(4 * ((size_t)V + 1));
         uint32_t* usrc = (uint32_t*)talloc(4 * std::max<uint64_t>(E, 1));
-        uint32_t* uw = weighted_ ? (uint32_t*)talloc(4 * std::max<uint64_t>(E, 1)) : nullptr;
+        uint32_t* uw = weights ? (uint32_t*)talloc(4 * std::max<uint64_t>(E, 1)) : nullptr;
         uint64_t at = 0;
         for (uint32_t p = 0; p < n_parts_; ++p) {
             cuda_check(launch_unify_csc(pd_[p], V, at, ucol, usrc, p + 1 == n_parts_, stream_), "slot CSC");
@@ -1504,9 +1509,9 @@ void Engine::build_out_edges() {
         deg = sdeg;
     }
     uint32_t* scratch = (uint32_t*)talloc(4 * out_edges_scratch_words(S, E));
-    cuda_check(launch_out_edges(in, V, S, E, deg, d_out_ptr_, scratch, d_out_dst_, weighted_ ? d_out_w_ : nullptr,
-                                stream_), "out-edges");
+    cuda_check(launch_out_edges(in, V, S, E, deg, d_out_ptr_, scratch, d_out_dst_, out_w, stream_), "out-edges");
     cuda_check(cudaStreamSynchronize(stream_), "out-edges");
+    d_out_w_ = out_w;
     out_ready_ = true;
 }
 
@@ -1692,10 +1697,10 @@ void Engine::build_lp() {
     // device, every superstep recomputes every row.
     if (n_parts_ == 1) {
         const uint64_t V = n_vertices_, E = total_edges_;
-        const uint64_t need = (out_ready_ ? 0 : 4 * pad4(V + 1) + (weighted_ ? 8 : 4) * E) + 5 * 4 * ((V + 31) / 32) + 128;
+        const uint64_t need = (out_ready_ ? 0 : 4 * pad4(V + 1) + 4 * E) + 5 * 4 * ((V + 31) / 32) + 128;
         const bool room = !cfg_.mem_budget || graph_bytes_ + need <= cfg_.mem_budget;
-        if (room && !out_ready_ && !if_it_fits([&] { build_out_edges(); }))
-            d_out_ptr_ = d_out_dst_ = d_out_w_ = nullptr;
+        if (room && !out_ready_ && !if_it_fits([&] { build_out_edges(false); }))
+            d_out_ptr_ = d_out_dst_ = nullptr;
         if (room && out_ready_) if_it_fits([&] {
             const size_t words = (V + 31) / 32;
             uint32_t* bits[5];   // all of them or none, as superstep() takes them

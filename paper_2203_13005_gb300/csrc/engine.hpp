@@ -221,7 +221,7 @@ private:
     uint64_t list_cap_ = 0;
     unsigned long long seed_all_ne_ = 0;   // the frontier count of all slots (a CC run's start), once known
     uint32_t n_slots_ = 0;         // push sources: the vertices, then (several partitions) the cached copies
-    void build_out_edges();
+    void build_out_edges(bool weights);
     void build_frontier_lists();
     void seed_frontier(uint32_t source_int);
     // label propagation: rows by in-degree class, hub hash tables, and for one
