@@ -648,6 +648,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sweep(const SweepArgs a, const 
     uint64_t passed = run.passed;   // grid barriers
     if (tid < 3) s_acc[tid] = 0ull;
     if (tid < 2) s_cnt[tid] = 0u;
+    __syncthreads();   // a push superstep has no other barrier before the warps add to them
     for (;;) {
         const StepStats* const in = a.stats + t % kStatRing;
         StepStats* const out = a.stats + (t + 1) % kStatRing;
