@@ -394,8 +394,9 @@ struct Pull {
 
     // Hub parts first, first + step, ... below n, lane-strided. The part of a
     // row that arrives last combines all of the row's parts, in part order.
-    // A partial is published as one word with its flag, so neither it nor the
-    // arrival needs a fence; the arrival's answer is looked at one part later,
+    // A partial is published as one word with its flag, by a relaxed atomic
+    // store that relaxed atomic loads poll, so neither it nor the arrival needs
+    // a fence; the arrival's answer is looked at one part later,
     // when it has come back, and the last arriver polls the row's words,
     // all of them stored by then, until it sees them.
     struct Row {
@@ -449,7 +450,7 @@ struct Pull {
                 finish(row.v, total);
                 pend.nparts = 0u;
             } else if (lane == 0) {
-                __stcg(&a.hub_val[i], ((unsigned long long)Op::to_bits(total) << 32) | 1ull);
+                st_relaxed_gpu(&a.hub_val[i], ((unsigned long long)Op::to_bits(total) << 32) | 1ull);
                 pend.arrived = atomicAdd(&a.hub_arrive[row.t0], 1u);
             }
             words = next;
@@ -464,16 +465,16 @@ struct Pull {
         if (r.nparts == 0u || __shfl_sync(kFull, r.arrived, 0) != r.nparts - 1u) return;
         T tot = Op::ident();   // parts in a fixed order: lane-strided, then a fixed tree
         for (uint32_t q = (uint32_t)lane; q < r.nparts; q += 32u) {
-            unsigned long long x = __ldcg(&a.hub_val[r.t0 + q]);
+            unsigned long long x = ld_relaxed_gpu(&a.hub_val[r.t0 + q]);
             for (uint32_t spin = 0; !(x & 1ull); ++spin) {   // stored already: its way to L2
                 if (spin == 1u << 22) {
                     atomicOr(a.err, kErrTimeout);
                     break;
                 }
-                x = atomicAdd(&a.hub_val[r.t0 + q], 0ull);
+                x = ld_relaxed_gpu(&a.hub_val[r.t0 + q]);
             }
             tot = Op::combine(tot, Op::from_bits((uint32_t)(x >> 32)));
-            __stcg(&a.hub_val[r.t0 + q], 0ull);   // ready for the next superstep
+            st_relaxed_gpu(&a.hub_val[r.t0 + q], 0ull);   // ready for the next superstep
         }
         if (lane == 0) a.hub_arrive[r.t0] = 0u;
         finish(r.v, warp_all<Op>(tot));
