@@ -23,7 +23,9 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // 16.8 M edges of a million-vertex R-MAT graph take 191 us read one source a
 // thread and 214 us read four: the reads do not bound it. A single partition's
 // CSC is therefore counted chunk by chunk behind its copy from the host (189 us
-// in eight chunks, next to 363 us of copies).
+// in eight chunks, next to 363 us of copies). Above them a warp adds once per
+// distinct source: loading 16.8 M edges that all leave one vertex above takes
+// 0.58 ms so and 10.7 ms with an atomic an edge; uniform sources 0.50 ms either way.
 constexpr uint32_t kOutdegHot = 8192;
 
 // kCheck: ids of n_local and above are not counted but reported (bit 1 of err).
@@ -41,8 +43,12 @@ __global__ void __launch_bounds__(256) k_outdeg(const uint32_t* __restrict__ src
             return;
         }
         const uint32_t g = u < n_own ? v_begin + u : ghost_gid[u - n_own];
-        if (g < kOutdegHot) atomicAdd(&hot[g], 1u);
-        else atomicAdd(&outdeg[g], 1u);
+        if (g < kOutdegHot) {
+            atomicAdd(&hot[g], 1u);
+            return;
+        }
+        const unsigned peers = __match_any_sync(__activemask(), g);
+        if ((threadIdx.x & 31) == (unsigned)(__ffs(peers) - 1)) atomicAdd(&outdeg[g], (uint32_t)__popc(peers));
     };
     // four sources a load (src is 16-byte aligned)
     const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
