@@ -602,17 +602,18 @@ void Engine::build_sell() {
         cuda_check(launch_sell_fill(col_ptr, ssrc, sw, perm, width, off, (uint32_t)ns, p, pd_[p].pad_id,
                                     sweep_cols_, sell_src, sell_w, part_desc[p], stream_), "fill slices");
         // 5. hub rows -> parts of T edges
+        const uint32_t max_parts = n_parts_ == 1 ? kMaxRowParts : kInf;
         uint32_t* hub_list = (uint32_t*)talloc(4 * nh_rows + 4);
         uint32_t* part_off = (uint32_t*)talloc(4 * nh_rows + 4);
         cuda_check(launch_hub_rows(col_ptr, n, hub_out, counts + nw, d_bases + nw, hub_list, (uint32_t)nh_rows,
-                                   T, part_off, stream_), "hub rows");
+                                   T, max_parts, part_off, stream_), "hub rows");
         uint32_t nparts = 0;
         d2h(&nparts, part_off + nh_rows, 4);
         if ((uint64_t)total_hubs + nparts > 0xFFFFFFF0ull) fail(GXP_E_INVAL, "too many hub parts");
         part_hubs[p] = (HubPart*)talloc(sizeof(HubPart) * ((size_t)nparts + 1));
         part_nh[p] = nparts;
-        cuda_check(launch_hub_parts(col_ptr, hub_list, part_off, (uint32_t)nh_rows, T, p, total_hubs,
-                                    part_hubs[p], stream_), "hub parts");
+        cuda_check(launch_hub_parts(col_ptr, hub_list, part_off, (uint32_t)nh_rows, T, max_parts, p,
+                                    total_hubs, part_hubs[p], stream_), "hub parts");
         pd_[p].sell_src = sell_src;
         pd_[p].sell_w = sell_w;
         pd_[p].perm = perm;
@@ -724,7 +725,7 @@ void Engine::build_sell_sorted(uint32_t H, uint32_t T) {
     } free_tmp{tmp, stream_};
     // (the hub rows' parts are counted first: the host waits for the count)
     uint32_t* part_off = (uint32_t*)talloc(4 * (size_t)nh + 4);
-    cuda_check(launch_hub_offsets(col, nh, T, part_off, stream_), "hub rows");
+    cuda_check(launch_hub_offsets(col, nh, T, kMaxRowParts, part_off, stream_), "hub rows");
     uint32_t n_parts = 0;
     cuda_check(cudaMemcpyAsync(&n_parts, part_off + nh, 4, cudaMemcpyDeviceToHost, stream_), "read counts");
     uint32_t* ssrc = (uint32_t*)dalloc_ordered(4 * pad4(E));
@@ -743,7 +744,7 @@ void Engine::build_sell_sorted(uint32_t H, uint32_t T) {
     n_hubs_ = n_parts;
     const size_t nh1 = std::max<size_t>(n_parts, 1);
     d_hubs_ = (HubPart*)dalloc_ordered(sizeof(HubPart) * nh1);
-    cuda_check(launch_hub_parts(col, nullptr, part_off, nh, T, 0u, 0u, d_hubs_, stream_), "hub parts");
+    cuda_check(launch_hub_parts(col, nullptr, part_off, nh, T, kMaxRowParts, 0u, 0u, d_hubs_, stream_), "hub parts");
     d_hub_val_ = (unsigned long long*)dalloc_ordered(8 * nh1);
     cuda_check(cudaMemsetAsync(d_hub_val_, 0, 8 * nh1, stream_), "memset");
     d_hub_arrive_ = (uint32_t*)dalloc_ordered(4 * nh1);

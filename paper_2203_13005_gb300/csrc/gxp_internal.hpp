@@ -691,15 +691,21 @@ cudaError_t launch_sell_fill(const uint32_t* col_ptr, const uint32_t* ssrc, cons
 cudaError_t launch_sell_fill_sorted(const uint32_t* col_ptr, const uint32_t* ssrc, const uint32_t* sw, uint32_t n_rows,
                                     uint32_t first_row, const uint64_t* at, uint32_t n_slices, uint32_t cols,
                                     uint32_t* sell_src, uint32_t* sell_w, SellSlice* desc, cudaStream_t s);
+// Hub rows are cut into parts of T edges, a row of more than max_parts of them
+// into longer ones. One partition cuts a row into at most kMaxRowParts, about a
+// part for each of its kernel's 4,864 warps: the row's last part combines
+// them all, a warp's 128 loads a lane. Rows of up to 2 M in-edges (T = 512; 8 M
+// at T = 2048) are below it.
+constexpr uint32_t kMaxRowParts = 4096;
 // exclusive prefix of the parts of hub rows 0 .. n_hub_rows - 1, and their total
-cudaError_t launch_hub_offsets(const uint32_t* col_ptr, uint32_t n_hub_rows, uint32_t T, uint32_t* part_off,
-                               cudaStream_t s);
+cudaError_t launch_hub_offsets(const uint32_t* col_ptr, uint32_t n_hub_rows, uint32_t T, uint32_t max_parts,
+                               uint32_t* part_off, cudaStream_t s);
 cudaError_t launch_hub_rows(const uint32_t* col_ptr, uint32_t n, const uint32_t* hub_out, const uint32_t* hub_cnt,
                             const uint32_t* hub_base, uint32_t* hub_list, uint32_t n_hub_rows, uint32_t T,
-                            uint32_t* part_off, cudaStream_t s);
+                            uint32_t max_parts, uint32_t* part_off, cudaStream_t s);
 cudaError_t launch_hub_parts(const uint32_t* col_ptr, const uint32_t* hub_list, const uint32_t* part_off,
-                             uint32_t n_hub_rows, uint32_t T, uint32_t part, uint32_t part_base, HubPart* hubs,
-                             cudaStream_t s);   // hub_list nullptr: rows 0 .. n_hub_rows - 1
+                             uint32_t n_hub_rows, uint32_t T, uint32_t max_parts, uint32_t part, uint32_t part_base,
+                             HubPart* hubs, cudaStream_t s);   // hub_list nullptr: rows 0 .. n_hub_rows - 1
 // slices by decreasing width (stable); afterwards word b of
 // order_slices_starts(scratch, n) holds the number of slices wider than b
 // (b <= kOrderExact)

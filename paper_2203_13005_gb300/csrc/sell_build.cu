@@ -594,10 +594,16 @@ __global__ void k_hub_rows(const uint32_t* hub_out, const uint32_t* hub_cnt, con
     for (uint32_t i = threadIdx.x; i < cnt; i += blockDim.x) hub_list[base + i] = hub_out[w0 + i];
 }
 
+// Edges per part of a hub row of d in-edges: T, or as many more as keep it to
+// max_parts parts.
+__device__ __forceinline__ uint32_t hub_part_edges(uint32_t d, uint32_t T, uint32_t max_parts) {
+    return d / T < max_parts ? T : ((d / max_parts) | 31u) + 1u;
+}
+
 // single CTA: exclusive prefix of the parts of each hub row (hub_list, or rows
 // 0 .. n - 1 of a renumbered partition); out[n] = total
 __global__ void __launch_bounds__(1024) k_scan_parts(const uint32_t* col_ptr, const uint32_t* hub_list, uint32_t n,
-                                                     uint32_t T, uint32_t* out) {
+                                                     uint32_t T, uint32_t max_parts, uint32_t* out) {
     __shared__ uint32_t part[1024];
     const uint32_t t = threadIdx.x;
     const uint32_t per = (n + 1023) / 1024;
@@ -605,7 +611,7 @@ __global__ void __launch_bounds__(1024) k_scan_parts(const uint32_t* col_ptr, co
     auto parts = [&](uint32_t h) {
         const uint32_t v = hub_list ? hub_list[h] : h;
         const uint32_t d = col_ptr[v + 1] - col_ptr[v];
-        return (d + T - 1) / T;
+        return (d - 1u) / hub_part_edges(d, T, max_parts) + 1u;   // (a hub row has in-edges)
     };
     uint32_t s = 0;
     for (uint32_t i = a; i < b; ++i) s += parts(i);
@@ -626,15 +632,16 @@ __global__ void __launch_bounds__(1024) k_scan_parts(const uint32_t* col_ptr, co
 }
 
 __global__ void k_hub_parts(const uint32_t* col_ptr, const uint32_t* hub_list, const uint32_t* part_off, uint32_t n,
-                            uint32_t T, uint32_t part, uint32_t part_base, HubPart* hubs) {
+                            uint32_t T, uint32_t max_parts, uint32_t part, uint32_t part_base, HubPart* hubs) {
     // a warp per row: the longest have hundreds of parts
     const uint32_t lane = threadIdx.x & 31u;
     for (uint32_t h = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; h < n; h += (gridDim.x * blockDim.x) >> 5) {
         const uint32_t v = hub_list ? hub_list[h] : h;
         const uint32_t b = col_ptr[v], d = col_ptr[v + 1] - b;
-        const uint32_t np = (d + T - 1) / T, local = part_off[h], t0 = part_base + local;
+        const uint32_t per = hub_part_edges(d, T, max_parts);
+        const uint32_t np = (d - 1u) / per + 1u, local = part_off[h], t0 = part_base + local;
         for (uint32_t k = lane; k < np; k += 32u)   // this partition's array; t0 indexes all partitions' parts
-            hubs[local + k] = HubPart{v, part, b + k * T, min(T, d - k * T), t0, np, {0u, 0u}};
+            hubs[local + k] = HubPart{v, part, b + k * per, min(per, d - k * per), t0, np, {0u, 0u}};
     }
 }
 
@@ -960,27 +967,27 @@ cudaError_t launch_sell_fill_sorted(const uint32_t* col_ptr, const uint32_t* ssr
     return cudaGetLastError();
 }
 
-cudaError_t launch_hub_offsets(const uint32_t* col_ptr, uint32_t n_hub_rows, uint32_t T, uint32_t* part_off,
-                               cudaStream_t s) {
-    k_scan_parts<<<1, 1024, 0, s>>>(col_ptr, nullptr, n_hub_rows, T, part_off);
+cudaError_t launch_hub_offsets(const uint32_t* col_ptr, uint32_t n_hub_rows, uint32_t T, uint32_t max_parts,
+                               uint32_t* part_off, cudaStream_t s) {
+    k_scan_parts<<<1, 1024, 0, s>>>(col_ptr, nullptr, n_hub_rows, T, max_parts, part_off);
     return cudaGetLastError();
 }
 
 cudaError_t launch_hub_rows(const uint32_t* col_ptr, uint32_t n, const uint32_t* hub_out, const uint32_t* hub_cnt,
                             const uint32_t* hub_base, uint32_t* hub_list, uint32_t n_hub_rows, uint32_t T,
-                            uint32_t* part_off, cudaStream_t s) {
+                            uint32_t max_parts, uint32_t* part_off, cudaStream_t s) {
     const uint32_t nw = (n + kSellWindow - 1) / kSellWindow;
     if (nw) k_hub_rows<<<nw, 256, 0, s>>>(hub_out, hub_cnt, hub_base, hub_list);
-    k_scan_parts<<<1, 1024, 0, s>>>(col_ptr, hub_list, n_hub_rows, T, part_off);
+    k_scan_parts<<<1, 1024, 0, s>>>(col_ptr, hub_list, n_hub_rows, T, max_parts, part_off);
     return cudaGetLastError();
 }
 
 cudaError_t launch_hub_parts(const uint32_t* col_ptr, const uint32_t* hub_list, const uint32_t* part_off,
-                             uint32_t n_hub_rows, uint32_t T, uint32_t part, uint32_t part_base, HubPart* hubs,
-                             cudaStream_t s) {
+                             uint32_t n_hub_rows, uint32_t T, uint32_t max_parts, uint32_t part, uint32_t part_base,
+                             HubPart* hubs, cudaStream_t s) {
     if (n_hub_rows == 0) return cudaSuccess;
-    k_hub_parts<<<grid_warps(n_hub_rows, 256), 256, 0, s>>>(col_ptr, hub_list, part_off, n_hub_rows, T, part, part_base,
-                                                         hubs);
+    k_hub_parts<<<grid_warps(n_hub_rows, 256), 256, 0, s>>>(col_ptr, hub_list, part_off, n_hub_rows, T, max_parts, part,
+                                                            part_base, hubs);
     return cudaGetLastError();
 }
 
