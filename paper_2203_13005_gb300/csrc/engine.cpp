@@ -165,7 +165,7 @@ void Engine::free_graph_device() {
     if (stream_) cudaStreamSynchronize(stream_);
     free_batch();   // graphs and pinned buffers that refer to the device buffers below
     d_bar_ = nullptr;
-    bar_passed_ = 0;
+    bar_arrived_ = 0;
     h_old2new_.clear();
     n_lookups_ = 0;
     lp_ = LpLists{};
@@ -1744,51 +1744,59 @@ uint32_t Engine::run(gxp_algo algo, uint32_t source, float damping, uint32_t max
     const gxp_apply ap = algo_ == Algo::PR ? GXP_APPLY_PAGERANK : algo_ == Algo::LP ? GXP_APPLY_SET : GXP_APPLY_MIN;
     uint32_t steps = 0;
     // SSSP, CC and PageRank on one partition: at most kRunChunk supersteps per
-    // persistent cooperative launch (a grid barrier between supersteps) and
-    // one host read per launch. Its barriers are device waits: a context
-    // whose timeout_ns was set below the default takes a launch per superstep,
-    // which waits for nothing.
-    if (n_parts_ == 1 && algo_ != Algo::LP && cfg_.timeout_ns >= kDefaultTimeoutNs) {
-        const SweepArgs sa = sweep_args();
-        if (!h_run_) cuda_check(cudaHostAlloc(&h_run_, sizeof(RunOut), cudaHostAllocMapped), "pinned run report");
-        if (!d_bar_) {
-            d_bar_ = (GridBar*)dalloc(sizeof(GridBar));
-            cuda_check(cudaMemsetAsync(d_bar_, 0, sizeof(GridBar), stream_), "memset");
-            bar_passed_ = 0;
-        }
-        while (steps < max_steps) {
-            RunArgs r{};
-            r.t0 = step_;
-            r.limit = step_ + std::min<uint32_t>(kRunChunk, max_steps - steps);
-            r.quiet_stop = algo_ != Algo::PR ? 1u : 0u;
-            r.force = faults_.timeout ? 1u : 0u;
-            r.timeout_ns = cfg_.timeout_ns;
-            r.passed = bar_passed_;
-            r.bar = d_bar_;
-            r.out = h_run_;   // mapped: the same address on the device
-            h_run_->step = 0;
-            cuda_check(cudaEventRecord(ev_a_, stream_), "event");
-            cuda_check(launch_sweep(algo_, sa, r, sms_, stream_), "run");
-            ++st_.persistent_launches;
-            cuda_check(cudaEventRecord(ev_b_, stream_), "event");
-            cuda_check(cudaStreamSynchronize(stream_), "run");
-            const uint64_t done = h_run_->step;
-            err_unread_ = false;
-            if (done == 0 || h_run_->err != 0) check_device_error();   // a wait that ran out, a bad index
-            if (done <= r.t0 || done > r.limit) fail(GXP_E_CUDA, "device-driven run lost its step counter");
-            bar_passed_ = h_run_->passed;
-            const uint32_t n_run = (uint32_t)(done - r.t0);
-            for (uint32_t i = 0; i < n_run; ++i) account_step(h_run_->sum[i]);
-            steps += n_run;
-            step_ = accounted_ = done;
-            cur_ = (int)(step_ & 1u);
-            float ms = 0.f;
-            if (cudaEventElapsedTime(&ms, ev_a_, ev_b_) == cudaSuccess)
-                st_.last_superstep_ms = st_.last_kernel_ms = ms / (double)n_run;
-            if (r.quiet_stop && st_.last_changed == 0) return steps;
-        }
-        return steps;
+    // persistent launch (a grid barrier between supersteps) and one host read
+    // per launch. Its barriers are device waits: a context whose timeout_ns
+    // was set below the default takes a launch per superstep, which waits for
+    // no other CTA, and so does a run whose CTAs did not all get onto the
+    // device (other work holds an SM).
+    bool resident = n_parts_ == 1 && algo_ != Algo::LP && cfg_.timeout_ns >= kDefaultTimeoutNs;
+    const SweepArgs sa = resident ? sweep_args() : SweepArgs{};
+    if (resident && !h_run_) {   // and what a launch per superstep would have to set up
+        cuda_check(load_sweep_list(), "load kernels");
+        cuda_check(load_step_sums(), "load kernels");
+        if (!h_steps_) cuda_check(cudaHostAlloc(&h_steps_, sizeof(StepReport), cudaHostAllocMapped), "pinned reports");
+        cuda_check(cudaHostAlloc(&h_run_, sizeof(RunOut), cudaHostAllocMapped), "pinned run report");
     }
+    if (resident && !d_bar_) d_bar_ = (GridBar*)dalloc(sizeof(GridBar));
+    while (resident && steps < max_steps) {
+        if (bar_arrived_ == 0) cuda_check(cudaMemsetAsync(d_bar_, 0, sizeof(GridBar), stream_), "memset");
+        RunArgs r{};
+        r.t0 = step_;
+        r.limit = step_ + std::min<uint32_t>(kRunChunk, max_steps - steps);
+        r.quiet_stop = algo_ != Algo::PR ? 1u : 0u;
+        r.force = faults_.timeout ? 1u : 0u;
+        r.timeout_ns = cfg_.timeout_ns;
+        r.arrived = bar_arrived_;
+        r.bar = d_bar_;
+        r.out = h_run_;   // mapped: the same address on the device
+        h_run_->step = 0;
+        h_run_->err = 0;
+        bar_arrived_ = 0;   // zeroed again unless the launch reports where it left the counter
+        cuda_check(cudaEventRecord(ev_a_, stream_), "event");
+        cuda_check(launch_sweep(algo_, sa, r, sms_, stream_), "run");
+        cuda_check(cudaEventRecord(ev_b_, stream_), "event");
+        cuda_check(cudaStreamSynchronize(stream_), "run");
+        const uint64_t done = h_run_->step;
+        err_unread_ = false;
+        if (done == 0 || h_run_->err != 0) check_device_error();   // a wait that ran out, a bad index
+        if (done == 0) {   // nothing was done
+            resident = false;
+            break;
+        }
+        if (done <= r.t0 || done > r.limit) fail(GXP_E_CUDA, "device-driven run lost its step counter");
+        ++st_.persistent_launches;
+        bar_arrived_ = h_run_->arrived;
+        const uint32_t n_run = (uint32_t)(done - r.t0);
+        for (uint32_t i = 0; i < n_run; ++i) account_step(h_run_->sum[i]);
+        steps += n_run;
+        step_ = accounted_ = done;
+        cur_ = (int)(step_ & 1u);
+        float ms = 0.f;
+        if (cudaEventElapsedTime(&ms, ev_a_, ev_b_) == cudaSuccess)
+            st_.last_superstep_ms = st_.last_kernel_ms = ms / (double)n_run;
+        if (r.quiet_stop && st_.last_changed == 0) return steps;
+    }
+    if (resident) return steps;
     struct Guard {
         bool &early_exit, &queue, &timed;
         ~Guard() {

@@ -249,7 +249,7 @@ private:
     // runs of several supersteps per launch (one partition)
     uint32_t* d_bits_[3] = {nullptr, nullptr, nullptr};   // changed vertices of the pull supersteps (frontier lists)
     GridBar* d_bar_ = nullptr;     // the run's grid barrier, zero when allocated
-    uint64_t bar_passed_ = 0;      // barriers passed on it
+    uint64_t bar_arrived_ = 0;     // its counter
     RunOut* h_run_ = nullptr;      // pinned: what a launch of a run reports
     StepReport* h_steps_ = nullptr;   // pinned: what other supersteps report
     bool timed_ = true;            // the coming superstep records its events (inside gxp_run: a chunk's last)

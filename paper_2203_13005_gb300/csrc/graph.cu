@@ -502,6 +502,11 @@ cudaError_t launch_count_dangling(const uint32_t* outdeg, uint32_t n, unsigned l
     return cudaGetLastError();
 }
 
+cudaError_t load_step_sums() {
+    cudaFuncAttributes at;
+    return cudaFuncGetAttributes(&at, k_step_sums);
+}
+
 cudaError_t launch_step_sums(const StepStats* ring, uint64_t first, uint64_t last, const uint32_t* err, StepReport* out,
                              cudaStream_t s) {
     if (last < first || last - first >= (uint64_t)kStatRing) return cudaErrorInvalidValue;

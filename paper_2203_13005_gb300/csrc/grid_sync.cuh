@@ -21,9 +21,11 @@ __device__ __forceinline__ uint64_t global_ns() {
     return t;
 }
 
-// Barrier of all CTAs of a cooperative grid: an arrival counter that only
-// grows, zero when the launch starts; `passed` is the caller's count of the
-// barriers this launch has passed. A CTA's arrival is a fire-and-forget add
+// Barrier of all CTAs of a grid: an arrival counter that only grows. `arrived`
+// is the caller's count of the arrivals there are once every CTA has passed
+// the barriers before: 0 at first in a launch whose counter was zeroed
+// (msssp.cu), the counter's value where it is carried from launch to launch
+// (sweep.cu). A CTA's arrival is a fire-and-forget add
 // and every CTA polls the counter itself, so a barrier costs a fence, the
 // add's and the last poll's way to L2: with a generation word to read,
 // release and poll, and an error word to read after it, a barrier and the
@@ -32,14 +34,18 @@ __device__ __forceinline__ uint64_t global_ns() {
 // `force`, an injected fault) sets kErrTimeout and the counter's top bit and
 // gives up. Returns false when this CTA gave up or saw that another one had;
 // the caller then returns.
+// kMeet: a barrier before which nothing was done. A wait gives up only while an
+// arrival is missing, so that either every CTA passes or none, and it is no
+// error (but for an injected one).
 constexpr unsigned long long kBarGaveUp = 1ull << 63;
-__device__ inline bool grid_barrier(GridBar* b, uint32_t n_ctas, uint64_t& passed, uint64_t timeout_ns, bool force,
+template <bool kMeet = false>
+__device__ inline bool grid_barrier(GridBar* b, uint32_t n_ctas, uint64_t& arrived, uint64_t timeout_ns, bool force,
                                     uint32_t* err) {
     __shared__ uint32_t s_ok;
-    ++passed;
+    arrived += n_ctas;
     __syncthreads();
     if (threadIdx.x == 0) {
-        const unsigned long long all = passed * n_ctas;
+        const unsigned long long all = arrived;
         fence_acq_rel_gpu();
         atomicAdd(&b->count, 1ull);   // result unused: a reduction
         unsigned long long c = ld_relaxed_gpu(&b->count);
@@ -47,9 +53,10 @@ __device__ inline bool grid_barrier(GridBar* b, uint32_t n_ctas, uint64_t& passe
             const uint64_t t0 = global_ns();
             while ((c = ld_relaxed_gpu(&b->count)) < all) {   // the top bit ends every wait
                 if (force || global_ns() - t0 > timeout_ns) {
-                    atomicOr(err, kErrTimeout);
+                    if (kMeet && atomicCAS(&b->count, c, c | kBarGaveUp) != c) continue;   // another arrival
+                    if (!kMeet || force) atomicOr(err, kErrTimeout);
                     c = kBarGaveUp;
-                    atomicOr(&b->count, kBarGaveUp);
+                    if (!kMeet) atomicOr(&b->count, kBarGaveUp);
                     break;
                 }
             }

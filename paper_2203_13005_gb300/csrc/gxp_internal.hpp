@@ -548,16 +548,16 @@ cudaError_t launch_init_ghosts(Algo a, uint32_t n_ghost_total, const uint32_t* g
 cudaError_t launch_superstep(Algo a, const SuperstepArgs& args, uint32_t sms, cudaStream_t s);
 cudaError_t launch_superstep_sell(Algo a, const SellArgs& args, cudaStream_t s);
 
-// Grid barrier state of a persistent launch, zero when it starts.
+// Grid barrier state of a persistent launch (grid_barrier).
 struct GridBar {
-    unsigned long long count;   // arrivals so far; top bit: a wait gave up
+    unsigned long long count;   // arrivals since it was zeroed; top bit: a wait gave up
 };
 constexpr uint32_t kRunChunk = 32;   // supersteps per launch of a run (the stat ring holds 64)
 // What a launch of several supersteps leaves in pinned host memory. The host
 // clears `step` before the launch; a launch that gave up leaves it zero.
 struct RunOut {
     uint64_t step;          // supersteps done since gxp_begin
-    uint64_t passed;        // grid barriers passed since the counter was zeroed
+    uint64_t arrived;       // the barrier counter
     uint32_t err, pad;      // the error word
     StepSum sum[kRunChunk]; // of the launch's supersteps
 };
@@ -566,14 +566,20 @@ struct RunArgs {
     uint64_t t0, limit;
     uint32_t quiet_stop, force;   // force: every barrier wait gives up (an injected fault)
     uint64_t timeout_ns;
-    uint64_t passed;        // the barrier counter's value in barriers
+    uint64_t arrived;       // the barrier counter's value
     GridBar* bar;           // nullptr: superstep t0 alone, in a launch that waits for nothing
     RunOut* out;
 };
 // Supersteps of a single-partition graph (sweep.cu), one CTA on each of the
-// `sms` multiprocessors, in one cooperative launch; a barrier wait past
-// timeout_ns sets kErrTimeout in args.err and ends the launch.
+// `sms` multiprocessors, in one launch. If its CTAs don't all get onto the
+// device in time, none of them does anything (run.out->step stays zero, and
+// the barrier's top bit is set); a later barrier wait past timeout_ns sets
+// kErrTimeout in args.err and ends the launch.
 cudaError_t launch_sweep(Algo a, const SweepArgs& args, const RunArgs& run, uint32_t sms, cudaStream_t s);
+// Load the kernels that a launch per superstep takes besides: the first launch
+// of one not loaded yet waits for whatever runs on the device.
+cudaError_t load_sweep_list();
+cudaError_t load_step_sums();
 // Values to stage per CTA.
 uint32_t sweep_hot_values(uint64_t n_vertices, uint64_t n_edges, bool by_degree);
 

@@ -254,7 +254,6 @@ __global__ void __launch_bounds__(kMsBlock, 4)
                  uint32_t* steps_out) {
     uint32_t* const F[3] = {f0, f1, f2};
     __shared__ uint32_t s_more;
-    uint64_t passed = 0;
     for (uint32_t t = 0; t < max_steps; ++t) {
         a.frontier_cur = F[t % 3];
         a.frontier_next = F[(t + 1) % 3];
@@ -264,7 +263,8 @@ __global__ void __launch_bounds__(kMsBlock, 4)
             clear[i] = 0u;
         if (blockIdx.x == 0 && threadIdx.x == 0) changed[(t + 2) % 4] = 0ull;
         msssp_block<LG, false, false, true, kNoSat>(a);
-        if (!grid_barrier(bar, gridDim.x, passed, timeout_ns, force != 0u, err)) return;
+        uint64_t arrived = (uint64_t)t * gridDim.x;
+        if (!grid_barrier(bar, gridDim.x, arrived, timeout_ns, force != 0u, err)) return;
         if (threadIdx.x == 0) s_more = __ldcg(changed + t % 4) != 0ull ? 1u : 0u;
         __syncthreads();
         if (!s_more || t + 1 == max_steps) {

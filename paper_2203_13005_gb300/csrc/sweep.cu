@@ -58,6 +58,13 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kThreads = 1024;   // one CTA per SM: 64 registers a thread
 constexpr int kWarps = kThreads / 32;
 constexpr int kZeroGroup = 4;      // slices of rows without in-edges per item
+// How long the first CTAs of a run wait for the others. Not a cooperative
+// launch, which the device holds back until every SM is free at once: beside a
+// kernel of 0.3 s on one SM a PageRank run of 0.41 ms took 279 ms. So it takes
+// 0.79 ms (0.94 / 1.74 ms with a limit of 200 / 1,000 us, 0.74 ms if every run
+// were a launch per superstep); beside a busy query server 0.43 .. 0.56 ms
+// with each of the limits. Alone, all of 3,000 runs met; meeting costs 1.6 us.
+constexpr uint64_t kGatherNs = 50000;
 constexpr uint32_t kMaxHot = 32768;     // staged values: 208 KB of the 227 KB a CTA may have
 
 // Columns (gathers) in flight per lane. More of them spill registers and run
@@ -661,10 +668,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_sweep(const SweepArgs a, const 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool loop = run.bar != nullptr;
     uint64_t t = run.t0;
-    uint64_t passed = run.passed;   // grid barriers
+    uint64_t arrived = run.arrived;   // at the grid barriers so far
     if (tid < 3) s_acc[tid] = 0ull;
     if (tid < 2) s_cnt[tid] = 0u;
     __syncthreads();   // a push superstep has no other barrier before the warps add to them
+    // The grid's barriers wait for CTAs that may not be on an SM yet, and never
+    // get there while something else holds it. So nothing is done before all
+    // of them have met here, within kGatherNs of the first; else none does
+    // anything and the host takes a launch per superstep.
+    if (loop && !grid_barrier<true>(run.bar, gridDim.x, arrived, kGatherNs, run.force != 0u, a.err)) return;
     for (;;) {
         const StepStats* const in = a.stats + t % kStatRing;
         StepStats* const out = a.stats + (t + 1) % kStatRing;
@@ -692,7 +704,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sweep(const SweepArgs a, const 
             pushes = sweep_pushes(fc, in, &needs_list);   // the same in every thread of the grid
             if (pushes && needs_list && loop) {
                 build_list(a, t, lane);
-                if (!grid_barrier(run.bar, gridDim.x, passed, run.timeout_ns, run.force != 0u, a.err)) return;
+                if (!grid_barrier(run.bar, gridDim.x, arrived, run.timeout_ns, run.force != 0u, a.err)) return;
             }
             if (blockIdx.x == 0 && tid == 0 && fc.list_out) {
                 if (pushes) {
@@ -777,7 +789,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sweep(const SweepArgs a, const 
             s_cnt[0] = s_cnt[1] = 0u;
         }
         if (!loop) return;
-        if (!grid_barrier(run.bar, gridDim.x, passed, run.timeout_ns, run.force != 0u, a.err)) return;
+        if (!grid_barrier(run.bar, gridDim.x, arrived, run.timeout_ns, run.force != 0u, a.err)) return;
         ++t;   // supersteps done; slot t holds the last one's counts
         bool more = t < run.limit;
         if (more && run.quiet_stop) {   // every warp reads the counts itself
@@ -793,7 +805,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sweep(const SweepArgs a, const 
                 report_step(st, &run.out->sum[warp], a.err, &run.out->err);
             }
             if (tid == 0) {
-                run.out->passed = passed;
+                run.out->arrived = arrived;
                 run.out->step = t;
             }
         }
@@ -818,11 +830,15 @@ cudaError_t launch_t(const SweepArgs& args, const RunArgs& run, uint32_t sms, cu
     SweepArgs a = args;
     RunArgs r = run;
     void* params[] = {&a, &r};
-    if (run.bar) return cudaLaunchCooperativeKernel(fn, dim3(sms), dim3(kThreads), params, smem, s);
     return cudaLaunchKernel(fn, dim3(sms), dim3(kThreads), params, smem, s);
 }
 
 }  // namespace
+
+cudaError_t load_sweep_list() {
+    cudaFuncAttributes at;
+    return cudaFuncGetAttributes(&at, k_sweep_list);
+}
 
 // All values of a graph that fits, else of a renumbered graph's first
 // vertices (its hottest), else none. Staging takes ~2 us for 128 KB, which a
