@@ -571,7 +571,7 @@ struct RunArgs {
     RunOut* out;
 };
 // Supersteps of a single-partition graph (sweep.cu), one CTA on each of the
-// `sms` multiprocessors, in one launch. If its CTAs don't all get onto the
+// `sms` multiprocessors (fewer on small graphs), in one launch. If its CTAs don't all get onto the
 // device in time, none of them does anything (run.out->step stays zero, and
 // the barrier's top bit is set); a later barrier wait past timeout_ns sets
 // kErrTimeout in args.err and ends the launch.

@@ -822,7 +822,7 @@ __global__ void __launch_bounds__(256) k_sweep_list(const SweepArgs a, uint64_t 
 }
 
 template <Algo A, bool kCheck>
-cudaError_t launch_t(const SweepArgs& args, const RunArgs& run, uint32_t sms, cudaStream_t s) {
+cudaError_t launch_t(const SweepArgs& args, const RunArgs& run, uint32_t ctas, cudaStream_t s) {
     const void* fn = (const void*)k_sweep<A, kCheck>;
     const size_t smem = 4 * (size_t)args.n_hot;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * (int)kMaxHot);
@@ -830,7 +830,7 @@ cudaError_t launch_t(const SweepArgs& args, const RunArgs& run, uint32_t sms, cu
     SweepArgs a = args;
     RunArgs r = run;
     void* params[] = {&a, &r};
-    return cudaLaunchKernel(fn, dim3(sms), dim3(kThreads), params, smem, s);
+    return cudaLaunchKernel(fn, dim3(ctas), dim3(kThreads), params, smem, s);
 }
 
 }  // namespace
@@ -860,6 +860,15 @@ cudaError_t launch_sweep(Algo alg, const SweepArgs& args, const RunArgs& run, ui
     if (args.n_hot > kMaxHot || args.n_hot % 4 || sms == 0) return cudaErrorInvalidValue;
     if (args.cols != 4 && args.cols != 8 && args.cols != 16) return cudaErrorInvalidValue;
     if (run.bar && (run.limit <= run.t0 || run.limit - run.t0 > kRunChunk || !run.out)) return cudaErrorInvalidValue;
+    // A CTA for every kWarps items at least: on a small graph the barriers of
+    // fewer CTAs cost less than a warp's second item. Runs of many supersteps
+    // of little work, an item or more a CTA / 16 / 32 (us a superstep): SSSP
+    // along a path of 20,000 vertices 9.3 / - / 7.1, on a 300 x 300 mesh 10.0 /
+    // 10.0 / 8.7; PageRank of R-MAT 12 9.9 / 8.6 / 9.4. (64: 6.9, 8.1, -, but a
+    // warp's items then follow one another on graphs that fill the chip.)
+    uint64_t items = args.n_hubs + (args.n_slices - args.n_lanes[4]);
+    for (int c = 0; c < 5; ++c) items += (uint64_t)(args.n_lanes[c] - (c ? args.n_lanes[c - 1] : 0u)) << (5 - c);
+    const uint32_t ctas = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(sms, (items + kWarps - 1) / kWarps));
     const bool chk = args.check_bounds != 0;
     if (!run.bar && alg != Algo::PR && args.fc.list_out && args.fc.direction != GXP_DIR_PULL) {
         k_sweep_list<<<sms, 256, 0, s>>>(args, run.t0);
@@ -867,12 +876,12 @@ cudaError_t launch_sweep(Algo alg, const SweepArgs& args, const RunArgs& run, ui
         if (e != cudaSuccess) return e;
     }
     switch (alg) {
-        case Algo::SSSP: return chk ? launch_t<Algo::SSSP, true>(args, run, sms, s)
-                                    : launch_t<Algo::SSSP, false>(args, run, sms, s);
-        case Algo::CC: return chk ? launch_t<Algo::CC, true>(args, run, sms, s)
-                                  : launch_t<Algo::CC, false>(args, run, sms, s);
-        case Algo::PR: return chk ? launch_t<Algo::PR, true>(args, run, sms, s)
-                                  : launch_t<Algo::PR, false>(args, run, sms, s);
+        case Algo::SSSP: return chk ? launch_t<Algo::SSSP, true>(args, run, ctas, s)
+                                    : launch_t<Algo::SSSP, false>(args, run, ctas, s);
+        case Algo::CC: return chk ? launch_t<Algo::CC, true>(args, run, ctas, s)
+                                  : launch_t<Algo::CC, false>(args, run, ctas, s);
+        case Algo::PR: return chk ? launch_t<Algo::PR, true>(args, run, ctas, s)
+                                  : launch_t<Algo::PR, false>(args, run, ctas, s);
         default: return cudaErrorInvalidValue;
     }
 }

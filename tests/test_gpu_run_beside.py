@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.fixture(scope="module")
 def graph():
-    wl = synth.SSSP_RMAT16.scaled(14)
+    wl = synth.SSSP_RMAT16.scaled(17)   # enough work for a CTA on every SM
     src, dst, w = wl.edges()
     return wl.n_vertices, src, dst, w
 
