@@ -1322,6 +1322,7 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
     } else if (n_parts_ == 1) {
         RunArgs one{};
         one.t0 = step_;
+        one.quiet_stop = early_exit_ && step_ > 0 ? 1u : 0u;
         cuda_check(launch_sweep(algo_, sweep_args(), one, sms_, stream_), "superstep kernel");
     } else {
         const SellArgs a = sell_args();

@@ -561,7 +561,8 @@ struct RunOut {
     uint32_t err, pad;      // the error word
     StepSum sum[kRunChunk]; // of the launch's supersteps
 };
-// Supersteps t0, t0 + 1, ... below limit, or until one that changed nothing.
+// Supersteps t0, t0 + 1, ... below limit, with quiet_stop until one that
+// changed nothing (a lone superstep then returns at once after such a one).
 struct RunArgs {
     uint64_t t0, limit;
     uint32_t quiet_stop, force;   // force: every barrier wait gives up (an injected fault)

@@ -677,6 +677,24 @@ __global__ void __launch_bounds__(kThreads, 1) k_sweep(const SweepArgs a, const 
     // of them have met here, within kGatherNs of the first; else none does
     // anything and the host takes a launch per superstep.
     if (loop && !grid_barrier<true>(run.bar, gridDim.x, arrived, kGatherNs, run.force != 0u, a.err)) return;
+    auto clear_ahead = [&]() {   // what superstep t clears for those after it
+        if (blockIdx.x == gridDim.x - 1) {
+            unsigned long long* z = reinterpret_cast<unsigned long long*>(a.stats + (t + 2) % kStatRing);
+            for (uint32_t i = tid; i < sizeof(StepStats) / 8; i += kThreads) z[i] = 0ull;
+        }
+        if (A != Algo::PR && a.fc.list_out) {
+            uint32_t* z = a.bits[(t + 1) % 3];
+            const uint32_t words = (a.n_vertices + 31u) / 32u;
+            for (uint32_t i = blockIdx.x * kThreads + tid; i < words; i += gridDim.x * kThreads) z[i] = 0u;
+        }
+    };
+    if (A != Algo::PR && !loop && run.quiet_stop) {   // a lone superstep after one that changed nothing
+        const StepStats* const in = a.stats + t % kStatRing;
+        if (!__any_sync(kFull, (__ldcg(&in->changed[lane]) + __ldcg(&in->changed[lane + 32])) != 0ull)) {
+            clear_ahead();
+            return;
+        }
+    }
     for (;;) {
         const StepStats* const in = a.stats + t % kStatRing;
         StepStats* const out = a.stats + (t + 1) % kStatRing;
@@ -689,17 +707,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_sweep(const SweepArgs a, const 
         s.bits = a.bits[t % 3];
         s.hot = (uint32_t)__cvta_generic_to_shared(s_hot);
         s.base = s.base_src = 0.0f;
-        if (blockIdx.x == gridDim.x - 1) {
-            unsigned long long* z = reinterpret_cast<unsigned long long*>(a.stats + (t + 2) % kStatRing);
-            for (uint32_t i = tid; i < sizeof(StepStats) / 8; i += kThreads) z[i] = 0ull;
-        }
+        clear_ahead();
         bool pushes = false;
         if constexpr (A != Algo::PR) {
-            if (fc.list_out) {
-                uint32_t* z = a.bits[(t + 1) % 3];
-                const uint32_t words = (a.n_vertices + 31u) / 32u;
-                for (uint32_t i = blockIdx.x * kThreads + tid; i < words; i += gridDim.x * kThreads) z[i] = 0u;
-            }
             bool needs_list;
             pushes = sweep_pushes(fc, in, &needs_list);   // the same in every thread of the grid
             if (pushes && needs_list && loop) {

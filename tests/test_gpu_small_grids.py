@@ -35,3 +35,31 @@ def test_items_at_the_borders(gpu, direction, timeout_ns):
             c.run(gxp.GXP_ALGO_PAGERANK, max_steps=35)
             r, ref = c.values().astype(np.float64), oracle.pagerank(n, src, dst, 0.85, 35)[0]
             assert (np.abs(r - ref) / ref).max() <= 1e-4, items
+
+
+@pytest.mark.parametrize("direction", [gxp.GXP_DIR_AUTO, gxp.GXP_DIR_PULL, gxp.GXP_DIR_PUSH])
+@pytest.mark.parametrize("algo", [gxp.GXP_ALGO_SSSP, gxp.GXP_ALGO_CC])
+def test_superstep_after_a_run(gpu, algo, direction):
+    """A run of launches of their own ends in supersteps enqueued past the fixed
+    point, which return at once; supersteps driven by the caller go on from there."""
+    n = 3000
+    rng = np.random.default_rng(8)
+    src, dst = rng.integers(0, n, 9000).astype(np.uint32), rng.integers(0, n, 9000).astype(np.uint32)
+    w = rng.integers(1, 100, 9000).astype(np.uint32)
+    sssp = algo == gxp.GXP_ALGO_SSSP
+    ref, steps, _ = oracle.sssp(n, src, dst, w, 4) if sssp else oracle.cc(n, src, dst)
+    step = (lambda x: oracle.sssp_step(n, src, dst, w, x)) if sssp else (lambda x: oracle.cc_step(n, src, dst, x))
+    with gxp.Context(0, timeout_ns=1000, direction=direction) as c:
+        c.create_graph(n, 1)
+        c.load_coo(src, dst, w)
+        for _ in range(2):
+            assert c.run(algo, source=4) == steps
+            assert c.superstep() == 0
+            assert np.array_equal(c.values(), ref)
+            x = ref.copy()
+            x[rng.integers(0, n, 5)] = 0
+            c.set_values(x)
+            for _ in range(6):
+                x, changed = step(x)
+                assert c.superstep() == changed
+                assert np.array_equal(c.values(), x)
