@@ -212,7 +212,7 @@ typedef struct gxp_stats {
                                        device-driven loop: the average superstep */
     uint64_t persistent_launches;   /* gxp_run launches of the persistent superstep kernel since
                                        gxp_begin (single-partition SSSP, CC and PageRank: one
-                                       cooperative kernel runs up to 32 supersteps) */
+                                       launch runs up to 32 supersteps) */
     uint64_t reserved[2];
 } gxp_stats;
 
@@ -327,10 +327,12 @@ GXP_API gxp_status gxp_cache_get(gxp_ctx* ctx, uint32_t part, uint32_t* ids, uin
  * PageRank; LP need not settle: the paper caps it at 15). Starts with
  * gxp_begin(algo, source, damping). *steps_done (nullable) counts supersteps
  * run, including the final one that changed nothing. SSSP, CC and PageRank on
- * one partition run the loop on the device (a persistent cooperative kernel,
- * up to 32 supersteps and one host synchronization per launch; with a
- * timeout_ns below the default a launch per superstep, which waits for
- * nothing); the others enqueue supersteps in chunks and read their changed
+ * one partition run the loop on the device (a persistent kernel, up to 32
+ * supersteps and one host synchronization per launch). They take a launch per
+ * superstep instead, none of whose thread blocks waits for another one to
+ * start, when timeout_ns is below 100 ms, and when the kernel's blocks don't
+ * all get onto the device within 50 us because other work holds it; the values
+ * are the same. The others enqueue supersteps in chunks and read their changed
  * counts once per chunk. */
 GXP_API gxp_status gxp_run(gxp_ctx* ctx, gxp_algo algo, uint32_t source, float damping,
                            uint32_t max_steps, uint32_t* steps_done);

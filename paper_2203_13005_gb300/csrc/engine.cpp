@@ -25,6 +25,10 @@ void cuda_check(cudaError_t e, const char* what) {
 namespace {
 
 constexpr uint64_t kDefaultTimeoutNs = 2000000000ull;
+// gxp_run waits at grid barriers only in contexts that allow them this long: a
+// CTA waits there for the slowest one's share of a superstep, and reading all
+// of the device's memory once takes 40 ms.
+constexpr uint64_t kBarrierTimeoutNs = 100000000ull;
 constexpr uint32_t kDefaultTile = 2048;   // edges per hub part; rows above tile/2 in-edges are hubs
 
 inline size_t pad4(size_t n) { return ((n + 3) & ~size_t(3)) + 4; }
@@ -1747,10 +1751,10 @@ uint32_t Engine::run(gxp_algo algo, uint32_t source, float damping, uint32_t max
     // SSSP, CC and PageRank on one partition: at most kRunChunk supersteps per
     // persistent launch (a grid barrier between supersteps) and one host read
     // per launch. Its barriers are device waits: a context whose timeout_ns
-    // was set below the default takes a launch per superstep, which waits for
+    // is below kBarrierTimeoutNs takes a launch per superstep, which waits for
     // no other CTA, and so does a run whose CTAs did not all get onto the
     // device (other work holds an SM).
-    bool resident = n_parts_ == 1 && algo_ != Algo::LP && cfg_.timeout_ns >= kDefaultTimeoutNs;
+    bool resident = n_parts_ == 1 && algo_ != Algo::LP && cfg_.timeout_ns >= kBarrierTimeoutNs;
     const SweepArgs sa = resident ? sweep_args() : SweepArgs{};
     if (resident && !h_run_) {   // and what a launch per superstep would have to set up
         cuda_check(load_sweep_list(), "load kernels");

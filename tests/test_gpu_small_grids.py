@@ -14,7 +14,7 @@ ITEMS = [1, 2, 31, 32, 33, 63, 64, 65, 151, 153, 32 * 151, 32 * 152 - 1, 32 * 15
 
 
 @pytest.mark.parametrize("direction", [gxp.GXP_DIR_AUTO, gxp.GXP_DIR_PULL])
-@pytest.mark.parametrize("timeout_ns", [0, 1_000_000_000])   # the second: a launch per superstep
+@pytest.mark.parametrize("timeout_ns", [0, 1_000_000])   # the second: a launch per superstep
 def test_items_at_the_borders(gpu, direction, timeout_ns):
     with gxp.Context(0, direction=direction, timeout_ns=timeout_ns) as c:
         for items in ITEMS:
@@ -63,3 +63,14 @@ def test_superstep_after_a_run(gpu, algo, direction):
                 x, changed = step(x)
                 assert c.superstep() == changed
                 assert np.array_equal(c.values(), x)
+
+
+@pytest.mark.parametrize("timeout_ns,persistent", [(0, True), (500_000_000, True), (100_000_000, True), (99_999_999, False)])
+def test_timeout_that_allows_barriers(gpu, timeout_ns, persistent):
+    n = 1000
+    src, dst = np.arange(n - 1, dtype=np.uint32), np.arange(1, n, dtype=np.uint32)
+    with gxp.Context(0, timeout_ns=timeout_ns) as c:
+        c.create_graph(n, 1)
+        c.load_coo(src, dst)
+        c.run(gxp.GXP_ALGO_PAGERANK, max_steps=5)
+        assert (c.stats()["persistent_launches"] > 0) == persistent
