@@ -44,6 +44,10 @@ constexpr int kGatherUnroll = 4;
 constexpr int kBigBlock = 1024;
 constexpr uint32_t kBigSlots = 16384;      // 128 KB of keys and counts
 constexpr uint32_t kBigPerPass = 8192;     // labels a pass aims at
+constexpr uint32_t kBigProbes = 256;       // of a label in a pass, in the first kBigTries tries
+constexpr uint32_t kBigTries = 8;
+constexpr uint32_t kAllProbes = 2 * kLpChunk - 1;   // of a label in the tables of shorter rows, all of their slots
+constexpr uint32_t kLpHash = 0x9E3779B1u;  // a label's first slot: the top bits of its product
 
 // the label of in-edge source s of partition P (previous superstep)
 __device__ __forceinline__ uint32_t lp_label(const LpArgs& a, const LpPart& P, uint32_t s) {
@@ -231,7 +235,7 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_slices(const LpArgs a) {
 __device__ __forceinline__ uint32_t lp_table_add(uint32_t* keys, uint32_t* counts, uint32_t log2_size,
                                                  uint32_t label, uint32_t count) {
     const uint32_t mask = log2_size >= 32u ? 0xFFFFFFFFu : (1u << log2_size) - 1u;
-    uint32_t slot = (label * 0x9E3779B1u) >> (32u - log2_size);
+    uint32_t slot = (label * kLpHash) >> (32u - log2_size);
     for (uint64_t probe = 0; probe <= mask; ++probe) {
         const uint32_t k = atomicCAS(keys + slot, kInf, label);
         if (k == kInf || k == label) {
@@ -245,10 +249,11 @@ __device__ __forceinline__ uint32_t lp_table_add(uint32_t* keys, uint32_t* count
 
 // Add a warp's labels (where `has`) to a shared-memory table of 2^log2_size
 // slots. A slot's count is its label's occurrences less one, so a label
-// that occurs once costs the compare-and-swap alone. Returns false for a lane
-// whose label found no slot (a full table). All 32 lanes must call it.
-__device__ __forceinline__ bool lp_warp_add(uint32_t* keys, uint32_t* more, uint32_t log2_size, uint32_t label, bool has,
-                                            int lane) {
+// that occurs once costs the compare-and-swap alone. `hash` is the label's, its
+// top bits the first slot. Returns false for a lane whose label found no slot
+// in `probes` + 1 of them. All 32 lanes must call it.
+__device__ __forceinline__ bool lp_warp_add(uint32_t* keys, uint32_t* more, uint32_t log2_size, uint32_t label,
+                                            uint32_t hash, uint32_t probes, bool has, int lane) {
     const unsigned act = __ballot_sync(kFull, has);
     if (act == 0u) return true;
     // lanes that carry the first lane's label count as one
@@ -258,8 +263,8 @@ __device__ __forceinline__ bool lp_warp_add(uint32_t* keys, uint32_t* more, uint
     if (!has || (label == l0 && lane != first)) return true;
     const uint32_t c = lane == first ? (uint32_t)__popc(same) : 1u;
     const uint32_t mask = (1u << log2_size) - 1u;
-    uint32_t slot = (label * 0x9E3779B1u) >> (32u - log2_size);
-    for (uint32_t probe = 0; probe <= mask; ++probe) {
+    uint32_t slot = hash >> (32u - log2_size);
+    for (uint32_t probe = 0; probe <= probes; ++probe) {
         const uint32_t k = atomicCAS(keys + slot, kInf, label);
         if (k == kInf || k == label) {
             const uint32_t add = k == kInf ? c - 1u : c;
@@ -340,7 +345,8 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_warp_rows(const LpArgs a) {
             }
 #pragma unroll
             for (int q = 0; q < kGatherUnroll; ++q)   // (a table of 2n slots never fills)
-                lp_warp_add(keys, more, lg, lab[q], i0 + 32u * q + (uint32_t)lane < n, lane);
+                lp_warp_add(keys, more, lg, lab[q], lab[q] * kLpHash, kAllProbes,
+                            i0 + 32u * q + (uint32_t)lane < n, lane);
         }
         __syncwarp();
         unsigned long long best = 0ull;
@@ -405,7 +411,8 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_rows(const LpArgs a) {
             }
 #pragma unroll
             for (int q = 0; q < kGatherUnroll; ++q)
-                lp_warp_add(t_key, t_more, lg, lab[q], i0 + (uint32_t)q * kLpBlock + (uint32_t)tid < n, lane);
+                lp_warp_add(t_key, t_more, lg, lab[q], lab[q] * kLpHash, kAllProbes,
+                            i0 + (uint32_t)q * kLpBlock + (uint32_t)tid < n, lane);
         }
         __syncthreads();
         // read the counts and empty the table for the next row
@@ -436,16 +443,31 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_rows(const LpArgs a) {
     if (tid < 32) lp_count(a, acc, lane, blockIdx.x);
 }
 
+// A permutation of the labels for each try but the first: MurmurHash3's 32-bit
+// finalizer (A. Appleby) of the label with the try's number mixed in.
+__device__ __forceinline__ uint32_t lp_rehash(uint32_t x, uint32_t attempt) {
+    x ^= attempt * 0x632BE5ABu;
+    x = (x ^ (x >> 16)) * 0x85EBCA6Bu;
+    x = (x ^ (x >> 13)) * 0xC2B2AE35u;
+    return x ^ (x >> 16);
+}
+
 // Rows of 2049..65,536 in-edges, a large CTA each: `passes` sweeps over the
 // row, pass p counting the labels whose second hash falls in its range. A
-// pass whose labels do not fit the table (they are as many as it aims at up
-// to the hash's spread) starts the row again with twice as many passes.
+// label that finds no slot within kBigProbes starts the row again with other
+// hashes, and with twice as many passes if the table had filled up. Labels can
+// be chosen to crowd under one hash (60,000 of them would have needed 262,144
+// passes under the first one), but few labels crowd under several: what five
+// tries in a row put into one pass is one 2^25th of the 32-bit numbers, 128
+// labels. After kBigTries a label may look at every slot. So a row takes at
+// most some hundreds of passes.
 __global__ void __launch_bounds__(kBigBlock) k_lp_big(const LpArgs a) {
     extern __shared__ uint32_t s_table[];
     uint32_t* t_key = s_table;
     uint32_t* t_more = s_table + kBigSlots;
     __shared__ unsigned long long s_red[kBigBlock / 32];
     __shared__ uint32_t s_want[kBigBlock / 32];
+    __shared__ uint32_t s_taken;   // slots, in a try that failed
     const int tid = threadIdx.x, lane = tid & 31;
     if (lp_quiet(a, lane)) return;
     const bool sparse = lp_sparse(a);
@@ -471,42 +493,59 @@ __global__ void __launch_bounds__(kBigBlock) k_lp_big(const LpArgs a) {
         while (lg < 14u && (1u << lg) < 2u * min(n, kBigPerPass)) ++lg;
         const uint32_t size = 1u << lg;
         unsigned long long best = 0ull;
+        uint32_t attempt = 0;
         for (uint32_t p = 0; p < passes; ++p) {
-            bool ok = true;
-            for (uint32_t i0 = 0; i0 < n; i0 += (uint32_t)kBigBlock * kGatherUnroll) {
-                uint32_t sv[kGatherUnroll], lab[kGatherUnroll];
+            // count the labels of pass p; false: one found no slot. The first
+            // try is compiled apart, without what the others need.
+            auto count = [&](auto first) {
+                constexpr bool kFirst = decltype(first)::value;
+                const uint32_t probes = kFirst || attempt < kBigTries ? kBigProbes : size - 1u;
+                bool ok = true;
+                for (uint32_t i0 = 0; i0 < n; i0 += (uint32_t)kBigBlock * kGatherUnroll) {
+                    uint32_t sv[kGatherUnroll], lab[kGatherUnroll];
 #pragma unroll
-                for (int q = 0; q < kGatherUnroll; ++q) {
-                    const uint32_t i = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid;
-                    sv[q] = i < n ? __ldg(P.src + r.e0 + i) : 0u;
-                }
+                    for (int q = 0; q < kGatherUnroll; ++q) {
+                        const uint32_t i = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid;
+                        sv[q] = i < n ? __ldg(P.src + r.e0 + i) : 0u;
+                    }
 #pragma unroll
-                for (int q = 0; q < kGatherUnroll; ++q) {
-                    const uint32_t i = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid;
-                    lab[q] = i < n ? lp_label(a, P, sv[q]) : 0u;
-                }
+                    for (int q = 0; q < kGatherUnroll; ++q) {
+                        const uint32_t i = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid;
+                        lab[q] = i < n ? lp_label(a, P, sv[q]) : 0u;
+                    }
 #pragma unroll
-                for (int q = 0; q < kGatherUnroll; ++q) {
-                    const bool mine = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid < n &&
-                                      __umulhi(lab[q] * 0x85EBCA6Bu, passes) == p;
-                    ok &= lp_warp_add(t_key, t_more, lg, lab[q], mine, lane);
+                    for (int q = 0; q < kGatherUnroll; ++q) {
+                        const uint32_t key = kFirst ? lab[q] : lp_rehash(lab[q], attempt);
+                        const bool mine = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid < n && (kFirst || ok) &&
+                                          __umulhi(key * 0x85EBCA6Bu, passes) == p;
+                        ok &= lp_warp_add(t_key, t_more, lg, lab[q], key * kLpHash, probes, mine, lane);
+                    }
                 }
-            }
+                return ok;
+            };
+            bool ok = attempt == 0u ? count(std::true_type{}) : count(std::false_type{});
+            if (tid == 0) s_taken = 0u;
             ok = __syncthreads_and(ok);
+            uint32_t taken = 0;
             for (uint32_t i = (uint32_t)tid; i < size; i += kBigBlock) {
                 const uint32_t k = t_key[i];
                 if (k != kInf) {
                     if (ok) best = max(best, mode_key(t_more[i] + 1u, k));
                     t_key[i] = kInf;
                     t_more[i] = 0u;
+                    ++taken;
                 }
             }
-            __syncthreads();
-            if (!ok) {   // again, with smaller passes (labels are distinct under the hash: this ends)
-                passes = min(2u * passes, 1u << 30);
+            if (!ok) {   // again, with other hashes (the same in every thread)
+                taken = __reduce_add_sync(kFull, taken);
+                if (lane == 0) atomicAdd(&s_taken, taken);
+                __syncthreads();
+                if (s_taken > size / 4u * 3u) passes = min(2u * passes, 1u << 30);
+                ++attempt;
                 best = 0ull;
                 p = 0xFFFFFFFFu;   // ++ -> 0
             }
+            __syncthreads();
         }
         best = block_max<kBigBlock>(best, s_red);
         if (tid == 0) lp_apply(a, r.g, ~(uint32_t)best, acc);
