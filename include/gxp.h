@@ -194,7 +194,10 @@ typedef struct gxp_ctx gxp_ctx;
 
 typedef struct gxp_stats {
     uint64_t supersteps;            /* supersteps run since the last gxp_begin */
-    uint64_t edges_scanned;         /* edges read by supersteps since gxp_begin */
+    uint64_t edges_scanned;         /* edges read by supersteps since gxp_begin: all of them, a pushing
+                                       superstep's the out-edges of its frontier, those of a
+                                       label-propagation superstep that recomputes some rows only
+                                       the in-edges of these */
     uint64_t last_changed;          /* vertices changed by the last superstep */
     uint64_t last_boundary_changed; /* of which boundary vertices uploaded by its sync */
     uint64_t syncs_done;            /* exchanges performed (Algorithm 3) */

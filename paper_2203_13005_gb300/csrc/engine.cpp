@@ -1318,6 +1318,7 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
             l.all_rows = lp_all_rows_ ? 1u : 0u;
             l.out_ptr = d_out_ptr_;
             l.out_dst = d_out_dst_;
+            l.col_ptr = work_[0].col;
         }
         lp_all_rows_ = false;
         l.n_vertices = (uint32_t)n_vertices_;
@@ -1399,7 +1400,7 @@ uint64_t Engine::superstep(gxp_algo algo, gxp_msggen g, gxp_merge m, gxp_apply a
 void Engine::account_step(const StepSum& s) {
     st_.supersteps++;
     st_.edges_scanned += s.pushed ? s.push_edges : total_edges_;
-    if (s.pushed) st_.push_supersteps++;
+    if (s.pushed == 1) st_.push_supersteps++;
     st_.last_changed = s.changed;
     if (algo_ == Algo::PR) {
         st_.last_dangling = fx_to_double(s.dangling_fx);

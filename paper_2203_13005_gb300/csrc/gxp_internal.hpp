@@ -144,8 +144,8 @@ struct StepStats {
     // items appended to its list (high 32 bits) and the out-edges of the
     // vertices they cover (low 32 bits), advanced together by one atomic
     unsigned long long list_ne;
-    unsigned long long pushed;                    // 1: the superstep ran in push direction,
-    unsigned long long push_edges;                //    relaxing this many out-edges
+    unsigned long long pushed;                    // 1: the superstep ran in push direction, 2: LP recomputed some
+    unsigned long long push_edges;                //    rows; out-edges relaxed, the rows' in-edges
     unsigned long long exchanged;                 // 1 once the superstep's exchange between
                                                   // partitions ran (skipped or not)
     unsigned long long downloads;                 // copies the superstep used that were not cached
@@ -462,6 +462,7 @@ struct LpArgs {
     uint32_t n_vertices;
     uint64_t n_edges;
     const uint32_t *out_ptr, *out_dst;
+    const uint32_t* col_ptr;    // one partition: row offsets, for the edges a superstep of some rows reads
 };
 cudaError_t launch_lp_superstep(const LpArgs& a, cudaStream_t s);
 

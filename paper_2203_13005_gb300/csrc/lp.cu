@@ -77,9 +77,10 @@ __device__ __forceinline__ bool lp_marked(const LpArgs& a, uint32_t g) {
     return (__ldg(a.active + (g >> 5)) >> (g & 31u)) & 1u;
 }
 
-// what a thread adds up: changed rows and the out-edges of their vertices
+// what a thread adds up: changed rows and the out-edges of their vertices, and
+// (if only the marked rows are recomputed) the in-edges of the rows
 struct LpAcc {
-    uint32_t changed = 0, edges = 0, boundary = 0;
+    uint32_t changed = 0, edges = 0, boundary = 0, read = 0;
 };
 
 // MSGApply
@@ -96,8 +97,10 @@ __device__ __forceinline__ void lp_apply(const LpArgs& a, uint32_t g, uint32_t l
 // a warp's sums into the superstep's stats
 __device__ __forceinline__ void lp_count(const LpArgs& a, const LpAcc& acc, int lane, uint64_t slot) {
     const uint32_t c = __reduce_add_sync(kFull, acc.changed), e = __reduce_add_sync(kFull, acc.edges),
-                   b = __reduce_add_sync(kFull, acc.boundary);
-    if (lane != 0 || c == 0u) return;
+                   b = __reduce_add_sync(kFull, acc.boundary), r = __reduce_add_sync(kFull, acc.read);
+    if (lane != 0) return;
+    if (r) atomicAdd(&a.stats_out->push_edges, (unsigned long long)r);
+    if (c == 0u) return;
     atomicAdd(&a.stats_out->changed[slot % kStatLanes], (unsigned long long)c);
     if (e) atomicAdd(&a.stats_out->list_ne, (unsigned long long)e);
     if (b) atomicAdd(&a.stats_out->boundary[slot % kStatLanes], (unsigned long long)b);
@@ -121,6 +124,7 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_mark(const LpArgs a) {
         a.changed_next[i] = 0u;
     }
     if (!lp_sparse(a)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.stats_out->pushed = 2ull;
     const uint32_t n_warps = gridDim.x * kLpWarps;
     for (uint32_t w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < words; w += n_warps) {
         const uint32_t bits = __ldg(a.changed_prev + w);
@@ -213,6 +217,7 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_slices(const LpArgs a) {
         if (sparse) {
             want = want && lp_marked(a, row);
             if (!__any_sync(kFull, want)) continue;
+            if (want) acc.read += __ldg(a.col_ptr + row + 1) - __ldg(a.col_ptr + row);
         }
         switch ((sl.width + 3u) / 4u) {
             case 1: lp_slice<kOnePart, 4>(a, P, sl, row, want, lane, acc); break;
@@ -360,7 +365,10 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_warp_rows(const LpArgs a) {
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(kFull, best, o));
-        if (lane == 0) lp_apply(a, r.g, ~(uint32_t)best, acc);
+        if (lane == 0) {
+            lp_apply(a, r.g, ~(uint32_t)best, acc);
+            if (sparse) acc.read += n;
+        }
         __syncwarp();
     }
     }
@@ -436,6 +444,7 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_rows(const LpArgs a) {
             best = block_max<kLpBlock>(best, s_red);
             if (tid == 0) lp_apply(a, r.g, ~(uint32_t)best, acc);
         }
+        if (tid == 0 && sparse) acc.read += n;
         __syncthreads();   // the table and s_red are reused by the next row
     }
     __syncthreads();   // s_want is read
@@ -548,7 +557,10 @@ __global__ void __launch_bounds__(kBigBlock) k_lp_big(const LpArgs a) {
             __syncthreads();
         }
         best = block_max<kBigBlock>(best, s_red);
-        if (tid == 0) lp_apply(a, r.g, ~(uint32_t)best, acc);
+        if (tid == 0) {
+            lp_apply(a, r.g, ~(uint32_t)best, acc);
+            if (sparse) acc.read += n;
+        }
         __syncthreads();   // s_red is reused by the next row
     }
     __syncthreads();   // s_want is read
