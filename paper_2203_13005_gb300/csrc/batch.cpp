@@ -310,7 +310,7 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
         std::string tune_key;
         gxp_tune_record cached{};
         bool from_cache = false;
-        if (!opts.block_edges && opts.tune_cache) {
+        if (!opts.block_edges && opts.tune_cache && E) {
             cudaDeviceProp prop{};
             cuda_check(cudaGetDeviceProperties(&prop, device_), "device properties");
             const double deg = V ? (double)E / (double)V : 0.0;
@@ -319,7 +319,7 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
                        " esize=" + std::to_string(b.esize) + " gpu=" + prop.name;
             from_cache = tune_cache_get(opts.tune_cache, tune_key.c_str(), &cached) && cached.block_edges >= 1.0;
         }
-        if (opts.block_edges) {
+        if (opts.block_edges || E == 0) {   // (without edges there is no block to time)
             block_edges = opts.block_edges;
         } else if (from_cache) {
             r.k1 = cached.k1;
@@ -470,7 +470,7 @@ void Engine::sssp_batch(const uint32_t* sources, uint32_t n_src, uint32_t* dist_
     // (k_msssp_loop, a grid barrier between supersteps, the changed count
     // tested on the device); streamed edges: one superstep (copies and
     // kernels of the pipeline) per launch, the changed count read between
-    bool persistent = !streamed;
+    bool persistent = !streamed && !b.units.empty();   // (without edges there is nothing to launch)
     if (persistent) {
         cuda_check(cudaMemsetAsync(b.d_frontier[1], 0, 4 * words, stream_), "memset");
         cuda_check(cudaMemsetAsync(b.d_loop_changed, 0, 8 * 4, stream_), "memset");

@@ -49,3 +49,22 @@ def test_batch_after_a_reload(gpu, first, streamed):
         _check_batch(c, b, streamed)
         _load(c, gxp.GXP_FMT_COO, *d)
         _check_batch(c, d, streamed)
+
+
+@pytest.mark.parametrize("use_graph", [False, True])
+@pytest.mark.parametrize("streamed,block_edges", [(False, 0), (True, 0), (True, 100)])
+def test_batch_without_edges(gpu, streamed, block_edges, use_graph):
+    """A graph without edges: every source reaches itself alone, in one
+    superstep that changes nothing; the context goes on with a real graph."""
+    none = np.zeros(0, np.uint32)
+    a = _edges(4, 5000)
+    with gxp.Context(0) as c:
+        c.create_graph(N, 1)
+        c.load_coo(none, none, none)
+        dist, rep = c.sssp_batch(SOURCES, streamed=streamed, block_edges=block_edges, use_graph=use_graph)
+        ref = np.full((N, len(SOURCES)), gxp.INF, np.uint32)
+        ref[SOURCES, np.arange(len(SOURCES))] = 0
+        assert np.array_equal(dist, ref)
+        assert rep["supersteps"] == 1
+        _load(c, gxp.GXP_FMT_CSC, *a)
+        _check_batch(c, a, streamed)
