@@ -1162,7 +1162,6 @@ SweepArgs Engine::sweep_args() const {
     SweepArgs a{};
     a.slices = d_slices_;
     a.n_slices = n_slices_;
-    a.cols = sweep_cols_;
     for (int j = 0; j < 5; ++j) a.n_lanes[j] = n_lanes_[j];
     a.n_gt8 = n_gt8_;
     a.n_gt4 = n_gt4_;

@@ -18,7 +18,6 @@ namespace gxp {
 constexpr uint32_t kInf = 0xFFFFFFFFu;
 constexpr int kBlock = 128;          // threads per superstep CTA (4 independent warps)
 constexpr uint32_t kVertexCost = 4;  // merge-path weight of a vertex end when cutting tiles
-constexpr int kMaxTileItems = 3072;  // tile_items + hub_items limit (shared-memory budget)
 constexpr int kStatLanes = 64;       // stat accumulators are spread over lanes to
                                      // avoid same-address atomic serialization
 constexpr int kStatRing = 64;        // superstep stat slots kept on the device
@@ -87,11 +86,6 @@ __host__ __device__ constexpr uint64_t sell_words(uint32_t width, uint32_t cols)
     if (!cols) return 32ull * width;
     const uint32_t l = sweep_lanes(width, cols);
     return 32ull * l * sweep_cols(width, l);
-}
-// element k of row slot r of a slice stored with L lanes per row, c columns per sub-slice
-__host__ __device__ constexpr uint64_t sweep_idx(uint32_t k, uint32_t r, uint32_t lanes, uint32_t c) {
-    const uint32_t rows = 32u / lanes, col = k / lanes, lane = (r % rows) * lanes + k % lanes;
-    return 32ull * c * (r / rows) + 128ull * (col >> 2) + 4ull * lane + (col & 3u);
 }
 constexpr uint32_t kSellWindow = 65536;      // rows sorted by degree within windows of this size
 
@@ -288,7 +282,6 @@ struct SellArgs {
 struct SweepArgs {
     const SellSlice* slices;     // decreasing width
     uint32_t n_slices;
-    uint32_t cols;               // columns per lane the layout aims at (sweep_lanes): 4, 8 or 16
     // slices spread over 32, 16, 8, 4, 2 lanes a row end at n_lanes[0..4];
     // then those wider than 8 columns, 4 and 0
     uint32_t n_lanes[5], n_gt8, n_gt4, n_gt0;

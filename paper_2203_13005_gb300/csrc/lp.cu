@@ -328,49 +328,49 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_warp_rows(const LpArgs a) {
     LpAcc acc;
     // the warp's next 32 rows, w0, w0 + nw, ...: lane j asks whether row j is wanted
     for (uint64_t r0 = w0; r0 < a.n_warp_rows; r0 += 32u * nw) {
-    const uint64_t mine = r0 + (uint64_t)lane * nw;
-    const bool want = mine < a.n_warp_rows && (!sparse || lp_marked(a, __ldg(&a.warp_rows[mine].g)));
-    for (unsigned todo = __ballot_sync(kFull, want); todo; todo &= todo - 1u) {
-        const LpRow r = a.warp_rows[r0 + (uint64_t)(__ffs(todo) - 1) * nw];
-        const LpPart P = a.parts[r.part];
-        const uint32_t n = r.n;
-        uint32_t lg = 1;
-        while ((1u << lg) < 2u * n) ++lg;
-        for (uint32_t i0 = 0; i0 < n; i0 += 32u * kGatherUnroll) {
-            uint32_t sv[kGatherUnroll], lab[kGatherUnroll];
+        const uint64_t mine = r0 + (uint64_t)lane * nw;
+        const bool want = mine < a.n_warp_rows && (!sparse || lp_marked(a, __ldg(&a.warp_rows[mine].g)));
+        for (unsigned todo = __ballot_sync(kFull, want); todo; todo &= todo - 1u) {
+            const LpRow r = a.warp_rows[r0 + (uint64_t)(__ffs(todo) - 1) * nw];
+            const LpPart P = a.parts[r.part];
+            const uint32_t n = r.n;
+            uint32_t lg = 1;
+            while ((1u << lg) < 2u * n) ++lg;
+            for (uint32_t i0 = 0; i0 < n; i0 += 32u * kGatherUnroll) {
+                uint32_t sv[kGatherUnroll], lab[kGatherUnroll];
 #pragma unroll
-            for (int q = 0; q < kGatherUnroll; ++q) {
-                const uint32_t i = i0 + 32u * q + (uint32_t)lane;
-                sv[q] = i < n ? __ldg(P.src + r.e0 + i) : 0u;
+                for (int q = 0; q < kGatherUnroll; ++q) {
+                    const uint32_t i = i0 + 32u * q + (uint32_t)lane;
+                    sv[q] = i < n ? __ldg(P.src + r.e0 + i) : 0u;
+                }
+#pragma unroll
+                for (int q = 0; q < kGatherUnroll; ++q) {
+                    const uint32_t i = i0 + 32u * q + (uint32_t)lane;
+                    lab[q] = i < n ? lp_label(a, P, sv[q]) : 0u;
+                }
+#pragma unroll
+                for (int q = 0; q < kGatherUnroll; ++q)   // (a table of 2n slots never fills)
+                    lp_warp_add(keys, more, lg, lab[q], lab[q] * kLpHash, kAllProbes,
+                                i0 + 32u * q + (uint32_t)lane < n, lane);
+            }
+            __syncwarp();
+            unsigned long long best = 0ull;
+            for (uint32_t i = (uint32_t)lane; i < (1u << lg); i += 32u) {
+                const uint32_t k = keys[i];
+                if (k != kInf) {
+                    best = max(best, mode_key(more[i] + 1u, k));
+                    keys[i] = kInf;
+                    more[i] = 0u;
+                }
             }
 #pragma unroll
-            for (int q = 0; q < kGatherUnroll; ++q) {
-                const uint32_t i = i0 + 32u * q + (uint32_t)lane;
-                lab[q] = i < n ? lp_label(a, P, sv[q]) : 0u;
+            for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(kFull, best, o));
+            if (lane == 0) {
+                lp_apply(a, r.g, ~(uint32_t)best, acc);
+                if (sparse) acc.read += n;
             }
-#pragma unroll
-            for (int q = 0; q < kGatherUnroll; ++q)   // (a table of 2n slots never fills)
-                lp_warp_add(keys, more, lg, lab[q], lab[q] * kLpHash, kAllProbes,
-                            i0 + 32u * q + (uint32_t)lane < n, lane);
+            __syncwarp();
         }
-        __syncwarp();
-        unsigned long long best = 0ull;
-        for (uint32_t i = (uint32_t)lane; i < (1u << lg); i += 32u) {
-            const uint32_t k = keys[i];
-            if (k != kInf) {
-                best = max(best, mode_key(more[i] + 1u, k));
-                keys[i] = kInf;
-                more[i] = 0u;
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(kFull, best, o));
-        if (lane == 0) {
-            lp_apply(a, r.g, ~(uint32_t)best, acc);
-            if (sparse) acc.read += n;
-        }
-        __syncwarp();
-    }
     }
     lp_count(a, acc, lane, w0);
 }
@@ -388,66 +388,66 @@ __global__ void __launch_bounds__(kLpBlock) k_lp_rows(const LpArgs a) {
     bool empty = false;   // the table is set up
     LpAcc acc;
     for (uint64_t c0 = blockIdx.x; c0 < a.n_chunks; c0 += (uint64_t)gridDim.x * kLpBlock) {
-    if (!lp_wanted<kLpBlock>(a, a.chunks, c0, gridDim.x, a.n_chunks, sparse, s_want)) continue;
-    if (!empty) {
-        for (uint32_t i = (uint32_t)tid; i < 2 * kLpChunk; i += kLpBlock) {
-            t_key[i] = kInf;
-            t_more[i] = 0u;
-        }
-        empty = true;
-        __syncthreads();
-    }
-    for (int wd = 0; wd < kLpWarps; ++wd)
-    for (unsigned todo = s_want[wd]; todo; todo &= todo - 1u) {
-        const LpRow r = a.chunks[c0 + (uint64_t)(32 * wd + __ffs(todo) - 1) * gridDim.x];
-        const LpPart P = a.parts[r.part];
-        const uint32_t n = r.n;
-        uint32_t lg = 1;
-        while ((1u << lg) < 2u * n) ++lg;
-        const uint32_t size = 1u << lg;
-        for (uint32_t i0 = 0; i0 < n; i0 += (uint32_t)kLpBlock * kGatherUnroll) {
-            uint32_t sv[kGatherUnroll], lab[kGatherUnroll];
-#pragma unroll
-            for (int q = 0; q < kGatherUnroll; ++q) {
-                const uint32_t i = i0 + (uint32_t)q * kLpBlock + (uint32_t)tid;
-                sv[q] = i < n ? __ldg(P.src + r.e0 + i) : 0u;
-            }
-#pragma unroll
-            for (int q = 0; q < kGatherUnroll; ++q) {
-                const uint32_t i = i0 + (uint32_t)q * kLpBlock + (uint32_t)tid;
-                lab[q] = i < n ? lp_label(a, P, sv[q]) : 0u;
-            }
-#pragma unroll
-            for (int q = 0; q < kGatherUnroll; ++q)
-                lp_warp_add(t_key, t_more, lg, lab[q], lab[q] * kLpHash, kAllProbes,
-                            i0 + (uint32_t)q * kLpBlock + (uint32_t)tid < n, lane);
-        }
-        __syncthreads();
-        // read the counts and empty the table for the next row
-        unsigned long long best = 0ull;
-        for (uint32_t i = (uint32_t)tid; i < size; i += kLpBlock) {
-            const uint32_t k = t_key[i];
-            if (k != kInf) {
-                const uint32_t cnt = t_more[i] + 1u;
-                if (r.hub == kInf) {
-                    best = max(best, mode_key(cnt, k));
-                } else {
-                    const LpHub H = a.hubs[r.hub];
-                    const uint32_t slot = lp_table_add(a.keys + H.table, a.counts + H.table, H.log2_size, k, cnt);
-                    a.seg_used[H.seg0 + slot / kLpSegment] = 1u;   // same value from every writer
-                }
+        if (!lp_wanted<kLpBlock>(a, a.chunks, c0, gridDim.x, a.n_chunks, sparse, s_want)) continue;
+        if (!empty) {
+            for (uint32_t i = (uint32_t)tid; i < 2 * kLpChunk; i += kLpBlock) {
                 t_key[i] = kInf;
                 t_more[i] = 0u;
             }
+            empty = true;
+            __syncthreads();
         }
-        if (r.hub == kInf) {
-            best = block_max<kLpBlock>(best, s_red);
-            if (tid == 0) lp_apply(a, r.g, ~(uint32_t)best, acc);
-        }
-        if (tid == 0 && sparse) acc.read += n;
-        __syncthreads();   // the table and s_red are reused by the next row
-    }
-    __syncthreads();   // s_want is read
+        for (int wd = 0; wd < kLpWarps; ++wd)
+            for (unsigned todo = s_want[wd]; todo; todo &= todo - 1u) {
+                const LpRow r = a.chunks[c0 + (uint64_t)(32 * wd + __ffs(todo) - 1) * gridDim.x];
+                const LpPart P = a.parts[r.part];
+                const uint32_t n = r.n;
+                uint32_t lg = 1;
+                while ((1u << lg) < 2u * n) ++lg;
+                const uint32_t size = 1u << lg;
+                for (uint32_t i0 = 0; i0 < n; i0 += (uint32_t)kLpBlock * kGatherUnroll) {
+                    uint32_t sv[kGatherUnroll], lab[kGatherUnroll];
+#pragma unroll
+                    for (int q = 0; q < kGatherUnroll; ++q) {
+                        const uint32_t i = i0 + (uint32_t)q * kLpBlock + (uint32_t)tid;
+                        sv[q] = i < n ? __ldg(P.src + r.e0 + i) : 0u;
+                    }
+#pragma unroll
+                    for (int q = 0; q < kGatherUnroll; ++q) {
+                        const uint32_t i = i0 + (uint32_t)q * kLpBlock + (uint32_t)tid;
+                        lab[q] = i < n ? lp_label(a, P, sv[q]) : 0u;
+                    }
+#pragma unroll
+                    for (int q = 0; q < kGatherUnroll; ++q)
+                        lp_warp_add(t_key, t_more, lg, lab[q], lab[q] * kLpHash, kAllProbes,
+                                    i0 + (uint32_t)q * kLpBlock + (uint32_t)tid < n, lane);
+                }
+                __syncthreads();
+                // read the counts and empty the table for the next row
+                unsigned long long best = 0ull;
+                for (uint32_t i = (uint32_t)tid; i < size; i += kLpBlock) {
+                    const uint32_t k = t_key[i];
+                    if (k != kInf) {
+                        const uint32_t cnt = t_more[i] + 1u;
+                        if (r.hub == kInf) {
+                            best = max(best, mode_key(cnt, k));
+                        } else {
+                            const LpHub H = a.hubs[r.hub];
+                            const uint32_t slot = lp_table_add(a.keys + H.table, a.counts + H.table, H.log2_size, k, cnt);
+                            a.seg_used[H.seg0 + slot / kLpSegment] = 1u;   // same value from every writer
+                        }
+                        t_key[i] = kInf;
+                        t_more[i] = 0u;
+                    }
+                }
+                if (r.hub == kInf) {
+                    best = block_max<kLpBlock>(best, s_red);
+                    if (tid == 0) lp_apply(a, r.g, ~(uint32_t)best, acc);
+                }
+                if (tid == 0 && sparse) acc.read += n;
+                __syncthreads();   // the table and s_red are reused by the next row
+            }
+        __syncthreads();   // s_want is read
     }
     if (tid < 32) lp_count(a, acc, lane, blockIdx.x);
 }
@@ -483,87 +483,87 @@ __global__ void __launch_bounds__(kBigBlock) k_lp_big(const LpArgs a) {
     bool empty = false;   // the table is set up
     LpAcc acc;
     for (uint64_t c0 = blockIdx.x; c0 < a.n_big; c0 += (uint64_t)gridDim.x * kBigBlock) {
-    if (!lp_wanted<kBigBlock>(a, a.big, c0, gridDim.x, a.n_big, sparse, s_want)) continue;
-    if (!empty) {
-        for (uint32_t i = (uint32_t)tid; i < kBigSlots; i += kBigBlock) {
-            t_key[i] = kInf;
-            t_more[i] = 0u;
-        }
-        empty = true;
-        __syncthreads();
-    }
-    for (int wd = 0; wd < kBigBlock / 32; ++wd)
-    for (unsigned todo = s_want[wd]; todo; todo &= todo - 1u) {
-        const LpRow r = a.big[c0 + (uint64_t)(32 * wd + __ffs(todo) - 1) * gridDim.x];
-        const LpPart P = a.parts[r.part];
-        const uint32_t n = r.n;
-        uint32_t passes = (n + kBigPerPass - 1) / kBigPerPass;
-        uint32_t lg = 12;
-        while (lg < 14u && (1u << lg) < 2u * min(n, kBigPerPass)) ++lg;
-        const uint32_t size = 1u << lg;
-        unsigned long long best = 0ull;
-        uint32_t attempt = 0;
-        for (uint32_t p = 0; p < passes; ++p) {
-            // count the labels of pass p; false: one found no slot. The first
-            // try is compiled apart, without what the others need.
-            auto count = [&](auto first) {
-                constexpr bool kFirst = decltype(first)::value;
-                const uint32_t probes = kFirst || attempt < kBigTries ? kBigProbes : size - 1u;
-                bool ok = true;
-                for (uint32_t i0 = 0; i0 < n; i0 += (uint32_t)kBigBlock * kGatherUnroll) {
-                    uint32_t sv[kGatherUnroll], lab[kGatherUnroll];
-#pragma unroll
-                    for (int q = 0; q < kGatherUnroll; ++q) {
-                        const uint32_t i = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid;
-                        sv[q] = i < n ? __ldg(P.src + r.e0 + i) : 0u;
-                    }
-#pragma unroll
-                    for (int q = 0; q < kGatherUnroll; ++q) {
-                        const uint32_t i = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid;
-                        lab[q] = i < n ? lp_label(a, P, sv[q]) : 0u;
-                    }
-#pragma unroll
-                    for (int q = 0; q < kGatherUnroll; ++q) {
-                        const uint32_t key = kFirst ? lab[q] : lp_rehash(lab[q], attempt);
-                        const bool mine = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid < n && (kFirst || ok) &&
-                                          __umulhi(key * 0x85EBCA6Bu, passes) == p;
-                        ok &= lp_warp_add(t_key, t_more, lg, lab[q], key * kLpHash, probes, mine, lane);
-                    }
-                }
-                return ok;
-            };
-            bool ok = attempt == 0u ? count(std::true_type{}) : count(std::false_type{});
-            if (tid == 0) s_taken = 0u;
-            ok = __syncthreads_and(ok);
-            uint32_t taken = 0;
-            for (uint32_t i = (uint32_t)tid; i < size; i += kBigBlock) {
-                const uint32_t k = t_key[i];
-                if (k != kInf) {
-                    if (ok) best = max(best, mode_key(t_more[i] + 1u, k));
-                    t_key[i] = kInf;
-                    t_more[i] = 0u;
-                    ++taken;
-                }
+        if (!lp_wanted<kBigBlock>(a, a.big, c0, gridDim.x, a.n_big, sparse, s_want)) continue;
+        if (!empty) {
+            for (uint32_t i = (uint32_t)tid; i < kBigSlots; i += kBigBlock) {
+                t_key[i] = kInf;
+                t_more[i] = 0u;
             }
-            if (!ok) {   // again, with other hashes (the same in every thread)
-                taken = __reduce_add_sync(kFull, taken);
-                if (lane == 0) atomicAdd(&s_taken, taken);
-                __syncthreads();
-                if (s_taken > size / 4u * 3u) passes = min(2u * passes, 1u << 30);
-                ++attempt;
-                best = 0ull;
-                p = 0xFFFFFFFFu;   // ++ -> 0
-            }
+            empty = true;
             __syncthreads();
         }
-        best = block_max<kBigBlock>(best, s_red);
-        if (tid == 0) {
-            lp_apply(a, r.g, ~(uint32_t)best, acc);
-            if (sparse) acc.read += n;
-        }
-        __syncthreads();   // s_red is reused by the next row
-    }
-    __syncthreads();   // s_want is read
+        for (int wd = 0; wd < kBigBlock / 32; ++wd)
+            for (unsigned todo = s_want[wd]; todo; todo &= todo - 1u) {
+                const LpRow r = a.big[c0 + (uint64_t)(32 * wd + __ffs(todo) - 1) * gridDim.x];
+                const LpPart P = a.parts[r.part];
+                const uint32_t n = r.n;
+                uint32_t passes = (n + kBigPerPass - 1) / kBigPerPass;
+                uint32_t lg = 12;
+                while (lg < 14u && (1u << lg) < 2u * min(n, kBigPerPass)) ++lg;
+                const uint32_t size = 1u << lg;
+                unsigned long long best = 0ull;
+                uint32_t attempt = 0;
+                for (uint32_t p = 0; p < passes; ++p) {
+                    // count the labels of pass p; false: one found no slot. The first
+                    // try is compiled apart, without what the others need.
+                    auto count = [&](auto first) {
+                        constexpr bool kFirst = decltype(first)::value;
+                        const uint32_t probes = kFirst || attempt < kBigTries ? kBigProbes : size - 1u;
+                        bool ok = true;
+                        for (uint32_t i0 = 0; i0 < n; i0 += (uint32_t)kBigBlock * kGatherUnroll) {
+                            uint32_t sv[kGatherUnroll], lab[kGatherUnroll];
+#pragma unroll
+                            for (int q = 0; q < kGatherUnroll; ++q) {
+                                const uint32_t i = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid;
+                                sv[q] = i < n ? __ldg(P.src + r.e0 + i) : 0u;
+                            }
+#pragma unroll
+                            for (int q = 0; q < kGatherUnroll; ++q) {
+                                const uint32_t i = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid;
+                                lab[q] = i < n ? lp_label(a, P, sv[q]) : 0u;
+                            }
+#pragma unroll
+                            for (int q = 0; q < kGatherUnroll; ++q) {
+                                const uint32_t key = kFirst ? lab[q] : lp_rehash(lab[q], attempt);
+                                const bool mine = i0 + (uint32_t)q * kBigBlock + (uint32_t)tid < n && (kFirst || ok) &&
+                                                  __umulhi(key * 0x85EBCA6Bu, passes) == p;
+                                ok &= lp_warp_add(t_key, t_more, lg, lab[q], key * kLpHash, probes, mine, lane);
+                            }
+                        }
+                        return ok;
+                    };
+                    bool ok = attempt == 0u ? count(std::true_type{}) : count(std::false_type{});
+                    if (tid == 0) s_taken = 0u;
+                    ok = __syncthreads_and(ok);
+                    uint32_t taken = 0;
+                    for (uint32_t i = (uint32_t)tid; i < size; i += kBigBlock) {
+                        const uint32_t k = t_key[i];
+                        if (k != kInf) {
+                            if (ok) best = max(best, mode_key(t_more[i] + 1u, k));
+                            t_key[i] = kInf;
+                            t_more[i] = 0u;
+                            ++taken;
+                        }
+                    }
+                    if (!ok) {   // again, with other hashes (the same in every thread)
+                        taken = __reduce_add_sync(kFull, taken);
+                        if (lane == 0) atomicAdd(&s_taken, taken);
+                        __syncthreads();
+                        if (s_taken > size / 4u * 3u) passes = min(2u * passes, 1u << 30);
+                        ++attempt;
+                        best = 0ull;
+                        p = 0xFFFFFFFFu;   // ++ -> 0
+                    }
+                    __syncthreads();
+                }
+                best = block_max<kBigBlock>(best, s_red);
+                if (tid == 0) {
+                    lp_apply(a, r.g, ~(uint32_t)best, acc);
+                    if (sparse) acc.read += n;
+                }
+                __syncthreads();   // s_red is reused by the next row
+            }
+        __syncthreads();   // s_want is read
     }
     if (tid < 32) lp_count(a, acc, lane, blockIdx.x + 31u);
 }

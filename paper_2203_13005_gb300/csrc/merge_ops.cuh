@@ -1,6 +1,6 @@
 // The algorithm template's operators (Section IV-A1: MSGGen, MSGMerge) and
-// the warp helpers shared by the two superstep kernels (sweep.cu: one
-// partition, sell.cu: several).
+// the warp helpers shared by the superstep kernels (sweep.cu: one partition,
+// sell.cu: several, superstep.cu: a CSC in the caller's memory).
 #pragma once
 
 #include "gxp_internal.hpp"
@@ -51,6 +51,8 @@ template <> struct Ops<Algo::PR> {
 __device__ __forceinline__ uint32_t ld_stream(const uint32_t* p) { return __ldcs(p); }
 __device__ __forceinline__ uint4 ld_stream4(const uint4* p) { return __ldcs(p); }
 
+// acq_rel arrival: orders this thread's earlier writes before the count
+// becomes visible, and makes earlier arrivals' writes visible to the last.
 __device__ __forceinline__ uint32_t arrive_acq_rel(uint32_t* ctr) {
     uint32_t old;
     asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(ctr) : "memory");

@@ -517,7 +517,7 @@ __device__ __forceinline__ void fill_lane_groups(const uint32_t* ssrc, const uin
     for (uint32_t sub = 0; sub < L; ++sub) {
         const int slot = (int)(sub * rows + (uint32_t)lane / L);   // this lane's row
         const uint32_t rb = __shfl_sync(kFull, b, slot), rd = __shfl_sync(kFull, d, slot);
-        const uint64_t at0 = o + 32ull * c * sub + 4u * lane;   // sweep_idx
+        const uint64_t at0 = o + 32ull * c * sub + 4u * lane;
         for (uint32_t g = 0; g < c / 4u; ++g) {
             uint32_t x[4], y[4];
 #pragma unroll

@@ -25,7 +25,8 @@
 // cuts the tiles.
 #include <algorithm>
 
-#include "gxp_internal.hpp"
+#include "grid_sync.cuh"
+#include "merge_ops.cuh"
 
 namespace gxp {
 namespace {
@@ -72,12 +73,6 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
         : "memory");
 }
 
-__device__ __forceinline__ uint64_t global_ns() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
 // Wait for phase `parity` of `bar`, giving up after timeout_ns (and after a
 // fixed iteration cap as a backstop). Returns false on give-up. With
 // `give_up` set (the injected timeout fault) it gives up at once, whether or
@@ -93,45 +88,8 @@ __device__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, uint64_t timeo
     return false;
 }
 
-// acq_rel arrival: orders this thread's earlier writes before the count
-// becomes visible, and makes earlier arrivals' writes visible to the last.
-__device__ __forceinline__ uint32_t arrive_acq_rel(uint32_t* ctr) {
-    uint32_t old;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(ctr) : "memory");
-    return old;
-}
-
-// ------------------------------------------------------ algorithm traits
-
-template <Algo A> struct Traits;
-
-template <> struct Traits<Algo::SSSP> {
-    using T = uint32_t;
-    static constexpr bool kWeighted = true;
-    static constexpr int kUnroll = 8;   // gathers in flight per lane
-    __device__ static T ident() { return kInf; }
-    __device__ static T combine(T a, T b) { return min(a, b); }
-    __device__ static T from_bits(uint32_t x) { return x; }
-    __device__ static uint32_t to_bits(T x) { return x; }
-    // MSGGen: relax; unreachable sources send nothing.
-    __device__ static T gen(uint32_t du, uint32_t w) {
-        if (du == kInf) return kInf;
-        uint32_t s = du + w;
-        if (s < du || s == kInf) s = kInf - 1u;   // saturate below INF
-        return s;
-    }
-};
-
-template <> struct Traits<Algo::CC> {
-    using T = uint32_t;
-    static constexpr bool kWeighted = false;
-    static constexpr int kUnroll = 16;
-    __device__ static T ident() { return kInf; }
-    __device__ static T combine(T a, T b) { return min(a, b); }
-    __device__ static T from_bits(uint32_t x) { return x; }
-    __device__ static uint32_t to_bits(T x) { return x; }
-    __device__ static T gen(uint32_t lu, uint32_t) { return lu; }
-};
+// Gathers in flight per lane.
+template <Algo A> constexpr int kGathers = A == Algo::SSSP ? 8 : 16;
 
 // Merge-path split of a tile: the merged sequence interleaves the tile's
 // edges 0..ne-1 with its vertex ends 0..n_ends-1, vertex end r coming right
@@ -149,13 +107,6 @@ __device__ __forceinline__ void merge_split(uint32_t d, uint32_t n_ends, uint32_
     }
     r = lo;
     j = d - lo;
-}
-
-template <class Tr>
-__device__ __forceinline__ typename Tr::T warp_combine_all(typename Tr::T v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = Tr::combine(v, __shfl_xor_sync(kFull, v, o));
-    return v;
 }
 
 __device__ __forceinline__ uint32_t round4(uint32_t x) { return (x + 3u) & ~3u; }
@@ -178,9 +129,9 @@ __host__ __device__ inline Geometry geometry(Algo a, uint32_t max_items) {
 
 template <Algo A>
 __global__ void __launch_bounds__(kBlock, 8) k_superstep(const SuperstepArgs args) {
-    using Tr = Traits<A>;
-    using T = typename Tr::T;
-    constexpr int kU = Tr::kUnroll;
+    using Op = Ops<A>;
+    using T = typename Op::T;
+    constexpr int kU = kGathers<A>;
 
     extern __shared__ __align__(128) uint32_t smem[];
     __shared__ uint64_t s_bar[kWarps][kStages];
@@ -250,13 +201,13 @@ __global__ void __launch_bounds__(kBlock, 8) k_superstep(const SuperstepArgs arg
             const uint32_t e_lo = d.e0 & ~3u, e_hi = round4(d.e0 + d.ne);
             const uint32_t g_lo = g0 & ~3u, g_hi = round4(g0 + d.nv);
             const uint32_t bc = (c_hi - c_lo) * 4u, be = (e_hi - e_lo) * 4u, bg = (g_hi - g_lo) * 4u;
-            const uint32_t total = bc + be * (Tr::kWeighted ? 2u : 1u) + bg;
+            const uint32_t total = bc + be * (Op::kWeighted ? 2u : 1u) + bg;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive_expect_tx(&s_bar[warp][s], total);
             bulk_g2s(st_col(s), P.col_ptr + c_lo, bc, &s_bar[warp][s]);   // bc >= 16
             if (be) {
                 bulk_g2s(st_src(s), P.src + e_lo, be, &s_bar[warp][s]);
-                if (Tr::kWeighted) bulk_g2s(st_w(s), P.w + e_lo, be, &s_bar[warp][s]);
+                if (Op::kWeighted) bulk_g2s(st_w(s), P.w + e_lo, be, &s_bar[warp][s]);
             }
             if (bg) bulk_g2s(st_vx(s), args.own_cur + g_lo, bg, &s_bar[warp][s]);
         }
@@ -323,7 +274,7 @@ __global__ void __launch_bounds__(kBlock, 8) k_superstep(const SuperstepArgs arg
                 for (int q = 0; q < kU; ++q) {
                     const uint32_t j = jb + (uint32_t)q * 32u + (uint32_t)lane;
                     if (j < ne)
-                        s_msg[j] = Tr::to_bits(valid[q] ? Tr::gen(x[q], Tr::kWeighted ? s_w[j] : 0u) : Tr::ident());
+                        s_msg[j] = Op::to_bits(valid[q] ? Op::gen(x[q], Op::kWeighted ? s_w[j] : 0u) : Op::ident());
                 }
             }
         }
@@ -337,8 +288,8 @@ __global__ void __launch_bounds__(kBlock, 8) k_superstep(const SuperstepArgs arg
         merge_split(d0, n_ends, ne, s_end, e0, r0, j);
         __syncwarp();   // every lane has searched before row values overwrite s_end
         uint32_t r = r0;
-        T acc = Tr::ident();
-        T first = Tr::ident();
+        T acc = Op::ident();
+        T first = Op::ident();
         bool have_first = false;
         for (uint32_t k = 0; k < cnt; ++k) {
             if (r < n_ends && s_end[r] - e0 <= j) {
@@ -346,12 +297,12 @@ __global__ void __launch_bounds__(kBlock, 8) k_superstep(const SuperstepArgs arg
                     first = acc;
                     have_first = true;
                 } else {
-                    s_col[r + 1] = Tr::to_bits(acc);   // no other lane reads slot r+1 any more
+                    s_col[r + 1] = Op::to_bits(acc);   // no other lane reads slot r+1 any more
                 }
-                acc = Tr::ident();
+                acc = Op::ident();
                 ++r;
             } else {
-                acc = Tr::combine(acc, Tr::from_bits(s_msg[j]));
+                acc = Op::combine(acc, Op::from_bits(s_msg[j]));
                 ++j;
             }
         }
@@ -362,14 +313,14 @@ __global__ void __launch_bounds__(kBlock, 8) k_superstep(const SuperstepArgs arg
         for (int off = 1; off < 32; off <<= 1) {
             const uint32_t ku = __shfl_up_sync(kFull, key, off);
             const T vu = __shfl_up_sync(kFull, val, off);
-            if (lane >= off && ku == key) val = Tr::combine(vu, val);
+            if (lane >= off && ku == key) val = Op::combine(vu, val);
         }
         T prev = __shfl_up_sync(kFull, val, 1);
         const uint32_t kprev = __shfl_up_sync(kFull, key, 1);
-        if (lane == 0 || kprev != r0) prev = Tr::ident();
+        if (lane == 0 || kprev != r0) prev = Op::ident();
         const T tail_part = __shfl_sync(kFull, val, 31);   // the open tail row's partial
         __syncwarp();   // the previous lane's last check of slot r0+1 is done
-        if (have_first) s_col[r0 + 1] = Tr::to_bits(Tr::combine(prev, first));
+        if (have_first) s_col[r0 + 1] = Op::to_bits(Op::combine(prev, first));
         __syncwarp();
 
         // ---- MSGApply of row rr (staged old values) with merged message m
@@ -391,7 +342,7 @@ __global__ void __launch_bounds__(kBlock, 8) k_superstep(const SuperstepArgs arg
                 slot = &args.part_head[tix];
                 t0 = tile.hub_t0;
                 vrow = 0u;
-                part = (n_ends > 0u) ? Tr::from_bits(s_col[1]) : tail_part;   // n_ends 0: inside one row
+                part = (n_ends > 0u) ? Op::from_bits(s_col[1]) : tail_part;   // n_ends 0: inside one row
             } else if (pass == 1 && tail_open && !(head_open && nv == 1u)) {
                 slot = &args.part_tail[tix];
                 t0 = tix;
@@ -402,17 +353,17 @@ __global__ void __launch_bounds__(kBlock, 8) k_superstep(const SuperstepArgs arg
             }
             uint32_t np = 0;
             if (lane == 0) {
-                __stcg(slot, Tr::to_bits(part));
+                __stcg(slot, Op::to_bits(part));
                 const uint32_t n = __ldg(&args.tiles[t0].nparts);
                 np = arrive_acq_rel(&args.hub_cnt[t0]) == n - 1u ? n : 0u;
             }
             np = __shfl_sync(kFull, np, 0);
             if (np) {
                 __threadfence();
-                T tot = Tr::ident();
+                T tot = Op::ident();
                 for (uint32_t q = (uint32_t)lane; q < np; q += 32u)
-                    tot = Tr::combine(tot, Tr::from_bits(__ldcg(q == 0u ? &args.part_tail[t0] : &args.part_head[t0 + q])));
-                tot = warp_combine_all<Tr>(tot);
+                    tot = Op::combine(tot, Op::from_bits(__ldcg(q == 0u ? &args.part_tail[t0] : &args.part_head[t0 + q])));
+                tot = warp_all<Op>(tot);
                 if (lane == 0) {
                     args.hub_cnt[t0] = 0u;   // ready for the next superstep
                     if (apply(vrow, tot)) ++n_changed;
@@ -423,7 +374,7 @@ __global__ void __launch_bounds__(kBlock, 8) k_superstep(const SuperstepArgs arg
         // complete rows, lanes on consecutive rows
         for (uint32_t rb = head_open ? 1u : 0u; rb < n_ends; rb += 32u) {
             const uint32_t rr = rb + (uint32_t)lane;
-            const bool ch = rr < n_ends && apply(rr, Tr::from_bits(s_col[rr + 1]));
+            const bool ch = rr < n_ends && apply(rr, Op::from_bits(s_col[rr + 1]));
             const unsigned mask = __ballot_sync(kFull, ch);
             if (lane == 0) n_changed += __popc(mask);
         }

@@ -765,10 +765,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_sweep(const SweepArgs a, const 
                 const uint32_t n = p.n_subs();
                 p.subs(n, deal(n), n_warps);
             }
-            constexpr int kN8 = kU >= 16 ? kU / 8 : 1, kN4 = kU / 4;
+            constexpr int kN4 = kU / 4;
             if constexpr (kU >= 8)
-                p.template groups<kN8>(a.n_gt8, a.n_gt4, deal((a.n_gt4 - a.n_gt8 + kN8 - 1) / kN8), n_warps,
-                                       [&](uint32_t wd, uint32_t n) { p.template narrow<kN8>(wd, n); });
+                p.template groups<1>(a.n_gt8, a.n_gt4, deal(a.n_gt4 - a.n_gt8), n_warps,
+                                     [&](uint32_t wd, uint32_t n) { p.template narrow<1>(wd, n); });
             p.template groups<kN4>(a.n_gt4, a.n_gt0, deal((a.n_gt0 - a.n_gt4 + kN4 - 1) / kN4), n_warps,
                                    [&](uint32_t wd, uint32_t n) { p.template narrow<kN4>(wd, n); });
         }
@@ -868,7 +868,6 @@ cudaError_t launch_sweep(Algo alg, const SweepArgs& args, const RunArgs& run, ui
         at = end;
     }
     if (args.n_hot > kMaxHot || args.n_hot % 4 || sms == 0) return cudaErrorInvalidValue;
-    if (args.cols != 4 && args.cols != 8 && args.cols != 16) return cudaErrorInvalidValue;
     if (run.bar && (run.limit <= run.t0 || run.limit - run.t0 > kRunChunk || !run.out)) return cudaErrorInvalidValue;
     // A CTA for every kWarps items at least: on a small graph the barriers of
     // fewer CTAs cost less than a warp's second item. Runs of many supersteps
