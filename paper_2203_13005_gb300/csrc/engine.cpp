@@ -519,10 +519,7 @@ void Engine::build_sell() {
             T = std::max<uint32_t>(512, T);
         }
     }
-    // One partition: columns a lane gathers per work item (sweep_lanes). 16
-    // fill a batch; a small graph takes fewer, so that its items still cover
-    // the chip's ~4,900 resident warps.
-    sweep_cols_ = n_parts_ > 1 ? 0u : total_edges_ >= (1ull << 23) ? 16u : total_edges_ >= (1ull << 21) ? 8u : 4u;
+    sweep_cols_ = n_parts_ > 1 ? 0u : kSweepCols;
     if (n_parts_ == 1 && relabeled_ && H <= kOrderExact) {
         build_sell_sorted(H, T);
         return;

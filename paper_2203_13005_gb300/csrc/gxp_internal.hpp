@@ -72,7 +72,12 @@ constexpr uint32_t kSellPad = 0xFFFFFFFFu;   // empty row slot of a slice (perm)
 // two (at most 32) that brings its columns down to `cols`: the slice is L
 // sub-slices of 32 / L rows, edge k of a row in lane k % L of its lane group
 // and column k / L, and columns are stored in groups of 4, so that a lane
-// reads 4 of its sources with one 128-bit load.
+// reads 4 of its sources with one 128-bit load. kSweepCols: fewer columns, so
+// more items and lanes, pad more and measured no faster at any size (R-MAT and
+// uniform graphs of 2^19 to 2^24 edges at 4 / 8 / 16, us a run: PageRank R-MAT
+// 2^20 edges 263 / 242 / 235, 2^22 468 / 409 / 389, 2^24 1,135 / 946 / 865; SSSP
+// 179 / 174 / 167, 238 / 228 / 220, 520 / 492 / 462).
+constexpr uint32_t kSweepCols = 16;
 __host__ __device__ constexpr uint32_t sweep_lanes(uint32_t width, uint32_t cols) {
     uint32_t l = 1;
     while (l < 32u && width > cols * l) l *= 2;
