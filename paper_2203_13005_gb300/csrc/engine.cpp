@@ -4,6 +4,8 @@
 #include "engine.hpp"
 #include "trace.hpp"
 
+#include <cuda.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -225,6 +227,25 @@ void Engine::check_device_error() {
     if (err & kErrTimeout) fail(GXP_E_TIMEOUT, "a device-side wait exceeded timeout_ns");
     if (err & kErrBounds) fail(GXP_E_BOUNDS, "a device-side bounds check failed");
     if (err & kErrInput) fail(GXP_E_BOUNDS, "a device-side check found CSC offsets out of order");
+}
+
+// Bytes from p to the end of its device allocation; 0 if the driver doesn't say.
+static size_t allocation_room(const void* p) {
+    using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const Range range = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found{};
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess)
+            fn = nullptr;
+        cudaGetLastError();
+        return reinterpret_cast<Range>(fn);
+    }();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    if (!range || range(&base, &size, at) != CUDA_SUCCESS || at < base || at >= base + size) return 0;
+    return base + size - at;
 }
 
 // ------------------------------------------------------------------ graph
@@ -1848,9 +1869,14 @@ void Engine::get_values(uint32_t part, void* out, uint64_t n) {
     const void* src = algo_ == Algo::PR ? (const void*)(d_rank_[cur_] + off) : (const void*)(d_own_[cur_] + off);
     if (relabeled_) {   // internal order -> input ids, straight into the caller's array if it is this device's
         cudaPointerAttributes at{};
-        const bool direct = cudaPointerGetAttributes(&at, out) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
-                            at.device == device_ && ((uintptr_t)out & 3u) == 0;
+        bool direct = cudaPointerGetAttributes(&at, out) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
+                      at.device == device_ && ((uintptr_t)out & 3u) == 0;
         if (!direct) cudaGetLastError();
+        if (direct) {   // (a copy into it would be checked, a kernel's stores are not)
+            const size_t room = allocation_room(out);
+            if (room == 0) direct = false;
+            else if (room < 4 * cnt) fail(GXP_E_INVAL, "output array ends before n values");
+        }
         uint32_t* to = direct ? (uint32_t*)out : d_perm_tmp_;
         cuda_check(launch_permute_u32((const uint32_t*)src, d_old2new_, (uint32_t)cnt, to, false, stream_), "map values");
         src = to;
