@@ -371,7 +371,7 @@ def run_sssp(args):
         "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": "u32", "data": "synthetic",
         "config": {"workload": wl.name, "vertices": n, "edges": m, "source": 0, "supersteps": steps,
-                   "step": (f"one gxp_run to convergence: {st['persistent_launches']} persistent cooperative "
+                   "step": (f"one gxp_run to convergence: {st['persistent_launches']} persistent "
                             "launch(es), grid barrier between supersteps"),
                    "value": "supersteps x edges / run time (the Jacobi sweeps the run stands for)",
                    "l2": (f"{bytes_sweep / 1e6:.0f} MB working set: "
@@ -387,9 +387,8 @@ def run_sssp(args):
                      "algorithmic_bytes_per_launch": bytes_sweep},
         "e2e": {"value": steps * m / e2e_s / 1e9, "unit": "GTEPS", "h2d_bytes_per_step": 8 * (n + 1) + 8 * m,
                 "d2h_bytes_per_step": 4 * n, "ms_per_step": e2e_s * 1e3},
-        # per run: initial values, identity slot and frontier seed, then the
-        # persistent kernel's launches
-        "gpu_launches": reps * (3 + st["persistent_launches"]),
+        # per run: the initial state, then the persistent kernel's launches
+        "gpu_launches": reps * (1 + st["persistent_launches"]),
         "clocks": clk.summary(),
     }
     line.update(cpu)
@@ -1060,8 +1059,8 @@ def main():
             "e2e": {"value": ITERS * m / e2e_s / 1e9, "unit": "GTEPS",
                     "h2d_bytes_per_step": 8 * (n + 1) + 4 * m, "d2h_bytes_per_step": 4 * n,
                     "ms_per_step": e2e_s * 1e3},
-            # per step: initial values, the identity slots, 20 supersteps
-            "gpu_launches": args.steps * (ITERS + 2),
+            # per step: the initial state, 20 supersteps
+            "gpu_launches": args.steps * (ITERS + 1),
             "clocks": clk.summary(),
         }
         if base is not None:

@@ -252,6 +252,10 @@ GXP_API gxp_status gxp_create_graph(gxp_ctx* ctx, uint64_t n_vertices, uint32_t 
  * of the edge list for COO). The engine builds its dst-sorted edge blocks and
  * the vertex-edge mapping table from it (Section II-B: fixed-size edge blocks
  * paired with vertex blocks). Ownership of the arrays stays with the caller.
+ * fp32 PageRank sums a vertex's in-edges in an order that follows the order in
+ * which they are loaded (one partition, unless keep_ids) or their source ids: the
+ * same arrays give the same bits, the same edges in another order may differ
+ * in rounding. Integer values don't depend on it.
  * Errors: GXP_E_INVAL for an out-of-range id, a destination outside the
  * partition, a non-monotone offset array, or more than 2^32-1 edges. */
 GXP_API gxp_status gxp_load_partition(gxp_ctx* ctx, uint32_t part, gxp_format fmt,

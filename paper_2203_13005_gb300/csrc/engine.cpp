@@ -514,15 +514,14 @@ uint32_t* Engine::upload_u32(const std::vector<uint32_t>& h, size_t n_pad) {
     return d;
 }
 
-// Sliced-ELL layout of the rows with at most H in-edges (SELL-32-sigma: rows
-// sorted by in-degree within windows of kSellWindow rows, grouped in 32-row
-// slices stored column-major, each row's in-edges in ascending source order)
-// and hub parts of T edges for the rows with more. Built on first use by a
-// superstep (the batched path does not need it).
-// Sliced-ELL layout of every partition, built on the device (sell_build.cu):
-// rows sorted by source, windows sorted by in-degree, slices filled, hub rows
-// split into parts; then all slices ordered heavy-first. A few small counts
-// come back to the host to size the arrays.
+// Sliced-ELL layout of the rows with at most H in-edges, and hub parts of T
+// edges for the rows with more, of every partition, built on the device
+// (sell_build.cu) on first use by a superstep (the batched path does not need
+// it): rows sorted by source, windows of kSellWindow rows sorted by in-degree,
+// 32-row slices filled, hub rows split into parts; then all slices ordered
+// heavy-first. A few small counts come back to the host to size the arrays. A
+// renumbered partition's rows are in order of in-degree as they stand and keep
+// the order of their in-edges as loaded (build_sell_sorted).
 void Engine::build_sell() {
     TraceRange trace_("gxp layout build");
     uint32_t T = cfg_.tile_items, H = cfg_.hub_items;
@@ -1769,8 +1768,8 @@ uint32_t Engine::run(gxp_algo algo, uint32_t source, float damping, uint32_t max
     // SSSP, CC and PageRank on one partition: at most kRunChunk supersteps per
     // persistent launch (a grid barrier between supersteps) and one host read
     // per launch. Its barriers are device waits: a context whose timeout_ns
-    // is below kBarrierTimeoutNs takes a launch per superstep, which waits for
-    // no other CTA, and so does a run whose CTAs did not all get onto the
+    // is below kBarrierTimeoutNs takes a launch per superstep, no CTA of which
+    // waits for one that has yet to start, and so does a run whose CTAs did not all get onto the
     // device (other work holds an SM).
     bool resident = n_parts_ == 1 && algo_ != Algo::LP && cfg_.timeout_ns >= kBarrierTimeoutNs;
     const SweepArgs sa = resident ? sweep_args() : SweepArgs{};

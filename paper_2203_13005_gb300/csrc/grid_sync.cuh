@@ -1,5 +1,6 @@
-// Grid-wide barrier of a cooperative launch, with a bounded wait: used by
-// the persistent superstep loops (sell.cu, msssp.cu).
+// Grid-wide barrier with a bounded wait, of launches all of whose CTAs are on
+// the device: a cooperative one (msssp.cu), or one whose CTAs have met at it
+// before anything was done (sweep.cu).
 #pragma once
 
 #include "gxp_internal.hpp"

@@ -1,6 +1,7 @@
 // Supersteps of a single-partition graph (SSSP, CC, PageRank, personalized
 // PageRank): MSGGen + MSGMerge + MSGApply over the sliced-ELL layout in one
-// persistent CTA per SM, one superstep or many per launch.
+// persistent CTA per SM (fewer for small graphs), one superstep or many per
+// launch.
 //
 // What bounds it: the gathers of the sources' values. On a power-law graph a
 // warp's 32 gathers touch ~30 different sectors, so large graphs run at the
@@ -11,9 +12,9 @@
 //    (2.7 us) in place of a launch, and no prologue and epilogue per 8 work
 //    items;
 //  * work items of one size: a row of up to 512 in-edges is spread over as
-//    many lanes (1 .. 32) as bring it down to `cols` columns (sweep_lanes),
-//    so an item is one batch of gathers for most rows, and items are dealt
-//    out evenly with neither a queue nor a long item to wait for. With whole
+//    many lanes (1 .. 32) as bring it down to 16 columns (sweep_lanes), so
+//    an item is at most two batches of gathers (four for SSSP), and items are
+//    dealt out evenly with neither a queue nor a long item to wait for. With whole
 //    rows per lane, up to 1,024 columns, the longest slice alone took as long
 //    as the superstep should;
 //  * a warp's loads run ahead: the next item's descriptor, then its sources,
@@ -30,7 +31,7 @@
 // Per superstep, launch gaps included, before (a launch per superstep, one
 // warp per slice, 8 warps a CTA) and after: PageRank R-MAT 22 187 -> 153 us,
 // 1 M vertices and 16.8 M edges 73 -> 42 us, 200 K vertices and 3.2 M edges
-// 31 -> 19 us; a whole SSSP run of R-MAT 22 1,635 -> 1,119 us.
+// 31 -> 17 us; a whole SSSP run of R-MAT 22 1,635 -> 1,119 us.
 //
 // Work items, in order: for PageRank groups of slices of rows without
 // in-edges (the min-label algorithms leave such rows alone: both value
@@ -65,9 +66,10 @@ constexpr int kZeroGroup = 4;      // slices of rows without in-edges per item
 // were a launch per superstep); beside a busy query server 0.43 .. 0.56 ms
 // with each of the limits. Alone, all of 3,000 runs met; meeting costs 1.6 us.
 constexpr uint64_t kGatherNs = 50000;
-constexpr uint32_t kMaxHot = 32768;     // staged values: 208 KB of the 227 KB a CTA may have
+constexpr uint32_t kMaxHot = 32768;     // staged values: 128 KB, the rest of an SM's 256 KB is L1
 
-// Columns (gathers) in flight per lane. More of them spill registers and run
+// Columns (gathers) in flight per lane. Of 64 registers a thread these spill
+// 80 bytes (PageRank), 112 (CC) and 36 (SSSP); more of them spill more and run
 // slower: PageRank on R-MAT 22 at 16, 12 and 8 took 207, 179 and 163 us a
 // superstep, SSSP at 8 and 4 together 1,002 and 933 us a run.
 template <Algo A> constexpr int kCols = A == Algo::SSSP ? 4 : 8;
