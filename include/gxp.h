@@ -278,7 +278,9 @@ GXP_API gxp_status gxp_begin(gxp_ctx* ctx, gxp_algo algo, uint32_t source, float
 
 /* Copy the current values of the vertices owned by `part` (in local order,
  * n = owned count) to `out`: uint32 for SSSP/CC/LP, fp32 ranks for PageRank.
- * part = UINT32_MAX copies all partitions in global id order (n = n_vertices). */
+ * part = UINT32_MAX copies all partitions in global id order (n = n_vertices).
+ * Errors: GXP_E_INVAL (n differs, null, a device array whose allocation ends
+ * before n values), GXP_E_STATE (before gxp_begin). */
 GXP_API gxp_status gxp_get_values(gxp_ctx* ctx, uint32_t part, void* out, uint64_t n);
 
 /* Overwrite the current values (same layout as gxp_get_values) and mark every
